@@ -180,9 +180,9 @@ signtri_status signtri_set_verification(int full);
 
 /* Leaf (recursion cutoff) size b of the float64 Parlett-Higham forms: the
    order of the diagonal and off-diagonal blocks solved element by element
-   (Section 6 uses 16).  b in {16, 32, 64}, or 0 (the default): by size, the
-   fastest measured on GB300 -- the efficient form 16 below n = 4096, 32
-   below 8192, then 64; the matrix-multiply form 16 up to n = 4096, then 32.
+   (Section 6 uses 16).  b in {16, 32, 64}, or 0 (the default): 16, the
+   fastest measured on GB300 at every size; 32 and 64 run separate block-sum
+   and leaf launches and are kept for comparison.
    The mixed variants' tensor-core tiles are 64 whatever b.  signtri_info
    reports the b a call used.  Process-wide setting. */
 signtri_status signtri_set_cutoff(int b);
@@ -225,7 +225,7 @@ signtri_status sign_tri_batched(int count, const int *n, const double *const *T,
                                 void *stream);
 
 /* Leaf-size table of the batched path: b[k] (16, 32, 64, or 0 = the
-   process-wide cutoff, by size when that is 0) for problems with
+   process-wide cutoff, 16 when that is 0) for problems with
    floor(log2 n) == k, k < len <= 32. */
 signtri_status signtri_set_cutoff_table(const int *b, int len);
 signtri_status signtri_get_cutoff_table(int *b, int len);

@@ -37,7 +37,7 @@ struct DeviceState {
 
 std::mutex g_mu;
 DeviceState g_dev[kMaxDevices];
-// 0: by size (default_cutoff); else the leaf size set by signtri_set_cutoff
+// 0: kDefaultCutoff; else the leaf size set by signtri_set_cutoff
 int g_cutoff = 0;
 // leaf size per size bucket floor(log2 n) for the batched path; 0 = g_cutoff
 int g_cutoff_table[32] = {};
@@ -126,28 +126,24 @@ signtri_status get_workspace(DeviceState &s, size_t need, Arena &a)
     return SIGNTRI_OK;
 }
 
-// swaps < 0: the worst case over inertia (n^2/4 swaps).
-// Leaf size of the float64 forms when none is set: measured on GB300 (p = 0.5
-// random), the fastest of 16, 32, 64 per size -- small leaves while the leaf
-// latency dominates, larger ones once the block sums do: the efficient form
-// 16 below n = 4096, 32 below 8192, then 64; the matrix-multiply form 16 up
-// to 4096, then 32.
-int default_cutoff(int n, signtri_variant v)
-{
-    if (v == SIGNTRI_PH_FP64_EFFICIENT || v == SIGNTRI_AUTO) return n < 4096 ? 16 : (n < 8192 ? 32 : 64);
-    return n <= 4096 ? 16 : 32;
-}
+// Leaf size of the float64 forms when none is set.  16 runs one launch per
+// anti-diagonal (ph_level.cuh) and is the fastest measured on GB300 at every
+// size: the efficient form takes 0.22 / 1.0 / 5.0 / 32 / 262 ms at n = 256 /
+// 1001 / 2000 / 4000 / 8192 with leaves of 16, against 1.2 / 5.6 / 14.5 / 51 /
+// 312 ms with 32 and 2.0 / 8.6 / 22 / 65 / 309 ms with 64 (p = 0.3 random).
+constexpr int kDefaultCutoff = 16;
 
 // the leaf size a float64 form runs with (callers hold g_mu)
-int cutoff_of(int n, signtri_variant v)
+int current_cutoff_locked()
 {
-    return g_cutoff ? g_cutoff : default_cutoff(n, v);
+    return g_cutoff ? g_cutoff : kDefaultCutoff;
 }
 
+// swaps < 0: the worst case over inertia (n^2/4 swaps).
 size_t workspace_need(int n, signtri_variant v, long long swaps)
 {
     if (swaps < 0) swaps = (long long)n * n / 4;
-    const int cutoff = cutoff_of(n, v == SIGNTRI_PH_FP64_EFFICIENT || v == SIGNTRI_AUTO ? v : SIGNTRI_PH_FP64);
+    const int cutoff = current_cutoff_locked();
     switch (v) {
     case SIGNTRI_PH_FP64:
         return ph_fp64_workspace_bytes(n, cutoff);
@@ -224,7 +220,7 @@ double window_launch_seconds(double kw)
 signtri_variant choose_variant(int n, const ScanResult &r)
 {
     const double nd = n;
-    const int b = cutoff_of(n, SIGNTRI_PH_FP64_EFFICIENT);
+    const int b = current_cutoff_locked();
     const double nb = std::ceil(nd / b);
     double w_ph = 0.0, w_ps = 0.0;
     work_estimates(n, r, &w_ph, &w_ps);
@@ -251,7 +247,7 @@ signtri_status run_variant(int n, const double *T, int ldt, double *U, int ldu, 
                            const ScanResult &r, cudaStream_t st, DeviceState &s)
 {
     Arena ws;
-    const int b = cutoff_of(n, v == SIGNTRI_PH_FP64_EFFICIENT ? v : SIGNTRI_PH_FP64);
+    const int b = current_cutoff_locked();
     signtri_status rs = get_workspace(s, workspace_need(n, v, r.swaps), ws);
     if (rs != SIGNTRI_OK) return rs;
     switch (v) {
@@ -353,7 +349,7 @@ int size_bucket(int n)
 int cutoff_for(int n)
 {
     const int k = size_bucket(n);
-    return g_cutoff_table[k] ? g_cutoff_table[k] : cutoff_of(n, SIGNTRI_PH_FP64_EFFICIENT);
+    return g_cutoff_table[k] ? g_cutoff_table[k] : current_cutoff_locked();
 }
 
 // Synthetic upper-triangular T for the autotuner: counter-based hash
@@ -384,10 +380,10 @@ __global__ void synth_kernel(int n, double *T, unsigned long long seed)
 
 }  // namespace
 
-int signtri::current_cutoff(int n)
+int signtri::current_cutoff()
 {
     std::lock_guard<std::mutex> lk(g_mu);
-    return cutoff_of(n, SIGNTRI_PH_FP64);
+    return current_cutoff_locked();
 }
 
 extern "C" {
@@ -933,7 +929,7 @@ signtri_status signtri_funm(int n, const double *T, int ldt, double *F, int ldf,
     DeviceState *s = nullptr;
     signtri_status rs = current_state(&s);
     if (rs != SIGNTRI_OK) return rs;
-    const int b = cutoff_of(n, SIGNTRI_PH_FP64);
+    const int b = current_cutoff_locked();
     Arena ws;
     rs = get_workspace(*s, funm_workspace_bytes(n, b), ws);
     if (rs != SIGNTRI_OK) return rs;

@@ -112,7 +112,7 @@ template <int B>
 signtri_status funm_b(int n, const double *T, int ldt, double *F, int ldf, int phi, Arena &ws, cudaStream_t st)
 {
     const int nb = (n + B - 1) / B;
-    const size_t slabs = max_slabs(n, B);
+    const size_t slabs = B == 16 ? 0 : max_slabs(n, B);
     double *PX = nullptr, *PY = nullptr;
     if (slabs > 0) {
         PX = static_cast<double *>(ws.take(slabs * B * B * sizeof(double)));
@@ -130,6 +130,7 @@ signtri_status funm_b(int n, const double *T, int ldt, double *F, int ldf, int p
         funm_diag_leaf_kernel<B><<<nb, kThreads, diag_smem<B>(), st>>>(n, T, ldt, F, ldf, phi);
         SGT_LAUNCH_CHECK();
     }
+    if (B == 16) return levels_f64(n, T, ldt, F, ldf, true, ws, st);
     for (int d = 1; d < nb; d++) {
         const int ntiles = nb - d;
         const long long W = (long long)ntiles * sk_chunks_per_tile(d, B);

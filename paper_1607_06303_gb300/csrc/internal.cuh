@@ -118,12 +118,17 @@ signtri_status launch_fill_batched(int count, const BatchDesc *d_mats, const int
                                    cudaStream_t st);
 signtri_status launch_zero_strict_lower(int n, double *U, int ldu, cudaStream_t st);
 
-// Leaf size the float64 matrix-multiply form runs with at order n (api.cu).
-int current_cutoff(int n);
+// Leaf size the float64 forms run with (api.cu).
+int current_cutoff();
 
 // Recursive Parlett-Higham, float64 (ph_fp64.cu)
 size_t ph_fp64_workspace_bytes(int n, int b);
 signtri_status diag_leaves_f64(int n, const double *T, int ldt, double *U, int ldu, int b, cudaStream_t st);
+// every off-diagonal block of U in blocks of 16, the diagonal blocks being
+// solved; general: U = phi(T), every entry from TU = UT.  Workspace:
+// ph_fp64_workspace_bytes(n, 16)
+signtri_status levels_f64(int n, const double *T, int ldt, double *U, int ldu, bool general, Arena &ws,
+                          cudaStream_t st);
 signtri_status ph_fp64_run(int n, const double *T, int ldt, double *U, int ldu, int b,
                            Arena &ws, cudaStream_t st);
 // arithmetic-efficient form (one sum per entry)

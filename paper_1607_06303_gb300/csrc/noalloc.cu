@@ -12,6 +12,7 @@
 
 #include "internal.cuh"
 #include "ph_bodies.cuh"
+#include "ph_level.cuh"
 
 namespace signtri {
 
@@ -21,20 +22,21 @@ constexpr int kNoallocMaxN = 1024;
 // The first 256 bytes hold the scan result; the rest is the float64 path's
 // block-sum slabs.  Their size grows with n, so n = 1024 bounds every smaller
 // problem; at n = 1024 the cutoffs need 15.7 MB (b = 64: 240 slabs of 64 x 64
-// doubles per set), 8.4 MB (b = 32: 512 slabs) and 2.8 MB (b = 16: 672), two
-// sets each.  The array is sized from that bound, checked at compile time.
+// doubles per set) and 8.4 MB (b = 32: 512 slabs), two sets each, and 0.9 MB
+// (b = 16, ph_level.cuh: its slabs depend little on n).  The array is sized
+// from that bound, checked at compile time.
 constexpr size_t kScanSlot = 256;
 constexpr size_t noalloc_need()
 {
     size_t m = 0;
-    for (int b = 16; b <= 64; b *= 2)
+    for (int b = 32; b <= 64; b *= 2)
         if (ph::mm_form_workspace_bytes(kNoallocMaxN, b) > m) m = ph::mm_form_workspace_bytes(kNoallocMaxN, b);
     return m;
 }
 constexpr size_t kNoallocBytes = ((kScanSlot + noalloc_need() + 4095) / 4096) * 4096;
 static_assert(ph::mm_form_workspace_bytes(kNoallocMaxN, 64) <= kNoallocBytes - kScanSlot, "b = 64 at the maximum n");
 static_assert(ph::mm_form_workspace_bytes(kNoallocMaxN, 32) <= kNoallocBytes - kScanSlot, "b = 32 at the maximum n");
-static_assert(ph::mm_form_workspace_bytes(kNoallocMaxN, 16) <= kNoallocBytes - kScanSlot, "b = 16 at the maximum n");
+static_assert(lvl::level_workspace_bytes(kNoallocMaxN) <= kNoallocBytes - kScanSlot, "b = 16 at the maximum n");
 static_assert(kNoallocBytes <= ((size_t)16 << 20), "the array stays modest");
 
 __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocBytes];
@@ -70,7 +72,7 @@ extern "C" signtri_status sign_tri_noalloc(int n, const double *T, int ldt, doub
         if (e != cudaSuccess || p == nullptr) return SIGNTRI_ERR_CUDA;
         na_base[dev] = static_cast<char *>(p);
     }
-    const int b = current_cutoff(n);
+    const int b = current_cutoff();
     Arena ws;
     ws.base = na_base[dev] + kScanSlot;
     ws.bytes = kNoallocBytes - kScanSlot;

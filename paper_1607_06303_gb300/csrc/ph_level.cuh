@@ -1,0 +1,400 @@
+// ph_level.cuh -- one launch per block anti-diagonal: the float64
+// Parlett-Higham leaves of blocks of 16 and, beside them in the same launch,
+// the block sums of the next anti-diagonal.  Used by the single-matrix
+// (ph_fp64.cu), batched (batched.cu) and general-phi (funm.cu) paths.
+//
+// Entry (p, q) of block (I, J), J = I + d, is fixed by (Algorithm 6, 1x1 case)
+//   signs differ: (t_pp - t_qq) v_pq = t_pq (u_pp - u_qq) + sum_k (u_pk t_kq - t_pk u_kq)
+//   signs agree:  (u_pp + u_qq) v_pq = - sum_k u_pk u_kq
+// with k running over every index strictly between p and q.  Only the terms
+//   - m_pk u_kq  for k in block I + 1     (u_kq: anti-diagonal d - 1)
+//   + u_pk n_kq  for k in block J - 1     (u_pk: anti-diagonal d - 1)
+// and those inside blocks I and J that hold v itself need the anti-diagonal
+// just before; all others ("early" terms) need d - 2 or less, or the diagonal
+// blocks.  (m = t, n = t where the signs differ; m = u, n = -u where they
+// agree.)  So launch d runs two kinds of CTAs that do not depend on each
+// other:
+//   leaf CTAs, one per block of anti-diagonal d: add the early sums (partial
+//     slabs of launch d - 1), the two near blocks, and solve the block;
+//   far CTAs: the early sums of anti-diagonal d + 1.
+// One launch per anti-diagonal instead of two, and the block sums hide behind
+// the leaves, which bound small problems: a leaf is a chain of 31 dependent
+// steps of float64 arithmetic, whose pipe takes one warp instruction per 64
+// cycles and sub-partition on GB300.  Launches are programmatic dependents:
+// a leaf loads its operands and forms its reciprocals before it waits for the
+// launch before it.
+//
+// Inside a leaf one thread owns one entry.  A solved entry is pushed at once
+// into the later entries that need it (one multiply-add for the row, one for
+// the column), so a step's critical path is a product, a barrier and two
+// multiply-adds, whatever the length of the entry's sum; threads are numbered
+// along the block's anti-diagonals, so whole warps fall idle as the solve
+// proceeds and leave the float64 pipe to the others.
+#pragma once
+
+#include "internal.cuh"
+#include "level_split.h"
+#include "ph_bodies.cuh"
+
+namespace signtri {
+namespace lvl {
+
+constexpr int LT = LB * LB;     // threads of a leaf, and of each half of a far CTA: one per entry
+constexpr int kLevelThreads = 2 * LT;
+constexpr int LD = LB + 1;      // shared-memory pitch of a block
+constexpr int BLK = LB * LD;    // doubles per staged block
+
+// Wait for the launch this one programmatically depends on (all of it, with
+// its writes visible); let the next launch start its independent part.
+__device__ __forceinline__ void dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void dependency_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// barrier of one half of a CTA
+__device__ __forceinline__ void half_sync(int half)
+{
+    asm volatile("bar.sync %0, %1;" ::"r"(half + 1), "n"(LT) : "memory");
+}
+
+// the position of set bit number r of a 16-bit mask
+__device__ __forceinline__ int nth_bit(unsigned mask, int r)
+{
+    for (int i = 0; i < r; i++) mask &= mask - 1;
+    return __ffs(mask) - 1;
+}
+
+union alignas(16) Smem {
+    struct {
+        double AU[2][LB * LB], AT[2][LB * LB];   // [buffer][k * 16 + row]
+        double BU[2][BLK], BT[2][BLK];           // [buffer][column * 17 + k]
+    } far[2];                                    // per half of the CTA
+    struct {
+        double TI[BLK], UI[BLK], TJ[BLK], UJ[BLK];       // diagonal blocks, [row + column * 17]
+        double T1[BLK], U1[BLK], T2[BLK], U2[BLK];       // blocks (I, I+1) and (J-1, J)
+        double X1[BLK], X2[BLK];                         // U of blocks (I+1, J) and (I, J-1)
+        double C[BLK], V[BLK];
+        double urow[LB], ucol[LB];
+    } leaf;
+};
+
+// Shared memory a CTA of a launch of G asks for: an SM's, divided by the CTAs
+// an SM gets, so that they spread evenly (left to itself the scheduler puts
+// 152 CTAs on 123 SMs, and a leaf that shares its SM takes twice as long).
+// Small launches ask for less, so that they start beside the one before and
+// have their operands loaded when it ends.
+constexpr int kSmallLaunch = 64;
+constexpr int level_smem(int G)
+{
+    const int per = (G + kSms - 1) / kSms;
+    const int b = (227 - per) / per * 1024;
+    return G > kSmallLaunch && b > (int)sizeof(Smem) ? b : (int)sizeof(Smem);
+}
+constexpr size_t level_workspace_bytes(int n)
+{
+    return level_slabs(n) == 0 ? 0 : 2 * (level_slabs(n) * LT * sizeof(double) + 256);
+}
+
+// Early sums of tile (I, J) over the K-blocks [kb0, kb1) of I .. J, written to
+// slab (entry (p, q) at p + 16 q): where the signs differ
+//   sum u_pk t_kq over K = I (k > p) and I < K <= J - 2, minus
+//   sum t_pk u_kq over I + 2 <= K < J and K = J (k < q);
+// where they agree sum u_pk u_kq over I + 2 <= K <= J - 2.  general: every
+// entry takes the first form.  Entries are dealt to threads by kind (rows and
+// columns gathered by sign), so a warp issues one multiply-add a term or two,
+// not both kinds for every entry; at most one warp of a half holds both, and
+// the second half deals them in reverse, so that every sub-partition gets
+// both kinds.  The two halves of the CTA take every other K-block, each at
+// its own pace (one fills the float64 pipes while the other waits at its
+// barrier), and add up at the end; the next K-block is in flight in registers
+// while one is summed.
+template <bool general>
+__device__ __forceinline__ void far_sums(int n, const double *__restrict__ T, int ldt, const double *__restrict__ U,
+                                         int ldu, int I, int J, int kb0, int kb1, double *__restrict__ slab,
+                                         Smem &sm)
+{
+    const int r0 = I * LB, c0 = J * LB;
+    const int bj = min(LB, n - c0);
+    const int half = threadIdx.x / LT, tid = threadIdx.x % LT;
+    const int lo = tid % LB, hi = tid / LB, lane = tid & 31;
+    double au, at, bu, bt;
+    auto fetch = [&](int kb) {
+        const bool useUT = kb == I || kb <= J - 2, useTU = kb == J || kb >= I + 2;
+        const int k0 = kb * LB;
+        au = at = bu = bt = 0.0;
+        // A: rows of block I (lo = row), B: columns of block J (hi = column);
+        // only the last block of all can be ragged
+        if (useUT) {
+            au = SGT_AT(U, ldu, r0 + lo, k0 + hi);
+            if (hi < bj) bt = SGT_AT(T, ldt, k0 + lo, c0 + hi);
+        }
+        if (useTU) {
+            if (kb < J || hi < bj) at = SGT_AT(T, ldt, r0 + lo, k0 + hi);
+            if (hi < bj && (kb < J || lo < bj)) bu = SGT_AT(U, ldu, k0 + lo, c0 + hi);
+        }
+    };
+    if (kb0 + half < kb1) fetch(kb0 + half);
+    int p = lo, q = hi;
+    bool opp = true;
+    if (!general) {
+        const int g = (lane < LB) ? r0 + lane : c0 + lane - LB;
+        const unsigned pos = __ballot_sync(0xffffffffu, g < n && SGT_AT(T, ldt, g < n ? g : 0, g < n ? g : 0) > 0.0);
+        const unsigned rm = pos & 0xffffu, cm = pos >> 16;
+        const int rp = __popc(rm), cp = __popc(cm), rn = LB - rp, cn = LB - cp;
+        int t = half ? LT - 1 - tid : tid;
+        unsigned rset, cset;
+        int len;
+        if (t < rp * cp) { rset = rm; cset = cm; len = rp; opp = false; }
+        else if ((t -= rp * cp) < rn * cn) { rset = ~rm; cset = ~cm; len = rn; opp = false; }
+        else if ((t -= rn * cn) < rp * cn) { rset = rm; cset = ~cm; len = rp; }
+        else { t -= rp * cn; rset = ~rm; cset = cm; len = rn; }
+        p = nth_bit(rset & 0xffffu, t % len);
+        q = nth_bit(cset & 0xffffu, t / len);
+    }
+    const bool any_opp = __any_sync(0xffffffffu, opp), all_opp = __all_sync(0xffffffffu, opp);
+    // acc restarts every few K-blocks, its sum so far added to `total`: long
+    // sums round as two short chains, at 1 addition in 64 terms
+    double acc = 0.0, total = 0.0;
+    __syncthreads();   // the buffers may still be read for the CTA's work before
+    for (int kb = kb0 + half, buf = 0; kb < kb1; kb += 2, buf ^= 1) {
+        auto &F = sm.far[half];
+        double *AU = F.AU[buf], *AT = F.AT[buf], *BU = F.BU[buf], *BT = F.BT[buf];
+        AU[hi * LB + lo] = au;
+        AT[hi * LB + lo] = at;
+        BU[hi * LD + lo] = bu;
+        BT[hi * LD + lo] = bt;
+        half_sync(half);
+        if (kb + 2 < kb1) fetch(kb + 2);
+        const double *A1 = AU + p, *A2 = AT + p, *B1 = (opp ? BT : BU) + q * LD, *B2 = BU + q * LD;
+        if (kb >= I + 2 && kb <= J - 2) {
+            if (all_opp) {
+#pragma unroll
+                for (int k = 0; k < LB; k++) {
+                    acc = fma(A1[k * LB], B1[k], acc);
+                    acc = fma(-A2[k * LB], B2[k], acc);
+                }
+            } else if (any_opp) {
+#pragma unroll 4
+                for (int k = 0; k < LB; k++) {
+                    acc = fma(A1[k * LB], B1[k], acc);
+                    const double r = fma(-A2[k * LB], B2[k], acc);
+                    if (opp) acc = r;
+                }
+            } else {
+#pragma unroll
+                for (int k = 0; k < LB; k++) acc = fma(A1[k * LB], B1[k], acc);
+            }
+        } else if (any_opp) {
+            // the first and last two K-blocks: one part only, and inside a
+            // diagonal block only the terms between p and q
+            if (kb == I || kb <= J - 2) {
+                const int k1 = kb == I ? p : -1;
+#pragma unroll 4
+                for (int k = 0; k < LB; k++) {
+                    const double r = fma(A1[k * LB], B1[k], acc);
+                    if (opp && k > k1) acc = r;
+                }
+            }
+            if (kb == J || kb >= I + 2) {
+                const int k1 = kb == J ? q : LB;
+#pragma unroll 4
+                for (int k = 0; k < LB; k++) {
+                    const double r = fma(-A2[k * LB], B2[k], acc);
+                    if (opp && k < k1) acc = r;
+                }
+            }
+        }
+        if (((kb - kb0) & 6) == 6) {
+            total += acc;
+            acc = 0.0;
+        }
+        // the other buffer is refilled next; its readers passed the barrier
+        // above only after they had finished with it
+    }
+    acc += total;
+    __syncthreads();
+    double *part = sm.far[0].AU[0];
+    if (half == 1) part[p + q * LB] = acc;
+    __syncthreads();
+    if (half == 0) slab[p + q * LB] = acc + part[p + q * LB];
+}
+
+// Leaf of block (I, J): nslab partial slabs from slab0 on, LT doubles each.
+// Everything that a launch before the last has written may be read before
+// dependency_wait(); for d <= 2 the blocks next to the diagonal are not yet
+// among it.  Run by the first half of the CTA.
+template <bool general>
+__device__ __forceinline__ void leaf(int n, const double *__restrict__ T, int ldt, double *__restrict__ U, int ldu,
+                                     int I, int J, int nslab, const double *__restrict__ slab0, Smem &sm)
+{
+    auto &s = sm.leaf;
+    const int d = J - I;
+    const int r0 = I * LB, c0 = J * LB;
+    const int bj = min(LB, n - c0);
+    const int lo = threadIdx.x % LB, hi = threadIdx.x / LB;
+    const int at = lo + hi * LD;
+    const bool up = lo <= hi, in = hi < bj;
+    s.TI[at] = up ? SGT_AT(T, ldt, r0 + lo, r0 + hi) : 0.0;
+    s.UI[at] = up ? SGT_AT(U, ldu, r0 + lo, r0 + hi) : 0.0;
+    s.TJ[at] = up && in ? SGT_AT(T, ldt, c0 + lo, c0 + hi) : 0.0;
+    s.UJ[at] = up && in ? SGT_AT(U, ldu, c0 + lo, c0 + hi) : 0.0;
+    const double tij = in ? SGT_AT(T, ldt, r0 + lo, c0 + hi) : 0.0;
+    if (d >= 2) {
+        s.T1[at] = SGT_AT(T, ldt, r0 + lo, r0 + LB + hi);
+        s.T2[at] = in ? SGT_AT(T, ldt, c0 - LB + lo, c0 + hi) : 0.0;
+    }
+    if (d >= 3) {
+        s.U1[at] = SGT_AT(U, ldu, r0 + lo, r0 + LB + hi);
+        s.U2[at] = in ? SGT_AT(U, ldu, c0 - LB + lo, c0 + hi) : 0.0;
+    }
+    if (threadIdx.x < LB) {
+        const int i = threadIdx.x;
+        s.urow[i] = SGT_AT(U, ldu, r0 + i, r0 + i);
+        s.ucol[i] = i < bj ? SGT_AT(U, ldu, c0 + i, c0 + i) : 1.0;
+    }
+    // the thread's entry: number threadIdx.x along the anti-diagonals
+    // step = 15 - p + q, from the bottom-left corner
+    const int m = threadIdx.x < 136 ? threadIdx.x : 255 - threadIdx.x;
+    int a = (int)((sqrtf(8.f * m + 1.f) - 1.f) * 0.5f);
+    if ((a + 1) * (a + 2) / 2 <= m) a++;
+    if (a * (a + 1) / 2 > m) a--;
+    int q = m - a * (a + 1) / 2, p = LB - 1 - a + q;
+    if (threadIdx.x >= 136) { p = LB - 1 - p; q = LB - 1 - q; }
+    const int step = LB - 1 - p + q;
+    half_sync(0);
+    const double upp = s.urow[p], uqq = s.ucol[q];
+    const bool opp = general || upp + uqq == 0.0;
+    // signs agree: 1 / (u_pp + u_qq) is +-1/2 exactly
+    const double rinv = opp ? 1.0 / (s.TI[p + p * LD] - s.TJ[q + q * LD]) : 0.5 * upp;
+    // flips the sign of the row terms where the signs agree
+    const unsigned long long flip = opp ? 0ull : 0x8000000000000000ull;
+    const double *M = opp ? s.TI : s.UI, *N = opp ? s.TJ : s.UJ;
+    const double *M1 = opp ? s.T1 : s.U1, *N2 = opp ? s.T2 : s.U2;
+
+    dependency_wait();
+    dependency_release();
+    // all of the launch before's results in flight together
+    double x1 = 0.0, x2 = 0.0, u1 = 0.0, u2 = 0.0, v[8];
+    if (d >= 2) {
+        if (in) x1 = SGT_AT(U, ldu, r0 + LB + lo, c0 + hi);
+        x2 = SGT_AT(U, ldu, r0 + lo, c0 - LB + hi);
+    }
+    if (d == 2) {
+        u1 = SGT_AT(U, ldu, r0 + lo, r0 + LB + hi);
+        if (in) u2 = SGT_AT(U, ldu, c0 - LB + lo, c0 + hi);
+    }
+#pragma unroll
+    for (int t = 0; t < 8; t++) v[t] = t < nslab ? slab0[(size_t)t * LT + threadIdx.x] : 0.0;
+    double sum = v[0];
+#pragma unroll
+    for (int t = 1; t < 8; t++)
+        if (t < nslab) sum += v[t];
+    for (int t0 = 8; t0 < nslab; t0 += 8) {
+#pragma unroll
+        for (int t = 0; t < 8; t++) v[t] = t0 + t < nslab ? slab0[(size_t)(t0 + t) * LT + threadIdx.x] : 0.0;
+#pragma unroll
+        for (int t = 0; t < 8; t++)
+            if (t0 + t < nslab) sum += v[t];
+    }
+    if (d >= 2) {
+        s.X1[at] = x1;
+        s.X2[at] = x2;
+    }
+    if (d == 2) {
+        s.U1[at] = u1;
+        s.U2[at] = u2;
+    }
+    const double ui = s.urow[lo], uj = s.ucol[hi];
+    const bool o = general || ui + uj == 0.0;
+    s.C[at] = o ? sum : -sum;
+    s.V[at] = o ? tij * (ui - uj) : 0.0;
+    half_sync(0);
+    // t_pq (u_pp - u_qq) is as a rule far larger than the terms summed below,
+    // so it joins them last, when only the terms of one step are still to come
+    double acc = s.C[p + q * LD];
+    const double base = s.V[p + q * LD];
+    if (d >= 2) {
+        // (d = 2: both near blocks are the same, and a sum of U U counts it once)
+        const bool row = d > 2 || opp;
+#pragma unroll 8
+        for (int k = 0; k < LB; k++) {
+            acc = fma(-M1[p + k * LD], s.X1[k + q * LD], acc);
+            const double x = __longlong_as_double(__double_as_longlong(s.X2[p + k * LD]) ^ flip);
+            const double r = fma(x, N2[k + q * LD], acc);
+            if (row) acc = r;
+        }
+    }
+    if (step == 0) acc += base;
+    half_sync(0);   // every base is read: V now takes the solution
+    for (int st = 0; st < 2 * LB - 1; st++) {
+        if (step == st || step == st + 1) {
+            // the entry's value, or its base term: one instruction for both
+            // kinds of lane (x * 1 + base and x * rinv - 0 round as the plain
+            // sum and product)
+            const bool now = step == st;
+            acc = fma(acc, now ? rinv : 1.0, now ? -0.0 : base);
+            if (now) s.V[p + q * LD] = acc;
+        }
+        half_sync(0);
+        if (st < step) {
+            const int k1 = LB - 1 + q - st;   // solved at this step in the entry's column ...
+            const int k2 = st - (LB - 1) + p;   // ... and in its row
+            if (k2 >= 0) {
+                const double x = __longlong_as_double(__double_as_longlong(s.V[p + k2 * LD]) ^ flip);
+                acc = fma(x, N[k2 + q * LD], acc);
+            }
+            if (k1 < LB) acc = fma(-M[p + k1 * LD], s.V[k1 + q * LD], acc);
+        }
+    }
+    if (in) SGT_AT(U, ldu, r0 + lo, c0 + hi) = s.V[at];
+}
+
+// Diagonal block (r0, r0): Algorithm 3 with the plain float64 algorithm's own
+// rounding (separate multiply, add and divide, sums in ascending k).  By
+// anti-diagonal: the products of all the anti-diagonal's terms first, spread
+// over the threads, then each entry's sum, one addition after another, by a
+// thread of its own; the quotients t_ij (u_ii - u_jj) / (t_ii - t_jj), which
+// need no sum, once at the start.
+__device__ __forceinline__ void diag_leaf(int n, const double *__restrict__ T, int ldt, double *__restrict__ U,
+                                          int ldu, int blk, double *Ts, double *Us, double *Pr, double *Q1)
+{
+    const int r0 = blk * LB, bs = min(LB, n - r0);
+    const int lo = threadIdx.x % LB, hi = threadIdx.x / LB, at = lo + hi * LD;
+    const bool in = lo <= hi && hi < bs;
+    const double t = in ? SGT_AT(T, ldt, r0 + lo, r0 + hi) : 0.0;
+    Ts[at] = t;
+    Us[at] = lo == hi ? ph::sgn(t) : 0.0;
+    __syncthreads();
+    {
+        const double ui = Us[lo * (LD + 1)], uj = Us[hi * (LD + 1)];
+        if (in && lo < hi && __dadd_rn(ui, uj) == 0.0)
+            Q1[at] = __ddiv_rn(__dmul_rn(t, __dsub_rn(ui, uj)), __dsub_rn(Ts[lo * (LD + 1)], Ts[hi * (LD + 1)]));
+    }
+    for (int d = 1; d < bs; d++) {
+        const int terms = d - 1;
+        if (terms > 0 && threadIdx.x < (bs - d) * terms) {   // at most 8 * 7 of them
+            const int i = threadIdx.x / terms, k = i + 1 + threadIdx.x % terms, j = i + d;
+            const double uk = Us[i + k * LD], ukj = Us[k + j * LD];
+            const bool opp = __dadd_rn(Us[i * (LD + 1)], Us[j * (LD + 1)]) == 0.0;
+            double v = __dmul_rn(uk, opp ? Ts[k + j * LD] : ukj);
+            if (opp) v = __dsub_rn(v, __dmul_rn(Ts[i + k * LD], ukj));
+            Pr[i * LD + (k - i - 1)] = v;
+        }
+        __syncthreads();
+        if (threadIdx.x < bs - d) {
+            const int i = threadIdx.x, j = i + d;
+            double s = 0.0;
+            for (int k = 0; k < terms; k++) s = __dadd_rn(s, Pr[i * LD + k]);
+            const double uii = Us[i * (LD + 1)], ujj = Us[j * (LD + 1)];
+            double r;
+            if (__dadd_rn(uii, ujj) == 0.0)
+                r = __dadd_rn(Q1[i + j * LD], __ddiv_rn(s, __dsub_rn(Ts[i * (LD + 1)], Ts[j * (LD + 1)])));
+            else
+                r = __dmul_rn(-s, __dmul_rn(0.5, uii));   // -s / (+-2), exactly
+            Us[i + j * LD] = r;
+        }
+        __syncthreads();
+    }
+    if (in) SGT_AT(U, ldu, r0 + lo, r0 + hi) = Us[at];
+}
+
+}  // namespace lvl
+}  // namespace signtri
