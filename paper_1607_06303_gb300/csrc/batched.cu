@@ -16,6 +16,7 @@
 
 #include "internal.cuh"
 #include "ph_bodies.cuh"
+#include "ph_level.cuh"
 #include "batched_plan.h"
 
 namespace signtri {
@@ -84,6 +85,52 @@ batched_leaf_kernel(const BatchDesc *__restrict__ mats, const int *__restrict__ 
                          PY + (size_t)t.slot0 * B * B, (size_t)B * B);
 }
 
+// Leaf blocks of 16: as diag_level_kernel and level_kernel of ph_fp64.cu,
+// over the tiles of all matrices.
+__global__ void __launch_bounds__(lvl::LT)
+batched_diag_level_kernel(const BatchDesc *__restrict__ mats, const int *__restrict__ members,
+                          const DiagTask *__restrict__ tasks)
+{
+    __shared__ double Ts[lvl::BLK], Us[lvl::BLK], Pr[lvl::BLK], Q1[lvl::BLK];
+    const DiagTask t = tasks[blockIdx.x];
+    const BatchDesc M = mats[members[t.m]];
+    lvl::diag_leaf(M.n, M.T, M.ldt, M.U, M.ldu, t.blk, Ts, Us, Pr, Q1);
+}
+
+__global__ void __launch_bounds__(lvl::kLevelThreads)
+batched_level_kernel(const BatchDesc *__restrict__ mats, const int *__restrict__ members, int d, int leaves,
+                     const LevelTile *__restrict__ tiles, const __grid_constant__ lvl::Split sin,
+                     const double *__restrict__ in, const LevelTile *__restrict__ next,
+                     const __grid_constant__ lvl::Split sout, double *__restrict__ out)
+{
+    using namespace lvl;
+    extern __shared__ __align__(16) unsigned char raw[];
+    Smem &sm = *reinterpret_cast<Smem *>(raw);
+    const int c = blockIdx.x;
+    if (c < leaves && threadIdx.x < LT) {
+        const LevelTile t = tiles[c];
+        const BatchDesc M = mats[members[t.m]];
+        const int f = split_owner(sin, (long long)c * sin.cpt), l = split_owner(sin, (long long)(c + 1) * sin.cpt - 1);
+        leaf<false>(M.n, M.T, M.ldt, M.U, M.ldu, t.I, t.I + d, l - f + 1, in + (size_t)(f + c) * LT, sm);
+    } else {
+        dependency_wait();
+        dependency_release();
+    }
+    if (c >= sout.G) return;
+    __syncthreads();   // the leaf's shared memory is free
+    const int e = d + 1, cpt = sout.cpt;
+    const long long x1 = split_start(sout, c + 1);
+    for (long long x = split_start(sout, c); x < x1;) {
+        const int k = (int)(x / cpt);
+        const long long t0 = (long long)k * cpt, xe = min(x1, t0 + cpt);
+        const LevelTile t = next[k];
+        const BatchDesc M = mats[members[t.m]];
+        far_sums<false>(M.n, M.T, M.ldt, M.U, M.ldu, t.I, t.I + e, t.I + (int)(x - t0), t.I + (int)(xe - t0),
+                        out + (size_t)(c + k) * LT, sm);
+        x = xe;
+    }
+}
+
 // A group's device task tables and instantiated graph, kept for the next
 // call that runs the same group: same leaf size and form, same member sizes
 // and indices, and the same descriptor array and partial-slab addresses
@@ -125,14 +172,22 @@ signtri_status run_group(const BatchDesc *d_mats, const std::vector<int> &member
     GroupCache &gc = g_cache[dev][B == 16 ? 0 : (B == 32 ? 1 : 2)];
     const bool same_shape = gc.valid && gc.split == split && gc.ns == ns && gc.members == members &&
                             gc.d_mats == d_mats;
+    // leaves of 16: one launch per level over lp (both forms are the same);
+    // else separate block-sum and leaf launches over p
+    constexpr bool levels = B == lvl::LB;
     Plan p;
-    if (!same_shape) make_plan(ns, B, p);
-    const size_t slots = std::max<size_t>(same_shape ? gc.max_slots : p.max_slots, 1);
+    LevelPlan lp;
+    auto plan = [&] {
+        if (levels) make_level_plan(ns, lp);
+        else make_plan(ns, B, p);
+    };
+    if (!same_shape) plan();
+    const size_t slots = std::max<size_t>(same_shape ? gc.max_slots : (levels ? 2 * lp.slabs : p.max_slots), 1);
     // the partial slabs come first from the workspace, so a group of the same
     // shape finds them at the same address
     double *PX = static_cast<double *>(ws.take(slots * B * B * sizeof(double)));
     // the efficient form keeps one sum per entry: X and Y share the slabs
-    double *PY = split ? PX : static_cast<double *>(ws.take(slots * B * B * sizeof(double)));
+    double *PY = split || levels ? PX : static_cast<double *>(ws.take(slots * B * B * sizeof(double)));
     if (!PX || !PY) return SIGNTRI_ERR_NO_WORKSPACE;
     if (same_shape && gc.PX == PX) {
         gc.hits++;
@@ -144,19 +199,22 @@ signtri_status run_group(const BatchDesc *d_mats, const std::vector<int> &member
         SGT_CUDA_TRY(cudaGraphLaunch(gc.exec, st));
         return SIGNTRI_OK;
     }
-    if (same_shape) make_plan(ns, B, p);   // same shape, moved workspace: rebuild
+    if (same_shape) plan();   // same shape, moved workspace: rebuild
+    const std::vector<DiagTask> &diag = levels ? lp.diag : p.diag;
+    const bool perms = split && !levels;
     cache_drop(gc);
     // tables: members, diagonal / block-sum / leaf tasks, sign permutations
     // and their offsets, each 256-byte aligned
     auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
-    const size_t b_mem = al(members.size() * sizeof(int)), b_diag = al(std::max<size_t>(p.diag.size(), 1) * sizeof(DiagTask));
+    const size_t b_mem = al(members.size() * sizeof(int)), b_diag = al(std::max<size_t>(diag.size(), 1) * sizeof(DiagTask));
     const size_t b_gemm = al(std::max<size_t>(p.gemm.size(), 1) * sizeof(GemmTask));
     const size_t b_leaf = al(std::max<size_t>(p.leaf.size(), 1) * sizeof(LeafTask));
-    const size_t b_perm = split ? al(std::max<size_t>(p.perm_len, 1) * sizeof(short)) : 0;
-    const size_t b_npos = split ? al(std::max<size_t>(p.npos_len, 1) * sizeof(int)) : 0;
-    const size_t b_off = split ? 2 * al(p.poff.size() * sizeof(int)) : 0;
+    const size_t b_tile = al(std::max<size_t>(lp.tiles.size(), 1) * sizeof(LevelTile));
+    const size_t b_perm = perms ? al(std::max<size_t>(p.perm_len, 1) * sizeof(short)) : 0;
+    const size_t b_npos = perms ? al(std::max<size_t>(p.npos_len, 1) * sizeof(int)) : 0;
+    const size_t b_off = perms ? 2 * al(p.poff.size() * sizeof(int)) : 0;
     char *tb = nullptr;
-    if (cudaMalloc(&tb, b_mem + b_diag + b_gemm + b_leaf + b_perm + b_npos + b_off) != cudaSuccess) {
+    if (cudaMalloc(&tb, b_mem + b_diag + b_gemm + b_leaf + b_tile + b_perm + b_npos + b_off) != cudaSuccess) {
         cudaGetLastError();
         return SIGNTRI_ERR_NO_WORKSPACE;
     }
@@ -165,10 +223,11 @@ signtri_status run_group(const BatchDesc *d_mats, const std::vector<int> &member
     auto *d_diag = reinterpret_cast<DiagTask *>(tb + b_mem);
     auto *d_gemm = reinterpret_cast<GemmTask *>(tb + b_mem + b_diag);
     auto *d_leaf = reinterpret_cast<LeafTask *>(tb + b_mem + b_diag + b_gemm);
-    char *rest = tb + b_mem + b_diag + b_gemm + b_leaf;
+    auto *d_tile = reinterpret_cast<LevelTile *>(tb + b_mem + b_diag + b_gemm + b_leaf);
+    char *rest = tb + b_mem + b_diag + b_gemm + b_leaf + b_tile;
     short *d_perm = nullptr;
     int *d_npos = nullptr, *d_poff = nullptr, *d_noff = nullptr;
-    if (split) {
+    if (perms) {
         d_perm = reinterpret_cast<short *>(rest);
         d_npos = reinterpret_cast<int *>(rest + b_perm);
         d_poff = reinterpret_cast<int *>(rest + b_perm + b_npos);
@@ -177,17 +236,24 @@ signtri_status run_group(const BatchDesc *d_mats, const std::vector<int> &member
         SGT_CUDA_TRY(cudaMemcpyAsync(d_noff, p.noff.data(), p.noff.size() * sizeof(int), cudaMemcpyHostToDevice, st));
     }
     SGT_CUDA_TRY(cudaMemcpyAsync(d_members, members.data(), members.size() * sizeof(int), cudaMemcpyHostToDevice, st));
-    SGT_CUDA_TRY(cudaMemcpyAsync(d_diag, p.diag.data(), p.diag.size() * sizeof(DiagTask), cudaMemcpyHostToDevice, st));
+    SGT_CUDA_TRY(cudaMemcpyAsync(d_diag, diag.data(), diag.size() * sizeof(DiagTask), cudaMemcpyHostToDevice, st));
     if (!p.gemm.empty())
         SGT_CUDA_TRY(cudaMemcpyAsync(d_gemm, p.gemm.data(), p.gemm.size() * sizeof(GemmTask), cudaMemcpyHostToDevice, st));
     if (!p.leaf.empty())
         SGT_CUDA_TRY(cudaMemcpyAsync(d_leaf, p.leaf.data(), p.leaf.size() * sizeof(LeafTask), cudaMemcpyHostToDevice, st));
+    if (!lp.tiles.empty())
+        SGT_CUDA_TRY(cudaMemcpyAsync(d_tile, lp.tiles.data(), lp.tiles.size() * sizeof(LevelTile), cudaMemcpyHostToDevice, st));
     // the host tables are pageable and local
     SGT_CUDA_TRY(cudaStreamSynchronize(st));
-    SGT_CUDA_TRY(cudaFuncSetAttribute(batched_leaf_kernel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)leaf_smem<B>()));
-    SGT_CUDA_TRY(cudaFuncSetAttribute(batched_diag_kernel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)diag_smem<B>()));
+    if constexpr (levels) {
+        SGT_CUDA_TRY(cudaFuncSetAttribute(batched_level_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          lvl::level_smem(lvl::kSms)));
+    } else {
+        SGT_CUDA_TRY(cudaFuncSetAttribute(batched_leaf_kernel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)leaf_smem<B>()));
+        SGT_CUDA_TRY(cudaFuncSetAttribute(batched_diag_kernel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)diag_smem<B>()));
+    }
     // the level loop, captured into one graph on a private stream
     if (!gc.capture) {
         cudaStream_t cs = nullptr;
@@ -201,28 +267,54 @@ signtri_status run_group(const BatchDesc *d_mats, const std::vector<int> &member
     long long nk[3] = {0, 0, 0};
     if (rs == SIGNTRI_OK) {
         prof_pause(true);
-        if (split) {
-            batched_perm_kernel<B><<<(unsigned)p.diag.size(), B, 0, cs>>>(d_mats, d_members, d_diag, d_perm, d_npos,
-                                                                          d_poff, d_noff);
+        if constexpr (levels) {
+            batched_diag_level_kernel<<<(unsigned)diag.size(), lvl::LT, 0, cs>>>(d_mats, d_members, d_diag);
             nk[0]++;
-        }
-        batched_diag_kernel<B><<<(unsigned)p.diag.size(), kThreads, diag_smem<B>(), cs>>>(d_mats, d_members, d_diag);
-        nk[0]++;
-        for (int d = 1; d < p.nbmax; d++) {
-            const int g0 = p.gemm_off[d], g1 = p.gemm_off[d + 1];
-            const int l0 = p.leaf_off[d], l1 = p.leaf_off[d + 1];
-            if (g1 > g0) {
-                if (split)
-                    batched_gemm_split_kernel<B><<<g1 - g0, kThreads, 0, cs>>>(d_mats, d_members, d_gemm + g0, d_perm,
-                                                                               d_npos, d_poff, d_noff, PX);
-                else
-                    batched_gemm_kernel<B><<<g1 - g0, kThreads, 0, cs>>>(d_mats, d_members, d_gemm + g0, PX, PY);
-                nk[1]++;
-            }
-            if (l1 > l0) {
-                batched_leaf_kernel<B><<<l1 - l0, kThreads, leaf_smem<B>(), cs>>>(d_mats, d_members, d_leaf + l0, PX,
-                                                                                 PY);
+            cudaLaunchAttribute attr{};
+            attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            attr.val.programmaticStreamSerializationAllowed = 1;
+            cudaLaunchConfig_t cfg{};
+            cfg.blockDim = dim3(lvl::kLevelThreads);
+            cfg.stream = cs;
+            cfg.attrs = &attr;
+            cfg.numAttrs = 1;
+            double *slab[2] = {PX, PX + slots / 2 * B * B};
+            for (int d = 0; d < lp.nbmax; d++) {
+                const int leaves = d > 0 ? lp.off[d + 1] - lp.off[d] : 0, e = d + 1;
+                const lvl::Split sin = lp.split[d], sout = e < lp.nbmax ? lp.split[e] : lvl::Split{};
+                cfg.gridDim = dim3(std::max(leaves, sout.G));
+                if (cfg.gridDim.x == 0) continue;   // a group of single blocks
+                cfg.dynamicSmemBytes = lvl::level_smem((int)cfg.gridDim.x);
+                if (cudaLaunchKernelEx(&cfg, batched_level_kernel, d_mats, (const int *)d_members, d, leaves,
+                                       (const LevelTile *)(d_tile + lp.off[d]), sin, (const double *)slab[d & 1],
+                                       (const LevelTile *)(d_tile + lp.off[e]), sout, slab[e & 1]) != cudaSuccess)
+                    rs = SIGNTRI_ERR_CUDA;
                 nk[2]++;
+            }
+        } else {
+            if (split) {
+                batched_perm_kernel<B><<<(unsigned)p.diag.size(), B, 0, cs>>>(d_mats, d_members, d_diag, d_perm, d_npos,
+                                                                              d_poff, d_noff);
+                nk[0]++;
+            }
+            batched_diag_kernel<B><<<(unsigned)p.diag.size(), kThreads, diag_smem<B>(), cs>>>(d_mats, d_members, d_diag);
+            nk[0]++;
+            for (int d = 1; d < p.nbmax; d++) {
+                const int g0 = p.gemm_off[d], g1 = p.gemm_off[d + 1];
+                const int l0 = p.leaf_off[d], l1 = p.leaf_off[d + 1];
+                if (g1 > g0) {
+                    if (split)
+                        batched_gemm_split_kernel<B><<<g1 - g0, kThreads, 0, cs>>>(d_mats, d_members, d_gemm + g0, d_perm,
+                                                                                   d_npos, d_poff, d_noff, PX);
+                    else
+                        batched_gemm_kernel<B><<<g1 - g0, kThreads, 0, cs>>>(d_mats, d_members, d_gemm + g0, PX, PY);
+                    nk[1]++;
+                }
+                if (l1 > l0) {
+                    batched_leaf_kernel<B><<<l1 - l0, kThreads, leaf_smem<B>(), cs>>>(d_mats, d_members, d_leaf + l0, PX,
+                                                                                     PY);
+                    nk[2]++;
+                }
             }
         }
         prof_pause(false);
@@ -270,6 +362,7 @@ void batched_cache_stats(long long *hits, long long *builds)
 size_t batched_workspace_bytes(int count, const int *n, int B)
 {
     std::vector<int> ns(n, n + count);
+    if (B == lvl::LB) return level_bytes_bound(ns) + 4096;
     Plan p;
     make_plan(ns, B, p);
     return std::max(plan_bytes(p, B), plan_bytes_bound(ns, B)) + (size_t)count * sizeof(int) + 4096;

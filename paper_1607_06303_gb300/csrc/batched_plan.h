@@ -11,6 +11,8 @@
 #include <cstddef>
 #include <vector>
 
+#include "level_split.h"
+
 namespace signtri {
 
 // K splits per tile at most, and the CTAs a level's block-sum launch aims at
@@ -128,6 +130,64 @@ inline size_t plan_bytes_bound(const std::vector<int> &ns, int B)
     return diag * sizeof(DiagTask) + gemm * sizeof(GemmTask) + leaf * sizeof(LeafTask) +
            2 * std::max<size_t>(slots, 1) * B * B * sizeof(double) + perm * sizeof(short) + npos * sizeof(int) +
            2 * ns.size() * sizeof(int) + 12 * 256;
+}
+
+// Leaf blocks of 16 run one launch per level (ph_level.cuh): the level's
+// leaves and the early sums of the next level.  tiles: (matrix, row block) of
+// every level's tiles, level d's from off[d]; all tiles of a level have the
+// same number of K-blocks, so a level is cut like that of a single matrix.
+struct LevelTile {
+    int m, I;
+};
+struct LevelPlan {
+    std::vector<DiagTask> diag;
+    std::vector<LevelTile> tiles;
+    std::vector<int> off;                // per level d (size nbmax + 1)
+    std::vector<lvl::Split> split;       // split[e]: the early sums of level e
+    int nbmax = 0;
+    size_t slabs = 0;                    // partial slabs of one level, at most
+};
+
+inline void make_level_plan(const std::vector<int> &ns, LevelPlan &p)
+{
+    const int cnt = (int)ns.size(), B = lvl::LB;
+    p = LevelPlan();
+    for (int k = 0; k < cnt; k++) {
+        const int nb = (ns[k] + B - 1) / B;
+        p.nbmax = std::max(p.nbmax, nb);
+        for (int b = 0; b < nb; b++) p.diag.push_back({k, b});
+    }
+    p.off.assign(p.nbmax + 1, 0);
+    p.split.assign(p.nbmax + 1, lvl::Split{});
+    for (int d = 1; d < p.nbmax; d++) {
+        p.off[d] = (int)p.tiles.size();
+        for (int k = 0; k < cnt; k++)
+            for (int I = 0; I + d < (ns[k] + B - 1) / B; I++) p.tiles.push_back({k, I});
+    }
+    p.off[p.nbmax] = (int)p.tiles.size();
+    for (int e = 1; e < p.nbmax; e++) {
+        const int tiles = p.off[e + 1] - p.off[e], leaves = e > 1 ? p.off[e] - p.off[e - 1] : 0;
+        p.split[e] = lvl::make_split(tiles, e, leaves);
+        p.slabs = std::max(p.slabs, (size_t)p.split[e].G + tiles);
+    }
+}
+
+// An upper bound of a level plan's workspace (two slab sets) over every
+// subset of the matrices ns: tiles and leaves only shrink with the subset.
+inline size_t level_bytes_bound(const std::vector<int> &ns)
+{
+    const int B = lvl::LB;
+    int nbmax = 0;
+    for (int n : ns) nbmax = std::max(nbmax, (n + B - 1) / B);
+    size_t slabs = 0;
+    long long before = 0;
+    for (int d = 1; d < nbmax; d++) {
+        long long tiles = 0;
+        for (int n : ns) tiles += std::max(0, (n + B - 1) / B - d);
+        slabs = std::max(slabs, lvl::slabs_bound(tiles, before));
+        before = tiles;
+    }
+    return 2 * slabs * B * B * sizeof(double) + 2 * 256;
 }
 
 }  // namespace signtri

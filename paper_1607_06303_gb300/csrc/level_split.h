@@ -16,19 +16,22 @@ namespace lvl {
 
 constexpr int LB = 16;   // block order
 
-// Anti-diagonal e has nb - e tiles of e + 1 K-blocks (K = I .. J), W in all,
-// numbered tile by tile.  The launch has G CTAs, of which the first L solve
+// Anti-diagonal e has tiles (nb - e of them in one matrix) of e + 1 K-blocks
+// (K = I .. J), W in all, numbered tile by tile.  The launch has G CTAs, of which the first L solve
 // a leaf first, worth about kLeafBlocks K-blocks of float64 work.  CTA c sums
 // the K-blocks [start(c), start(c + 1)), the leaf CTAs fewer, so that all end
 // together; when that leaves them fewer than kFarShare, they sum nothing and
 // the others share W evenly, in ranges of about kFarShare at least (a tile's
 // leaf adds its partials one after another, 128 cycles each).  One CTA (or as
 // many as the leaves need) per SM: its sixteen warps keep the float64 pipes
-// busy, and a leaf that shares them takes longer.  The cut depends on sizes
-// only, so results do not depend on the GPU.
+// busy, and a leaf that shares them takes longer.  With more than kManyLeaves
+// leaves (batches) every SM solves several in turn whatever the placement,
+// and the sums go to kManyFar CTAs behind them.  The cut depends on sizes only, so results do not depend on the GPU.
 constexpr int kSms = 152;
 constexpr int kLeafBlocks = 5;
 constexpr int kFarShare = 4;
+constexpr int kManyLeaves = 4 * kSms;
+constexpr int kManyFar = 16 * kSms;
 
 struct Split {
     long long W;   // K-blocks
@@ -38,12 +41,13 @@ struct Split {
     int lam;       // K-blocks a leaf counts for; 0: leaf CTAs sum nothing
 };
 
-SGT_HD constexpr Split make_split(int nb, int e, int leaves)
+SGT_HD constexpr Split make_split(int tiles, int e, int leaves)
 {
-    const int cpt = e + 1, tiles = nb - e;
+    const int cpt = e + 1;
     Split s{(long long)tiles * cpt, cpt, leaves, kSms, kLeafBlocks};
-    while (s.G < leaves + kSms / 8) s.G += kSms;
-    if (s.W + (long long)kLeafBlocks * leaves < (long long)(kLeafBlocks + kFarShare) * s.G) {
+    if (leaves > kManyLeaves) s.G = leaves + kManyFar;
+    else while (s.G < leaves + kSms / 8) s.G += kSms;
+    if (leaves > kManyLeaves || s.W + (long long)kLeafBlocks * leaves < (long long)(kLeafBlocks + kFarShare) * s.G) {
         long long g = s.G - leaves;
         const long long most = (long long)tiles * ((cpt + kFarShare - 1) / kFarShare);
         if (g > most) g = most;
@@ -86,10 +90,16 @@ constexpr size_t level_slabs(int n)
     const int nb = (n + LB - 1) / LB;
     int most = 0;
     for (int e = 1; e < nb; e++) {
-        const int g = make_split(nb, e, far_leaves(nb, e)).G + nb - e;
+        const int g = make_split(nb - e, e, far_leaves(nb, e)).G + nb - e;
         if (g > most) most = g;
     }
     return (size_t)most;
+}
+
+// The same for any set of at most `tiles` tiles and `leaves` leaves.
+SGT_HD constexpr size_t slabs_bound(long long tiles, long long leaves)
+{
+    return (size_t)(tiles + leaves + kManyFar + 2 * kSms);
 }
 
 }  // namespace lvl

@@ -242,7 +242,7 @@ static signtri_status launch_levels(int n, const double *T, int ldt, double *U, 
     for (int d = 0; d < nb; d++) {
         const int leaves = d > 0 ? nb - d : 0, e = d + 1;
         lvl::Split sout{};
-        if (e < nb) sout = lvl::make_split(nb, e, leaves);
+        if (e < nb) sout = lvl::make_split(nb - e, e, leaves);
         cfg.gridDim = dim3(std::max(leaves, sout.G));
         cfg.dynamicSmemBytes = lvl::level_smem((int)cfg.gridDim.x);
         ProfScope ps(SIGNTRI_KC_OFFDIAG_LEAF, st);

@@ -11,7 +11,7 @@ using namespace signtri::lvl;
 
 static int check(int nb, int e, int stride, long long slabs)
 {
-    const Split s = make_split(nb, e, far_leaves(nb, e));
+    const Split s = make_split(nb - e, e, far_leaves(nb, e));
     if (split_start(s, 0) != 0 || split_start(s, s.G) != s.W) return 1;
     for (int c = 0; c < s.G; c++) {
         const long long len = split_start(s, c + 1) - split_start(s, c);
