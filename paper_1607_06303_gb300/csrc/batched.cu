@@ -105,7 +105,7 @@ batched_level_kernel(const BatchDesc *__restrict__ mats, const int *__restrict__
 {
     using namespace lvl;
     extern __shared__ __align__(16) unsigned char raw[];
-    Smem &sm = *reinterpret_cast<Smem *>(raw);
+    Smem<double> &sm = *reinterpret_cast<Smem<double> *>(raw);
     const int c = blockIdx.x;
     if (c < leaves && threadIdx.x < LT) {
         const LevelTile t = tiles[c];
@@ -247,7 +247,7 @@ signtri_status run_group(const BatchDesc *d_mats, const std::vector<int> &member
     SGT_CUDA_TRY(cudaStreamSynchronize(st));
     if constexpr (levels) {
         SGT_CUDA_TRY(cudaFuncSetAttribute(batched_level_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          lvl::level_smem(lvl::kSms)));
+                                          lvl::level_smem<double>(lvl::kSms)));
     } else {
         SGT_CUDA_TRY(cudaFuncSetAttribute(batched_leaf_kernel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           (int)leaf_smem<B>()));
@@ -284,7 +284,7 @@ signtri_status run_group(const BatchDesc *d_mats, const std::vector<int> &member
                 const lvl::Split sin = lp.split[d], sout = e < lp.nbmax ? lp.split[e] : lvl::Split{};
                 cfg.gridDim = dim3(std::max(leaves, sout.G));
                 if (cfg.gridDim.x == 0) continue;   // a group of single blocks
-                cfg.dynamicSmemBytes = lvl::level_smem((int)cfg.gridDim.x);
+                cfg.dynamicSmemBytes = lvl::level_smem<double>((int)cfg.gridDim.x);
                 if (cudaLaunchKernelEx(&cfg, batched_level_kernel, d_mats, (const int *)d_members, d, leaves,
                                        (const LevelTile *)(d_tile + lp.off[d]), sin, (const double *)slab[d & 1],
                                        (const LevelTile *)(d_tile + lp.off[e]), sout, slab[e & 1]) != cudaSuccess)

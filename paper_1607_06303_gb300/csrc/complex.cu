@@ -8,13 +8,10 @@
 //   signs differ: u_ij = t_ij (u_ii - u_jj) / (t_ii - t_jj)
 //                        + [sum_{i<k<j} (u_ik t_kj - t_ik u_kj)] / (t_ii - t_jj)
 //   signs agree:  u_ij = -[sum_{i<k<j} u_ik u_kj] / (u_ii + u_jj)
-// in complex float64 arithmetic.  Entries are computed by anti-diagonal
-// d = j - i (each depends on smaller d only), one launch per anti-diagonal,
-// one warp per entry: the lanes split the terms of the sum and reduce by
-// shuffles.  Row i of U and of T is read from row-major copies (UR, TR, the
-// entry's writer storing u_ij in both layouts), so every sum reads
-// contiguous runs.  This path runs at the float64 rate of the SMs; it is the
-// general-spectrum building block, not a tuned hot path.
+// in complex float64 arithmetic, blocked as the real float64 path: blocks of
+// 16, one launch per block anti-diagonal (ph_level.cuh, on double2 entries),
+// bound by the float64 pipes.  (Entry by entry, one launch per element
+// anti-diagonal, n = 1000 took 21 ms; blocked 3.3 ms.)
 //
 // The route's products W = U Q^H and S = Q W are complex: each is four real
 // emulated-float64 tensor-core products of the real and imaginary planes
@@ -27,6 +24,7 @@
 #include <climits>
 
 #include "internal.cuh"
+#include "ph_level.cuh"
 
 namespace signtri {
 
@@ -52,64 +50,65 @@ __device__ __forceinline__ double2 cdiv(double2 a, double2 b)
     return make_double2((a.x * r + a.y) / den, (a.y * r - a.x) / den);
 }
 
-// Diagonal check (first bad index: 4 i + status, as the real scan) and
-// signs; U zeroed with its diagonal set; TR = rows of T's upper triangle.
+// Diagonal check (first bad index: 4 i + status, as the real scan); strictly
+// lower part of U zeroed.
 __global__ void complex_init_kernel(int n, const double2 *__restrict__ T, int ldt, double2 *__restrict__ U, int ldu,
-                                    double2 *__restrict__ UR, double2 *__restrict__ TR, signed char *__restrict__ sg,
                                     int *__restrict__ bad)
 {
     const int j = blockIdx.x;
-    const double2 tjj = T[(size_t)j + (size_t)j * ldt];
-    const double s = tjj.x > 0.0 ? 1.0 : -1.0;
     if (threadIdx.x == 0) {
+        const double2 tjj = T[(size_t)j + (size_t)j * ldt];
         int key = INT_MAX;
         if (!isfinite(tjj.x) || !isfinite(tjj.y)) key = 4 * j + SIGNTRI_ERR_NONFINITE;
         else if (tjj.x == 0.0) key = 4 * j + SIGNTRI_ERR_ZERO_EIGENVALUE;
         if (key != INT_MAX) atomicMin(bad, key);
-        sg[j] = (signed char)s;
     }
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        const double2 v = make_double2(i == j ? s : 0.0, 0.0);
-        U[(size_t)i + (size_t)j * ldu] = v;
-        UR[(size_t)j * n + i] = (i == j) ? v : make_double2(0.0, 0.0);   // UR row j
-        TR[(size_t)j * n + i] = (i >= j) ? T[(size_t)j + (size_t)i * ldt] : make_double2(0.0, 0.0);
-    }
+    for (int i = j + 1 + threadIdx.x; i < n; i += blockDim.x) SGT_AT(U, ldu, i, j) = make_double2(0.0, 0.0);
 }
 
-// Anti-diagonal d: entries (i, i + d), i < n - d, one warp each.
-__global__ void __launch_bounds__(kThreads)
-complex_antidiag_kernel(int n, int d, const double2 *__restrict__ T, int ldt, const double2 *__restrict__ TR,
-                        double2 *__restrict__ U, int ldu, double2 *__restrict__ UR, const signed char *__restrict__ sg)
+// Diagonal blocks of 16, by anti-diagonal: the products of all the
+// anti-diagonal's terms spread over the threads, then each entry's sum and
+// quotient by a thread of its own; the quotients that need no sum at the start.
+__global__ void __launch_bounds__(lvl::LT)
+complex_diag_kernel(int n, const double2 *__restrict__ T, int ldt, double2 *__restrict__ U, int ldu)
 {
-    const int i = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) / 32), lane = threadIdx.x & 31;
-    if (i >= n - d) return;
-    const int j = i + d;
-    const bool opp = sg[i] != sg[j];
-    const double2 *urow = UR + (size_t)i * n, *trow = TR + (size_t)i * n;
-    const double2 *ucol = U + (size_t)j * ldu, *tcol = T + (size_t)j * ldt;
-    double2 s = make_double2(0.0, 0.0);
-    if (opp) {
-        for (int k = i + 1 + lane; k < j; k += 32) s = cadd(s, csub(cmul(urow[k], tcol[k]), cmul(trow[k], ucol[k])));
-    } else {
-        for (int k = i + 1 + lane; k < j; k += 32) s = cadd(s, cmul(urow[k], ucol[k]));
+    using namespace lvl;
+    __shared__ double2 Ts[BLK], Us[BLK], Pr[BLK], Q1[BLK];
+    const int r0 = blockIdx.x * LB, bs = min(LB, n - r0);
+    const int lo = threadIdx.x % LB, hi = threadIdx.x / LB, at = lo + hi * LD;
+    const bool in = lo <= hi && hi < bs;
+    const double2 zero = make_double2(0.0, 0.0);
+    const double2 t = in ? SGT_AT(T, ldt, r0 + lo, r0 + hi) : zero;
+    Ts[at] = t;
+    Us[at] = lo == hi ? make_double2(t.x > 0.0 ? 1.0 : -1.0, 0.0) : zero;
+    __syncthreads();
+    {
+        const double ui = Us[lo * (LD + 1)].x, uj = Us[hi * (LD + 1)].x;
+        if (in && lo < hi && ui + uj == 0.0)
+            Q1[at] = cdiv(scaled(t, ui - uj), csub(Ts[lo * (LD + 1)], Ts[hi * (LD + 1)]));
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
-        s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
+    for (int d = 1; d < bs; d++) {
+        const int terms = d - 1;
+        if (terms > 0 && threadIdx.x < (bs - d) * terms) {   // at most 8 * 7 of them
+            const int i = threadIdx.x / terms, k = i + 1 + threadIdx.x % terms, j = i + d;
+            const bool opp = Us[i * (LD + 1)].x != Us[j * (LD + 1)].x;
+            const double2 ik = Us[i + k * LD], kj = Us[k + j * LD];
+            Pr[i * LD + (k - i - 1)] = opp ? csub(cmul(ik, Ts[k + j * LD]), cmul(Ts[i + k * LD], kj)) : cmul(ik, kj);
+        }
+        __syncthreads();
+        if (threadIdx.x < bs - d) {
+            const int i = threadIdx.x, j = i + d;
+            double2 s = zero;
+            for (int k = 0; k < terms; k++) s = cadd(s, Pr[i * LD + k]);
+            const double uii = Us[i * (LD + 1)].x, ujj = Us[j * (LD + 1)].x;
+            if (uii + ujj == 0.0)
+                Us[i + j * LD] = cadd(Q1[i + j * LD], cdiv(s, csub(Ts[i * (LD + 1)], Ts[j * (LD + 1)])));
+            else
+                Us[i + j * LD] = scaled(s, -0.5 * uii);   // -s / (+-2)
+        }
+        __syncthreads();
     }
-    if (lane != 0) return;
-    const double uii = sg[i], ujj = sg[j];
-    double2 v;
-    if (opp) {
-        const double2 den = csub(trow[i], tcol[j]);
-        const double2 tij = tcol[i];
-        v = cadd(cdiv(make_double2(tij.x * (uii - ujj), tij.y * (uii - ujj)), den), cdiv(s, den));
-    } else {
-        v = make_double2(-s.x / (uii + ujj), -s.y / (uii + ujj));
-    }
-    U[(size_t)i + (size_t)j * ldu] = v;
-    UR[(size_t)i * n + j] = v;
+    if (in) SGT_AT(U, ldu, r0 + lo, r0 + hi) = Us[at];
 }
 
 // Real and imaginary planes of an n x n complex matrix (ld in complex
@@ -147,27 +146,22 @@ __global__ void join_planes_kernel(int n, const double *__restrict__ re, const d
 size_t complex_workspace_bytes(int n)
 {
     if (n <= 0) return 0;
-    const size_t nn = (size_t)n * n;
-    return 2 * nn * sizeof(double2) + (size_t)n + sizeof(int) + 4 * 256;
+    return lvl::level_workspace_bytes<double2>(n) + sizeof(int) + 256;
 }
 
 signtri_status complex_sign_run(int n, const double *T, int ldt, double *U, int ldu, Arena &ws, int *bad_index,
                                 cudaStream_t st)
 {
     if (n <= 0) return SIGNTRI_OK;
-    const size_t nn = (size_t)n * n;
-    auto *UR = static_cast<double2 *>(ws.take(nn * sizeof(double2)));
-    auto *TR = static_cast<double2 *>(ws.take(nn * sizeof(double2)));
-    auto *sg = static_cast<signed char *>(ws.take((size_t)n));
     auto *bad = static_cast<int *>(ws.take(sizeof(int)));
-    if (!UR || !TR || !sg || !bad) return SIGNTRI_ERR_NO_WORKSPACE;
+    if (!bad) return SIGNTRI_ERR_NO_WORKSPACE;
     const auto *Tc = reinterpret_cast<const double2 *>(T);
     auto *Uc = reinterpret_cast<double2 *>(U);
     const int big = INT_MAX;
     SGT_CUDA_TRY(cudaMemcpyAsync(bad, &big, sizeof(int), cudaMemcpyHostToDevice, st));
     {
         ProfScope ps(SIGNTRI_KC_SCAN, st);
-        complex_init_kernel<<<n, kThreads, 0, st>>>(n, Tc, ldt, Uc, ldu, UR, TR, sg, bad);
+        complex_init_kernel<<<n, kThreads, 0, st>>>(n, Tc, ldt, Uc, ldu, bad);
         SGT_LAUNCH_CHECK();
     }
     int key = INT_MAX;
@@ -177,14 +171,12 @@ signtri_status complex_sign_run(int n, const double *T, int ldt, double *U, int 
         if (bad_index) *bad_index = key / 4;
         return (signtri_status)(key % 4);
     }
-    for (int d = 1; d < n; d++) {
-        const int entries = n - d;
-        const unsigned blocks = (unsigned)(((size_t)entries * 32 + kThreads - 1) / kThreads);
-        ProfScope ps(SIGNTRI_KC_OFFDIAG_LEAF, st);
-        complex_antidiag_kernel<<<blocks, kThreads, 0, st>>>(n, d, Tc, ldt, TR, Uc, ldu, UR, sg);
+    {
+        ProfScope ps(SIGNTRI_KC_DIAG_LEAF, st);
+        complex_diag_kernel<<<(n + lvl::LB - 1) / lvl::LB, lvl::LT, 0, st>>>(n, Tc, ldt, Uc, ldu);
         SGT_LAUNCH_CHECK();
     }
-    return SIGNTRI_OK;
+    return lvl::launch_levels<false>(n, Tc, ldt, Uc, ldu, ws, st);
 }
 
 size_t complex_schur_workspace_bytes(int n)

@@ -36,7 +36,7 @@ constexpr size_t noalloc_need()
 constexpr size_t kNoallocBytes = ((kScanSlot + noalloc_need() + 4095) / 4096) * 4096;
 static_assert(ph::mm_form_workspace_bytes(kNoallocMaxN, 64) <= kNoallocBytes - kScanSlot, "b = 64 at the maximum n");
 static_assert(ph::mm_form_workspace_bytes(kNoallocMaxN, 32) <= kNoallocBytes - kScanSlot, "b = 32 at the maximum n");
-static_assert(lvl::level_workspace_bytes(kNoallocMaxN) <= kNoallocBytes - kScanSlot, "b = 16 at the maximum n");
+static_assert(lvl::level_workspace_bytes<double>(kNoallocMaxN) <= kNoallocBytes - kScanSlot, "b = 16 at the maximum n");
 static_assert(kNoallocBytes <= ((size_t)16 << 20), "the array stays modest");
 
 __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocBytes];

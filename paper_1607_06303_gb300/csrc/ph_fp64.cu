@@ -120,39 +120,6 @@ diag_level_kernel(int n, const double *__restrict__ T, int ldt, double *__restri
     lvl::diag_leaf(n, T, ldt, U, ldu, blockIdx.x, Ts, Us, Pr, Q1);
 }
 
-// CTAs [0, leaves): the leaves of anti-diagonal d, their early sums in `in`
-// (split sin).  Then every CTA: its share of the early sums of d + 1 into
-// `out` (split sout).
-template <bool general>
-__global__ void __launch_bounds__(lvl::kLevelThreads)
-level_kernel(int n, const double *__restrict__ T, int ldt, double *__restrict__ U, int ldu, int d, int leaves,
-             const __grid_constant__ lvl::Split sin, const double *__restrict__ in,
-             const __grid_constant__ lvl::Split sout, double *__restrict__ out)
-{
-    using namespace lvl;
-    extern __shared__ __align__(16) unsigned char raw[];
-    Smem &sm = *reinterpret_cast<Smem *>(raw);
-    const int c = blockIdx.x;
-    if (c < leaves && threadIdx.x < LT) {
-        const int f = split_owner(sin, (long long)c * sin.cpt), l = split_owner(sin, (long long)(c + 1) * sin.cpt - 1);
-        leaf<general>(n, T, ldt, U, ldu, c, c + d, l - f + 1, in + (size_t)(f + c) * LT, sm);
-    } else {
-        dependency_wait();
-        dependency_release();
-    }
-    if (c >= sout.G) return;
-    __syncthreads();   // the leaf's shared memory is free
-    const int e = d + 1, cpt = sout.cpt;
-    const long long x1 = split_start(sout, c + 1);
-    for (long long x = split_start(sout, c); x < x1;) {
-        const int I = (int)(x / cpt);
-        const long long t0 = (long long)I * cpt, xe = min(x1, t0 + cpt);
-        far_sums<general>(n, T, ldt, U, ldu, I, I + e, I + (int)(x - t0), I + (int)(xe - t0),
-                          out + (size_t)(c + I) * LT, sm);
-        x = xe;
-    }
-}
-
 // One schedule for both forms: per anti-diagonal d, the block sums (if any
 // K-block lies between) then the in-block leaves.  split = true runs the
 // arithmetic-efficient form (one sum per entry, X or Y by the sign pair).
@@ -218,45 +185,10 @@ signtri_status run_b(int n, const double *T, int ldt, double *U, int ldu, bool s
 
 }  // namespace
 
-template <bool general>
-static signtri_status launch_levels(int n, const double *T, int ldt, double *U, int ldu, Arena &ws, cudaStream_t st)
-{
-    const int nb = (n + lvl::LB - 1) / lvl::LB;
-    if (nb < 2) return SIGNTRI_OK;
-    double *slab[2];
-    for (double *&s : slab) {
-        s = static_cast<double *>(ws.take(lvl::level_slabs(n) * lvl::LT * sizeof(double)));
-        if (!s) return SIGNTRI_ERR_NO_WORKSPACE;
-    }
-    SGT_CUDA_TRY(cudaFuncSetAttribute(level_kernel<general>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      lvl::level_smem(lvl::kSms)));
-    cudaLaunchAttribute attr{};
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg{};
-    cfg.blockDim = dim3(lvl::kLevelThreads);
-    cfg.stream = st;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    lvl::Split sin{};
-    for (int d = 0; d < nb; d++) {
-        const int leaves = d > 0 ? nb - d : 0, e = d + 1;
-        lvl::Split sout{};
-        if (e < nb) sout = lvl::make_split(nb - e, e, leaves);
-        cfg.gridDim = dim3(std::max(leaves, sout.G));
-        cfg.dynamicSmemBytes = lvl::level_smem((int)cfg.gridDim.x);
-        ProfScope ps(SIGNTRI_KC_OFFDIAG_LEAF, st);
-        SGT_CUDA_TRY(cudaLaunchKernelEx(&cfg, level_kernel<general>, n, T, ldt, U, ldu, d, leaves, sin,
-                                        (const double *)slab[d & 1], sout, slab[e & 1]));
-        sin = sout;
-    }
-    return SIGNTRI_OK;
-}
-
 signtri_status levels_f64(int n, const double *T, int ldt, double *U, int ldu, bool general, Arena &ws,
                           cudaStream_t st)
 {
-    return general ? launch_levels<true>(n, T, ldt, U, ldu, ws, st) : launch_levels<false>(n, T, ldt, U, ldu, ws, st);
+    return general ? lvl::launch_levels<true>(n, T, ldt, U, ldu, ws, st) : lvl::launch_levels<false>(n, T, ldt, U, ldu, ws, st);
 }
 
 static signtri_status run_16(int n, const double *T, int ldt, double *U, int ldu, Arena &ws, cudaStream_t st)
@@ -297,13 +229,13 @@ signtri_status diag_leaves_f64(int n, const double *T, int ldt, double *U, int l
 size_t ph_fp64_workspace_bytes(int n, int b)
 {
     if (n <= 0 || (b != 16 && b != 32 && b != 64)) return 0;
-    return b == lvl::LB ? lvl::level_workspace_bytes(n) : mm_form_workspace_bytes(n, b);
+    return b == lvl::LB ? lvl::level_workspace_bytes<double>(n) : mm_form_workspace_bytes(n, b);
 }
 
 size_t ph_fp64_split_workspace_bytes(int n, int b)
 {
     if (n <= 0 || (b != 16 && b != 32 && b != 64)) return 0;
-    if (b == lvl::LB) return lvl::level_workspace_bytes(n);
+    if (b == lvl::LB) return lvl::level_workspace_bytes<double>(n);
     const size_t nb = (size_t)(n + b - 1) / b;
     const size_t slabs = max_slabs(n, b);
     const size_t z = slabs == 0 ? 0 : slabs * b * b * sizeof(double) + 256;

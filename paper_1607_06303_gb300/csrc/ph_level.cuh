@@ -32,6 +32,8 @@
 // proceeds and leave the float64 pipe to the others.
 #pragma once
 
+#include <algorithm>
+
 #include "internal.cuh"
 #include "level_split.h"
 #include "ph_bodies.cuh"
@@ -49,6 +51,50 @@ constexpr int BLK = LB * LD;    // doubles per staged block
 __device__ __forceinline__ void dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void dependency_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// ---- arithmetic of real (double) and complex (double2) entries ------------
+__device__ __forceinline__ double mac(double a, double b, double c) { return fma(a, b, c); }     // c + a b
+__device__ __forceinline__ double nmac(double a, double b, double c) { return fma(-a, b, c); }   // c - a b
+__device__ __forceinline__ double2 mac(double2 a, double2 b, double2 c)
+{
+    return make_double2(fma(a.x, b.x, fma(-a.y, b.y, c.x)), fma(a.x, b.y, fma(a.y, b.x, c.y)));
+}
+__device__ __forceinline__ double2 nmac(double2 a, double2 b, double2 c)
+{
+    return make_double2(fma(-a.x, b.x, fma(a.y, b.y, c.x)), fma(-a.x, b.y, fma(-a.y, b.x, c.y)));
+}
+__device__ __forceinline__ double add(double a, double b) { return a + b; }
+__device__ __forceinline__ double2 add(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ double flip_sign(double a, unsigned long long m)
+{
+    return __longlong_as_double(__double_as_longlong(a) ^ m);
+}
+__device__ __forceinline__ double2 flip_sign(double2 a, unsigned long long m)
+{
+    return make_double2(flip_sign(a.x, m), flip_sign(a.y, m));
+}
+__device__ __forceinline__ double re(double a) { return a; }
+__device__ __forceinline__ double re(double2 a) { return a.x; }
+__device__ __forceinline__ double scaled(double a, double r) { return a * r; }
+__device__ __forceinline__ double2 scaled(double2 a, double r) { return make_double2(a.x * r, a.y * r); }
+template <class S>
+__device__ __forceinline__ S real_value(double r);
+template <>
+__device__ __forceinline__ double real_value<double>(double r) { return r; }
+template <>
+__device__ __forceinline__ double2 real_value<double2>(double r) { return make_double2(r, 0.0); }
+// 1 / (a - b); complex by R. L. Smith's algorithm (CACM 5(8), 1962)
+__device__ __forceinline__ double inv_diff(double a, double b) { return 1.0 / (a - b); }
+__device__ __forceinline__ double2 inv_diff(double2 a, double2 b)
+{
+    const double x = a.x - b.x, y = a.y - b.y;
+    if (fabs(x) >= fabs(y)) {
+        const double r = y / x, den = fma(y, r, x);
+        return make_double2(1.0 / den, -r / den);
+    }
+    const double r = x / y, den = fma(x, r, y);
+    return make_double2(r / den, -1.0 / den);
+}
+
 // barrier of one half of a CTA
 __device__ __forceinline__ void half_sync(int half)
 {
@@ -62,17 +108,18 @@ __device__ __forceinline__ int nth_bit(unsigned mask, int r)
     return __ffs(mask) - 1;
 }
 
+template <class S>
 union alignas(16) Smem {
     struct {
-        double AU[2][LB * LB], AT[2][LB * LB];   // [buffer][k * 16 + row]
-        double BU[2][BLK], BT[2][BLK];           // [buffer][column * 17 + k]
+        S AU[2][LB * LB], AT[2][LB * LB];   // [buffer][k * 16 + row]
+        S BU[2][BLK], BT[2][BLK];           // [buffer][column * 17 + k]
     } far[2];                                    // per half of the CTA
     struct {
-        double TI[BLK], UI[BLK], TJ[BLK], UJ[BLK];       // diagonal blocks, [row + column * 17]
-        double T1[BLK], U1[BLK], T2[BLK], U2[BLK];       // blocks (I, I+1) and (J-1, J)
-        double X1[BLK], X2[BLK];                         // U of blocks (I+1, J) and (I, J-1)
-        double C[BLK], V[BLK];
-        double urow[LB], ucol[LB];
+        S TI[BLK], UI[BLK], TJ[BLK], UJ[BLK];       // diagonal blocks, [row + column * 17]
+        S T1[BLK], U1[BLK], T2[BLK], U2[BLK];       // blocks (I, I+1) and (J-1, J)
+        S X1[BLK], X2[BLK];                         // U of blocks (I+1, J) and (I, J-1)
+        S C[BLK], V[BLK];
+        S urow[LB], ucol[LB];
     } leaf;
 };
 
@@ -82,15 +129,17 @@ union alignas(16) Smem {
 // Small launches ask for less, so that they start beside the one before and
 // have their operands loaded when it ends.
 constexpr int kSmallLaunch = 64;
+template <class S>
 constexpr int level_smem(int G)
 {
     const int per = (G + kSms - 1) / kSms;
     const int b = (227 - per) / per * 1024;
-    return G > kSmallLaunch && b > (int)sizeof(Smem) ? b : (int)sizeof(Smem);
+    return G > kSmallLaunch && b > (int)sizeof(Smem<S>) ? b : (int)sizeof(Smem<S>);
 }
+template <class S>
 constexpr size_t level_workspace_bytes(int n)
 {
-    return level_slabs(n) == 0 ? 0 : 2 * (level_slabs(n) * LT * sizeof(double) + 256);
+    return level_slabs(n) == 0 ? 0 : 2 * (level_slabs(n) * LT * sizeof(S) + 256);
 }
 
 // Early sums of tile (I, J) over the K-blocks [kb0, kb1) of I .. J, written to
@@ -106,20 +155,20 @@ constexpr size_t level_workspace_bytes(int n)
 // its own pace (one fills the float64 pipes while the other waits at its
 // barrier), and add up at the end; the next K-block is in flight in registers
 // while one is summed.
-template <bool general>
-__device__ __forceinline__ void far_sums(int n, const double *__restrict__ T, int ldt, const double *__restrict__ U,
-                                         int ldu, int I, int J, int kb0, int kb1, double *__restrict__ slab,
-                                         Smem &sm)
+template <bool general, class S>
+__device__ __forceinline__ void far_sums(int n, const S *__restrict__ T, int ldt, const S *__restrict__ U,
+                                         int ldu, int I, int J, int kb0, int kb1, S *__restrict__ slab,
+                                         Smem<S> &sm)
 {
     const int r0 = I * LB, c0 = J * LB;
     const int bj = min(LB, n - c0);
     const int half = threadIdx.x / LT, tid = threadIdx.x % LT;
     const int lo = tid % LB, hi = tid / LB, lane = tid & 31;
-    double au, at, bu, bt;
+    S au, at, bu, bt;
     auto fetch = [&](int kb) {
         const bool useUT = kb == I || kb <= J - 2, useTU = kb == J || kb >= I + 2;
         const int k0 = kb * LB;
-        au = at = bu = bt = 0.0;
+        au = at = bu = bt = real_value<S>(0.0);
         // A: rows of block I (lo = row), B: columns of block J (hi = column);
         // only the last block of all can be ragged
         if (useUT) {
@@ -136,7 +185,7 @@ __device__ __forceinline__ void far_sums(int n, const double *__restrict__ T, in
     bool opp = true;
     if (!general) {
         const int g = (lane < LB) ? r0 + lane : c0 + lane - LB;
-        const unsigned pos = __ballot_sync(0xffffffffu, g < n && SGT_AT(T, ldt, g < n ? g : 0, g < n ? g : 0) > 0.0);
+        const unsigned pos = __ballot_sync(0xffffffffu, g < n && re(SGT_AT(T, ldt, g < n ? g : 0, g < n ? g : 0)) > 0.0);
         const unsigned rm = pos & 0xffffu, cm = pos >> 16;
         const int rp = __popc(rm), cp = __popc(cm), rn = LB - rp, cn = LB - cp;
         int t = half ? LT - 1 - tid : tid;
@@ -152,35 +201,35 @@ __device__ __forceinline__ void far_sums(int n, const double *__restrict__ T, in
     const bool any_opp = __any_sync(0xffffffffu, opp), all_opp = __all_sync(0xffffffffu, opp);
     // acc restarts every few K-blocks, its sum so far added to `total`: long
     // sums round as two short chains, at 1 addition in 64 terms
-    double acc = 0.0, total = 0.0;
+    S acc = real_value<S>(0.0), total = acc;
     __syncthreads();   // the buffers may still be read for the CTA's work before
     for (int kb = kb0 + half, buf = 0; kb < kb1; kb += 2, buf ^= 1) {
         auto &F = sm.far[half];
-        double *AU = F.AU[buf], *AT = F.AT[buf], *BU = F.BU[buf], *BT = F.BT[buf];
+        S *AU = F.AU[buf], *AT = F.AT[buf], *BU = F.BU[buf], *BT = F.BT[buf];
         AU[hi * LB + lo] = au;
         AT[hi * LB + lo] = at;
         BU[hi * LD + lo] = bu;
         BT[hi * LD + lo] = bt;
         half_sync(half);
         if (kb + 2 < kb1) fetch(kb + 2);
-        const double *A1 = AU + p, *A2 = AT + p, *B1 = (opp ? BT : BU) + q * LD, *B2 = BU + q * LD;
+        const S *A1 = AU + p, *A2 = AT + p, *B1 = (opp ? BT : BU) + q * LD, *B2 = BU + q * LD;
         if (kb >= I + 2 && kb <= J - 2) {
             if (all_opp) {
-#pragma unroll
+#pragma unroll (sizeof(S) == 8 ? LB : LB / 4)
                 for (int k = 0; k < LB; k++) {
-                    acc = fma(A1[k * LB], B1[k], acc);
-                    acc = fma(-A2[k * LB], B2[k], acc);
+                    acc = mac(A1[k * LB], B1[k], acc);
+                    acc = nmac(A2[k * LB], B2[k], acc);
                 }
             } else if (any_opp) {
 #pragma unroll 4
                 for (int k = 0; k < LB; k++) {
-                    acc = fma(A1[k * LB], B1[k], acc);
-                    const double r = fma(-A2[k * LB], B2[k], acc);
+                    acc = mac(A1[k * LB], B1[k], acc);
+                    const S r = nmac(A2[k * LB], B2[k], acc);
                     if (opp) acc = r;
                 }
             } else {
-#pragma unroll
-                for (int k = 0; k < LB; k++) acc = fma(A1[k * LB], B1[k], acc);
+#pragma unroll (sizeof(S) == 8 ? LB : LB / 4)
+                for (int k = 0; k < LB; k++) acc = mac(A1[k * LB], B1[k], acc);
             }
         } else if (any_opp) {
             // the first and last two K-blocks: one part only, and inside a
@@ -189,7 +238,7 @@ __device__ __forceinline__ void far_sums(int n, const double *__restrict__ T, in
                 const int k1 = kb == I ? p : -1;
 #pragma unroll 4
                 for (int k = 0; k < LB; k++) {
-                    const double r = fma(A1[k * LB], B1[k], acc);
+                    const S r = mac(A1[k * LB], B1[k], acc);
                     if (opp && k > k1) acc = r;
                 }
             }
@@ -197,58 +246,59 @@ __device__ __forceinline__ void far_sums(int n, const double *__restrict__ T, in
                 const int k1 = kb == J ? q : LB;
 #pragma unroll 4
                 for (int k = 0; k < LB; k++) {
-                    const double r = fma(-A2[k * LB], B2[k], acc);
+                    const S r = nmac(A2[k * LB], B2[k], acc);
                     if (opp && k < k1) acc = r;
                 }
             }
         }
         if (((kb - kb0) & 6) == 6) {
-            total += acc;
-            acc = 0.0;
+            total = add(total, acc);
+            acc = real_value<S>(0.0);
         }
         // the other buffer is refilled next; its readers passed the barrier
         // above only after they had finished with it
     }
-    acc += total;
+    acc = add(acc, total);
     __syncthreads();
-    double *part = sm.far[0].AU[0];
+    S *part = sm.far[0].AU[0];
     if (half == 1) part[p + q * LB] = acc;
     __syncthreads();
-    if (half == 0) slab[p + q * LB] = acc + part[p + q * LB];
+    if (half == 0) slab[p + q * LB] = add(acc, part[p + q * LB]);
 }
 
 // Leaf of block (I, J): nslab partial slabs from slab0 on, LT doubles each.
 // Everything that a launch before the last has written may be read before
 // dependency_wait(); for d <= 2 the blocks next to the diagonal are not yet
 // among it.  Run by the first half of the CTA.
-template <bool general>
-__device__ __forceinline__ void leaf(int n, const double *__restrict__ T, int ldt, double *__restrict__ U, int ldu,
-                                     int I, int J, int nslab, const double *__restrict__ slab0, Smem &sm)
+template <bool general, class S>
+__device__ __forceinline__ void leaf(int n, const S *__restrict__ T, int ldt, S *__restrict__ U, int ldu,
+                                     int I, int J, int nslab, const S *__restrict__ slab0, Smem<S> &sm)
 {
     auto &s = sm.leaf;
+    const S zero = real_value<S>(0.0);
     const int d = J - I;
     const int r0 = I * LB, c0 = J * LB;
     const int bj = min(LB, n - c0);
     const int lo = threadIdx.x % LB, hi = threadIdx.x / LB;
     const int at = lo + hi * LD;
     const bool up = lo <= hi, in = hi < bj;
-    s.TI[at] = up ? SGT_AT(T, ldt, r0 + lo, r0 + hi) : 0.0;
-    s.UI[at] = up ? SGT_AT(U, ldu, r0 + lo, r0 + hi) : 0.0;
-    s.TJ[at] = up && in ? SGT_AT(T, ldt, c0 + lo, c0 + hi) : 0.0;
-    s.UJ[at] = up && in ? SGT_AT(U, ldu, c0 + lo, c0 + hi) : 0.0;
-    const double tij = in ? SGT_AT(T, ldt, r0 + lo, c0 + hi) : 0.0;
+    s.TI[at] = up ? SGT_AT(T, ldt, r0 + lo, r0 + hi) : zero;
+    s.UI[at] = up ? SGT_AT(U, ldu, r0 + lo, r0 + hi) : zero;
+    s.TJ[at] = up && in ? SGT_AT(T, ldt, c0 + lo, c0 + hi) : zero;
+    s.UJ[at] = up && in ? SGT_AT(U, ldu, c0 + lo, c0 + hi) : zero;
+    const S tij = in ? SGT_AT(T, ldt, r0 + lo, c0 + hi) : zero;
     if (d >= 2) {
         s.T1[at] = SGT_AT(T, ldt, r0 + lo, r0 + LB + hi);
-        s.T2[at] = in ? SGT_AT(T, ldt, c0 - LB + lo, c0 + hi) : 0.0;
+        s.T2[at] = in ? SGT_AT(T, ldt, c0 - LB + lo, c0 + hi) : zero;
     }
     if (d >= 3) {
         s.U1[at] = SGT_AT(U, ldu, r0 + lo, r0 + LB + hi);
-        s.U2[at] = in ? SGT_AT(U, ldu, c0 - LB + lo, c0 + hi) : 0.0;
+        s.U2[at] = in ? SGT_AT(U, ldu, c0 - LB + lo, c0 + hi) : zero;
     }
     if (threadIdx.x < LB) {
         const int i = threadIdx.x;
         s.urow[i] = SGT_AT(U, ldu, r0 + i, r0 + i);
-        s.ucol[i] = i < bj ? SGT_AT(U, ldu, c0 + i, c0 + i) : 1.0;
+        s.ucol[i] = i < bj ? SGT_AT(U, ldu, c0 + i, c0 + i) : real_value<S>(1.0);
     }
     // the thread's entry: number threadIdx.x along the anti-diagonals
     // step = 15 - p + q, from the bottom-left corner
@@ -260,19 +310,19 @@ __device__ __forceinline__ void leaf(int n, const double *__restrict__ T, int ld
     if (threadIdx.x >= 136) { p = LB - 1 - p; q = LB - 1 - q; }
     const int step = LB - 1 - p + q;
     half_sync(0);
-    const double upp = s.urow[p], uqq = s.ucol[q];
-    const bool opp = general || upp + uqq == 0.0;
+    const S upp = s.urow[p], uqq = s.ucol[q];
+    const bool opp = general || re(upp) + re(uqq) == 0.0;
     // signs agree: 1 / (u_pp + u_qq) is +-1/2 exactly
-    const double rinv = opp ? 1.0 / (s.TI[p + p * LD] - s.TJ[q + q * LD]) : 0.5 * upp;
+    const S rinv = opp ? inv_diff(s.TI[p + p * LD], s.TJ[q + q * LD]) : scaled(upp, 0.5);
     // flips the sign of the row terms where the signs agree
     const unsigned long long flip = opp ? 0ull : 0x8000000000000000ull;
-    const double *M = opp ? s.TI : s.UI, *N = opp ? s.TJ : s.UJ;
-    const double *M1 = opp ? s.T1 : s.U1, *N2 = opp ? s.T2 : s.U2;
+    const S *M = opp ? s.TI : s.UI, *N = opp ? s.TJ : s.UJ;
+    const S *M1 = opp ? s.T1 : s.U1, *N2 = opp ? s.T2 : s.U2;
 
     dependency_wait();
     dependency_release();
     // all of the launch before's results in flight together
-    double x1 = 0.0, x2 = 0.0, u1 = 0.0, u2 = 0.0, v[8];
+    S x1 = zero, x2 = zero, u1 = zero, u2 = zero, v[8];
     if (d >= 2) {
         if (in) x1 = SGT_AT(U, ldu, r0 + LB + lo, c0 + hi);
         x2 = SGT_AT(U, ldu, r0 + lo, c0 - LB + hi);
@@ -282,17 +332,17 @@ __device__ __forceinline__ void leaf(int n, const double *__restrict__ T, int ld
         if (in) u2 = SGT_AT(U, ldu, c0 - LB + lo, c0 + hi);
     }
 #pragma unroll
-    for (int t = 0; t < 8; t++) v[t] = t < nslab ? slab0[(size_t)t * LT + threadIdx.x] : 0.0;
-    double sum = v[0];
+    for (int t = 0; t < 8; t++) v[t] = t < nslab ? slab0[(size_t)t * LT + threadIdx.x] : zero;
+    S sum = v[0];
 #pragma unroll
     for (int t = 1; t < 8; t++)
-        if (t < nslab) sum += v[t];
+        if (t < nslab) sum = add(sum, v[t]);
     for (int t0 = 8; t0 < nslab; t0 += 8) {
 #pragma unroll
-        for (int t = 0; t < 8; t++) v[t] = t0 + t < nslab ? slab0[(size_t)(t0 + t) * LT + threadIdx.x] : 0.0;
+        for (int t = 0; t < 8; t++) v[t] = t0 + t < nslab ? slab0[(size_t)(t0 + t) * LT + threadIdx.x] : zero;
 #pragma unroll
         for (int t = 0; t < 8; t++)
-            if (t0 + t < nslab) sum += v[t];
+            if (t0 + t < nslab) sum = add(sum, v[t]);
     }
     if (d >= 2) {
         s.X1[at] = x1;
@@ -302,27 +352,27 @@ __device__ __forceinline__ void leaf(int n, const double *__restrict__ T, int ld
         s.U1[at] = u1;
         s.U2[at] = u2;
     }
-    const double ui = s.urow[lo], uj = s.ucol[hi];
+    // (u_ii and u_jj are real)
+    const double ui = re(s.urow[lo]), uj = re(s.ucol[hi]);
     const bool o = general || ui + uj == 0.0;
-    s.C[at] = o ? sum : -sum;
-    s.V[at] = o ? tij * (ui - uj) : 0.0;
+    s.C[at] = o ? sum : flip_sign(sum, 0x8000000000000000ull);
+    s.V[at] = o ? scaled(tij, ui - uj) : zero;
     half_sync(0);
     // t_pq (u_pp - u_qq) is as a rule far larger than the terms summed below,
     // so it joins them last, when only the terms of one step are still to come
-    double acc = s.C[p + q * LD];
-    const double base = s.V[p + q * LD];
+    S acc = s.C[p + q * LD];
+    const S base = s.V[p + q * LD];
     if (d >= 2) {
         // (d = 2: both near blocks are the same, and a sum of U U counts it once)
         const bool row = d > 2 || opp;
-#pragma unroll 8
+#pragma unroll (sizeof(S) == 8 ? 8 : 4)
         for (int k = 0; k < LB; k++) {
-            acc = fma(-M1[p + k * LD], s.X1[k + q * LD], acc);
-            const double x = __longlong_as_double(__double_as_longlong(s.X2[p + k * LD]) ^ flip);
-            const double r = fma(x, N2[k + q * LD], acc);
+            acc = nmac(M1[p + k * LD], s.X1[k + q * LD], acc);
+            const S r = mac(flip_sign(s.X2[p + k * LD], flip), N2[k + q * LD], acc);
             if (row) acc = r;
         }
     }
-    if (step == 0) acc += base;
+    if (step == 0) acc = add(acc, base);
     half_sync(0);   // every base is read: V now takes the solution
     for (int st = 0; st < 2 * LB - 1; st++) {
         if (step == st || step == st + 1) {
@@ -330,7 +380,7 @@ __device__ __forceinline__ void leaf(int n, const double *__restrict__ T, int ld
             // kinds of lane (x * 1 + base and x * rinv - 0 round as the plain
             // sum and product)
             const bool now = step == st;
-            acc = fma(acc, now ? rinv : 1.0, now ? -0.0 : base);
+            acc = mac(acc, now ? rinv : real_value<S>(1.0), now ? real_value<S>(-0.0) : base);
             if (now) s.V[p + q * LD] = acc;
         }
         half_sync(0);
@@ -338,10 +388,9 @@ __device__ __forceinline__ void leaf(int n, const double *__restrict__ T, int ld
             const int k1 = LB - 1 + q - st;   // solved at this step in the entry's column ...
             const int k2 = st - (LB - 1) + p;   // ... and in its row
             if (k2 >= 0) {
-                const double x = __longlong_as_double(__double_as_longlong(s.V[p + k2 * LD]) ^ flip);
-                acc = fma(x, N[k2 + q * LD], acc);
+                acc = mac(flip_sign(s.V[p + k2 * LD], flip), N[k2 + q * LD], acc);
             }
-            if (k1 < LB) acc = fma(-M[p + k1 * LD], s.V[k1 + q * LD], acc);
+            if (k1 < LB) acc = nmac(M[p + k1 * LD], s.V[k1 + q * LD], acc);
         }
     }
     if (in) SGT_AT(U, ldu, r0 + lo, c0 + hi) = s.V[at];
@@ -394,6 +443,75 @@ __device__ __forceinline__ void diag_leaf(int n, const double *__restrict__ T, i
         __syncthreads();
     }
     if (in) SGT_AT(U, ldu, r0 + lo, r0 + hi) = Us[at];
+}
+
+// CTAs [0, leaves): the leaves of anti-diagonal d, their early sums in `in`
+// (split sin).  Then every CTA: its share of the early sums of d + 1 into
+// `out` (split sout).
+template <bool general, class S>
+__global__ void __launch_bounds__(kLevelThreads)
+level_kernel(int n, const S *__restrict__ T, int ldt, S *__restrict__ U, int ldu, int d, int leaves,
+             const __grid_constant__ Split sin, const S *__restrict__ in,
+             const __grid_constant__ Split sout, S *__restrict__ out)
+{
+    extern __shared__ __align__(16) unsigned char raw[];
+    Smem<S> &sm = *reinterpret_cast<Smem<S> *>(raw);
+    const int c = blockIdx.x;
+    if (c < leaves && threadIdx.x < LT) {
+        const int f = split_owner(sin, (long long)c * sin.cpt), l = split_owner(sin, (long long)(c + 1) * sin.cpt - 1);
+        leaf<general>(n, T, ldt, U, ldu, c, c + d, l - f + 1, in + (size_t)(f + c) * LT, sm);
+    } else {
+        dependency_wait();
+        dependency_release();
+    }
+    if (c >= sout.G) return;
+    __syncthreads();   // the leaf's shared memory is free
+    const int e = d + 1, cpt = sout.cpt;
+    const long long x1 = split_start(sout, c + 1);
+    for (long long x = split_start(sout, c); x < x1;) {
+        const int I = (int)(x / cpt);
+        const long long t0 = (long long)I * cpt, xe = min(x1, t0 + cpt);
+        far_sums<general>(n, T, ldt, U, ldu, I, I + e, I + (int)(x - t0), I + (int)(xe - t0),
+                          out + (size_t)(c + I) * LT, sm);
+        x = xe;
+    }
+}
+
+// Every off-diagonal block of U, the diagonal blocks being solved; workspace:
+// level_workspace_bytes.
+template <bool general, class S>
+signtri_status launch_levels(int n, const S *T, int ldt, S *U, int ldu, Arena &ws, cudaStream_t st)
+{
+    const int nb = (n + LB - 1) / LB;
+    if (nb < 2) return SIGNTRI_OK;
+    S *slab[2];
+    for (S *&s : slab) {
+        s = static_cast<S *>(ws.take(level_slabs(n) * LT * sizeof(S)));
+        if (!s) return SIGNTRI_ERR_NO_WORKSPACE;
+    }
+    SGT_CUDA_TRY(cudaFuncSetAttribute(level_kernel<general, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      level_smem<S>(kSms)));
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.blockDim = dim3(kLevelThreads);
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    Split sin{};
+    for (int d = 0; d < nb; d++) {
+        const int leaves = d > 0 ? nb - d : 0, e = d + 1;
+        Split sout{};
+        if (e < nb) sout = make_split(nb - e, e, leaves);
+        cfg.gridDim = dim3(std::max(leaves, sout.G));
+        cfg.dynamicSmemBytes = level_smem<S>((int)cfg.gridDim.x);
+        ProfScope ps(SIGNTRI_KC_OFFDIAG_LEAF, st);
+        SGT_CUDA_TRY(cudaLaunchKernelEx(&cfg, level_kernel<general, S>, n, T, ldt, U, ldu, d, leaves, sin,
+                                        (const S *)slab[d & 1], sout, slab[e & 1]));
+        sin = sout;
+    }
+    return SIGNTRI_OK;
 }
 
 }  // namespace lvl
