@@ -47,8 +47,16 @@ typedef enum {
        by default Parlett-Sylvester when no swaps are needed and the batched
        Parlett-Higham (efficient form) otherwise. */
     SIGNTRI_AUTO = 0,
-    /* Recursive Parlett-Higham (Algorithms 3-6), float64 throughout; block
-       sums in matrix-multiply form (both X and Y for every entry). */
+    /* Recursive Parlett-Higham (Algorithms 3-6) in float64; with leaves of
+       32 or 64 (signtri_set_cutoff) the block sums in matrix-multiply form
+       (both X and Y for every entry), with leaves of 16 as
+       SIGNTRI_PH_FP64_EFFICIENT.  From n = 1600 on with leaves of 16 the sums
+       between superblocks of 128 run on the tensor cores, exact but for
+       rounding their operands to 53 or more bits of their row's or column's
+       largest entry (no larger an error against 64 bits than the float64
+       sums measured); rows or columns that one scale does not suit (graded by
+       more than about 2^24) and non-finite entries of T or U are left to the
+       float64 sums. */
     SIGNTRI_PH_FP64 = 1,
     /* Parlett-Sylvester for the sign function (Section 2, Section 3,
        Section 5.1): reorder by sign with adjacent Givens swaps, solve
@@ -78,9 +86,9 @@ typedef enum {
     SIGNTRI_PH_MIXED_BF16 = 4,
     /* Arithmetic-efficient recursive Parlett-Higham (Section 5.3), float64:
        each entry's block sum is X (signs differ) or Y (signs agree) only,
-       n^3/3..2n^3/3 flops instead of n^3.  Every sum runs over the same
-       terms in the same order as in SIGNTRI_PH_FP64, so the two results
-       agree bit for bit (up to the sign of zero).  Workspace: see
+       n^3/3..2n^3/3 flops instead of n^3.  For one leaf size every sum runs
+       over the same terms in the same order as in SIGNTRI_PH_FP64, so the two
+       results agree bit for bit (up to the sign of zero).  Workspace: see
        signtri_workspace_bytes. */
     SIGNTRI_PH_FP64_EFFICIENT = 5,
     /* As SIGNTRI_PH_MIXED_TF32, with each block-update operand split into
@@ -139,7 +147,10 @@ typedef struct {
 const char *signtri_status_string(signtri_status s);
 
 /* Bytes of device workspace sign_tri needs for size n and variant v with the
-   current cutoff (0 when none).  Returns 0 for invalid arguments. */
+   current cutoff (0 when none).  Returns 0 for invalid arguments.  The float64
+   Parlett-Higham forms also run in less (a caller's workspace without room
+   for the superblocks' operands), down to the leaves' partial sums, by
+   float64 sums alone. */
 size_t signtri_workspace_bytes(int n, signtri_variant v);
 
 /* Use caller-owned device memory [dev_ptr, dev_ptr+bytes) as the workspace of
@@ -190,7 +201,8 @@ signtri_status signtri_set_cutoff(int b);
 /* U = sign(T).  T, U device pointers (see conventions).  Enqueued on
    `stream`; the host waits after the inertia scan to read three integers
    (n_pos, n_neg, swaps) and the error flags.  The float64 Parlett-Higham
-   forms then enqueue their launches and return without waiting for them;
+   forms then enqueue their launches and return without waiting for them
+   (from n = 1600 on with leaves of 16 they return after U is written);
    Parlett-Sylvester also waits while it builds its swap schedule from the
    diagonal, and the mixed variants wait a few times (diagonal signs,
    residual norms) and return after U is written.

@@ -139,6 +139,25 @@ int current_cutoff_locked()
     return g_cutoff ? g_cutoff : kDefaultCutoff;
 }
 
+// From this order on the float64 Parlett-Higham forms with leaves of 16 run
+// by superblocks with their sums on the tensor cores (ph_super.cu): 2.95 /
+// 4.1 / 11.8 / 40.7 ms at n = 1537 / 2000 / 4096 / 8192, against 2.7 / 5.0 /
+// 32 / 270 ms by float64 sums alone (p = 0.3 random).
+constexpr int kSuperMin = 1600;
+bool super_runs(int n, int cutoff) { return n >= kSuperMin && cutoff == 16; }
+
+// What the float64 Parlett-Higham forms work in; with less (a caller's
+// workspace), down to the plain path's, the plain path runs.
+size_t ph_plain_need(int n, int cutoff, bool split)
+{
+    return split ? ph_fp64_split_workspace_bytes(n, cutoff) : ph_fp64_workspace_bytes(n, cutoff);
+}
+size_t ph_workspace_need(int n, int cutoff, bool split)
+{
+    const size_t plain = ph_plain_need(n, cutoff, split);
+    return super_runs(n, cutoff) ? std::max(plain, ph_super_workspace_bytes(n)) : plain;
+}
+
 // swaps < 0: the worst case over inertia (n^2/4 swaps).
 size_t workspace_need(int n, signtri_variant v, long long swaps)
 {
@@ -146,9 +165,9 @@ size_t workspace_need(int n, signtri_variant v, long long swaps)
     const int cutoff = current_cutoff_locked();
     switch (v) {
     case SIGNTRI_PH_FP64:
-        return ph_fp64_workspace_bytes(n, cutoff);
+        return ph_workspace_need(n, cutoff, false);
     case SIGNTRI_PH_FP64_EFFICIENT:
-        return ph_fp64_split_workspace_bytes(n, cutoff);
+        return ph_workspace_need(n, cutoff, true);
     case SIGNTRI_PH_MIXED_TF32:
     case SIGNTRI_PH_MIXED_BF16:
     case SIGNTRI_PH_MIXED_FP16:
@@ -158,7 +177,7 @@ size_t workspace_need(int n, signtri_variant v, long long swaps)
     case SIGNTRI_PS_FP64:
         return ps_workspace_bytes(n, swaps);
     case SIGNTRI_AUTO:
-        return std::max(ph_fp64_split_workspace_bytes(n, cutoff), ps_workspace_bytes(n, swaps));
+        return std::max(ph_workspace_need(n, cutoff, true), ps_workspace_bytes(n, swaps));
     }
     return 0;
 }
@@ -243,20 +262,39 @@ signtri_variant choose_variant(int n, const ScanResult &r)
     return t_ps < t_ph ? SIGNTRI_PS_FP64 : SIGNTRI_PH_FP64_EFFICIENT;
 }
 
+// The float64 Parlett-Higham forms with leaf size b.
+signtri_status run_ph_fp64(int n, const double *T, int ldt, double *U, int ldu, int b, bool split, cudaStream_t st,
+                           DeviceState &s)
+{
+    Arena ws;
+    if (super_runs(n, b) && get_workspace(s, ph_workspace_need(n, b, split), ws) == SIGNTRI_OK) {
+        SGT_CUDA_TRY(cudaMemsetAsync(s.err_dev, 0, sizeof(int), st));
+        int *flags = reinterpret_cast<int *>(s.norms_host);
+        signtri_status rs = ph_super_run(n, T, ldt, U, ldu, ws, s.err_dev, flags, st);
+        if (rs != SIGNTRI_OK) return rs;
+        SGT_CUDA_TRY(cudaMemcpyAsync(s.err_host, s.err_dev, sizeof(int), cudaMemcpyDeviceToHost, st));
+        SGT_CUDA_TRY(cudaStreamSynchronize(st));
+        if (*s.err_host) return SIGNTRI_ERR_TIMEOUT;
+        if (!*flags) return SIGNTRI_OK;
+        // entries that one scale per row does not suit, or not finite
+    }
+    signtri_status rs = get_workspace(s, ph_plain_need(n, b, split), ws);
+    if (rs != SIGNTRI_OK) return rs;
+    return split ? ph_fp64_split_run(n, T, ldt, U, ldu, b, ws, st) : ph_fp64_run(n, T, ldt, U, ldu, b, ws, st);
+}
+
 signtri_status run_variant(int n, const double *T, int ldt, double *U, int ldu, signtri_variant v,
                            const ScanResult &r, cudaStream_t st, DeviceState &s)
 {
     Arena ws;
     const int b = current_cutoff_locked();
+    if (v == SIGNTRI_PH_FP64 || v == SIGNTRI_PH_FP64_EFFICIENT) {
+        g_info.cutoff = b;
+        return run_ph_fp64(n, T, ldt, U, ldu, b, v == SIGNTRI_PH_FP64_EFFICIENT, st, s);
+    }
     signtri_status rs = get_workspace(s, workspace_need(n, v, r.swaps), ws);
     if (rs != SIGNTRI_OK) return rs;
     switch (v) {
-    case SIGNTRI_PH_FP64:
-        g_info.cutoff = b;
-        return ph_fp64_run(n, T, ldt, U, ldu, b, ws, st);
-    case SIGNTRI_PH_FP64_EFFICIENT:
-        g_info.cutoff = b;
-        return ph_fp64_split_run(n, T, ldt, U, ldu, b, ws, st);
     case SIGNTRI_PS_FP64: {
         SGT_CUDA_TRY(cudaMemsetAsync(s.err_dev, 0, sizeof(int), st));
         rs = ps_fp64_run(n, T, ldt, U, ldu, r.n_pos, r.swaps, ws, s.err_dev, st);
@@ -291,10 +329,7 @@ signtri_status run_variant(int n, const double *T, int ldt, double *U, int ldu, 
             // the residual did not contract: plain float64 path
             g_info.variant = SIGNTRI_PH_FP64;
             g_info.cutoff = b;
-            Arena ws2;
-            rs = get_workspace(s, ph_fp64_workspace_bytes(n, b), ws2);
-            if (rs != SIGNTRI_OK) return rs;
-            return ph_fp64_run(n, T, ldt, U, ldu, b, ws2, st);
+            return run_ph_fp64(n, T, ldt, U, ldu, b, false, st, s);
         }
         return SIGNTRI_OK;
     }

@@ -129,6 +129,12 @@ signtri_status diag_leaves_f64(int n, const double *T, int ldt, double *U, int l
 // ph_fp64_workspace_bytes(n, 16)
 signtri_status levels_f64(int n, const double *T, int ldt, double *U, int ldu, bool general, Arena &ws,
                           cudaStream_t st);
+signtri_status ph_fp64_near_run(int n, const double *T, int ldt, double *U, int ldu, int last, Arena &ws,
+                                cudaStream_t st);
+// superblocks of 128, their sums on the tensor cores (ph_super.cu)
+size_t ph_super_workspace_bytes(int n);
+signtri_status ph_super_run(int n, const double *T, int ldt, double *U, int ldu, Arena &ws, int *d_err,
+                            int *flags_host, cudaStream_t st);
 signtri_status ph_fp64_run(int n, const double *T, int ldt, double *U, int ldu, int b,
                            Arena &ws, cudaStream_t st);
 // arithmetic-efficient form (one sum per entry)

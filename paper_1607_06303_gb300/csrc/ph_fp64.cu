@@ -191,7 +191,10 @@ signtri_status levels_f64(int n, const double *T, int ldt, double *U, int ldu, b
     return general ? lvl::launch_levels<true>(n, T, ldt, U, ldu, ws, st) : lvl::launch_levels<false>(n, T, ldt, U, ldu, ws, st);
 }
 
-static signtri_status run_16(int n, const double *T, int ldt, double *U, int ldu, Arena &ws, cudaStream_t st)
+// zero lower part, diagonal blocks and block anti-diagonals 1 .. last, leaves
+// of 16
+signtri_status ph_fp64_near_run(int n, const double *T, int ldt, double *U, int ldu, int last, Arena &ws,
+                                cudaStream_t st)
 {
     signtri_status rs = launch_zero_strict_lower(n, U, ldu, st);
     if (rs != SIGNTRI_OK) return rs;
@@ -200,7 +203,7 @@ static signtri_status run_16(int n, const double *T, int ldt, double *U, int ldu
         diag_level_kernel<<<(n + lvl::LB - 1) / lvl::LB, lvl::LT, 0, st>>>(n, T, ldt, U, ldu);
         SGT_LAUNCH_CHECK();
     }
-    return levels_f64(n, T, ldt, U, ldu, false, ws, st);
+    return lvl::launch_levels<false>(n, T, ldt, U, ldu, ws, st, last);
 }
 
 signtri_status diag_leaves_f64(int n, const double *T, int ldt, double *U, int ldu, int b, cudaStream_t st)
@@ -246,7 +249,7 @@ signtri_status ph_fp64_split_run(int n, const double *T, int ldt, double *U, int
                                  cudaStream_t st)
 {
     switch (b) {
-    case 16: return run_16(n, T, ldt, U, ldu, ws, st);
+    case 16: return ph_fp64_near_run(n, T, ldt, U, ldu, INT_MAX, ws, st);
     case 32: return run_b<32>(n, T, ldt, U, ldu, true, ws, st);
     case 64: return run_b<64>(n, T, ldt, U, ldu, true, ws, st);
     default: return SIGNTRI_ERR_BAD_ARG;
@@ -257,7 +260,7 @@ signtri_status ph_fp64_run(int n, const double *T, int ldt, double *U, int ldu, 
                            cudaStream_t st)
 {
     switch (b) {
-    case 16: return run_16(n, T, ldt, U, ldu, ws, st);
+    case 16: return ph_fp64_near_run(n, T, ldt, U, ldu, INT_MAX, ws, st);
     case 32: return run_b<32>(n, T, ldt, U, ldu, false, ws, st);
     case 64: return run_b<64>(n, T, ldt, U, ldu, false, ws, st);
     default: return SIGNTRI_ERR_BAD_ARG;

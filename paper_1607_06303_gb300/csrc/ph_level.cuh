@@ -266,6 +266,52 @@ __device__ __forceinline__ void far_sums(int n, const S *__restrict__ T, int ldt
     if (half == 0) slab[p + q * LB] = add(acc, part[p + q * LB]);
 }
 
+// Entry number t of a block along its anti-diagonals step = 15 - p + q, from
+// the bottom-left corner.
+__device__ __forceinline__ void entry_of(int t, int &p, int &q)
+{
+    const int m = t < 136 ? t : 255 - t;
+    int a = (int)((sqrtf(8.f * m + 1.f) - 1.f) * 0.5f);
+    if ((a + 1) * (a + 2) / 2 <= m) a++;
+    if (a * (a + 1) / 2 > m) a--;
+    q = m - a * (a + 1) / 2;
+    p = LB - 1 - a + q;
+    if (t >= 136) { p = LB - 1 - p; q = LB - 1 - q; }
+}
+
+// The block's solve: the thread's entry (p, q) starts as acc (the sums of all
+// terms outside the block) and base (its own term), and takes
+//   - M[p, k] v_kq (k > p)   and   + v_pk N[k, q] (k < q; sign flipped by flip)
+// as the entries of V are solved, step by step; V must not be in use.  The
+// base is as a rule far larger than the other terms, so it joins them last,
+// when only the terms of one step are still to come.
+template <class S>
+__device__ __forceinline__ void solve16(S acc, S base, S rinv, unsigned long long flip, const S *M, const S *N, S *V,
+                                        int p, int q, int step)
+{
+    if (step == 0) acc = add(acc, base);
+    half_sync(0);   // every base is read: V now takes the solution
+    for (int st = 0; st < 2 * LB - 1; st++) {
+        if (step == st || step == st + 1) {
+            // the entry's value, or its base term: one instruction for both
+            // kinds of lane (x * 1 + base and x * rinv - 0 round as the plain
+            // sum and product)
+            const bool now = step == st;
+            acc = mac(acc, now ? rinv : real_value<S>(1.0), now ? real_value<S>(-0.0) : base);
+            if (now) V[p + q * LD] = acc;
+        }
+        half_sync(0);
+        if (st < step) {
+            const int k1 = LB - 1 + q - st;   // solved at this step in the entry's column ...
+            const int k2 = st - (LB - 1) + p;   // ... and in its row
+            if (k2 >= 0) {
+                acc = mac(flip_sign(V[p + k2 * LD], flip), N[k2 + q * LD], acc);
+            }
+            if (k1 < LB) acc = nmac(M[p + k1 * LD], V[k1 + q * LD], acc);
+        }
+    }
+}
+
 // Leaf of block (I, J): nslab partial slabs from slab0 on, LT doubles each.
 // Everything that a launch before the last has written may be read before
 // dependency_wait(); for d <= 2 the blocks next to the diagonal are not yet
@@ -300,14 +346,8 @@ __device__ __forceinline__ void leaf(int n, const S *__restrict__ T, int ldt, S 
         s.urow[i] = SGT_AT(U, ldu, r0 + i, r0 + i);
         s.ucol[i] = i < bj ? SGT_AT(U, ldu, c0 + i, c0 + i) : real_value<S>(1.0);
     }
-    // the thread's entry: number threadIdx.x along the anti-diagonals
-    // step = 15 - p + q, from the bottom-left corner
-    const int m = threadIdx.x < 136 ? threadIdx.x : 255 - threadIdx.x;
-    int a = (int)((sqrtf(8.f * m + 1.f) - 1.f) * 0.5f);
-    if ((a + 1) * (a + 2) / 2 <= m) a++;
-    if (a * (a + 1) / 2 > m) a--;
-    int q = m - a * (a + 1) / 2, p = LB - 1 - a + q;
-    if (threadIdx.x >= 136) { p = LB - 1 - p; q = LB - 1 - q; }
+    int p, q;
+    entry_of(threadIdx.x, p, q);
     const int step = LB - 1 - p + q;
     half_sync(0);
     const S upp = s.urow[p], uqq = s.ucol[q];
@@ -358,8 +398,6 @@ __device__ __forceinline__ void leaf(int n, const S *__restrict__ T, int ldt, S 
     s.C[at] = o ? sum : flip_sign(sum, 0x8000000000000000ull);
     s.V[at] = o ? scaled(tij, ui - uj) : zero;
     half_sync(0);
-    // t_pq (u_pp - u_qq) is as a rule far larger than the terms summed below,
-    // so it joins them last, when only the terms of one step are still to come
     S acc = s.C[p + q * LD];
     const S base = s.V[p + q * LD];
     if (d >= 2) {
@@ -372,27 +410,7 @@ __device__ __forceinline__ void leaf(int n, const S *__restrict__ T, int ldt, S 
             if (row) acc = r;
         }
     }
-    if (step == 0) acc = add(acc, base);
-    half_sync(0);   // every base is read: V now takes the solution
-    for (int st = 0; st < 2 * LB - 1; st++) {
-        if (step == st || step == st + 1) {
-            // the entry's value, or its base term: one instruction for both
-            // kinds of lane (x * 1 + base and x * rinv - 0 round as the plain
-            // sum and product)
-            const bool now = step == st;
-            acc = mac(acc, now ? rinv : real_value<S>(1.0), now ? real_value<S>(-0.0) : base);
-            if (now) s.V[p + q * LD] = acc;
-        }
-        half_sync(0);
-        if (st < step) {
-            const int k1 = LB - 1 + q - st;   // solved at this step in the entry's column ...
-            const int k2 = st - (LB - 1) + p;   // ... and in its row
-            if (k2 >= 0) {
-                acc = mac(flip_sign(s.V[p + k2 * LD], flip), N[k2 + q * LD], acc);
-            }
-            if (k1 < LB) acc = nmac(M[p + k1 * LD], s.V[k1 + q * LD], acc);
-        }
-    }
+    solve16(acc, base, rinv, flip, M, N, s.V, p, q, step);
     if (in) SGT_AT(U, ldu, r0 + lo, c0 + hi) = s.V[at];
 }
 
@@ -477,10 +495,10 @@ level_kernel(int n, const S *__restrict__ T, int ldt, S *__restrict__ U, int ldu
     }
 }
 
-// Every off-diagonal block of U, the diagonal blocks being solved; workspace:
-// level_workspace_bytes.
+// Every off-diagonal block of U up to block anti-diagonal `last`, the diagonal
+// blocks being solved; workspace: level_workspace_bytes.
 template <bool general, class S>
-signtri_status launch_levels(int n, const S *T, int ldt, S *U, int ldu, Arena &ws, cudaStream_t st)
+signtri_status launch_levels(int n, const S *T, int ldt, S *U, int ldu, Arena &ws, cudaStream_t st, int last = INT_MAX)
 {
     const int nb = (n + LB - 1) / LB;
     if (nb < 2) return SIGNTRI_OK;
@@ -500,10 +518,10 @@ signtri_status launch_levels(int n, const S *T, int ldt, S *U, int ldu, Arena &w
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     Split sin{};
-    for (int d = 0; d < nb; d++) {
+    for (int d = 0; d < nb && d <= last; d++) {
         const int leaves = d > 0 ? nb - d : 0, e = d + 1;
         Split sout{};
-        if (e < nb) sout = make_split(nb - e, e, leaves);
+        if (e < nb && e <= last) sout = make_split(nb - e, e, leaves);
         cfg.gridDim = dim3(std::max(leaves, sout.G));
         cfg.dynamicSmemBytes = level_smem<S>((int)cfg.gridDim.x);
         ProfScope ps(SIGNTRI_KC_OFFDIAG_LEAF, st);

@@ -1,0 +1,58 @@
+// rns.cuh -- float64 products on the tensor cores through residues (rns.cu).
+#pragma once
+
+#include <cuda_bf16.h>
+
+#include "internal.cuh"
+
+namespace signtri {
+namespace rns {
+
+// Pairwise coprime moduli; their product is 2^125.3.
+constexpr int kMods = 16;
+constexpr int kModulus[kMods] = {256, 255, 253, 251, 247, 241, 239, 233, 229, 227, 223, 217, 211, 199, 197, 193};
+constexpr int kPanel = 128;                    // rows of a panel, and edge of a product tile
+constexpr int kTileElems = kPanel * 64;        // one panel's K-block of 64, one modulus: 16 KB of bf16
+
+// Bits kept of each operand entry below its row's (column's) power-of-two
+// scale: products of K terms then stay below half the moduli's product.
+constexpr int operand_bits(int K)
+{
+    int lg = 0;
+    while ((1 << lg) < K) lg++;
+    return (124 - lg) / 2;
+}
+
+// The residues of a matrix cut into panels of 128 rows (a row form: rows of
+// M) or of 128 columns (a column form: columns of M), K-contiguous: tile
+// (panel, modulus, K-block) at ((panel * kMods + modulus) * nkb + kblock) *
+// kTileElems, already in the 128-byte swizzle the MMA descriptor names.
+struct Form {
+    __nv_bfloat16 *tiles;
+    int *exps;      // per row (column): entries are below 2^exps
+    int panels;
+    int nkb;
+};
+inline size_t form_tile_bytes(int panels, int nkb) { return (size_t)panels * kMods * nkb * kTileElems * 2; }
+
+// One 128 x 128 product: panel pa of source `src`'s A form times panel pb of
+// its B form over K-blocks [kb0, kb1).
+struct Tile {
+    int src, pa, pb, kb0, kb1;
+};
+struct Source {
+    const __nv_bfloat16 *A, *B;
+    int nkbA, nkbB;
+};
+struct Sources {
+    Source s[3];
+};
+
+// Residues of tiles [0, ntiles) of d_tiles, `per` consecutive tiles sharing
+// panels: out[tile][modulus][row][column], int8, already multiplied by the
+// modulus's cofactor inverse.
+signtri_status gemm(const Sources &src, const Tile *d_tiles, int ntiles, int per, int8_t *out, int *d_err, int cls,
+                    cudaStream_t st);
+
+}  // namespace rns
+}  // namespace signtri

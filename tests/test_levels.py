@@ -40,3 +40,62 @@ def test_levels_vs_oracle(gpu_lib, oracle_mod, n, n_neg):
     # of the sum's size: n eps covers both sides
     assert np.linalg.norm(U - ref) <= n * np.finfo(float).eps * np.linalg.norm(ref)
     assert np.array_equal(np.diag(U), np.sign(np.diag(T))) and np.all(np.tril(U, -1) == 0)
+
+
+# ---- superblocks with residue products (ph_super.cu) ------------------------
+
+def _plain(p, T):
+    """sign(T) by the plain float64 path: a caller's workspace that holds only
+    the leaves' partial sums leaves no room for the superblocks'."""
+    import torch
+    ws = torch.empty(32 << 20, dtype=torch.uint8, device="cuda")
+    assert p.signtri_set_workspace(ws.data_ptr(), ws.numel()) == 0
+    try:
+        U = p.to_numpy(p.sign(p.to_device(T), p.Variant.PH_FP64_EFFICIENT))
+        torch.cuda.synchronize()
+    finally:
+        p.signtri_set_workspace(0, 0)
+    return U
+
+
+def _super(p, T):
+    import torch
+    U = p.to_numpy(p.sign(p.to_device(T), p.Variant.PH_FP64_EFFICIENT))
+    torch.cuda.synchronize()
+    return U
+
+
+# whole superblocks of 128, one row beyond, one short, and a ragged block of 16
+@pytest.mark.gpu
+@pytest.mark.parametrize("n", [1792, 1793, 1919, 2075])
+@pytest.mark.parametrize("n_neg,order", [(1, "random"), (None, "random"), (None, "sorted")])
+def test_superblocks_vs_oracle(gpu_lib, oracle_mod, n, n_neg, order):
+    T = make_T(n, 0.4, seed=n, n_neg=n_neg, order=order)
+    U = _super(gpu_lib, T)
+    ref = oracle_mod.sign_tri(T, schedule="antidiag")
+    # as above; the residue products keep 53 bits of every operand
+    assert np.linalg.norm(U - ref) <= n * np.finfo(float).eps * np.linalg.norm(ref)
+    assert np.array_equal(np.diag(U), np.sign(np.diag(T))) and np.all(np.tril(U, -1) == 0)
+
+
+@pytest.mark.gpu
+def test_superblocks_leave_graded_and_nonfinite_data_to_the_plain_path(gpu_lib):
+    n = 1800
+    T0 = make_T(n, 0.4, seed=5)
+    U0 = _plain(gpu_lib, T0)
+    # T = D^-1 T0 D with powers of two: the plain path's every operation
+    # scales exactly, so it returns D^-1 U0 D to the last bit
+    g = np.round(np.linspace(0.0, 300.0, n)).astype(int)
+    T = np.asfortranarray(np.ldexp(T0, g[None, :] - g[:, None]))
+    U = _super(gpu_lib, T)
+    assert np.array_equal(np.ldexp(U, g[:, None] - g[None, :]), U0)
+    # a NaN in the last corner, which enters the result only if the signs of
+    # its row and column differ, and one where they do
+    s = np.sign(np.diag(T0))
+    opposite = int(np.max(np.nonzero(s != s[0])[0]))
+    for j in (n - 1, opposite):
+        T = T0.copy(order="F")
+        T[0, j] = np.nan
+        U = _super(gpu_lib, T)
+        assert np.array_equal(U, _plain(gpu_lib, T), equal_nan=True)
+        assert np.isnan(U[0, j]) == (s[0] != s[j])
