@@ -293,14 +293,17 @@ signtri_status run_variant(int n, const double *T, int ldt, double *U, int ldu, 
         return run_ph_fp64(n, T, ldt, U, ldu, b, v == SIGNTRI_PH_FP64_EFFICIENT, st, s);
     }
     signtri_status rs = get_workspace(s, workspace_need(n, v, r.swaps), ws);
+    if (rs == SIGNTRI_ERR_NO_WORKSPACE && v == SIGNTRI_PS_FP64)
+        rs = get_workspace(s, ps_workspace_bytes(n, r.swaps, false), ws);   // a caller's, without room for superblocks
     if (rs != SIGNTRI_OK) return rs;
     switch (v) {
     case SIGNTRI_PS_FP64: {
         SGT_CUDA_TRY(cudaMemsetAsync(s.err_dev, 0, sizeof(int), st));
-        rs = ps_fp64_run(n, T, ldt, U, ldu, r.n_pos, r.swaps, ws, s.err_dev, st);
+        rs = ps_fp64_run(n, T, ldt, U, ldu, r.n_pos, r.swaps, ws, s.err_dev, reinterpret_cast<int *>(s.norms_host), st);
         if (rs != SIGNTRI_OK) return rs;
-        if (r.swaps > 0 && n >= kBlockedReorderMin) {
-            // the blocked reorder's tensor-core products wait with a bound
+        if ((r.swaps > 0 && n >= kBlockedReorderMin) || n > 256) {
+            // the tensor-core products (of the blocked reorder, of the
+            // Sylvester solve's superblocks) wait with a bound
             SGT_CUDA_TRY(cudaMemcpyAsync(s.err_host, s.err_dev, sizeof(int), cudaMemcpyDeviceToHost, st));
             SGT_CUDA_TRY(cudaStreamSynchronize(st));
             if (*s.err_host) return SIGNTRI_ERR_TIMEOUT;
@@ -992,9 +995,19 @@ signtri_status signtri_sylvester(int m, int p, const double *A, int lda, const d
     signtri_status rs = current_state(&s);
     if (rs != SIGNTRI_OK) return rs;
     Arena ws;
-    rs = get_workspace(*s, sylvester_workspace_bytes(m, p), ws);
+    // a caller's workspace may hold the plain solve's sums only
+    const size_t plain = sylvester_workspace_bytes(m, p);
+    rs = get_workspace(*s, std::max(plain, sylvester_super_workspace_bytes(m, p)), ws);
+    if (rs == SIGNTRI_ERR_NO_WORKSPACE) rs = get_workspace(*s, plain, ws);
     if (rs != SIGNTRI_OK) return rs;
-    return sylvester_run(m, p, A, lda, B, ldb, C, ldc, 1.0, X, ldx, ws, static_cast<cudaStream_t>(stream));
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    SGT_CUDA_TRY(cudaMemsetAsync(s->err_dev, 0, sizeof(int), st));
+    rs = sylvester_any_run(m, p, A, lda, B, ldb, C, ldc, 1.0, X, ldx, ws, s->err_dev,
+                           reinterpret_cast<int *>(s->norms_host), st);
+    if (rs != SIGNTRI_OK || m + p <= 256) return rs;
+    SGT_CUDA_TRY(cudaMemcpyAsync(s->err_host, s->err_dev, sizeof(int), cudaMemcpyDeviceToHost, st));
+    SGT_CUDA_TRY(cudaStreamSynchronize(st));
+    return *s->err_host ? SIGNTRI_ERR_TIMEOUT : SIGNTRI_OK;
 }
 
 signtri_status signtri_set_workspace(void *dev_ptr, size_t bytes)

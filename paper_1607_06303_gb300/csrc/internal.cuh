@@ -135,6 +135,11 @@ signtri_status ph_fp64_near_run(int n, const double *T, int ldt, double *U, int 
 size_t ph_super_workspace_bytes(int n);
 signtri_status ph_super_run(int n, const double *T, int ldt, double *U, int ldu, Arena &ws, int *d_err,
                             int *flags_host, cudaStream_t st);
+size_t sylvester_super_workspace_bytes(int m, int p);
+size_t sylvester_super_workspace_bound(int n);   // for every m + p = n
+signtri_status sylvester_super_run(int m, int p, const double *A, int lda, const double *B, int ldb, const double *C,
+                                   int ldc, double cscale, double *X, int ldx, Arena &ws, int *d_err, int *flags_host,
+                                   cudaStream_t st);
 signtri_status ph_fp64_run(int n, const double *T, int ldt, double *U, int ldu, int b,
                            Arena &ws, cudaStream_t st);
 // arithmetic-efficient form (one sum per entry)
@@ -149,6 +154,11 @@ signtri_status gemm_f64(bool transA, bool transB, int m, int n, int k, double al
 
 // Parlett-Sylvester pieces (ps_fp64.cu)
 size_t sylvester_workspace_bytes(int m, int p);
+// by superblocks where ws has room for them, else (or where the data does not
+// suit them) by sylvester_run
+signtri_status sylvester_any_run(int m, int p, const double *A, int lda, const double *Bm, int ldb, const double *C,
+                                 int ldc, double cscale, double *X, int ldx, Arena &ws, int *d_err, int *flags_host,
+                                 cudaStream_t st);
 signtri_status sylvester_run(int m, int p, const double *A, int lda, const double *Bm, int ldb, const double *C,
                              int ldc, double cscale, double *X, int ldx, Arena &ws, cudaStream_t st);
 signtri_status copy_upper_identity(int n, const double *T, int ldt, double *Tr, int ldtr, double *Q, int ldq,
@@ -167,9 +177,10 @@ signtri_status reorder_blocked_run(int n, const double *T, int ldt, double *Tr, 
 size_t reorder_any_workspace_bytes(int n, long long swaps);
 signtri_status reorder_any_run(int n, const double *T, int ldt, double *Tr, int ldtr, double *Q, int ldq,
                                long long *swaps_out, Arena &ws, int *d_err, cudaStream_t st);
-size_t ps_workspace_bytes(int n, long long swaps);
+// super = false: without room for the Sylvester solve's superblocks
+size_t ps_workspace_bytes(int n, long long swaps, bool super = true);
 signtri_status ps_fp64_run(int n, const double *T, int ldt, double *U, int ldu, int npos, long long swaps,
-                           Arena &ws, int *d_err, cudaStream_t st);
+                           Arena &ws, int *d_err, int *flags_host, cudaStream_t st);
 
 // bf16 slices and the emulated-float64 GEMM (slices.cu)
 int pad64(int x);

@@ -56,23 +56,27 @@ __device__ __forceinline__ int exponent_above(double x)   // |x| < 2^result
     return ((__double2hiint(x) >> 20) & 0x7ff) - 1022;
 }
 
-// Entry (k, j) of the strictly upper part of the n x n matrix M, 0 elsewhere.
-__device__ __forceinline__ double strict_upper(const double *__restrict__ M, int ld, int n, int k, int j)
-{
-    return (k < j && j < n) ? SGT_AT(M, ld, k, j) : 0.0;
-}
+// A matrix read as rows x cols, or only its strictly upper part.
+struct Mat {
+    const double *M;
+    int ld, rows, cols;
+    bool strict;
+    __device__ __forceinline__ double operator()(int i, int j) const
+    {
+        return i < rows && j < cols && (!strict || i < j) ? SGT_AT(M, ld, i, j) : 0.0;
+    }
+};
 
 // Largest exponents of the rows and columns of superblock (A, B), in shared
 // memory; returns with the block synchronised.
-__device__ __forceinline__ void superblock_exps(const double *__restrict__ M, int ld, int n, int A, int B, int *rmax,
-                                                int *cmax)
+__device__ __forceinline__ void superblock_exps(const Mat &M, int A, int B, int *rmax, int *cmax)
 {
     if (threadIdx.x < SP) rmax[threadIdx.x] = cmax[threadIdx.x] = kNoExp;
     __syncthreads();
     const int i = threadIdx.x % SP, h = threadIdx.x / SP;
     int rm = kNoExp;
     for (int j = h; j < SP; j += kThreads / SP) {
-        const double x = strict_upper(M, ld, n, A * SP + i, B * SP + j);
+        const double x = M(A * SP + i, B * SP + j);
         const int e = x != 0.0 ? exponent_above(x) : kNoExp;
         rm = max(rm, e);
         const int cm = __reduce_max_sync(0xffffffffu, e);
@@ -84,28 +88,28 @@ __device__ __forceinline__ void superblock_exps(const double *__restrict__ M, in
 
 // The exponents of M's superblocks (the diagonal ones only, or all).
 __global__ void __launch_bounds__(kThreads)
-fixed_exps_kernel(const double *__restrict__ M, int ld, int n, bool diagonal_only, int *__restrict__ rexp,
+fixed_exps_kernel(const __grid_constant__ Mat M, bool diagonal_only, int *__restrict__ rexp,
                   int *__restrict__ cexp, int *__restrict__ flags)
 {
     const int A = blockIdx.x, B = diagonal_only ? A : blockIdx.y;
     if (A > B) return;
     __shared__ int rmax[SP], cmax[SP];
-    superblock_exps(M, ld, n, A, B, rmax, cmax);
+    superblock_exps(M, A, B, rmax, cmax);
     if (threadIdx.x < SP) {
-        atomicMax(&rexp[A * SP + threadIdx.x], rmax[threadIdx.x]);
-        atomicMax(&cexp[B * SP + threadIdx.x], cmax[threadIdx.x]);
+        if (rexp) atomicMax(&rexp[A * SP + threadIdx.x], rmax[threadIdx.x]);
+        if (cexp) atomicMax(&cexp[B * SP + threadIdx.x], cmax[threadIdx.x]);
         if (rmax[threadIdx.x] > 1024) atomicOr(flags, 1);
     }
 }
 
-// The exponents of U's new superblocks (t, t + D) that outgrow their row or
+// The exponents of the new superblocks (a0 + t, b0 + t) that outgrow their row or
 // column, and which panels to convert anew.  rnew, cnew: the new superblocks'
 // largest, gathered by the leaves that solved them and reset here.
 __global__ void __launch_bounds__(SP)
-grow_exps_kernel(int D, int *__restrict__ rnew, int *__restrict__ cnew, int *__restrict__ rexp, int *__restrict__ cexp,
+grow_exps_kernel(int a0, int b0, int *__restrict__ rnew, int *__restrict__ cnew, int *__restrict__ rexp, int *__restrict__ cexp,
                  int *__restrict__ rgrown, int *__restrict__ cgrown, int *__restrict__ flags)
 {
-    const int A = blockIdx.x, B = A + D;
+    const int A = a0 + blockIdx.x, B = b0 + blockIdx.x;
     const int r = A * SP + threadIdx.x, c = B * SP + threadIdx.x;
     const int er = rnew[r], ec = cnew[c];
     rnew[r] = kNoExp;
@@ -139,11 +143,10 @@ constexpr ConvConst make_conv_const()
 }
 __constant__ ConvConst c_conv = make_conv_const();
 
-// Residues of one 128 x 128 superblock of M's strictly upper part into panel
-// P's K-blocks 2 K, 2 K + 1.  rows: P holds rows, K counts columns; else P
+// Residues of one 128 x 128 superblock of M into panel P's K-blocks 2 K, 2 K + 1.  rows: P holds rows, K counts columns; else P
 // holds columns and K counts rows.  Part `part` of kConvParts of it.
 constexpr int kConvParts = SP * SP / 8 / kThreads;
-__device__ __forceinline__ void convert_superblock(const double *__restrict__ M, int ld, int n, int bits, bool rows,
+__device__ __forceinline__ void convert_superblock(const Mat &M, int bits, bool rows,
                                                    int P, int K, int part, const int *__restrict__ exps,
                                                    __nv_bfloat16 *__restrict__ tiles, int nkb, int *flags)
 {
@@ -160,7 +163,7 @@ __device__ __forceinline__ void convert_superblock(const double *__restrict__ M,
 #pragma unroll
         for (int t = 0; t < 8; t++) {
             const int k = K * SP + ch * 8 + t;
-            const double x = rows ? strict_upper(M, ld, n, g, k) : strict_upper(M, ld, n, k, g);
+            const double x = rows ? M(g, k) : M(k, g);
             if (x != 0.0) {
                 some++;
                 small += exponent_above(x) < e - kWideBits;
@@ -201,32 +204,39 @@ __device__ __forceinline__ void convert_superblock(const double *__restrict__ M,
     if (threadIdx.x == 0 && some > kThreads / 2) atomicOr(flags, 2);
 }
 
-// All of T's superblocks, both forms and their parts (blockIdx.z).  A row form needs the
-// columns beyond its own superblock, a column form the rows before it.
+// All superblocks above the diagonal ones of a triangular M, both forms (rt,
+// ct; null: not wanted) and their parts (blockIdx.z).
 __global__ void __launch_bounds__(kThreads)
-convert_fixed_kernel(const double *__restrict__ M, int ld, int n, int bits, const int *__restrict__ rexp,
+convert_fixed_kernel(const __grid_constant__ Mat M, int bits, const int *__restrict__ rexp,
                      const int *__restrict__ cexp, __nv_bfloat16 *__restrict__ rt, __nv_bfloat16 *__restrict__ ct,
-                     int nkb, int *__restrict__ flags)
+                     int nkb, bool with_diagonal, int *__restrict__ flags)
 {
-    const int A = blockIdx.x, B = blockIdx.y;
-    if (A >= B) return;
-    const int part = blockIdx.z / 2;
-    if (blockIdx.z % 2 == 0) convert_superblock(M, ld, n, bits, true, A, B, part, rexp, rt, nkb, flags);
-    else convert_superblock(M, ld, n, bits, false, B, A, part, cexp, ct, nkb, flags);
+    const int A = blockIdx.x, B = blockIdx.y, part = blockIdx.z / 2;
+    if (A > B || (A == B && !with_diagonal)) return;
+    if (blockIdx.z % 2 == 0) {
+        if (rt) convert_superblock(M, bits, true, A, B, part, rexp, rt, nkb, flags);
+    } else {
+        if (ct) convert_superblock(M, bits, false, B, A, part, cexp, ct, nkb, flags);
+    }
 }
 
-// U's new superblocks (t, t + D), and the whole of a panel whose scale grew.
+// The new superblocks (A, B) = (a0 + t, b0 + t), and the whole of a panel whose
+// scale grew: of row panel A the superblocks before B (down to low, or to the
+// diagonal when low < 0), of column panel B those below A (up to high, or to
+// the diagonal).
 __global__ void __launch_bounds__(kThreads)
-convert_new_kernel(const double *__restrict__ M, int ld, int n, int bits, int D, const int *__restrict__ rexp,
-                   const int *__restrict__ cexp, const int *__restrict__ rgrown, const int *__restrict__ cgrown,
-                   __nv_bfloat16 *__restrict__ rt, __nv_bfloat16 *__restrict__ ct, int nkb, int *__restrict__ flags)
+convert_new_kernel(const __grid_constant__ Mat M, int bits, int a0, int b0, int low, int high,
+                   const int *__restrict__ rexp, const int *__restrict__ cexp, const int *__restrict__ rgrown,
+                   const int *__restrict__ cgrown, __nv_bfloat16 *__restrict__ rt, int nkbr,
+                   __nv_bfloat16 *__restrict__ ct, int nkbc, int *__restrict__ flags)
 {
-    const int A = blockIdx.x, B = A + D, y = blockIdx.y;
-    const int part = blockIdx.z / 2;
+    const int A = a0 + blockIdx.x, B = b0 + blockIdx.x, y = blockIdx.y, part = blockIdx.z / 2;
     if (blockIdx.z % 2 == 0) {
-        if (y == D || rgrown[A]) convert_superblock(M, ld, n, bits, true, A, A + y, part, rexp, rt, nkb, flags);
+        if (B - y >= (low < 0 ? A : low) && (y == 0 || rgrown[A]))
+            convert_superblock(M, bits, true, A, B - y, part, rexp, rt, nkbr, flags);
     } else {
-        if (y == D || cgrown[B]) convert_superblock(M, ld, n, bits, false, B, B - y, part, cexp, ct, nkb, flags);
+        if (A + y <= (high < 0 ? B : high) && (y == 0 || cgrown[B]))
+            convert_superblock(M, bits, false, B, A + y, part, cexp, ct, nkbc, flags);
     }
 }
 
@@ -244,6 +254,22 @@ __global__ void tiles_kernel(int ns, rns::Tile *__restrict__ tiles)
         t[0] = {0, A, B, 2 * A, 2 * B};
         t[1] = {1, A, B, 2 * (A + 1), 2 * (B + 1)};
         t[2] = {2, A, B, 2 * (A + 1), 2 * B};
+    }
+}
+
+// The products of A X - X B's superblocks, step by step (superblocks (a, b),
+// a = nr - 1 - s + b): X B and A X.
+__global__ void sylvester_tiles_kernel(int nr, int nc, rns::Tile *__restrict__ tiles)
+{
+    const int s = blockIdx.x;
+    int base = 0;
+    for (int u = 0; u < s; u++) base += min(nc - 1, u) - max(0, u - (nr - 1)) + 1;
+    const int b0 = max(0, s - (nr - 1)), b1 = min(nc - 1, s);
+    for (int b = b0 + threadIdx.x; b <= b1; b += blockDim.x) {
+        const int a = nr - 1 - s + b;
+        rns::Tile *t = tiles + 2 * (base + b - b0);
+        t[0] = {0, a, b, 0, 2 * b};
+        t[1] = {1, a, b, 2 * (a + 1), 2 * nr};
     }
 }
 
@@ -304,13 +330,16 @@ struct Wave {
     int *rnew, *cnew;
     int ldrt, ldru, ldct, ldcu, ldc0, ldv;
     int rows, cols, a0, b0, tiles, bits;
+    int products;      // a tile's products in res: 3, or 2 without UU; 0: no sums
+    double own;        // an entry's own term is own (u_pp - u_qq) C0
 };
 
 // The residue sums of entry (i, j) of superblock t, in row panel A and column
 // panel B.
 __device__ __forceinline__ double residue_sum(const Wave &w, int t, int i, int j, bool opp)
 {
-    const int8_t *y = w.res + (size_t)t * 3 * rns::kMods * SP * SP + i * SP + j;
+    if (w.products == 0) return 0.0;
+    const int8_t *y = w.res + (size_t)t * w.products * rns::kMods * SP * SP + i * SP + j;
     const int r = (w.a0 + t) * SP + i, c = (w.b0 + t) * SP + j;
     if (!opp)
         return -scalbn(crt(y + (size_t)2 * rns::kMods * SP * SP), max(w.er0[r], kMinExp) + max(w.ec1[c], kMinExp) - 2 * w.bits);
@@ -412,7 +441,8 @@ __device__ __forceinline__ void wave_far(const Wave &w, int b, int l, double *__
     slabs[(((size_t)k.t * SB + k.jj) * kParts + part) * LT + p + q * LB] = acc;
 }
 
-__device__ __forceinline__ void wave_leaf(const Wave &w, int b, int l, const double *__restrict__ slabs, WaveSmem &sm)
+__device__ __forceinline__ void wave_leaf(const Wave &w, int b, int l, bool first, const double *__restrict__ slabs,
+                                          WaveSmem &sm)
 {
     auto &s = sm.leaf;
     const WaveBlock k = wave_block(w, b, l);
@@ -425,7 +455,7 @@ __device__ __forceinline__ void wave_leaf(const Wave &w, int b, int l, const dou
     }
     const int lo = threadIdx.x % LB, hi = threadIdx.x / LB, at = lo + hi * LD;
     const bool up = lo <= hi, hasU = w.RU != nullptr;
-    if (l == 0) lvl::dependency_wait();   // the residues come from the launch before
+    if (first) lvl::dependency_wait();   // the residues come from the launch before
     const bool inr = r0 + lo < w.rows, inc = c0 + hi < w.cols, in = inr && inc;
     const double *RT = w.RT, *RU = hasU ? w.RU : w.RT, *CT = w.CT, *CU = hasU ? w.CU : w.CT;
     const int ldru = hasU ? w.ldru : w.ldrt, ldcu = hasU ? w.ldcu : w.ldct;
@@ -481,7 +511,7 @@ __device__ __forceinline__ void wave_leaf(const Wave &w, int b, int l, const dou
     s.X2[at] = x2;
     const double ui = s.urow[lo], uj = s.ucol[hi];
     s.C[at] = sum;
-    s.V[at] = ui + uj == 0.0 ? own * (ui - uj) : 0.0;
+    s.V[at] = ui + uj == 0.0 ? own * (w.own * (ui - uj)) : 0.0;
     __syncthreads();
     double acc = s.C[p + q * LD];
     const double base = s.V[p + q * LD];
@@ -509,12 +539,12 @@ __device__ __forceinline__ void wave_leaf(const Wave &w, int b, int l, const dou
 // Step l of every superblock of the launch: its leaves, and beside them the
 // sums of step l + 1 over finished blocks that this step does not change.
 __global__ void __launch_bounds__(kThreads)
-wave_kernel(const __grid_constant__ Wave w, int l, const double *__restrict__ in, double *__restrict__ out)
+wave_kernel(const __grid_constant__ Wave w, int l, bool first, const double *__restrict__ in, double *__restrict__ out)
 {
     __shared__ WaveSmem sm;
     const int leaves = w.tiles * wave_blocks(l), b = blockIdx.x;
     if (b < leaves) {
-        wave_leaf(w, b, l, in, sm);
+        wave_leaf(w, b, l, first, in, sm);
     } else {
         lvl::dependency_wait();
         lvl::dependency_release();
@@ -522,7 +552,7 @@ wave_kernel(const __grid_constant__ Wave w, int l, const double *__restrict__ in
     }
 }
 
-signtri_status run_wave(const Wave &w, double *slab0, double *slab1, cudaStream_t st)
+signtri_status run_wave(const Wave &w, double *slab0, double *slab1, int cls, cudaStream_t st)
 {
     cudaLaunchAttribute attr{};
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -533,10 +563,14 @@ signtri_status run_wave(const Wave &w, double *slab0, double *slab1, cudaStream_
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     double *slab[2] = {slab0, slab1};
-    for (int l = 0; l < 2 * SB - 1; l++) {
+    // the steps that hold blocks (a ragged panel has fewer rows or columns of
+    // them; the first superblock has the most)
+    const int nbr = std::min(SB, (w.rows + LB - 1) / LB - w.a0 * SB), nbc = std::min(SB, (w.cols + LB - 1) / LB - w.b0 * SB);
+    const int l0 = SB - nbr, l1 = SB - 1 + nbc;
+    for (int l = l0; l < l1; l++) {
         cfg.gridDim = dim3(w.tiles * (wave_blocks(l) + kParts * wave_blocks(l + 1)));
-        ProfScope ps(SIGNTRI_KC_OFFDIAG_LEAF, st);
-        SGT_CUDA_TRY(cudaLaunchKernelEx(&cfg, wave_kernel, w, l, (const double *)slab[l & 1], slab[(l + 1) & 1]));
+        ProfScope ps(cls, st);
+        SGT_CUDA_TRY(cudaLaunchKernelEx(&cfg, wave_kernel, w, l, l == l0, (const double *)slab[l & 1], slab[(l + 1) & 1]));
     }
     return SIGNTRI_OK;
 }
@@ -578,6 +612,7 @@ signtri_status ph_super_run(int n, const double *T, int ldt, double *U, int ldu,
     auto *slab1 = static_cast<double *>(take(wave_slab_bytes(ns - 1)));
     int *flags = static_cast<int *>(take(sizeof(int)));
     if (!flags) return SIGNTRI_ERR_NO_WORKSPACE;
+    const Mat Tm{T, ldt, n, n, true}, Um{U, ldu, n, n, true};
     // the diagonal superblocks
     signtri_status rs = ph_fp64_near_run(n, T, ldt, U, ldu, SB - 1, ws, st);
     if (rs != SIGNTRI_OK) return rs;
@@ -587,20 +622,20 @@ signtri_status ph_super_run(int n, const double *T, int ldt, double *U, int ldu,
         SGT_CUDA_TRY(cudaMemsetAsync(flags, 0, sizeof(int), st));
         tiles_kernel<<<ns - 1, 128, 0, st>>>(ns, tiles);
         SGT_LAUNCH_CHECK();
-        fixed_exps_kernel<<<dim3(ns, ns), kThreads, 0, st>>>(T, ldt, n, false, exps[0], exps[1], flags);
+        fixed_exps_kernel<<<dim3(ns, ns), kThreads, 0, st>>>(Tm, false, exps[0], exps[1], flags);
         SGT_LAUNCH_CHECK();
-        convert_fixed_kernel<<<dim3(ns, ns, 2 * kConvParts), kThreads, 0, st>>>(T, ldt, n, bits, exps[0], exps[1], form[0], form[1],
-                                                                  nkb, flags);
+        convert_fixed_kernel<<<dim3(ns, ns, 2 * kConvParts), kThreads, 0, st>>>(Tm, bits, exps[0], exps[1], form[0],
+                                                                                form[1], nkb, false, flags);
         SGT_LAUNCH_CHECK();
-        fixed_exps_kernel<<<ns, kThreads, 0, st>>>(U, ldu, n, true, exps[4], exps[5], flags);
+        fixed_exps_kernel<<<ns, kThreads, 0, st>>>(Um, true, exps[4], exps[5], flags);
         SGT_LAUNCH_CHECK();
     }
     auto join = [&](int D) -> signtri_status {
         ProfScope ps(SIGNTRI_KC_CONVERT, st);
-        grow_exps_kernel<<<ns - D, SP, 0, st>>>(D, exps[4], exps[5], exps[2], exps[3], rgrown, cgrown, flags);
+        grow_exps_kernel<<<ns - D, SP, 0, st>>>(0, D, exps[4], exps[5], exps[2], exps[3], rgrown, cgrown, flags);
         SGT_LAUNCH_CHECK();
-        convert_new_kernel<<<dim3(ns - D, D + 1, 2 * kConvParts), kThreads, 0, st>>>(U, ldu, n, bits, D, exps[2], exps[3], rgrown,
-                                                                       cgrown, form[2], form[3], nkb, flags);
+        convert_new_kernel<<<dim3(ns - D, D + 1, 2 * kConvParts), kThreads, 0, st>>>(
+            Um, bits, 0, D, -1, -1, exps[2], exps[3], rgrown, cgrown, form[2], nkb, form[3], nkb, flags);
         SGT_LAUNCH_CHECK();
         return SIGNTRI_OK;
     };
@@ -613,10 +648,118 @@ signtri_status ph_super_run(int n, const double *T, int ldt, double *U, int ldu,
         if (rs != SIGNTRI_OK) return rs;
         at += nt;
         const Wave w{T, U, T, U, T, U, res, exps[2], exps[1], exps[0], exps[3], exps[4], exps[5], ldt, ldu, ldt, ldu, ldt, ldu,
-                     n, n, 0, D, nt, bits};
-        if ((rs = run_wave(w, slab0, slab1, st)) != SIGNTRI_OK) return rs;
+                     n, n, 0, D, nt, bits, 3, 1.0};
+        if ((rs = run_wave(w, slab0, slab1, SIGNTRI_KC_OFFDIAG_LEAF, st)) != SIGNTRI_OK) return rs;
         if (D + 1 < ns && (rs = join(D)) != SIGNTRI_OK) return rs;
     }
+    SGT_CUDA_TRY(cudaMemcpyAsync(flags_host, flags, sizeof(int), cudaMemcpyDeviceToHost, st));
+    SGT_CUDA_TRY(cudaStreamSynchronize(st));
+    return SIGNTRI_OK;
+}
+
+// ---- A X - X B = C -----------------------------------------------------------------
+
+static size_t sylvester_super_bytes(int nr, int nc, int nt)
+{
+    using namespace sup;
+    size_t b = 2 * (wave_slab_bytes(nt) + 256) + 3 * ((size_t)(nr + nc) * SP * sizeof(int) + 512) + 256;
+    if (nr + nc > 2)
+        b += rns::form_tile_bytes(nr, 2 * nr) + rns::form_tile_bytes(nc, 2 * nc) + rns::form_tile_bytes(nr, 2 * nc) +
+             rns::form_tile_bytes(nc, 2 * nr) + (size_t)nr * nc * 2 * sizeof(rns::Tile) +
+             (size_t)nt * 2 * rns::kMods * SP * SP + (size_t)(nr + nc) * sizeof(int) + 8 * 256;
+    return b;
+}
+
+size_t sylvester_super_workspace_bytes(int m, int p)
+{
+    if (m <= 0 || p <= 0) return 0;
+    const int nr = (m + sup::SP - 1) / sup::SP, nc = (p + sup::SP - 1) / sup::SP;
+    return sylvester_super_bytes(nr, nc, std::min(nr, nc));
+}
+
+// for every m + p = n: the forms take 2 (nr + nc)^2 tiles of K-blocks
+size_t sylvester_super_workspace_bound(int n)
+{
+    const int k = (n + sup::SP - 1) / sup::SP + 1;
+    return sylvester_super_bytes(k, 1, k / 2 + 1) + (size_t)k * k / 2 * sizeof(rns::Tile);
+}
+
+// X of A X - X B = cscale C by superblocks of 128 from the bottom-left one,
+// as ph_super_run: the terms between superblocks as residue products, those
+// inside one by wave_kernel.  flags_host (pinned) as there; one superblock
+// needs no products, sets no flag and returns without waiting.
+signtri_status sylvester_super_run(int m, int p, const double *A, int lda, const double *B, int ldb, const double *C,
+                                   int ldc, double cscale, double *X, int ldx, Arena &ws, int *d_err, int *flags_host,
+                                   cudaStream_t st)
+{
+    using namespace sup;
+    const int nr = (m + SP - 1) / SP, nc = (p + SP - 1) / SP, nt = std::min(nr, nc);
+    const int bits = rns::operand_bits(std::max(nr, nc) * SP);
+    const bool products = nr + nc > 2;
+    auto take = [&](size_t b) { return ws.take(b); };
+    auto *slab0 = static_cast<double *>(take(wave_slab_bytes(nt)));
+    auto *slab1 = static_cast<double *>(take(wave_slab_bytes(nt)));
+    // exponents: A's rows, B's columns, X's rows and columns, and of X's newest
+    int *ea = static_cast<int *>(take((size_t)nr * SP * sizeof(int))), *eb = static_cast<int *>(take((size_t)nc * SP * sizeof(int)));
+    int *er = static_cast<int *>(take((size_t)nr * SP * sizeof(int))), *ec = static_cast<int *>(take((size_t)nc * SP * sizeof(int)));
+    int *rnew = static_cast<int *>(take((size_t)nr * SP * sizeof(int))), *cnew = static_cast<int *>(take((size_t)nc * SP * sizeof(int)));
+    int *flags = static_cast<int *>(take(sizeof(int)));
+    if (!flags) return SIGNTRI_ERR_NO_WORKSPACE;
+    *flags_host = 0;
+    const Mat Am{A, lda, m, m, true}, Bm{B, ldb, p, p, true}, Xm{X, ldx, m, p, false};
+    __nv_bfloat16 *fa = nullptr, *fb = nullptr, *fr = nullptr, *fc = nullptr;
+    rns::Tile *tiles = nullptr;
+    int8_t *res = nullptr;
+    int *rgrown = nullptr, *cgrown = nullptr;
+    {
+        ProfScope ps(SIGNTRI_KC_CONVERT, st);
+        for (int *e : {ea, er, rnew}) SGT_CUDA_TRY(cudaMemsetAsync(e, 0xc0, (size_t)nr * SP * sizeof(int), st));
+        for (int *e : {eb, ec, cnew}) SGT_CUDA_TRY(cudaMemsetAsync(e, 0xc0, (size_t)nc * SP * sizeof(int), st));
+        if (products) {
+            fa = static_cast<__nv_bfloat16 *>(take(rns::form_tile_bytes(nr, 2 * nr)));
+            fb = static_cast<__nv_bfloat16 *>(take(rns::form_tile_bytes(nc, 2 * nc)));
+            fr = static_cast<__nv_bfloat16 *>(take(rns::form_tile_bytes(nr, 2 * nc)));
+            fc = static_cast<__nv_bfloat16 *>(take(rns::form_tile_bytes(nc, 2 * nr)));
+            tiles = static_cast<rns::Tile *>(take((size_t)nr * nc * 2 * sizeof(rns::Tile)));
+            res = static_cast<int8_t *>(take((size_t)nt * 2 * rns::kMods * SP * SP));
+            rgrown = static_cast<int *>(take((size_t)nr * sizeof(int)));
+            cgrown = static_cast<int *>(take((size_t)nc * sizeof(int)));
+            if (!cgrown) return SIGNTRI_ERR_NO_WORKSPACE;
+            SGT_CUDA_TRY(cudaMemsetAsync(flags, 0, sizeof(int), st));
+            sylvester_tiles_kernel<<<nr + nc - 1, 128, 0, st>>>(nr, nc, tiles);
+            SGT_LAUNCH_CHECK();
+            fixed_exps_kernel<<<dim3(nr, nr), kThreads, 0, st>>>(Am, false, ea, nullptr, flags);
+            SGT_LAUNCH_CHECK();
+            fixed_exps_kernel<<<dim3(nc, nc), kThreads, 0, st>>>(Bm, false, nullptr, eb, flags);
+            SGT_LAUNCH_CHECK();
+            convert_fixed_kernel<<<dim3(nr, nr, 2 * kConvParts), kThreads, 0, st>>>(Am, bits, ea, nullptr, fa, nullptr,
+                                                                                    2 * nr, false, flags);
+            SGT_LAUNCH_CHECK();
+            convert_fixed_kernel<<<dim3(nc, nc, 2 * kConvParts), kThreads, 0, st>>>(Bm, bits, nullptr, eb, nullptr, fb,
+                                                                                    2 * nc, false, flags);
+            SGT_LAUNCH_CHECK();
+        }
+    }
+    const rns::Sources src{{{fr, fb, 2 * nc, 2 * nc}, {fa, fc, 2 * nr, 2 * nr}, {}}};
+    size_t at = 0;
+    for (int s = 0; s < nr + nc - 1; s++) {
+        const int b0 = std::max(0, s - (nr - 1)), cnt = std::min(nc - 1, s) - b0 + 1, a0 = nr - 1 - s + b0;
+        signtri_status rs = SIGNTRI_OK;
+        if (s > 0 && (rs = rns::gemm(src, tiles + 2 * at, 2 * cnt, 2, res, d_err, SIGNTRI_KC_SYLV_SUMS, st)) != SIGNTRI_OK)
+            return rs;
+        at += cnt;
+        const Wave w{A, nullptr, B, nullptr, C, X, res, er, eb, ea, ec, rnew, cnew, lda, 0, ldb, 0, ldc, ldx,
+                     m, p, a0, b0, cnt, bits, s > 0 ? 2 : 0, 0.5 * cscale};
+        if ((rs = run_wave(w, slab0, slab1, SIGNTRI_KC_SYLV_LEAF, st)) != SIGNTRI_OK) return rs;
+        if (s + 1 == nr + nc - 1) break;
+        ProfScope ps(SIGNTRI_KC_CONVERT, st);
+        grow_exps_kernel<<<cnt, SP, 0, st>>>(a0, b0, rnew, cnew, er, ec, rgrown, cgrown, flags);
+        SGT_LAUNCH_CHECK();
+        convert_new_kernel<<<dim3(cnt, std::max(b0 + cnt, nr - a0), 2 * kConvParts), kThreads, 0, st>>>(
+            Xm, bits, a0, b0, 0, nr - 1, er, ec, rgrown, cgrown, fr, 2 * nc, fc, 2 * nr, flags);
+        SGT_LAUNCH_CHECK();
+    }
+    if (!products) return SIGNTRI_OK;
     SGT_CUDA_TRY(cudaMemcpyAsync(flags_host, flags, sizeof(int), cudaMemcpyDeviceToHost, st));
     SGT_CUDA_TRY(cudaStreamSynchronize(st));
     return SIGNTRI_OK;

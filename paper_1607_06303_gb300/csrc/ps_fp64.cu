@@ -416,6 +416,20 @@ signtri_status sylvester_run(int m, int p, const double *A, int lda, const doubl
     return SIGNTRI_OK;
 }
 
+signtri_status sylvester_any_run(int m, int p, const double *A, int lda, const double *Bm, int ldb, const double *C,
+                                 int ldc, double cscale, double *X, int ldx, Arena &ws, int *d_err, int *flags_host,
+                                 cudaStream_t st)
+{
+    const size_t mark = ws.used;
+    if (ws.bytes - ws.used >= sylvester_super_workspace_bytes(m, p)) {
+        const signtri_status rs =
+            sylvester_super_run(m, p, A, lda, Bm, ldb, C, ldc, cscale, X, ldx, ws, d_err, flags_host, st);
+        if (rs != SIGNTRI_OK || !*flags_host) return rs;
+        ws.used = mark;
+    }
+    return sylvester_run(m, p, A, lda, Bm, ldb, C, ldc, cscale, X, ldx, ws, st);
+}
+
 signtri_status copy_upper_identity(int n, const double *T, int ldt, double *Tr, int ldtr, double *Q, int ldq,
                                    cudaStream_t st)
 {
@@ -495,11 +509,13 @@ static size_t back_transform_workspace_bytes(int n, int npos)
     return std::max(emulated_product_workspace_bytes(npos, n, nneg), emulated_product_workspace_bytes(n, n, npos));
 }
 
-size_t ps_workspace_bytes(int n, long long swaps)
+size_t ps_workspace_bytes(int n, long long swaps, bool super)
 {
     if (n <= 0) return 0;
     const size_t nn = (size_t)n * n * sizeof(double) + 256;
-    size_t b = sylvester_workspace_bytes(n, n) + nn /* X */;
+    size_t syl = sylvester_workspace_bytes(n, n);
+    if (super) syl = std::max(syl, sylvester_super_workspace_bound(n));
+    size_t b = syl + nn /* X */;
     if (swaps > 0) {
         // T~, Q, W; then the reorder's space, reused by the Sylvester solve and
         // the back-transform (bounded over every inertia)
@@ -513,13 +529,13 @@ size_t ps_workspace_bytes(int n, long long swaps)
 }
 
 signtri_status ps_fp64_run(int n, const double *T, int ldt, double *U, int ldu, int npos, long long swaps,
-                           Arena &ws, int *d_err, cudaStream_t st)
+                           Arena &ws, int *d_err, int *flags_host, cudaStream_t st)
 {
     const int nneg = n - npos;
     if (swaps == 0) {
         // already grouped: T~ = T, Q = I, sign(T) = [I X; 0 -I]
-        signtri_status rs = sylvester_run(npos, nneg, T, ldt, &SGT_AT(T, ldt, npos, npos), ldt, &SGT_AT(T, ldt, 0, npos),
-                                          ldt, 2.0, &SGT_AT(U, ldu, 0, npos), ldu, ws, st);
+        signtri_status rs = sylvester_any_run(npos, nneg, T, ldt, &SGT_AT(T, ldt, npos, npos), ldt, &SGT_AT(T, ldt, 0, npos),
+                                          ldt, 2.0, &SGT_AT(U, ldu, 0, npos), ldu, ws, d_err, flags_host, st);
         if (rs != SIGNTRI_OK) return rs;
         ProfScope ps(SIGNTRI_KC_FILL, st);
         sorted_blocks_kernel<<<n, 256, 0, st>>>(n, npos, U, ldu);
@@ -536,8 +552,8 @@ signtri_status ps_fp64_run(int n, const double *T, int ldt, double *U, int ldu, 
     signtri_status rs = reorder_any_run(n, T, ldt, Tr, n, Q, n, &done, ws, d_err, st);
     if (rs != SIGNTRI_OK) return rs;
     ws.used = mark;   // the reorder's scratch is free again (stream order)
-    rs = sylvester_run(npos, nneg, Tr, n, &SGT_AT(Tr, n, npos, npos), n, &SGT_AT(Tr, n, 0, npos), n, 2.0, X, npos,
-                       ws, st);
+    rs = sylvester_any_run(npos, nneg, Tr, n, &SGT_AT(Tr, n, npos, npos), n, &SGT_AT(Tr, n, 0, npos), n, 2.0, X, npos,
+                           ws, d_err, flags_host, st);
     if (rs != SIGNTRI_OK) return rs;
     ws.used = mark;
     const double *Q1 = Q;

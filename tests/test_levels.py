@@ -99,3 +99,16 @@ def test_superblocks_leave_graded_and_nonfinite_data_to_the_plain_path(gpu_lib):
         U = _super(gpu_lib, T)
         assert np.array_equal(U, _plain(gpu_lib, T), equal_nan=True)
         assert np.isnan(U[0, j]) == (s[0] != s[j])
+
+
+# Parlett-Sylvester on a grouped diagonal: X of T11 X - X T22 = 2 T12 by
+# superblocks, whole ones, ragged rows, ragged columns, a few columns only
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,n_neg", [(20, 4), (256, 128), (146, 17), (559, 259), (417, 400), (1500, 3)])
+def test_sylvester_superblocks_vs_oracle(gpu_lib, oracle_mod, n, n_neg):
+    import torch
+    T = make_T(n, seed=n + n_neg, n_neg=n_neg, order="sorted")
+    U = gpu_lib.to_numpy(gpu_lib.sign(gpu_lib.to_device(T), gpu_lib.Variant.PS_FP64))
+    torch.cuda.synchronize()
+    ref = oracle_mod.sign_tri(T, schedule="antidiag")
+    assert np.linalg.norm(U - ref) <= n * np.finfo(float).eps * np.linalg.norm(ref)
