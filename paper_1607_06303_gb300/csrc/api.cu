@@ -155,7 +155,7 @@ size_t ph_plain_need(int n, int cutoff, bool split)
 size_t ph_workspace_need(int n, int cutoff, bool split)
 {
     const size_t plain = ph_plain_need(n, cutoff, split);
-    return super_runs(n, cutoff) ? std::max(plain, ph_super_workspace_bytes(n)) : plain;
+    return super_runs(n, cutoff) ? plain + ph_super_workspace_bytes(1, &n) : plain;
 }
 
 // swaps < 0: the worst case over inertia (n^2/4 swaps).
@@ -262,7 +262,17 @@ signtri_variant choose_variant(int n, const ScanResult &r)
     return t_ps < t_ph ? SIGNTRI_PS_FP64 : SIGNTRI_PH_FP64_EFFICIENT;
 }
 
-// The float64 Parlett-Higham forms with leaf size b.
+// The float64 Parlett-Higham forms with leaf size b, by float64 sums alone.
+signtri_status run_ph_plain(int n, const double *T, int ldt, double *U, int ldu, int b, bool split, cudaStream_t st,
+                            DeviceState &s)
+{
+    Arena ws;
+    signtri_status rs = get_workspace(s, ph_plain_need(n, b, split), ws);
+    if (rs != SIGNTRI_OK) return rs;
+    return split ? ph_fp64_split_run(n, T, ldt, U, ldu, b, ws, st) : ph_fp64_run(n, T, ldt, U, ldu, b, ws, st);
+}
+
+// The same, by superblocks where they are faster.
 signtri_status run_ph_fp64(int n, const double *T, int ldt, double *U, int ldu, int b, bool split, cudaStream_t st,
                            DeviceState &s)
 {
@@ -270,7 +280,10 @@ signtri_status run_ph_fp64(int n, const double *T, int ldt, double *U, int ldu, 
     if (super_runs(n, b) && get_workspace(s, ph_workspace_need(n, b, split), ws) == SIGNTRI_OK) {
         SGT_CUDA_TRY(cudaMemsetAsync(s.err_dev, 0, sizeof(int), st));
         int *flags = reinterpret_cast<int *>(s.norms_host);
-        signtri_status rs = ph_super_run(n, T, ldt, U, ldu, ws, s.err_dev, flags, st);
+        signtri_status rs = ph_fp64_near_run(n, T, ldt, U, ldu, kSuperNear, ws, st);
+        if (rs != SIGNTRI_OK) return rs;
+        const BatchDesc m{T, U, n, ldt, ldu, 0};
+        rs = ph_super_run(1, &m, ws, s.err_dev, flags, st);
         if (rs != SIGNTRI_OK) return rs;
         SGT_CUDA_TRY(cudaMemcpyAsync(s.err_host, s.err_dev, sizeof(int), cudaMemcpyDeviceToHost, st));
         SGT_CUDA_TRY(cudaStreamSynchronize(st));
@@ -278,9 +291,7 @@ signtri_status run_ph_fp64(int n, const double *T, int ldt, double *U, int ldu, 
         if (!*flags) return SIGNTRI_OK;
         // entries that one scale per row does not suit, or not finite
     }
-    signtri_status rs = get_workspace(s, ph_plain_need(n, b, split), ws);
-    if (rs != SIGNTRI_OK) return rs;
-    return split ? ph_fp64_split_run(n, T, ldt, U, ldu, b, ws, st) : ph_fp64_run(n, T, ldt, U, ldu, b, ws, st);
+    return run_ph_plain(n, T, ldt, U, ldu, b, split, st, s);
 }
 
 signtri_status run_variant(int n, const double *T, int ldt, double *U, int ldu, signtri_variant v,
@@ -388,6 +399,70 @@ int cutoff_for(int n)
 {
     const int k = size_bucket(n);
     return g_cutoff_table[k] ? g_cutoff_table[k] : current_cutoff_locked();
+}
+
+// In a batch, from this order on a problem's far sums run by superblocks
+// (ph_super.cu), whose launches all such problems share; in one go as many
+// problems as fit kBatchSuperRoom.
+constexpr int kBatchSuperMin = 512;
+constexpr size_t kBatchSuperRoom = (size_t)32 << 30;
+bool batch_super(int n, int b) { return b == 16 && n >= kBatchSuperMin; }
+
+// Workspace the superblocks of a batch's problems (orders n, leaf sizes b) are
+// given: all of them at once, up to kBatchSuperRoom.
+size_t batch_super_need(const std::vector<int> &n, const std::vector<int> &b)
+{
+    std::vector<int> ns;
+    size_t most = 0;
+    for (size_t k = 0; k < n.size(); k++)
+        if (batch_super(n[k], b[k])) {
+            ns.push_back(n[k]);
+            most = std::max(most, ph_super_workspace_bytes(1, &n[k]));
+        }
+    if (ns.empty()) return 0;
+    return std::max(most, std::min(ph_super_workspace_bytes((int)ns.size(), ns.data()), kBatchSuperRoom));
+}
+
+// The float64 Parlett-Higham problems of a batch (b[k] == 0: not among them):
+// one graph for the leaves and the sums of the smaller ones, then the larger
+// ones' superblocks where ws has room.  plainly: the problems that have to be
+// run on their own by float64 sums.
+signtri_status batched_float64(int cnt, const std::vector<BatchDesc> &h, const BatchDesc *d, const std::vector<int> &b,
+                               bool split, const Arena &ws, std::vector<int> &plainly, cudaStream_t st, DeviceState &s)
+{
+    std::vector<char> near(cnt, 0);
+    std::vector<int> large;
+    const size_t room = ws.bytes - ws.used;
+    for (int k = 0; k < cnt; k++)
+        if (b[k] && batch_super(h[k].n, b[k]) && ph_super_workspace_bytes(1, &h[k].n) + 4096 <= room) {
+            near[k] = 1;
+            large.push_back(k);
+        }
+    Arena sub = ws;
+    signtri_status rs = batched_ph_run(cnt, h.data(), d, b.data(), near.data(), split, sub, st);
+    if (rs != SIGNTRI_OK || large.empty()) return rs;
+    SGT_CUDA_TRY(cudaMemsetAsync(s.err_dev, 0, sizeof(int), st));
+    // the largest first, so that those of a run have about as many levels
+    std::stable_sort(large.begin(), large.end(), [&](int x, int y) { return h[x].n > h[y].n; });
+    for (size_t i = 0; i < large.size();) {
+        std::vector<BatchDesc> run;
+        std::vector<int> ns;
+        const size_t i0 = i;
+        while (i < large.size()) {
+            ns.push_back(h[large[i]].n);
+            if (!run.empty() && ph_super_workspace_bytes((int)ns.size(), ns.data()) + 4096 > room) break;
+            run.push_back(h[large[i++]]);
+        }
+        std::vector<int> flags(run.size());
+        Arena mine = ws;
+        rs = ph_super_run((int)run.size(), run.data(), mine, s.err_dev, flags.data(), st);
+        if (rs != SIGNTRI_OK) return rs;
+        for (size_t q = 0; q < run.size(); q++)
+            if (flags[q]) plainly.push_back(large[i0 + q]);
+    }
+    SGT_CUDA_TRY(cudaMemcpyAsync(s.err_host, s.err_dev, sizeof(int), cudaMemcpyDeviceToHost, st));
+    SGT_CUDA_TRY(cudaStreamSynchronize(st));
+    return *s.err_host ? SIGNTRI_ERR_TIMEOUT : SIGNTRI_OK;
 }
 
 // Synthetic upper-triangular T for the autotuner: counter-based hash
@@ -501,7 +576,8 @@ signtri_status sign_tri_batched(int count, const int *n, const double *const *T,
     const size_t fixed = (size_t)cnt * (sizeof(BatchDesc) + sizeof(ScanResult) + sizeof(int) + sizeof(double)) +
                          8 * 256;
     Arena ws;
-    rs = get_workspace(*s, fixed + plan, ws);
+    rs = get_workspace(*s, fixed + std::max(plan, batch_super_need(sizes, bs)), ws);
+    if (rs == SIGNTRI_ERR_NO_WORKSPACE) rs = get_workspace(*s, fixed + plan, ws);   // without superblocks
     if (rs != SIGNTRI_OK) return rs;
     auto *d_descs = static_cast<BatchDesc *>(ws.take(cnt * sizeof(BatchDesc)));
     auto *d_scan = static_cast<ScanResult *>(ws.take(cnt * sizeof(ScanResult)));
@@ -552,8 +628,13 @@ signtri_status sign_tri_batched(int count, const int *n, const double *const *T,
         if (rs != SIGNTRI_OK) return rs;
     }
     // the efficient form unless the matrix-multiply form was asked for
-    rs = batched_ph_run(cnt, descs.data(), d_descs, ph_bs.data(), v != SIGNTRI_PH_FP64, ws, st);
+    std::vector<int> plainly;
+    rs = batched_float64(cnt, descs, d_descs, ph_bs, v != SIGNTRI_PH_FP64, ws, plainly, st, *s);
     if (rs != SIGNTRI_OK) return rs;
+    for (int k : plainly) {
+        rs = run_ph_plain(sizes[k], descs[k].T, descs[k].ldt, descs[k].U, descs[k].ldu, ph_bs[k], true, st, *s);
+        if (rs != SIGNTRI_OK) info[owner[k]] = rs;
+    }
     for (auto &sv : singles) {
         const int k = sv.first;
         rs = run_variant(sizes[k], descs[k].T, descs[k].ldt, descs[k].U, descs[k].ldu, sv.second, sr[k], st, *s);
@@ -621,8 +702,11 @@ signtri_status signtri_autotune(int n_max, void *stream)
         size_t need = 0;
         std::vector<int> ns(c, nn);
         for (int b : {16, 32, 64}) need = std::max(need, batched_workspace_bytes(c, ns.data(), b));
+        const size_t with_super = std::max(need, batch_super_need(ns, std::vector<int>(c, 16)));
         Arena ws;
-        if ((rs = get_workspace(*s, need + c * sizeof(BatchDesc) + 512, ws)) != SIGNTRI_OK) break;
+        rs = get_workspace(*s, with_super + c * sizeof(BatchDesc) + 512, ws);
+        if (rs == SIGNTRI_ERR_NO_WORKSPACE) rs = get_workspace(*s, need + c * sizeof(BatchDesc) + 512, ws);
+        if (rs != SIGNTRI_OK) break;
         auto *d_h = static_cast<BatchDesc *>(ws.take(c * sizeof(BatchDesc)));
         SGT_CUDA_TRY(cudaMemcpyAsync(d_h, h.data(), c * sizeof(BatchDesc), cudaMemcpyHostToDevice, st));
         float best = 1e30f;
@@ -630,8 +714,8 @@ signtri_status signtri_autotune(int n_max, void *stream)
         for (int b : {16, 32, 64}) {
             std::vector<int> bs(c, b);
             float ms = 0.f;
-            Arena sub = ws;
-            rs = timed([&]() { return batched_ph_run(c, h.data(), d_h, bs.data(), true, sub, st); }, ms);
+            std::vector<int> plainly;
+            rs = timed([&]() { return batched_float64(c, h, d_h, bs, true, ws, plainly, st, *s); }, ms);
             if (rs != SIGNTRI_OK) break;
             if (ms < best) { best = ms; best_b = b; }
         }

@@ -12,6 +12,7 @@
 // are grouped by leaf size (from the cutoff table) because the kernels are
 // specialised on it.
 #include <algorithm>
+#include <climits>
 #include <vector>
 
 #include "internal.cuh"
@@ -140,7 +141,7 @@ batched_level_kernel(const BatchDesc *__restrict__ mats, const int *__restrict__
 struct GroupCache {
     bool valid = false;
     bool split = false;
-    std::vector<int> ns, members;
+    std::vector<int> ns, last, members;
     const BatchDesc *d_mats = nullptr;
     double *PX = nullptr;
     size_t max_slots = 0;
@@ -164,13 +165,13 @@ void cache_drop(GroupCache &gc)
 
 template <int B>
 signtri_status run_group(const BatchDesc *d_mats, const std::vector<int> &members, const std::vector<int> &ns,
-                         bool split, Arena &ws, cudaStream_t st)
+                         const std::vector<int> &last, bool split, Arena &ws, cudaStream_t st)
 {
     int dev = 0;
     SGT_CUDA_TRY(cudaGetDevice(&dev));
     if (dev < 0 || dev >= kCacheDevices) return SIGNTRI_ERR_CUDA;
     GroupCache &gc = g_cache[dev][B == 16 ? 0 : (B == 32 ? 1 : 2)];
-    const bool same_shape = gc.valid && gc.split == split && gc.ns == ns && gc.members == members &&
+    const bool same_shape = gc.valid && gc.split == split && gc.ns == ns && gc.last == last && gc.members == members &&
                             gc.d_mats == d_mats;
     // leaves of 16: one launch per level over lp (both forms are the same);
     // else separate block-sum and leaf launches over p
@@ -178,7 +179,7 @@ signtri_status run_group(const BatchDesc *d_mats, const std::vector<int> &member
     Plan p;
     LevelPlan lp;
     auto plan = [&] {
-        if (levels) make_level_plan(ns, lp);
+        if (levels) make_level_plan(ns, last, lp);
         else make_plan(ns, B, p);
     };
     if (!same_shape) plan();
@@ -331,6 +332,7 @@ signtri_status run_group(const BatchDesc *d_mats, const std::vector<int> &member
     gc.valid = true;
     gc.split = split;
     gc.ns = ns;
+    gc.last = last;
     gc.members = members;
     gc.d_mats = d_mats;
     gc.PX = PX;
@@ -369,24 +371,26 @@ size_t batched_workspace_bytes(int count, const int *n, int B)
 }
 
 // bs[m]: leaf size of matrix m (16, 32 or 64); matrices with bs[m] == 0 are
-// skipped (handled elsewhere).
+// skipped (handled elsewhere).  near[m] (leaves of 16): only the block
+// anti-diagonals within the diagonal superblocks.
 signtri_status batched_ph_run(int count, const BatchDesc *h_mats, const BatchDesc *d_mats, const int *bs,
-                              bool split, Arena &ws, cudaStream_t st)
+                              const char *near, bool split, Arena &ws, cudaStream_t st)
 {
     for (int B : {16, 32, 64}) {
-        std::vector<int> members, ns;
+        std::vector<int> members, ns, last;
         for (int m = 0; m < count; m++)
             if (bs[m] == B) {
                 members.push_back(m);
                 ns.push_back(h_mats[m].n);
+                last.push_back(near[m] ? kSuperNear : INT_MAX);
             }
         if (members.empty()) continue;
         Arena sub = ws;     // each group reuses the workspace after the previous one finished
         signtri_status rs;
         switch (B) {
-        case 16: rs = run_group<16>(d_mats, members, ns, split, sub, st); break;
-        case 32: rs = run_group<32>(d_mats, members, ns, split, sub, st); break;
-        default: rs = run_group<64>(d_mats, members, ns, split, sub, st); break;
+        case 16: rs = run_group<16>(d_mats, members, ns, last, split, sub, st); break;
+        case 32: rs = run_group<32>(d_mats, members, ns, last, split, sub, st); break;
+        default: rs = run_group<64>(d_mats, members, ns, last, split, sub, st); break;
         }
         if (rs != SIGNTRI_OK) return rs;
     }

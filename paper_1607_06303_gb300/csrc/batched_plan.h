@@ -148,13 +148,15 @@ struct LevelPlan {
     size_t slabs = 0;                    // partial slabs of one level, at most
 };
 
-inline void make_level_plan(const std::vector<int> &ns, LevelPlan &p)
+// last[k]: the last block anti-diagonal of matrix k to run here (the rest by
+// superblocks, ph_super.cu).
+inline void make_level_plan(const std::vector<int> &ns, const std::vector<int> &last, LevelPlan &p)
 {
     const int cnt = (int)ns.size(), B = lvl::LB;
     p = LevelPlan();
     for (int k = 0; k < cnt; k++) {
         const int nb = (ns[k] + B - 1) / B;
-        p.nbmax = std::max(p.nbmax, nb);
+        p.nbmax = std::max(p.nbmax, nb - 1 <= last[k] ? nb : last[k] + 1);
         for (int b = 0; b < nb; b++) p.diag.push_back({k, b});
     }
     p.off.assign(p.nbmax + 1, 0);
@@ -162,7 +164,7 @@ inline void make_level_plan(const std::vector<int> &ns, LevelPlan &p)
     for (int d = 1; d < p.nbmax; d++) {
         p.off[d] = (int)p.tiles.size();
         for (int k = 0; k < cnt; k++)
-            for (int I = 0; I + d < (ns[k] + B - 1) / B; I++) p.tiles.push_back({k, I});
+            for (int I = 0; d <= last[k] && I + d < (ns[k] + B - 1) / B; I++) p.tiles.push_back({k, I});
     }
     p.off[p.nbmax] = (int)p.tiles.size();
     for (int e = 1; e < p.nbmax; e++) {

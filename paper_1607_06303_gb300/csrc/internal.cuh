@@ -131,14 +131,19 @@ signtri_status levels_f64(int n, const double *T, int ldt, double *U, int ldu, b
                           cudaStream_t st);
 signtri_status ph_fp64_near_run(int n, const double *T, int ldt, double *U, int ldu, int last, Arena &ws,
                                 cudaStream_t st);
-// superblocks of 128, their sums on the tensor cores (ph_super.cu)
-size_t ph_super_workspace_bytes(int n);
-signtri_status ph_super_run(int n, const double *T, int ldt, double *U, int ldu, Arena &ws, int *d_err,
-                            int *flags_host, cudaStream_t st);
+// superblocks of 128, their sums on the tensor cores (ph_super.cu): everything
+// beyond the diagonal superblocks (ph_fp64_near_run with last = 7) of `count`
+// problems.  flags (host): nonzero where a problem's data did not suit one
+// scale per row and it has to be run plainly; waits for the stream.
+constexpr int kSuperNear = 7;
+size_t ph_super_workspace_bytes(int count, const int *n);
+signtri_status ph_super_run(int count, const BatchDesc *mats, Arena &ws, int *d_err, int *flags, cudaStream_t st);
+// X of A X - X B = cscale C likewise, from the bottom-left superblock; one
+// superblock needs no products, sets no flag and returns without waiting
 size_t sylvester_super_workspace_bytes(int m, int p);
 size_t sylvester_super_workspace_bound(int n);   // for every m + p = n
 signtri_status sylvester_super_run(int m, int p, const double *A, int lda, const double *B, int ldb, const double *C,
-                                   int ldc, double cscale, double *X, int ldx, Arena &ws, int *d_err, int *flags_host,
+                                   int ldc, double cscale, double *X, int ldx, Arena &ws, int *d_err, int *flags,
                                    cudaStream_t st);
 signtri_status ph_fp64_run(int n, const double *T, int ldt, double *U, int ldu, int b,
                            Arena &ws, cudaStream_t st);
@@ -199,7 +204,7 @@ signtri_status emulated_product(int m, int n, int k, const double *A, int lda, c
 // Batched float64 Parlett-Higham (batched.cu)
 size_t batched_workspace_bytes(int count, const int *n, int cutoff_for_all);
 signtri_status batched_ph_run(int count, const BatchDesc *h_mats, const BatchDesc *d_mats, const int *bs,
-                              bool split, Arena &ws, cudaStream_t st);
+                              const char *near, bool split, Arena &ws, cudaStream_t st);
 // Graph-cache counters of the batched path: launches of a cached graph, and
 // graphs built (tables, capture, instantiation), over all devices.
 void batched_cache_stats(long long *hits, long long *builds);

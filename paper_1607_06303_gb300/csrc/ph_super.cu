@@ -24,8 +24,13 @@
 // them.  Data that does not suit one scale per row (most of a superblock's
 // entries below 2^-24 of their row's or column's largest) or is not finite
 // sets a flag, and the caller runs the plain float64 path instead.
+//
+// The kernels work on lists of superblocks of any number of problems (a batch
+// shares its launches), and on A X - X B = C as well, where every entry is of
+// the first kind and rows and columns belong to different matrices.
 #include <algorithm>
 #include <climits>
+#include <vector>
 
 #include "internal.cuh"
 #include "ph_level.cuh"
@@ -49,6 +54,29 @@ constexpr int kWideBits = 24;
 
 namespace {
 
+// One problem: V (U of sign(T), or X) over a set of rows and a set of columns
+// with the operators m of the rows' (RT, RU) and n of the columns' (CT, CU) own
+// triangular matrices; RU, CU null: every entry takes RT, CT.
+struct Problem {
+    const double *RT, *RU, *CT, *CU, *C0;
+    double *V;
+    int ldrt, ldru, ldct, ldcu, ldc0, ldv;
+    int rows, cols;
+    double own;                                 // an entry's own term is own (u_pp - u_qq) C0
+    int bits;
+    bool triangular;                            // V strictly upper, rows and columns the same
+    int *er0, *ec0, *er1, *ec1;                 // exponents: V's rows, CT's columns, RT's rows, V's columns
+    int *rnew, *cnew;                           // of V's newest superblocks
+    int *rgrown, *cgrown;                       // panels whose exponents grew
+    __nv_bfloat16 *vr, *vc, *fm, *fn;           // row and column forms of V, row form of RT, column form of CT
+    int nkbr, nkbc;                             // K-blocks over the rows (vc, fm) and over the columns (vr, fn)
+    int *flags;
+};
+
+struct Super {   // superblock (A, B) of problem k
+    int k, A, B;
+};
+
 // ---- scales and residues ----------------------------------------------------
 
 __device__ __forceinline__ int exponent_above(double x)   // |x| < 2^result
@@ -67,16 +95,31 @@ struct Mat {
     }
 };
 
-// Largest exponents of the rows and columns of superblock (A, B), in shared
-// memory; returns with the block synchronised.
-__device__ __forceinline__ void superblock_exps(const Mat &M, int A, int B, int *rmax, int *cmax)
+// What a pass reads: the rows' operators by rows, the columns' by columns, or V
+// by both.
+enum { kRowOps = 0, kColOps = 1, kV = 2 };
+__device__ __forceinline__ Mat matrix_of(const Problem &p, int what)
 {
+    if (what == kRowOps) return {p.RT, p.ldrt, p.rows, p.rows, true};
+    if (what == kColOps) return {p.CT, p.ldct, p.cols, p.cols, true};
+    return {p.V, p.ldv, p.rows, p.cols, p.triangular};
+}
+
+// The largest exponents of the superblocks' rows (kRowOps), columns (kColOps)
+// or both (kV, into rnew and cnew).
+__global__ void __launch_bounds__(kThreads)
+exps_kernel(const Problem *__restrict__ probs, const Super *__restrict__ list, int what)
+{
+    const Super t = list[blockIdx.x];
+    const Problem p = probs[t.k];
+    const Mat M = matrix_of(p, what);
+    __shared__ int rmax[SP], cmax[SP];
     if (threadIdx.x < SP) rmax[threadIdx.x] = cmax[threadIdx.x] = kNoExp;
     __syncthreads();
     const int i = threadIdx.x % SP, h = threadIdx.x / SP;
     int rm = kNoExp;
     for (int j = h; j < SP; j += kThreads / SP) {
-        const double x = M(A * SP + i, B * SP + j);
+        const double x = M(t.A * SP + i, t.B * SP + j);
         const int e = x != 0.0 ? exponent_above(x) : kNoExp;
         rm = max(rm, e);
         const int cm = __reduce_max_sync(0xffffffffu, e);
@@ -84,42 +127,32 @@ __device__ __forceinline__ void superblock_exps(const Mat &M, int A, int B, int 
     }
     atomicMax(&rmax[i], rm);
     __syncthreads();
-}
-
-// The exponents of M's superblocks (the diagonal ones only, or all).
-__global__ void __launch_bounds__(kThreads)
-fixed_exps_kernel(const __grid_constant__ Mat M, bool diagonal_only, int *__restrict__ rexp,
-                  int *__restrict__ cexp, int *__restrict__ flags)
-{
-    const int A = blockIdx.x, B = diagonal_only ? A : blockIdx.y;
-    if (A > B) return;
-    __shared__ int rmax[SP], cmax[SP];
-    superblock_exps(M, A, B, rmax, cmax);
     if (threadIdx.x < SP) {
-        if (rexp) atomicMax(&rexp[A * SP + threadIdx.x], rmax[threadIdx.x]);
-        if (cexp) atomicMax(&cexp[B * SP + threadIdx.x], cmax[threadIdx.x]);
-        if (rmax[threadIdx.x] > 1024) atomicOr(flags, 1);
+        int *re = what == kRowOps ? p.er1 : p.rnew, *ce = what == kColOps ? p.ec0 : p.cnew;
+        if (what != kColOps) atomicMax(&re[t.A * SP + i], rmax[i]);
+        if (what != kRowOps) atomicMax(&ce[t.B * SP + i], cmax[i]);
+        if (rmax[i] > 1024) atomicOr(p.flags, 1);
     }
 }
 
-// The exponents of the new superblocks (a0 + t, b0 + t) that outgrow their row or
-// column, and which panels to convert anew.  rnew, cnew: the new superblocks'
-// largest, gathered by the leaves that solved them and reset here.
+// The exponents of V's new superblocks that outgrow their row or column, and
+// which panels to convert anew.  rnew, cnew: the new superblocks' largest,
+// gathered by the leaves that solved them and reset here.
 __global__ void __launch_bounds__(SP)
-grow_exps_kernel(int a0, int b0, int *__restrict__ rnew, int *__restrict__ cnew, int *__restrict__ rexp, int *__restrict__ cexp,
-                 int *__restrict__ rgrown, int *__restrict__ cgrown, int *__restrict__ flags)
+grow_exps_kernel(const Problem *__restrict__ probs, const Super *__restrict__ list)
 {
-    const int A = a0 + blockIdx.x, B = b0 + blockIdx.x;
-    const int r = A * SP + threadIdx.x, c = B * SP + threadIdx.x;
-    const int er = rnew[r], ec = cnew[c];
-    rnew[r] = kNoExp;
-    cnew[c] = kNoExp;
-    if (er > 1024) atomicOr(flags, 1);
-    const bool rg = er > rexp[r], cg = ec > cexp[c];
-    if (rg) rexp[r] = er + kHeadroom;
-    if (cg) cexp[c] = ec + kHeadroom;
+    const Super t = list[blockIdx.x];
+    const Problem p = probs[t.k];
+    const int r = t.A * SP + threadIdx.x, c = t.B * SP + threadIdx.x;
+    const int er = p.rnew[r], ec = p.cnew[c];
+    p.rnew[r] = kNoExp;
+    p.cnew[c] = kNoExp;
+    if (er > 1024) atomicOr(p.flags, 1);
+    const bool rg = er > p.er0[r], cg = ec > p.ec1[c];
+    if (rg) p.er0[r] = er + kHeadroom;
+    if (cg) p.ec1[c] = ec + kHeadroom;
     const int ra = __syncthreads_or(rg), ca = __syncthreads_or(cg);
-    if (threadIdx.x == 0) { rgrown[A] = ra; cgrown[B] = ca; }
+    if (threadIdx.x == 0) { p.rgrown[t.A] = ra; p.cgrown[t.B] = ca; }
 }
 
 struct ConvConst {
@@ -153,23 +186,28 @@ __device__ __forceinline__ void convert_superblock(const Mat &M, int bits, bool 
     int small = 0, some = 0;
     const int it = part * kThreads + threadIdx.x;
     {
-        // line `i` of the panel, 8 entries along K from 8 ch; the threads of a
-        // warp run along the matrix's columns, which are contiguous
-        const int i = rows ? it % SP : it / (SP / 8), ch = rows ? it / SP : it % (SP / 8);
+        // line `i` of the panel, 8 entries along K from 8 ch: eight threads write
+        // a line's 128 bytes of a tile (a line each wrote half sectors: 4x
+        // slower); along rows, four lines' entries of a column make a sector
+        const int i = rows ? it / 8 % SP : it / (SP / 8), ch = rows ? it % 8 + it / (8 * SP) * 8 : it % (SP / 8);
         const int g = P * SP + i;
         const int e = max(exps[g], kMinExp);
-        const double sc = __hiloint2double((1023 + bits - e) << 20, 0);
         float dig[8][5];
 #pragma unroll
         for (int t = 0; t < 8; t++) {
             const int k = K * SP + ch * 8 + t;
-            const double x = rows ? M(g, k) : M(k, g);
-            if (x != 0.0) {
-                some++;
-                small += exponent_above(x) < e - kWideBits;
-            }
+            const long long x = __double_as_longlong(rows ? M(g, k) : M(k, g));
+            // |x| 2^(bits - e), rounded, by integer operations (the float64 pipe
+            // is 1 / 64 of the others): the significand moved by the exponents'
+            // difference; subnormal numbers lie below every scale's last bit
+            const int ex = (int)(x >> 52) & 0x7ff;
+            const int sh = (e - bits) - (ex - 1075);
+            long long v = ex ? (x & 0xfffffffffffffll) | 0x10000000000000ll : 0;
+            v = sh <= 0 ? v << min(-sh, 10) : sh < 63 ? (v + (1ll << (sh - 1))) >> sh : 0;
+            if (x < 0) v = -v;
+            some += ex != 0;
+            small += ex != 0 && ex - 1022 < e - kWideBits;
             // bits <= 56: five balanced digits of 14 bits
-            long long v = __double2ll_rn(x * sc);
 #pragma unroll
             for (int d = 0; d < 5; d++) {
                 const int r = ((int)(v & 16383) ^ 8192) - 8192;
@@ -179,6 +217,7 @@ __device__ __forceinline__ void convert_superblock(const Mat &M, int bits, bool 
         }
         const int kb = 2 * K + ch / 8, c8 = ch & 7;
         __nv_bfloat16 *dst = tiles + ((size_t)P * rns::kMods * nkb + kb) * rns::kTileElems + i * 64 + ((c8 ^ (i & 7)) * 8);
+#pragma unroll 4
         for (int m = 0; m < rns::kMods; m++) {
             const float mm = c_conv.m[m], rm = c_conv.rm[m];
             float y[8];
@@ -204,73 +243,57 @@ __device__ __forceinline__ void convert_superblock(const Mat &M, int bits, bool 
     if (threadIdx.x == 0 && some > kThreads / 2) atomicOr(flags, 2);
 }
 
-// All superblocks above the diagonal ones of a triangular M, both forms (rt,
-// ct; null: not wanted) and their parts (blockIdx.z).
+// The operators' superblocks: row form of the rows' (kRowOps), column form of
+// the columns' (kColOps).  blockIdx.y: the parts.
 __global__ void __launch_bounds__(kThreads)
-convert_fixed_kernel(const __grid_constant__ Mat M, int bits, const int *__restrict__ rexp,
-                     const int *__restrict__ cexp, __nv_bfloat16 *__restrict__ rt, __nv_bfloat16 *__restrict__ ct,
-                     int nkb, bool with_diagonal, int *__restrict__ flags)
+convert_ops_kernel(const Problem *__restrict__ probs, const Super *__restrict__ list, int what)
 {
-    const int A = blockIdx.x, B = blockIdx.y, part = blockIdx.z / 2;
-    if (A > B || (A == B && !with_diagonal)) return;
-    if (blockIdx.z % 2 == 0) {
-        if (rt) convert_superblock(M, bits, true, A, B, part, rexp, rt, nkb, flags);
-    } else {
-        if (ct) convert_superblock(M, bits, false, B, A, part, cexp, ct, nkb, flags);
-    }
+    const Super t = list[blockIdx.x];
+    const Problem p = probs[t.k];
+    if (what == kRowOps)
+        convert_superblock(matrix_of(p, what), p.bits, true, t.A, t.B, blockIdx.y, p.er1, p.fm, p.nkbr, p.flags);
+    else
+        convert_superblock(matrix_of(p, what), p.bits, false, t.B, t.A, blockIdx.y, p.ec0, p.fn, p.nkbc, p.flags);
 }
 
-// The new superblocks (A, B) = (a0 + t, b0 + t), and the whole of a panel whose
-// scale grew: of row panel A the superblocks before B (down to low, or to the
-// diagonal when low < 0), of column panel B those below A (up to high, or to
-// the diagonal).
+// V's new superblocks (A, B), and the whole of a panel whose scale grew: of row
+// panel A the superblocks before B, of column panel B those below A, as far
+// as the panels hold any.  blockIdx.z: form and part.
 __global__ void __launch_bounds__(kThreads)
-convert_new_kernel(const __grid_constant__ Mat M, int bits, int a0, int b0, int low, int high,
-                   const int *__restrict__ rexp, const int *__restrict__ cexp, const int *__restrict__ rgrown,
-                   const int *__restrict__ cgrown, __nv_bfloat16 *__restrict__ rt, int nkbr,
-                   __nv_bfloat16 *__restrict__ ct, int nkbc, int *__restrict__ flags)
+convert_new_kernel(const Problem *__restrict__ probs, const Super *__restrict__ list)
 {
-    const int A = a0 + blockIdx.x, B = b0 + blockIdx.x, y = blockIdx.y, part = blockIdx.z / 2;
+    const Super t = list[blockIdx.x];
+    const Problem p = probs[t.k];
+    const Mat M = matrix_of(p, kV);
+    const int part = blockIdx.z / 2;
     if (blockIdx.z % 2 == 0) {
-        if (B - y >= (low < 0 ? A : low) && (y == 0 || rgrown[A]))
-            convert_superblock(M, bits, true, A, B - y, part, rexp, rt, nkbr, flags);
+        const int count = 1 + (p.rgrown[t.A] ? t.B - (p.triangular ? t.A : 0) : 0);
+        for (int y = blockIdx.y; y < count; y += gridDim.y)
+            convert_superblock(M, p.bits, true, t.A, t.B - y, part, p.er0, p.vr, p.nkbc, p.flags);
     } else {
-        if (A + y <= (high < 0 ? B : high) && (y == 0 || cgrown[B]))
-            convert_superblock(M, bits, false, B, A + y, part, cexp, ct, nkbc, flags);
+        const int count = 1 + (p.cgrown[t.B] ? (p.triangular ? t.B : p.nkbr / 2 - 1) - t.A : 0);
+        for (int y = blockIdx.y; y < count; y += gridDim.y)
+            convert_superblock(M, p.bits, false, t.B, t.A + y, part, p.ec1, p.vc, p.nkbr, p.flags);
     }
 }
 
 // ---- products ----------------------------------------------------------------
 
-// The products of every superblock, D by D: UT, TU, UU.
-__global__ void tiles_kernel(int ns, rns::Tile *__restrict__ tiles)
+// Every superblock's products: V N over the finished blocks of its row, M V over
+// those of its column, and, for sign(T), U U.  Triangular V: from the diagonal
+// superblock of the row and to that of the column, whose strictly upper parts
+// are known.
+__global__ void tiles_kernel(const Problem *__restrict__ probs, const Super *__restrict__ list, int count, int products,
+                             rns::Tile *__restrict__ tiles)
 {
-    const int D = blockIdx.x + 1;
-    // superblocks of smaller D: sum_{d < D} (ns - d)
-    const size_t base = (size_t)(D - 1) * ns - (size_t)(D - 1) * D / 2;
-    for (int A = threadIdx.x; A < ns - D; A += blockDim.x) {
-        const int B = A + D;
-        rns::Tile *t = tiles + 3 * (base + A);
-        t[0] = {0, A, B, 2 * A, 2 * B};
-        t[1] = {1, A, B, 2 * (A + 1), 2 * (B + 1)};
-        t[2] = {2, A, B, 2 * (A + 1), 2 * B};
-    }
-}
-
-// The products of A X - X B's superblocks, step by step (superblocks (a, b),
-// a = nr - 1 - s + b): X B and A X.
-__global__ void sylvester_tiles_kernel(int nr, int nc, rns::Tile *__restrict__ tiles)
-{
-    const int s = blockIdx.x;
-    int base = 0;
-    for (int u = 0; u < s; u++) base += min(nc - 1, u) - max(0, u - (nr - 1)) + 1;
-    const int b0 = max(0, s - (nr - 1)), b1 = min(nc - 1, s);
-    for (int b = b0 + threadIdx.x; b <= b1; b += blockDim.x) {
-        const int a = nr - 1 - s + b;
-        rns::Tile *t = tiles + 2 * (base + b - b0);
-        t[0] = {0, a, b, 0, 2 * b};
-        t[1] = {1, a, b, 2 * (a + 1), 2 * nr};
-    }
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= count) return;
+    const Super t = list[i];
+    const Problem &p = probs[t.k];
+    rns::Tile *o = tiles + (size_t)products * i;
+    o[0] = {3 * t.k, t.A, t.B, p.triangular ? 2 * t.A : 0, 2 * t.B};
+    o[1] = {3 * t.k + 1, t.A, t.B, 2 * (t.A + 1), p.triangular ? 2 * (t.B + 1) : p.nkbr};
+    if (products == 3) o[2] = {3 * t.k + 2, t.A, t.B, 2 * (t.A + 1), 2 * t.B};
 }
 
 struct CrtConst {
@@ -316,35 +339,26 @@ __device__ __forceinline__ double crt(const int8_t *__restrict__ y)
 
 // ---- the superblocks' own solve -----------------------------------------------
 
-// Superblock t of a launch: rows A = a0 + t of the row set, columns B = b0 + t
-// of the column set.  M = RT / RU and N = CT / CU are the sets' diagonal
-// superblocks (RU, CU null: every entry takes RT, CT).  The sums over the other superblocks come as residues, three
-// products to a tile: VN = sum v n (its row and column exponents er0, ec0), MV
-// = sum m v (er1, ec1), and, where the signs agree, UU (er0, ec1).  The new
-// entries' exponents go to rnew, cnew.
+// A launch: its superblocks, their residues (products to a superblock; 0: no
+// sums) and the problems they belong to.
 struct Wave {
-    const double *RT, *RU, *CT, *CU, *C0;
-    double *V;
+    const Problem *probs;
+    const Super *list;
     const int8_t *res;
-    const int *er0, *ec0, *er1, *ec1;
-    int *rnew, *cnew;
-    int ldrt, ldru, ldct, ldcu, ldc0, ldv;
-    int rows, cols, a0, b0, tiles, bits;
-    int products;      // a tile's products in res: 3, or 2 without UU; 0: no sums
-    double own;        // an entry's own term is own (u_pp - u_qq) C0
+    int tiles, products;
 };
 
-// The residue sums of entry (i, j) of superblock t, in row panel A and column
-// panel B.
-__device__ __forceinline__ double residue_sum(const Wave &w, int t, int i, int j, bool opp)
+// The residue sums of entry (i, j) of superblock t.
+__device__ __forceinline__ double residue_sum(const Wave &w, const Problem &pr, const Super &s, int t, int i, int j,
+                                              bool opp)
 {
     if (w.products == 0) return 0.0;
     const int8_t *y = w.res + (size_t)t * w.products * rns::kMods * SP * SP + i * SP + j;
-    const int r = (w.a0 + t) * SP + i, c = (w.b0 + t) * SP + j;
+    const int r = s.A * SP + i, c = s.B * SP + j, b2 = 2 * pr.bits;
     if (!opp)
-        return -scalbn(crt(y + (size_t)2 * rns::kMods * SP * SP), max(w.er0[r], kMinExp) + max(w.ec1[c], kMinExp) - 2 * w.bits);
-    return scalbn(crt(y), max(w.er0[r], kMinExp) + max(w.ec0[c], kMinExp) - 2 * w.bits) -
-           scalbn(crt(y + (size_t)rns::kMods * SP * SP), max(w.er1[r], kMinExp) + max(w.ec1[c], kMinExp) - 2 * w.bits);
+        return -scalbn(crt(y + (size_t)2 * rns::kMods * SP * SP), max(pr.er0[r], kMinExp) + max(pr.ec1[c], kMinExp) - b2);
+    return scalbn(crt(y), max(pr.er0[r], kMinExp) + max(pr.ec0[c], kMinExp) - b2) -
+           scalbn(crt(y + (size_t)rns::kMods * SP * SP), max(pr.er1[r], kMinExp) + max(pr.ec1[c], kMinExp) - b2);
 }
 
 // Blocks (i, j) of a superblock at step l = 7 - i + j.
@@ -354,6 +368,8 @@ constexpr int kParts = 3;
 
 struct WaveBlock {
     int t, jj, I, J, c, r;   // tile, place in the step, global blocks, finished blocks below and to the left
+    Super s;
+    Problem p;
 };
 __device__ __forceinline__ WaveBlock wave_block(const Wave &w, int b, int l)
 {
@@ -361,11 +377,12 @@ __device__ __forceinline__ WaveBlock wave_block(const Wave &w, int b, int l)
     const int cnt = wave_blocks(l);
     k.t = b / cnt;
     k.jj = b % cnt;
+    k.s = w.list[k.t];
+    k.p = w.probs[k.s.k];
     const int j = max(0, l - (SB - 1)) + k.jj, i = SB - 1 - (l - j);
-    const int A = w.a0 + k.t, B = w.b0 + k.t;
-    k.I = A * SB + i;
-    k.J = B * SB + j;
-    const int nbr = min(SB, (w.rows + LB - 1) / LB - A * SB);   // row blocks the panel has
+    k.I = k.s.A * SB + i;
+    k.J = k.s.B * SB + j;
+    const int nbr = min(SB, (k.p.rows + LB - 1) / LB - k.s.A * SB);   // row blocks the panel has
     k.c = nbr - 1 - i;
     k.r = j;
     return k;
@@ -391,10 +408,13 @@ __device__ __forceinline__ double at_or_zero(const double *__restrict__ M, int l
     return i < ni && j < nj ? SGT_AT(M, ld, i, j) : 0.0;
 }
 
-__device__ __forceinline__ void wave_far(const Wave &w, int b, int l, double *__restrict__ slabs, WaveSmem &sm)
+__device__ __forceinline__ void wave_far(const Wave &wv, int b, int l, double *__restrict__ slabs, WaveSmem &sm)
 {
-    const WaveBlock k = wave_block(w, b / kParts, l);
+    const WaveBlock k = wave_block(wv, b / kParts, l);
+    const Problem &w = k.p;
     const int part = b % kParts;
+    lvl::dependency_wait();
+    lvl::dependency_release();
     const int r0 = k.I * LB, c0 = k.J * LB;
     if (r0 >= w.rows || c0 >= w.cols) return;
     const int f = far_count(k), per = far_per(f), x0 = part * per, x1 = min(f, x0 + per);
@@ -441,11 +461,12 @@ __device__ __forceinline__ void wave_far(const Wave &w, int b, int l, double *__
     slabs[(((size_t)k.t * SB + k.jj) * kParts + part) * LT + p + q * LB] = acc;
 }
 
-__device__ __forceinline__ void wave_leaf(const Wave &w, int b, int l, bool first, const double *__restrict__ slabs,
+__device__ __forceinline__ void wave_leaf(const Wave &wv, int b, int l, bool first, const double *__restrict__ slabs,
                                           WaveSmem &sm)
 {
     auto &s = sm.leaf;
-    const WaveBlock k = wave_block(w, b, l);
+    const WaveBlock k = wave_block(wv, b, l);
+    const Problem &w = k.p;
     const int r0 = k.I * LB, c0 = k.J * LB;
     if (r0 >= w.rows || c0 >= w.cols) {
         // every CTA waits, so that a launch of absent blocks only does not end
@@ -491,7 +512,7 @@ __device__ __forceinline__ void wave_leaf(const Wave &w, int b, int l, bool firs
     const double *M = opp ? s.TI : s.UI, *N = opp ? s.TJ : s.UJ;
     const double *M1 = opp ? s.T1 : s.U1, *N2 = opp ? s.T2 : s.U2;
     // here a thread takes entry (hi, lo): residues lie row by row
-    s.C[hi + lo * LD] = residue_sum(w, k.t, (k.I % SB) * LB + hi, (k.J % SB) * LB + lo, s.urow[hi] + s.ucol[lo] == 0.0);
+    s.C[hi + lo * LD] = residue_sum(wv, w, k.s, k.t, (k.I % SB) * LB + hi, (k.J % SB) * LB + lo, s.urow[hi] + s.ucol[lo] == 0.0);
     __syncthreads();
 
     lvl::dependency_wait();
@@ -546,13 +567,12 @@ wave_kernel(const __grid_constant__ Wave w, int l, bool first, const double *__r
     if (b < leaves) {
         wave_leaf(w, b, l, first, in, sm);
     } else {
-        lvl::dependency_wait();
-        lvl::dependency_release();
         wave_far(w, b - leaves, l + 1, out, sm);
     }
 }
 
-signtri_status run_wave(const Wave &w, double *slab0, double *slab1, int cls, cudaStream_t st)
+// l0, l1: the first and one past the last step that hold blocks.
+signtri_status run_wave(const Wave &w, int l0, int l1, double *slab0, double *slab1, int cls, cudaStream_t st)
 {
     cudaLaunchAttribute attr{};
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -563,10 +583,6 @@ signtri_status run_wave(const Wave &w, double *slab0, double *slab1, int cls, cu
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     double *slab[2] = {slab0, slab1};
-    // the steps that hold blocks (a ragged panel has fewer rows or columns of
-    // them; the first superblock has the most)
-    const int nbr = std::min(SB, (w.rows + LB - 1) / LB - w.a0 * SB), nbc = std::min(SB, (w.cols + LB - 1) / LB - w.b0 * SB);
-    const int l0 = SB - nbr, l1 = SB - 1 + nbc;
     for (int l = l0; l < l1; l++) {
         cfg.gridDim = dim3(w.tiles * (wave_blocks(l) + kParts * wave_blocks(l + 1)));
         ProfScope ps(cls, st);
@@ -574,195 +590,276 @@ signtri_status run_wave(const Wave &w, double *slab0, double *slab1, int cls, cu
     }
     return SIGNTRI_OK;
 }
-size_t wave_slab_bytes(int tiles) { return (size_t)tiles * SB * kParts * LT * sizeof(double); }
+size_t wave_slab_bytes(size_t tiles) { return tiles * SB * kParts * LT * sizeof(double); }
+
+// ---- host side -------------------------------------------------------------------
+
+int panels_of(int n) { return (n + SP - 1) / SP; }
+
+// What a run of `levels` of superblocks works in besides its problems' own.
+size_t run_bytes(size_t problems, size_t superblocks, size_t ops, size_t widest, int products)
+{
+    return problems * (sizeof(Problem) + 3 * sizeof(rns::Source) + sizeof(int)) + (superblocks + ops) * sizeof(Super) +
+           superblocks * products * sizeof(rns::Tile) + widest * products * rns::kMods * SP * SP +
+           2 * wave_slab_bytes(widest) + 10 * 256;
+}
+// A problem's exponents, growth marks and forms.
+size_t problem_bytes(int nr, int nc, bool forms)
+{
+    size_t b = 3 * ((size_t)(nr + nc) * SP * sizeof(int) + 512) + (size_t)(nr + nc) * sizeof(int) + 512;
+    if (forms)
+        b += rns::form_tile_bytes(nr, 2 * nr) + rns::form_tile_bytes(nc, 2 * nc) + rns::form_tile_bytes(nr, 2 * nc) +
+             rns::form_tile_bytes(nc, 2 * nr) + 4 * 256;
+    return b;
+}
+
+// A set of problems whose superblocks are solved level by level, every level's
+// in the same launches.
+struct Run {
+    std::vector<Problem> probs;
+    std::vector<Super> list;        // level by level
+    std::vector<size_t> off{0};     // where the levels start
+    std::vector<Super> row_ops, col_ops, diagonal;
+    int products = 3;
+    int sums_from = 0;              // the first level with sums
+    int cls_sums, cls_leaf;
+
+    bool reserve(Arena &ws, Problem &p, int nr, int nc, bool forms)
+    {
+        auto ints = [&](size_t n) { return static_cast<int *>(ws.take(n * sizeof(int))); };
+        p.er0 = ints((size_t)nr * SP);
+        p.er1 = ints((size_t)nr * SP);
+        p.rnew = ints((size_t)nr * SP);
+        p.ec0 = ints((size_t)nc * SP);
+        p.ec1 = ints((size_t)nc * SP);
+        p.cnew = ints((size_t)nc * SP);
+        p.rgrown = ints(nr);
+        p.cgrown = ints(nc);
+        p.nkbr = 2 * nr;
+        p.nkbc = 2 * nc;
+        if (!forms) return p.cgrown != nullptr;
+        auto form = [&](int panels, int nkb) {
+            return static_cast<__nv_bfloat16 *>(ws.take(rns::form_tile_bytes(panels, nkb)));
+        };
+        p.fm = form(nr, 2 * nr);
+        p.fn = form(nc, 2 * nc);
+        p.vr = form(nr, 2 * nc);
+        p.vc = form(nc, 2 * nr);
+        return p.vc != nullptr;
+    }
+
+    // flags (host, one per problem): nonzero where the data did not suit one
+    // scale per row; waits for the stream.
+    signtri_status run(Arena &ws, int *d_err, int *flags, cudaStream_t st)
+    {
+        const int np = (int)probs.size(), levels = (int)off.size() - 1;
+        size_t widest = 0;
+        for (int l = 0; l < levels; l++) widest = std::max(widest, off[l + 1] - off[l]);
+        auto *d_probs = static_cast<Problem *>(ws.take(np * sizeof(Problem)));
+        auto *d_src = static_cast<rns::Source *>(ws.take(3 * (size_t)np * sizeof(rns::Source)));
+        auto *d_flags = static_cast<int *>(ws.take(np * sizeof(int)));
+        std::vector<Super> all = list;
+        for (auto *v : {&row_ops, &col_ops, &diagonal}) all.insert(all.end(), v->begin(), v->end());
+        auto *d_list = static_cast<Super *>(ws.take(all.size() * sizeof(Super)));
+        auto *tiles = static_cast<rns::Tile *>(ws.take(list.size() * products * sizeof(rns::Tile)));
+        auto *res = static_cast<int8_t *>(ws.take(widest * products * rns::kMods * SP * SP));
+        auto *slab0 = static_cast<double *>(ws.take(wave_slab_bytes(widest)));
+        auto *slab1 = static_cast<double *>(ws.take(wave_slab_bytes(widest)));
+        if (!slab1) return SIGNTRI_ERR_NO_WORKSPACE;
+        std::vector<rns::Source> src(3 * (size_t)np);
+        for (int k = 0; k < np; k++) {
+            Problem &p = probs[k];
+            p.flags = d_flags + k;
+            src[3 * k] = {p.vr, p.fn, p.nkbc, p.nkbc};
+            src[3 * k + 1] = {p.fm, p.vc, p.nkbr, p.nkbr};
+            src[3 * k + 2] = {p.vr, p.vc, p.nkbc, p.nkbr};
+        }
+        SGT_CUDA_TRY(cudaMemcpyAsync(d_probs, probs.data(), np * sizeof(Problem), cudaMemcpyHostToDevice, st));
+        SGT_CUDA_TRY(cudaMemcpyAsync(d_src, src.data(), src.size() * sizeof(rns::Source), cudaMemcpyHostToDevice, st));
+        SGT_CUDA_TRY(cudaMemcpyAsync(d_list, all.data(), all.size() * sizeof(Super), cudaMemcpyHostToDevice, st));
+        SGT_CUDA_TRY(cudaMemsetAsync(d_flags, 0, np * sizeof(int), st));
+        const bool sums = levels > sums_from;
+        {
+            ProfScope ps(SIGNTRI_KC_CONVERT, st);
+            for (const Problem &p : probs) {   // below every exponent
+                for (int *e : {p.er0, p.er1, p.rnew}) SGT_CUDA_TRY(cudaMemsetAsync(e, 0xc0, (size_t)p.nkbr / 2 * SP * sizeof(int), st));
+                for (int *e : {p.ec0, p.ec1, p.cnew}) SGT_CUDA_TRY(cudaMemsetAsync(e, 0xc0, (size_t)p.nkbc / 2 * SP * sizeof(int), st));
+            }
+            if (sums) {
+                tiles_kernel<<<(unsigned)((list.size() + 255) / 256), 256, 0, st>>>(d_probs, d_list, (int)list.size(),
+                                                                                    products, tiles);
+                SGT_LAUNCH_CHECK();
+                const Super *rl = d_list + list.size(), *cl = rl + row_ops.size();
+                for (int what : {kRowOps, kColOps}) {
+                    const Super *l = what == kRowOps ? rl : cl;
+                    const unsigned n = (unsigned)(what == kRowOps ? row_ops.size() : col_ops.size());
+                    exps_kernel<<<n, kThreads, 0, st>>>(d_probs, l, what);
+                    SGT_LAUNCH_CHECK();
+                    convert_ops_kernel<<<dim3(n, kConvParts), kThreads, 0, st>>>(d_probs, l, what);
+                    SGT_LAUNCH_CHECK();
+                }
+            }
+        }
+        // V's superblocks [l, l + n) join its forms
+        auto join = [&](const Super *l, size_t n, int longest) -> signtri_status {
+            ProfScope ps(SIGNTRI_KC_CONVERT, st);
+            grow_exps_kernel<<<(unsigned)n, SP, 0, st>>>(d_probs, l);
+            SGT_LAUNCH_CHECK();
+            convert_new_kernel<<<dim3((unsigned)n, std::min(longest, 8), 2 * kConvParts), kThreads, 0, st>>>(d_probs, l);
+            SGT_LAUNCH_CHECK();
+            return SIGNTRI_OK;
+        };
+        signtri_status rs = SIGNTRI_OK;
+        if (sums && !diagonal.empty()) {
+            const Super *l = d_list + all.size() - diagonal.size();
+            exps_kernel<<<(unsigned)diagonal.size(), kThreads, 0, st>>>(d_probs, l, kV);
+            SGT_LAUNCH_CHECK();
+            if ((rs = join(l, diagonal.size(), 1)) != SIGNTRI_OK) return rs;
+        }
+        for (int l = 0; l < levels; l++) {
+            const size_t n = off[l + 1] - off[l];
+            const Super *at = d_list + off[l];
+            const bool with_sums = l >= sums_from;
+            if (with_sums) {
+                rs = rns::gemm(d_src, tiles + products * off[l], (int)(products * n), products, res, d_err, cls_sums, st);
+                if (rs != SIGNTRI_OK) return rs;
+            }
+            // the steps that hold blocks: ragged panels have fewer rows or columns
+            int nbr = 0, nbc = 0;
+            for (size_t i = off[l]; i < off[l + 1]; i++) {
+                const Problem &p = probs[list[i].k];
+                nbr = std::max(nbr, std::min(SB, (p.rows + LB - 1) / LB - list[i].A * SB));
+                nbc = std::max(nbc, std::min(SB, (p.cols + LB - 1) / LB - list[i].B * SB));
+            }
+            const Wave w{d_probs, at, res, (int)n, with_sums ? products : 0};
+            if ((rs = run_wave(w, SB - nbr, SB - 1 + nbc, slab0, slab1, cls_leaf, st)) != SIGNTRI_OK) return rs;
+            if (l + 1 < levels && (rs = join(at, n, l + 2)) != SIGNTRI_OK) return rs;
+        }
+        if (!sums) {   // nothing that could have set a flag
+            for (int k = 0; k < np; k++) flags[k] = 0;
+            return SIGNTRI_OK;
+        }
+        SGT_CUDA_TRY(cudaMemcpyAsync(flags, d_flags, np * sizeof(int), cudaMemcpyDeviceToHost, st));
+        SGT_CUDA_TRY(cudaStreamSynchronize(st));
+        return SIGNTRI_OK;
+    }
+};
 
 }  // namespace
 }  // namespace sup
 
-// ---- the whole solve ------------------------------------------------------------
+// ---- sign(T) ------------------------------------------------------------------------
 
-size_t ph_super_workspace_bytes(int n)
+size_t ph_super_workspace_bytes(int count, const int *n)
 {
     using namespace sup;
-    const int ns = (n + SP - 1) / SP;
-    const size_t form = rns::form_tile_bytes(ns, 2 * ns);
-    return 4 * (form + 256) + 6 * ((size_t)ns * SP * sizeof(int) + 256) + 2 * ((size_t)ns * sizeof(int) + 256) +
-           (size_t)ns * (ns - 1) / 2 * 3 * sizeof(rns::Tile) + 256 + (size_t)(ns - 1) * 3 * rns::kMods * SP * SP + 256 +
-           2 * (wave_slab_bytes(ns - 1) + 256) + 256 +
-           lvl::level_workspace_bytes<double>(n);
+    size_t b = 0, superblocks = 0, ops = 0, widest = 0;
+    for (int k = 0; k < count; k++) {
+        const size_t ns = panels_of(n[k]);
+        b += problem_bytes((int)ns, (int)ns, true);
+        superblocks += ns * (ns - 1) / 2;
+        ops += ns * (ns + 1) + ns;
+        widest += ns - 1;
+    }
+    return b + run_bytes(count, superblocks, ops, widest, 3);
 }
 
-// flags_host (pinned): nonzero on return when the data did not suit one scale
-// per row and the plain path has to run; waits for the stream.
-signtri_status ph_super_run(int n, const double *T, int ldt, double *U, int ldu, Arena &ws, int *d_err,
-                            int *flags_host, cudaStream_t st)
+signtri_status ph_super_run(int count, const BatchDesc *mats, Arena &ws, int *d_err, int *flags, cudaStream_t st)
 {
     using namespace sup;
-    const int ns = (n + SP - 1) / SP, nkb = 2 * ns, bits = rns::operand_bits(ns * SP);
-    auto take = [&](size_t b) { return ws.take(b); };
-    __nv_bfloat16 *form[4];   // T rows, T columns, U rows, U columns
-    int *exps[6];             // of the same, and the newest superblocks' of U
-    for (auto *&f : form) f = static_cast<__nv_bfloat16 *>(take(rns::form_tile_bytes(ns, nkb)));
-    for (auto *&e : exps) e = static_cast<int *>(take((size_t)ns * SP * sizeof(int)));
-    int *rgrown = static_cast<int *>(take((size_t)ns * sizeof(int)));
-    int *cgrown = static_cast<int *>(take((size_t)ns * sizeof(int)));
-    auto *tiles = static_cast<rns::Tile *>(take((size_t)ns * (ns - 1) / 2 * 3 * sizeof(rns::Tile)));
-    auto *res = static_cast<int8_t *>(take((size_t)(ns - 1) * 3 * rns::kMods * SP * SP));
-    auto *slab0 = static_cast<double *>(take(wave_slab_bytes(ns - 1)));
-    auto *slab1 = static_cast<double *>(take(wave_slab_bytes(ns - 1)));
-    int *flags = static_cast<int *>(take(sizeof(int)));
-    if (!flags) return SIGNTRI_ERR_NO_WORKSPACE;
-    const Mat Tm{T, ldt, n, n, true}, Um{U, ldu, n, n, true};
-    // the diagonal superblocks
-    signtri_status rs = ph_fp64_near_run(n, T, ldt, U, ldu, SB - 1, ws, st);
-    if (rs != SIGNTRI_OK) return rs;
-    {
-        ProfScope ps(SIGNTRI_KC_CONVERT, st);
-        for (auto *e : exps) SGT_CUDA_TRY(cudaMemsetAsync(e, 0xc0, (size_t)ns * SP * sizeof(int), st));   // below every exponent
-        SGT_CUDA_TRY(cudaMemsetAsync(flags, 0, sizeof(int), st));
-        tiles_kernel<<<ns - 1, 128, 0, st>>>(ns, tiles);
-        SGT_LAUNCH_CHECK();
-        fixed_exps_kernel<<<dim3(ns, ns), kThreads, 0, st>>>(Tm, false, exps[0], exps[1], flags);
-        SGT_LAUNCH_CHECK();
-        convert_fixed_kernel<<<dim3(ns, ns, 2 * kConvParts), kThreads, 0, st>>>(Tm, bits, exps[0], exps[1], form[0],
-                                                                                form[1], nkb, false, flags);
-        SGT_LAUNCH_CHECK();
-        fixed_exps_kernel<<<ns, kThreads, 0, st>>>(Um, true, exps[4], exps[5], flags);
-        SGT_LAUNCH_CHECK();
+    Run r;
+    r.cls_sums = SIGNTRI_KC_BLOCK_SUMS_F64;
+    r.cls_leaf = SIGNTRI_KC_OFFDIAG_LEAF;
+    int most = 0;
+    for (int k = 0; k < count; k++) {
+        const BatchDesc &m = mats[k];
+        const int ns = panels_of(m.n);
+        most = std::max(most, ns);
+        Problem p{};
+        p.RT = p.CT = p.C0 = m.T;
+        p.RU = p.CU = m.U;
+        p.V = m.U;
+        p.ldrt = p.ldct = p.ldc0 = m.ldt;
+        p.ldru = p.ldcu = p.ldv = m.ldu;
+        p.rows = p.cols = m.n;
+        p.own = 1.0;
+        p.bits = rns::operand_bits(ns * SP);
+        p.triangular = true;
+        if (!r.reserve(ws, p, ns, ns, true)) return SIGNTRI_ERR_NO_WORKSPACE;
+        r.probs.push_back(p);
+        for (int A = 0; A < ns; A++) {
+            r.diagonal.push_back({k, A, A});
+            for (int B = A; B < ns; B++) r.row_ops.push_back({k, A, B});
+        }
     }
-    auto join = [&](int D) -> signtri_status {
-        ProfScope ps(SIGNTRI_KC_CONVERT, st);
-        grow_exps_kernel<<<ns - D, SP, 0, st>>>(0, D, exps[4], exps[5], exps[2], exps[3], rgrown, cgrown, flags);
-        SGT_LAUNCH_CHECK();
-        convert_new_kernel<<<dim3(ns - D, D + 1, 2 * kConvParts), kThreads, 0, st>>>(
-            Um, bits, 0, D, -1, -1, exps[2], exps[3], rgrown, cgrown, form[2], nkb, form[3], nkb, flags);
-        SGT_LAUNCH_CHECK();
-        return SIGNTRI_OK;
-    };
-    if ((rs = join(0)) != SIGNTRI_OK) return rs;
-    const rns::Sources src{{{form[2], form[1], nkb, nkb}, {form[0], form[3], nkb, nkb}, {form[2], form[3], nkb, nkb}}};
-    size_t at = 0;
-    for (int D = 1; D < ns; D++) {
-        const int nt = ns - D;
-        rs = rns::gemm(src, tiles + 3 * at, 3 * nt, 3, res, d_err, SIGNTRI_KC_BLOCK_SUMS_F64, st);
-        if (rs != SIGNTRI_OK) return rs;
-        at += nt;
-        const Wave w{T, U, T, U, T, U, res, exps[2], exps[1], exps[0], exps[3], exps[4], exps[5], ldt, ldu, ldt, ldu, ldt, ldu,
-                     n, n, 0, D, nt, bits, 3, 1.0};
-        if ((rs = run_wave(w, slab0, slab1, SIGNTRI_KC_OFFDIAG_LEAF, st)) != SIGNTRI_OK) return rs;
-        if (D + 1 < ns && (rs = join(D)) != SIGNTRI_OK) return rs;
+    r.col_ops = r.row_ops;
+    for (int D = 1; D < most; D++) {
+        for (int k = 0; k < count; k++)
+            for (int A = 0; A + D < panels_of(mats[k].n); A++) r.list.push_back({k, A, A + D});
+        r.off.push_back(r.list.size());
     }
-    SGT_CUDA_TRY(cudaMemcpyAsync(flags_host, flags, sizeof(int), cudaMemcpyDeviceToHost, st));
-    SGT_CUDA_TRY(cudaStreamSynchronize(st));
-    return SIGNTRI_OK;
+    return r.run(ws, d_err, flags, st);
 }
 
-// ---- A X - X B = C -----------------------------------------------------------------
+// ---- A X - X B = C ----------------------------------------------------------------
 
 static size_t sylvester_super_bytes(int nr, int nc, int nt)
 {
     using namespace sup;
-    size_t b = 2 * (wave_slab_bytes(nt) + 256) + 3 * ((size_t)(nr + nc) * SP * sizeof(int) + 512) + 256;
-    if (nr + nc > 2)
-        b += rns::form_tile_bytes(nr, 2 * nr) + rns::form_tile_bytes(nc, 2 * nc) + rns::form_tile_bytes(nr, 2 * nc) +
-             rns::form_tile_bytes(nc, 2 * nr) + (size_t)nr * nc * 2 * sizeof(rns::Tile) +
-             (size_t)nt * 2 * rns::kMods * SP * SP + (size_t)(nr + nc) * sizeof(int) + 8 * 256;
-    return b;
+    return problem_bytes(nr, nc, nr + nc > 2) +
+           run_bytes(1, (size_t)nr * nc, ((size_t)nr * (nr + 1) + (size_t)nc * (nc + 1)) / 2, nt, 2);
 }
 
 size_t sylvester_super_workspace_bytes(int m, int p)
 {
     if (m <= 0 || p <= 0) return 0;
-    const int nr = (m + sup::SP - 1) / sup::SP, nc = (p + sup::SP - 1) / sup::SP;
+    const int nr = sup::panels_of(m), nc = sup::panels_of(p);
     return sylvester_super_bytes(nr, nc, std::min(nr, nc));
 }
 
 // for every m + p = n: the forms take 2 (nr + nc)^2 tiles of K-blocks
 size_t sylvester_super_workspace_bound(int n)
 {
-    const int k = (n + sup::SP - 1) / sup::SP + 1;
-    return sylvester_super_bytes(k, 1, k / 2 + 1) + (size_t)k * k / 2 * sizeof(rns::Tile);
+    const int k = sup::panels_of(n) + 1;
+    return sylvester_super_bytes(k, 1, k / 2 + 1) +
+           (size_t)k * k / 2 * (2 * sizeof(rns::Tile) + sizeof(sup::Super));
 }
 
-// X of A X - X B = cscale C by superblocks of 128 from the bottom-left one,
-// as ph_super_run: the terms between superblocks as residue products, those
-// inside one by wave_kernel.  flags_host (pinned) as there; one superblock
-// needs no products, sets no flag and returns without waiting.
 signtri_status sylvester_super_run(int m, int p, const double *A, int lda, const double *B, int ldb, const double *C,
-                                   int ldc, double cscale, double *X, int ldx, Arena &ws, int *d_err, int *flags_host,
+                                   int ldc, double cscale, double *X, int ldx, Arena &ws, int *d_err, int *flags,
                                    cudaStream_t st)
 {
     using namespace sup;
-    const int nr = (m + SP - 1) / SP, nc = (p + SP - 1) / SP, nt = std::min(nr, nc);
-    const int bits = rns::operand_bits(std::max(nr, nc) * SP);
-    const bool products = nr + nc > 2;
-    auto take = [&](size_t b) { return ws.take(b); };
-    auto *slab0 = static_cast<double *>(take(wave_slab_bytes(nt)));
-    auto *slab1 = static_cast<double *>(take(wave_slab_bytes(nt)));
-    // exponents: A's rows, B's columns, X's rows and columns, and of X's newest
-    int *ea = static_cast<int *>(take((size_t)nr * SP * sizeof(int))), *eb = static_cast<int *>(take((size_t)nc * SP * sizeof(int)));
-    int *er = static_cast<int *>(take((size_t)nr * SP * sizeof(int))), *ec = static_cast<int *>(take((size_t)nc * SP * sizeof(int)));
-    int *rnew = static_cast<int *>(take((size_t)nr * SP * sizeof(int))), *cnew = static_cast<int *>(take((size_t)nc * SP * sizeof(int)));
-    int *flags = static_cast<int *>(take(sizeof(int)));
-    if (!flags) return SIGNTRI_ERR_NO_WORKSPACE;
-    *flags_host = 0;
-    const Mat Am{A, lda, m, m, true}, Bm{B, ldb, p, p, true}, Xm{X, ldx, m, p, false};
-    __nv_bfloat16 *fa = nullptr, *fb = nullptr, *fr = nullptr, *fc = nullptr;
-    rns::Tile *tiles = nullptr;
-    int8_t *res = nullptr;
-    int *rgrown = nullptr, *cgrown = nullptr;
-    {
-        ProfScope ps(SIGNTRI_KC_CONVERT, st);
-        for (int *e : {ea, er, rnew}) SGT_CUDA_TRY(cudaMemsetAsync(e, 0xc0, (size_t)nr * SP * sizeof(int), st));
-        for (int *e : {eb, ec, cnew}) SGT_CUDA_TRY(cudaMemsetAsync(e, 0xc0, (size_t)nc * SP * sizeof(int), st));
-        if (products) {
-            fa = static_cast<__nv_bfloat16 *>(take(rns::form_tile_bytes(nr, 2 * nr)));
-            fb = static_cast<__nv_bfloat16 *>(take(rns::form_tile_bytes(nc, 2 * nc)));
-            fr = static_cast<__nv_bfloat16 *>(take(rns::form_tile_bytes(nr, 2 * nc)));
-            fc = static_cast<__nv_bfloat16 *>(take(rns::form_tile_bytes(nc, 2 * nr)));
-            tiles = static_cast<rns::Tile *>(take((size_t)nr * nc * 2 * sizeof(rns::Tile)));
-            res = static_cast<int8_t *>(take((size_t)nt * 2 * rns::kMods * SP * SP));
-            rgrown = static_cast<int *>(take((size_t)nr * sizeof(int)));
-            cgrown = static_cast<int *>(take((size_t)nc * sizeof(int)));
-            if (!cgrown) return SIGNTRI_ERR_NO_WORKSPACE;
-            SGT_CUDA_TRY(cudaMemsetAsync(flags, 0, sizeof(int), st));
-            sylvester_tiles_kernel<<<nr + nc - 1, 128, 0, st>>>(nr, nc, tiles);
-            SGT_LAUNCH_CHECK();
-            fixed_exps_kernel<<<dim3(nr, nr), kThreads, 0, st>>>(Am, false, ea, nullptr, flags);
-            SGT_LAUNCH_CHECK();
-            fixed_exps_kernel<<<dim3(nc, nc), kThreads, 0, st>>>(Bm, false, nullptr, eb, flags);
-            SGT_LAUNCH_CHECK();
-            convert_fixed_kernel<<<dim3(nr, nr, 2 * kConvParts), kThreads, 0, st>>>(Am, bits, ea, nullptr, fa, nullptr,
-                                                                                    2 * nr, false, flags);
-            SGT_LAUNCH_CHECK();
-            convert_fixed_kernel<<<dim3(nc, nc, 2 * kConvParts), kThreads, 0, st>>>(Bm, bits, nullptr, eb, nullptr, fb,
-                                                                                    2 * nc, false, flags);
-            SGT_LAUNCH_CHECK();
-        }
+    const int nr = panels_of(m), nc = panels_of(p);
+    Run r;
+    r.cls_sums = SIGNTRI_KC_SYLV_SUMS;
+    r.cls_leaf = SIGNTRI_KC_SYLV_LEAF;
+    r.products = 2;
+    r.sums_from = 1;
+    Problem q{};
+    q.RT = A;
+    q.CT = B;
+    q.C0 = C;
+    q.V = X;
+    q.ldrt = lda;
+    q.ldct = ldb;
+    q.ldc0 = ldc;
+    q.ldv = ldx;
+    q.rows = m;
+    q.cols = p;
+    q.own = 0.5 * cscale;   // (rows and columns stand for u = 1 and -1)
+    q.bits = rns::operand_bits(std::max(nr, nc) * SP);
+    if (!r.reserve(ws, q, nr, nc, nr + nc > 2)) return SIGNTRI_ERR_NO_WORKSPACE;
+    r.probs.push_back(q);
+    for (int a = 0; a < nr; a++)
+        for (int b = a; b < nr; b++) r.row_ops.push_back({0, a, b});
+    for (int a = 0; a < nc; a++)
+        for (int b = a; b < nc; b++) r.col_ops.push_back({0, a, b});
+    for (int s = 0; s < nr + nc - 1; s++) {   // from the bottom-left superblock
+        for (int b = std::max(0, s - (nr - 1)); b <= std::min(nc - 1, s); b++) r.list.push_back({0, nr - 1 - s + b, b});
+        r.off.push_back(r.list.size());
     }
-    const rns::Sources src{{{fr, fb, 2 * nc, 2 * nc}, {fa, fc, 2 * nr, 2 * nr}, {}}};
-    size_t at = 0;
-    for (int s = 0; s < nr + nc - 1; s++) {
-        const int b0 = std::max(0, s - (nr - 1)), cnt = std::min(nc - 1, s) - b0 + 1, a0 = nr - 1 - s + b0;
-        signtri_status rs = SIGNTRI_OK;
-        if (s > 0 && (rs = rns::gemm(src, tiles + 2 * at, 2 * cnt, 2, res, d_err, SIGNTRI_KC_SYLV_SUMS, st)) != SIGNTRI_OK)
-            return rs;
-        at += cnt;
-        const Wave w{A, nullptr, B, nullptr, C, X, res, er, eb, ea, ec, rnew, cnew, lda, 0, ldb, 0, ldc, ldx,
-                     m, p, a0, b0, cnt, bits, s > 0 ? 2 : 0, 0.5 * cscale};
-        if ((rs = run_wave(w, slab0, slab1, SIGNTRI_KC_SYLV_LEAF, st)) != SIGNTRI_OK) return rs;
-        if (s + 1 == nr + nc - 1) break;
-        ProfScope ps(SIGNTRI_KC_CONVERT, st);
-        grow_exps_kernel<<<cnt, SP, 0, st>>>(a0, b0, rnew, cnew, er, ec, rgrown, cgrown, flags);
-        SGT_LAUNCH_CHECK();
-        convert_new_kernel<<<dim3(cnt, std::max(b0 + cnt, nr - a0), 2 * kConvParts), kThreads, 0, st>>>(
-            Xm, bits, a0, b0, 0, nr - 1, er, ec, rgrown, cgrown, fr, 2 * nc, fc, 2 * nr, flags);
-        SGT_LAUNCH_CHECK();
-    }
-    if (!products) return SIGNTRI_OK;
-    SGT_CUDA_TRY(cudaMemcpyAsync(flags_host, flags, sizeof(int), cudaMemcpyDeviceToHost, st));
-    SGT_CUDA_TRY(cudaStreamSynchronize(st));
-    return SIGNTRI_OK;
+    return r.run(ws, d_err, flags, st);
 }
 
 }  // namespace signtri

@@ -112,7 +112,7 @@ __device__ __forceinline__ Task task_of(int id, int per)
 }
 
 __global__ void __launch_bounds__(kThreads, 1)
-rns_gemm_kernel(const __grid_constant__ Sources src, const Tile *__restrict__ tiles, int ntasks, int per,
+rns_gemm_kernel(const Source *__restrict__ src, const Tile *__restrict__ tiles, int ntasks, int per,
                 int8_t *__restrict__ out, int *__restrict__ err)
 {
     extern __shared__ unsigned char smem_raw[];
@@ -151,7 +151,7 @@ rns_gemm_kernel(const __grid_constant__ Sources src, const Tile *__restrict__ ti
             for (int id = blockIdx.x; id < ntasks && ok; id += gridDim.x) {
                 const Task k = task_of(id, per);
                 const Tile t = tiles[k.tile];
-                const Source s = src.s[t.src];
+                const Source s = src[t.src];
                 const __nv_bfloat16 *a = s.A + ((size_t)t.pa * kMods + k.mod) * s.nkbA * kTileElems;
                 const __nv_bfloat16 *b = s.B + ((size_t)t.pb * kMods + k.mod) * s.nkbB * kTileElems;
                 for (int kb = t.kb0; kb < t.kb1; kb++) {
@@ -277,14 +277,14 @@ rns_gemm_kernel(const __grid_constant__ Sources src, const Tile *__restrict__ ti
 
 }  // namespace
 
-signtri_status gemm(const Sources &src, const Tile *d_tiles, int ntiles, int per, int8_t *out, int *d_err, int cls,
+signtri_status gemm(const Source *d_src, const Tile *d_tiles, int ntiles, int per, int8_t *out, int *d_err, int cls,
                     cudaStream_t st)
 {
     if (ntiles <= 0) return SIGNTRI_OK;
     SGT_CUDA_TRY(cudaFuncSetAttribute(rns_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
     const int ntasks = ntiles * kMods;
     ProfScope ps(cls, st);
-    rns_gemm_kernel<<<std::min(ntasks, 152), kThreads, kSmemBytes, st>>>(src, d_tiles, ntasks, per, out, d_err);
+    rns_gemm_kernel<<<std::min(ntasks, 152), kThreads, kSmemBytes, st>>>(d_src, d_tiles, ntasks, per, out, d_err);
     SGT_LAUNCH_CHECK();
     return SIGNTRI_OK;
 }

@@ -35,7 +35,7 @@ struct Form {
 };
 inline size_t form_tile_bytes(int panels, int nkb) { return (size_t)panels * kMods * nkb * kTileElems * 2; }
 
-// One 128 x 128 product: panel pa of source `src`'s A form times panel pb of
+// One 128 x 128 product: panel pa of source number `src`'s A form times panel pb of
 // its B form over K-blocks [kb0, kb1).
 struct Tile {
     int src, pa, pb, kb0, kb1;
@@ -44,14 +44,11 @@ struct Source {
     const __nv_bfloat16 *A, *B;
     int nkbA, nkbB;
 };
-struct Sources {
-    Source s[3];
-};
 
 // Residues of tiles [0, ntiles) of d_tiles, `per` consecutive tiles sharing
 // panels: out[tile][modulus][row][column], int8, already multiplied by the
 // modulus's cofactor inverse.
-signtri_status gemm(const Sources &src, const Tile *d_tiles, int ntiles, int per, int8_t *out, int *d_err, int cls,
+signtri_status gemm(const Source *d_src, const Tile *d_tiles, int ntiles, int per, int8_t *out, int *d_err, int cls,
                     cudaStream_t st);
 
 }  // namespace rns

@@ -112,3 +112,26 @@ def test_sylvester_superblocks_vs_oracle(gpu_lib, oracle_mod, n, n_neg):
     torch.cuda.synchronize()
     ref = oracle_mod.sign_tri(T, schedule="antidiag")
     assert np.linalg.norm(U - ref) <= n * np.finfo(float).eps * np.linalg.norm(ref)
+
+
+# a batch with problems on both sides of the superblocks' least order, ragged
+# ones, a graded one (left to the plain path) and a one-signed one
+@pytest.mark.gpu
+def test_batched_superblocks_vs_oracle(gpu_lib, oracle_mod):
+    import torch
+    p = gpu_lib
+    Ts = [make_T(n, 0.4, seed=n) for n in (511, 512, 513, 700, 1037, 64, 640, 530, 1281)]
+    g = np.round(np.linspace(0.0, 300.0, 700)).astype(int)
+    Ts[3] = np.asfortranarray(np.ldexp(Ts[3], g[None, :] - g[:, None]))
+    Ts[7][np.arange(530), np.arange(530)] = np.abs(np.diag(Ts[7]))
+    dev = [p.to_device(T) for T in Ts]
+    out = [torch.empty_like(t) for t in dev]
+    ns = [T.shape[0] for T in Ts]
+    st, info = p.sign_tri_batched(ns, [t.data_ptr() for t in dev], ns, [u.data_ptr() for u in out], ns,
+                                  p.Variant.PH_FP64_EFFICIENT, torch.cuda.current_stream().cuda_stream)
+    assert st == 0 and not any(info)
+    for k, T in enumerate(Ts):
+        U, ref = p.to_numpy(out[k]), oracle_mod.sign_tri(T, schedule="antidiag")
+        if k == 3:   # entries of very different size: compared at one size
+            U, ref = np.ldexp(U, g[:, None] - g[None, :]), np.ldexp(ref, g[:, None] - g[None, :])
+        assert np.linalg.norm(U - ref) <= ns[k] * np.finfo(float).eps * np.linalg.norm(ref), k
