@@ -101,8 +101,8 @@ batched_diag_level_kernel(const BatchDesc *__restrict__ mats, const int *__restr
 __global__ void __launch_bounds__(lvl::kLevelThreads)
 batched_level_kernel(const BatchDesc *__restrict__ mats, const int *__restrict__ members, int d, int leaves,
                      const LevelTile *__restrict__ tiles, const __grid_constant__ lvl::Split sin,
-                     const double *__restrict__ in, const LevelTile *__restrict__ next,
-                     const __grid_constant__ lvl::Split sout, double *__restrict__ out)
+                     const double *in, const LevelTile *__restrict__ next,
+                     const __grid_constant__ lvl::Split sout, double *out)
 {
     using namespace lvl;
     extern __shared__ __align__(16) unsigned char raw[];

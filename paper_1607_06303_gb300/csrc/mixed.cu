@@ -10,7 +10,7 @@
 //    variant), or a two-term fp16 split hi + lo with the three products of
 //    s + t <= 1 (about 2^-21; T, U and the correction scaled by powers of two
 //    into fp16's range, the FP16 variant); in-block recurrences (Algorithm 6,
-//    1x1 case) in fp32, a 64-row tile solved by 16 x 16 sub-blocks.
+//    1x1 case) in fp32, a 64-row tile solved by 4 x 4 micro-blocks.
 // 2. Refinement.  With U = U0 + E and E strictly upper triangular, UT = TU
 //    and U^2 = I become, entry by entry (i < j):
 //      signs differ: (t_ii - t_jj) e_ij = -Rc_ij + sum_{i<k<j} (e_ik t_kj - t_ik e_kj)
@@ -112,10 +112,16 @@ __device__ __forceinline__ void split_store4(float4 r, int S, bool f16, __nv_bfl
 // --------------------------------------------------------------- leaves ---
 
 constexpr int kLeafThreads = 256;
-constexpr int kSub = 16;             // sub-block edge of the in-tile solve
-constexpr int kLeafLD = MB + 4;      // leaf smem pitch: rows / columns stay 16-byte aligned for float4 reads
-constexpr int kNSub = MB / kSub;     // sub-blocks per tile edge
-constexpr int kLeafBufs = 6;         // M+, M-, N+, N-, V by columns, V by rows
+constexpr int kMicro = 4;            // micro-block edge of the in-tile solve: one thread's entries
+constexpr int kMicros = MB / kMicro; // micro-blocks per tile edge
+constexpr int kTri = kMicros * (kMicros + 1) / 2;   // micro-blocks of an upper triangular tile
+// words from one micro-block to the next in shared memory: eight consecutive
+// ones lie in different banks for 16-byte reads
+constexpr int kMicroPitch = kMicro * kMicro + 4;
+constexpr size_t kLeafSmem = (size_t)(4 * kTri + kMicros * kMicros) * kMicroPitch * sizeof(float);
+
+// Number of micro-block (r, c), r <= c, of an upper triangular tile, row by row.
+__host__ __device__ constexpr int tri_index(int r, int c) { return r * kMicros - r * (r - 1) / 2 + c - r; }
 
 // Per-sign operators of the in-block recurrences.  Entry (p, q) of a tile
 // (I, J) is fixed by
@@ -126,14 +132,16 @@ constexpr int kLeafBufs = 6;         // M+, M-, N+, N-, V by columns, V by rows
 // r of M^+ is A's row r if s_r = +, else T's, and M^- the other way round,
 // and the row part is + sum_k v_pk N^{s_p}_kq, where column c of N^+ is -A's
 // column c if s_c = +, else +T's, and N^- the other way round.  Per diagonal
-// block I, fp32, 64 x 64, zero on and below the diagonal (the diagonal terms
-// of T sit in the divisor t_pp - t_qq):
-//   OPS[(4 I + 0) 4096 ..]  M^+ row-major      OPS[(4 I + 1) 4096 ..]  M^- row-major
-//   OPS[(4 I + 2) 4096 ..]  N^+ column-major   OPS[(4 I + 3) 4096 ..]  N^- column-major
+// block I, fp32, zero on and below the diagonal (the diagonal terms of T sit
+// in the divisor t_pp - t_qq), the micro-blocks of the upper triangle one
+// after another (tri_index), M's row by row, N's column by column:
+//   OPS[(4 I + 0) 16 kTri ..]  M^+      OPS[(4 I + 1) 16 kTri ..]  M^-
+//   OPS[(4 I + 2) 16 kTri ..]  N^+      OPS[(4 I + 3) 16 kTri ..]  N^-
 // and DIAG[i] = (float) t_ii (0 beyond n).
 __global__ void leaf_ops_kernel(int n, const double *__restrict__ T, int ldt, const double *__restrict__ A, int lda,
                                 float *__restrict__ OPS, float *__restrict__ DIAG)
 {
+    constexpr int E = kMicro * kMicro;
     const int r0 = blockIdx.x * MB;
     __shared__ float sg[MB];
     for (int i = threadIdx.x; i < MB; i += blockDim.x) {
@@ -143,315 +151,229 @@ __global__ void leaf_ops_kernel(int n, const double *__restrict__ T, int ldt, co
         DIAG[r0 + i] = (float)t;
     }
     __syncthreads();
-    float *mp = OPS + (size_t)(4 * blockIdx.x) * MB * MB;
+    float *mp = OPS + (size_t)(4 * blockIdx.x) * E * kTri;
     for (int idx = threadIdx.x; idx < MB * MB; idx += blockDim.x) {
         const int i = idx % MB, j = idx / MB;   // element (i, j) of the block, i fastest
+        if (i / kMicro > j / kMicro) continue;
         const bool in = r0 + j < n && i < j;
         const float t = in ? (float)SGT_AT(T, ldt, r0 + i, r0 + j) : 0.f;
         const float a = in ? (float)SGT_AT(A, lda, r0 + i, r0 + j) : 0.f;
-        // row-major M: row i picks by the sign of i; column-major N: column j by the sign of j
-        mp[0 * MB * MB + i * MB + j] = sg[i] > 0.f ? a : t;
-        mp[1 * MB * MB + i * MB + j] = sg[i] > 0.f ? t : a;
-        mp[2 * MB * MB + j * MB + i] = sg[j] > 0.f ? -a : t;
-        mp[3 * MB * MB + j * MB + i] = sg[j] > 0.f ? t : -a;
+        // M: row i picks by the sign of i; N: column j by the sign of j
+        const int mb = tri_index(i / kMicro, j / kMicro) * E;
+        const int rm = mb + i % kMicro * kMicro + j % kMicro, cm = mb + j % kMicro * kMicro + i % kMicro;
+        mp[0 * E * kTri + rm] = sg[i] > 0.f ? a : t;
+        mp[1 * E * kTri + rm] = sg[i] > 0.f ? t : a;
+        mp[2 * E * kTri + cm] = sg[j] > 0.f ? -a : t;
+        mp[3 * E * kTri + cm] = sg[j] > 0.f ? t : -a;
     }
 }
 
-// One warp solves the 16 x 16 sub-block with rows R0.. and columns C0.. of a
-// leaf tile (the recurrences above restricted to it; the terms of the other,
-// already solved, sub-blocks are in VR and VC).  Lane (p, h) = p + 16 h owns
-// row R0 + p, columns C0 + 8h .. C0 + 8h + 7: its pending values c[j] start
-// as seed + row parts - column parts of the solved sub-blocks; entry (p, q)
-// is solved at step t = 15 - p + q by the lane of q's half, and each solved
-// value is pushed at once into the entries that depend on it -- into the
-// row's later entries by both lanes of the row (+ v N~, the value passed to
-// the other half by a shuffle), into the entries above it in its column by
-// the other rows' lanes of the same half, which receive it by shuffle
-// (- M v).  The coefficients M^{+-}[p][k] sit in each lane rotated by 8 h,
-// so that one constant register index serves both halves; the step's pending
-// value is picked by a three-level select tree and divided by a reciprocal
-// taken off the chain.  Both halves working halves the instructions per
-// step; the step loop is unrolled so that every register index is a
-// constant.
-__device__ __forceinline__ void subblock_solve(const float *__restrict__ Mp, const float *__restrict__ Mm,
-                                               const float *__restrict__ Np, const float *__restrict__ Nm,
-                                               float *__restrict__ VC, float *__restrict__ VR,
-                                               const float *__restrict__ srow, const float *__restrict__ scol,
-                                               const float *__restrict__ drow, const float *__restrict__ dcol, int R0,
-                                               int C0, int lane)
+// The seeds of anti-diagonal d's tiles (blockIdx.x): per entry the block sums
+// (their K range includes the diagonal blocks K = I and K = J, so they already
+// hold the in-block products of the known blocks: U_II T_IJ - T_IJ U_JJ for
+// opposite signs in mode 0, E_II T_IJ - T_IJ E_JJ and E_II U0_IJ + U0_IJ E_JJ in
+// mode 1; terms with the unknown V_IJ vanish, its slices being still zero),
+// float2 (hi, lo) partials summed in fp32 over the slots, and the base terms;
+// micro-block by micro-block as the leaf's threads own them, column by column.
+// A launch of its own: up to 16 slots of 64 to 96 KB a tile took one leaf CTA
+// up to 40 us to read, sixteen CTAs a few.
+template <int MODE>
+__global__ void __launch_bounds__(kLeafThreads)
+leaf_seed_kernel(int n, const double *__restrict__ T, int ldt, const float *__restrict__ DIAG,
+                 const double *__restrict__ Rc, const double *__restrict__ Rs, int ldr, int d,
+                 const int2 *__restrict__ tslot, const int2 *__restrict__ tslot2, const double *__restrict__ PA,
+                 const double *__restrict__ PB, float *__restrict__ SEED)
 {
-    constexpr int LD = kLeafLD;
-    const int p = lane & (kSub - 1), h = lane >> 4;
-    const int P = R0 + p;
-    // column signs of the sub-block, bit q for column C0 + q
-    const unsigned colmask = __ballot_sync(0xffffffffu, lane < kSub && scol[C0 + p] > 0.f) & 0xffffu;
-    const unsigned hmask = (colmask >> (8 * h)) & 0xffu;   // this half's columns
-    const float sp = srow[P], dp = drow[P];
-    float c[8], mr[24], nr[24];
-#pragma unroll
-    for (int j = 0; j < 8; j++) c[j] = VR[P * LD + C0 + 8 * h + j] - VC[(C0 + 8 * h + j) * LD + P];
-    // mr[x] = M^+[p][x - 8 + 8h], nr[x] = M^-[p][x - 8 + 8h] (0 outside the block)
-#pragma unroll
-    for (int x = 0; x < 24; x++) {
-        const int k = x - 8 + 8 * h;
-        const bool ok = k >= 0 && k < kSub;
-        mr[x] = ok ? Mp[P * LD + R0 + k] : 0.f;
-        nr[x] = ok ? Mm[P * LD + R0 + k] : 0.f;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the leaves may load their operators
+    const int I = blockIdx.x, J = I + d;
+    const int e = blockIdx.y * kLeafThreads + threadIdx.x, p = e % MB, q = e / MB;
+    const int gi = I * MB + p, gj = J * MB + q;
+    const int2 ts = tslot[I];
+    const int2 ts2 = (MODE == 0 && tslot2) ? tslot2[I] : make_int2(0, 0);
+    const bool sp = DIAG[gi] > 0.f, sq = gj >= n || DIAG[gj] > 0.f, opp = sp != sq;
+    const double own = gj >= n ? 0.0
+                       : MODE == 0 ? (opp ? SGT_AT(T, ldt, gi, gj) : 0.0)
+                                   : SGT_AT(opp ? Rc : Rs, ldr, gi, gj);
+    const float2 *PA2 = reinterpret_cast<const float2 *>(PA), *PB2 = reinterpret_cast<const float2 *>(PB);
+    float acc = 0.f;
+#pragma unroll 4
+    for (int s = 0; s < ts.y + ts2.y; s++) {
+        // mode 0: slots of PA, then (look-ahead pairing) slots of PB.  Signs
+        // differ: TL - BR of PA (X); agree: TR (Y, mode 0) or TL + BR of PB (Y^E)
+        const bool second = s >= ts.y;
+        const size_t at = (size_t)(second ? ts2.x + s - ts.y : ts.x + s) * 16384 + e;
+        const float2 *P0 = (second ? PB2 : PA2) + at;
+        const float2 *src = opp ? P0 : (MODE == 0 ? P0 + 4096 : PB2 + at);
+        const float2 l1 = src[0];
+        float2 l2 = make_float2(0.f, 0.f);
+        if (MODE == 1 || opp) l2 = src[3 * 4096];
+        const float sg = opp ? -1.f : 1.f;
+        acc += (l1.x + sg * l2.x) + (l1.y + sg * l2.y);
     }
-    const float *Nt = (sp > 0.f ? Np : Nm) + C0 * LD + C0;   // N~^{s_p}, this sub-block
-    const int base = 24 * h;
-    float vprev = 0.f;
-#pragma unroll
-    for (int t = 0; t < 2 * kSub - 1; t++) {
-        // column parts: column q = 8h + j takes row k = q + 16 - t, solved at
-        // the previous step by lane k + 16 h = k0 + 24 h (the same half;
-        // taken mod 32 where k is outside the block and the coefficient 0)
-#pragma unroll
-        for (int j = 0; j < 8; j++) {
-            const int k0 = j + kSub - t;   // k in half 0; k0 + 8 in half 1
-            if (t > 0 && k0 >= -8 && k0 < kSub) {
-                const int src = (base + k0) & 31;
-                const float vk = __shfl_sync(0xffffffffu, vprev, src);
-                c[j] = fmaf((hmask >> j) & 1u ? -mr[k0 + 8] : -nr[k0 + 8], vk, c[j]);
-            }
-        }
-        const int qp = t - (kSub - 1) + p;   // the row's column at this step
-        const int hc = qp >> 3;               // its half
-        const bool act = qp >= 0 && qp < kSub && hc == h;
-        const int qc = min(max(qp, 0), kSub - 1);
-        const bool sq = (colmask >> qc) & 1u;
-        const bool opp = (sp > 0.f) != sq;
-        const float den = opp ? dp - dcol[C0 + qc] : sp + (sq ? 1.f : -1.f);
-        const float rden = __fdividef(1.f, den);
-        const int jb = (qc - 8 * h) & 7;
-        const float s0 = (jb & 1) ? c[1] : c[0], s1 = (jb & 1) ? c[3] : c[2];
-        const float s2 = (jb & 1) ? c[5] : c[4], s3 = (jb & 1) ? c[7] : c[6];
-        const float u0 = (jb & 2) ? s1 : s0, u1 = (jb & 2) ? s3 : s2;
-        const float x = (jb & 4) ? u1 : u0;
-        const float v = act ? x * rden : 0.f;
-        // the row's solved value to both halves, then its row part
-        const float vrow = __shfl_sync(0xffffffffu, v, p + 16 * min(max(hc, 0), 1));
-        if (t < 2 * kSub - 2) {
-#pragma unroll
-            for (int j = 0; j < 8; j++) c[j] = fmaf(Nt[(8 * h + j) * LD + qc], vrow, c[j]);
-        }
-        if (act) {
-            VC[(C0 + qc) * LD + P] = v;
-            VR[P * LD + C0 + qc] = v;
-        }
-        vprev = v;
-    }
+    const float b = (float)own;
+    float c = opp ? acc : -acc;
+    if (MODE == 0) c += opp ? b * (sp ? 2.f : -2.f) : 0.f;
+    else c -= b;
+    if (gj >= n) c = 0.f;
+    SEED[(size_t)I * MB * MB + ((p / kMicro * kMicros + q / kMicro) * kMicro + q % kMicro) * kMicro + p % kMicro] = c;
 }
 
 // MODE 0: V = U (initial solve).  MODE 1: V = E (correction), with Rc, Rs.
-// Shared memory (fp32, pitch kLeafLD): the operators M^+, M^- of block I
-// (row-major) and N^+, N^- of block J (column-major), V by columns (VC) and
-// by rows (VR).  Until entry (p, q) is solved, VR[p][q] holds its seed (base
-// terms, block sums and the row parts of the solved sub-blocks) and VC[q][p]
-// the column parts of the solved sub-blocks.
+// Each of the 256 threads owns a 4 x 4 micro-block of the tile: its seeds (base
+// terms and block sums) wait in shared memory where its V will be, the in-tile
+// terms gather in registers.  Phase ph = 0 .. 30
+// solves the micro-blocks with 15 - mr + mc = ph, each by its thread (they
+// depend on those below and to the left only), and, after one barrier, every
+// later micro-block of the same rows or columns takes the phase's terms as
+// 4 x 4 x 4 products: 31 barriers and short register chains, where 16 x 16
+// sub-blocks solved by one warp each took 7 phases of 31 steps of shuffles
+// (100 thousand cycles a tile, 73 of them in the solve).
+// Shared memory (fp32): the operators of block I (M^+, M^-) and of block J
+// (N^+, N^-) and the solved V, micro-block by micro-block (V's columns of four).
 template <int MODE>
 __global__ void __launch_bounds__(kLeafThreads, 2)
-mixed_leaf_kernel(int n, const double *__restrict__ T, int ldt, double *__restrict__ V, int ldv,
-                  const float *__restrict__ OPS, const float *__restrict__ DIAG, const double *__restrict__ Rc,
-                  const double *__restrict__ Rs, int ldr, int d, const int2 *__restrict__ tslot,
-                  const int2 *__restrict__ tslot2,
-                  const double *__restrict__ PA, const double *__restrict__ PB, __nv_bfloat16 *__restrict__ Vr,
-                  __nv_bfloat16 *__restrict__ Vc, int S, int nbk, float sigma)
+mixed_leaf_kernel(int n, double *__restrict__ V, int ldv, const float *__restrict__ OPS, const float *__restrict__ DIAG,
+                  int d, const float *SEED, __nv_bfloat16 *__restrict__ Vr, __nv_bfloat16 *__restrict__ Vc,
+                  int S, int nbk, float sigma)
 {
-    constexpr int LD = kLeafLD;
-    constexpr int EPT = MB * MB / kLeafThreads;   // tile entries per thread
-    constexpr int QS = kLeafThreads / MB;
+    constexpr int E = kMicro * kMicro, PT = kMicroPitch;
+    static_assert(kLeafThreads == kMicros * kMicros, "one micro-block per thread");
     extern __shared__ float4 fsm4[];
-    float *Mp = reinterpret_cast<float *>(fsm4);
-    float *Mm = Mp + MB * LD;
-    float *Np = Mm + MB * LD;
-    float *Nm = Np + MB * LD;
-    float *VC = Nm + MB * LD;
-    float *VR = VC + MB * LD;
-    __shared__ float srow[MB], scol[MB], drow[MB], dcol[MB];
+    float *Mp = reinterpret_cast<float *>(fsm4), *Mm = Mp + kTri * PT, *Np = Mm + kTri * PT, *Nm = Np + kTri * PT;
+    float *Vs = Nm + kTri * PT;
     const int I = blockIdx.x, J = I + d;
     const int r0 = I * MB, c0 = J * MB;
     const int bj = min(MB, n - c0);
-    const int p = threadIdx.x % MB, q0 = threadIdx.x / MB;
-
-    // every global read before the first barrier: this tile's partial slots,
-    // the base terms of the seeds, the operators
-    const int2 ts = tslot[I];
-    const int2 ts2 = (MODE == 0 && tslot2) ? tslot2[I] : make_int2(0, 0);
-    // the partial block sums first (the largest read), with the signs of the
-    // thread's own row and columns taken from DIAG, so that they are in
-    // flight with the reads below: float2 (hi, lo) per element, summed in
-    // fp32 over the slots
-    float acc[EPT];
-    bool opp[EPT];
+    // a warp's micro-blocks: 8 rows of 4, so that its rows' and its columns'
+    // terms both come in few of the phases
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int mr = (warp >> 2) * 8 + (lane >> 2), mc = (warp & 3) * 4 + (lane & 3), own = mr * kMicros + mc;
+    auto four = [](const float *x) { return *reinterpret_cast<const float4 *>(x); };
+    // the operators, all loads in flight before the first store
     {
-        const float sgp = DIAG[r0 + p] > 0.f ? 1.f : -1.f;
+        const float4 *sm = reinterpret_cast<const float4 *>(OPS + (size_t)(4 * I) * E * kTri);
+        const float4 *sn = reinterpret_cast<const float4 *>(OPS + (size_t)(4 * J + 2) * E * kTri);
+        constexpr int N4 = 2 * E * kTri / 4, V4 = (N4 + kLeafThreads - 1) / kLeafThreads;
+        float4 vm[V4], vn[V4];
 #pragma unroll
-        for (int m = 0; m < EPT; m++) {
-            const int q = q0 + m * QS;
-            const float sgq = (q < bj) ? (DIAG[c0 + q] > 0.f ? 1.f : -1.f) : 1.f;
-            acc[m] = 0.f;
-            opp[m] = sgp + sgq == 0.f;
+        for (int i = 0; i < V4; i++) {
+            const int x = threadIdx.x + i * kLeafThreads;
+            if (x < N4) {
+                vm[i] = sm[x];
+                vn[i] = sn[x];
+            }
         }
-        const float2 *PA2 = reinterpret_cast<const float2 *>(PA);
-        const float2 *PB2 = reinterpret_cast<const float2 *>(PB);
-        #pragma unroll 2
-        for (int s = 0; s < ts.y + ts2.y; s++) {
-            // mode 0: slots of PA, then (look-ahead pairing) slots of PB
-            const bool second = s >= ts.y;
-            const float2 *P0 = second ? PB2 : PA2;
-            const size_t sb = ((size_t)(second ? ts2.x + s - ts.y : ts.x + s)) * 16384 + p;
 #pragma unroll
-            for (int m = 0; m < EPT; m++) {
-                const int q = q0 + m * QS;
-                // opposite signs: TL - BR of PA (X); equal signs: TR of PA
-                // (Y, mode 0) or TL + BR of PB (Y^E, mode 1)
-                const float2 *src = opp[m] ? P0 : (MODE == 0 ? P0 + 4096 : PB2);
-                const size_t e = sb + (size_t)q * 64;
-                const float2 l1 = src[e];
-                float2 l2 = make_float2(0.f, 0.f);
-                if (MODE == 1 || opp[m]) l2 = src[e + 3 * 4096];
-                const float sg = opp[m] ? -1.f : 1.f;
-                acc[m] += (l1.x + sg * l2.x) + (l1.y + sg * l2.y);
+        for (int i = 0; i < V4; i++) {
+            const int x = threadIdx.x + i * kLeafThreads;
+            if (x < N4) {
+                *reinterpret_cast<float4 *>(Mp + x / kMicro * PT + x % kMicro * kMicro) = vm[i];
+                *reinterpret_cast<float4 *>(Np + x / kMicro * PT + x % kMicro * kMicro) = vn[i];
             }
         }
     }
-    // base terms staged in VR (t_pq, or Rc_pq) and VC (Rs_pq) at the thread's
-    // own entries until the seeds replace them
-#pragma unroll 4
-    for (int m = 0; m < EPT; m++) {
-        const int q = q0 + m * QS;
-        const bool ok = q < bj;
-        VR[p * LD + q] = ok ? (float)SGT_AT(MODE == 0 ? T : Rc, MODE == 0 ? ldt : ldr, r0 + p, c0 + q) : 0.f;
-        VC[q * LD + p] = (MODE == 1 && ok) ? (float)SGT_AT(Rs, ldr, r0 + p, c0 + q) : 0.f;
-    }
+    bool sp[4], sq[4];         // signs of the rows and columns (beyond n: +)
+    float c[4][4], rd[4][4];   // [row][column]: pending values, reciprocal divisors t_pp - t_qq or s_p + s_q
     {
-        const float4 *src[4] = {reinterpret_cast<const float4 *>(OPS + (size_t)(4 * I + 0) * MB * MB),
-                                reinterpret_cast<const float4 *>(OPS + (size_t)(4 * I + 1) * MB * MB),
-                                reinterpret_cast<const float4 *>(OPS + (size_t)(4 * J + 2) * MB * MB),
-                                reinterpret_cast<const float4 *>(OPS + (size_t)(4 * J + 3) * MB * MB)};
-        float *dst[4] = {Mp, Mm, Np, Nm};
-        // all four operators' loads in flight before the first store
-        constexpr int V4 = MB * MB / 4 / kLeafThreads;
-        float4 v[4][V4];
+        const float4 a = four(DIAG + r0 + kMicro * mr), b = four(DIAG + c0 + kMicro * mc);
+        const float dp[4] = {a.x, a.y, a.z, a.w}, dq[4] = {b.x, b.y, b.z, b.w};
 #pragma unroll
-        for (int a = 0; a < 4; a++)
+        for (int i = 0; i < 4; i++) {
+            sp[i] = dp[i] > 0.f;
+            sq[i] = kMicro * mc + i >= bj || dq[i] > 0.f;
+        }
 #pragma unroll
-            for (int m = 0; m < V4; m++) v[a][m] = src[a][threadIdx.x + m * kLeafThreads];
+        for (int p = 0; p < 4; p++)
 #pragma unroll
-        for (int a = 0; a < 4; a++)
-#pragma unroll
-            for (int m = 0; m < V4; m++) {
-                const int e = 4 * (threadIdx.x + m * kLeafThreads);
-                // four consecutive entries of one row (M) or column (N)
-                *reinterpret_cast<float4 *>(dst[a] + (e / MB) * LD + e % MB) = v[a][m];
-            }
+            for (int q = 0; q < 4; q++)
+                rd[p][q] = __fdividef(1.f, sp[p] != sq[q] ? dp[p] - dq[q] : (sp[p] ? 2.f : -2.f));
     }
-    for (int i = threadIdx.x; i < MB; i += kLeafThreads) {
-        const float dr = DIAG[r0 + i], dc = DIAG[c0 + i];
-        drow[i] = dr;
-        dcol[i] = dc;
-        srow[i] = dr > 0.f ? 1.f : -1.f;
-        scol[i] = (i < bj) ? (dc > 0.f ? 1.f : -1.f) : 1.f;
+    // (SEED is written by the launch before: a restricted pointer's loads could
+    // be moved above the wait)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+        *reinterpret_cast<float4 *>(Vs + own * PT + q * kMicro) =
+            four(SEED + (size_t)I * MB * MB + (own * kMicro + q) * kMicro);
+        c[0][q] = c[1][q] = c[2][q] = c[3][q] = 0.f;
     }
     __syncthreads();
 
-    // seeds: block sums (their K range includes the diagonal blocks K = I
-    // and K = J, so they already hold the in-block products of the known
-    // blocks: U_II T_IJ - T_IJ U_JJ for opposite signs in mode 0, E_II T_IJ -
-    // T_IJ E_JJ and E_II U0_IJ + U0_IJ E_JJ in mode 1; terms with the unknown
-    // V_IJ vanish, its slices being still zero), summed into acc above, and
-    // the base terms.
-    {
+    const int mine = kMicros - 1 - mr + mc;
+    for (int ph = 0; ph < 2 * kMicros - 1; ph++) {
+        if (ph == mine) {
+            // the micro-block's own recurrence (Algorithm 6, 1x1 case), column by
+            // column from the bottom row up; the term solved last is added last
+            const int dm = tri_index(mr, mr) * PT, dn = tri_index(mc, mc) * PT;
+            float4 mp[3], mm[3], np[4], nm[4];
 #pragma unroll
-        for (int m = 0; m < EPT; m++) {
-            const int q = q0 + m * QS;
-            const float b0 = VR[p * LD + q], b1 = VC[q * LD + p];
-            float c = 0.f;
-            if (q < bj) {
-                if (opp[m]) c = (MODE == 0 ? b0 * (srow[p] - scol[q]) : -b0) + acc[m];
-                else c = (MODE == 0) ? -acc[m] : -b1 - acc[m];
+            for (int i = 0; i < 3; i++) {
+                mp[i] = four(Mp + dm + i * kMicro);
+                mm[i] = four(Mm + dm + i * kMicro);
+                np[i + 1] = four(Np + dn + (i + 1) * kMicro);
+                nm[i + 1] = four(Nm + dn + (i + 1) * kMicro);
             }
-            VR[p * LD + q] = c;
-            VC[q * LD + p] = 0.f;
-        }
-    }
-    __syncthreads();
-
-    // In-tile solve (Algorithm 6, 1x1 case) by 16 x 16 sub-blocks: entry
-    // (p, q) needs the entries below it in its column and left of it in its
-    // row, so sub-block (a, b) (rows 16a.., columns 16b..) needs the
-    // sub-blocks below and left of it, and phase s = (3 - a) + b holds up to
-    // four independent sub-blocks.  A phase first adds the sums over the solved
-    // sub-blocks -- the column parts into VC, the row parts into the seeds in
-    // VR, register-blocked 4 x 2 and 2 x 4 -- then one warp per sub-block
-    // solves it (subblock_solve).
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    for (int s = 0; s < 2 * kNSub - 1; s++) {
-        const int blo = max(0, s - (kNSub - 1)), nblk = min(kNSub - 1, s) - blo + 1;
-        if (s > 0) {
-            for (int it = threadIdx.x; it < 64 * nblk; it += kLeafThreads) {
-                const int b = blo + it / 64, w = it % 64, a = kNSub - 1 - s + b;
-                const int R0 = a * kSub, C0 = b * kSub;
-                if (w < 32) {
-                    // column parts of rows R0+4mr.. x columns C0+2mc..: sum over k >= 16(a+1)
-                    const int P = R0 + 4 * (w % 4), Q = C0 + 2 * (w / 4);
-                    float acc[4][2] = {};
-                    const float *mrow[4][2];
+            auto el = [](const float4 &v, int k) { return k == 0 ? v.x : k == 1 ? v.y : k == 2 ? v.z : v.w; };
 #pragma unroll
-                    for (int i = 0; i < 4; i++)
+            for (int q = 0; q < 4; q++) {
+                float *vq = Vs + own * PT + q * kMicro;
+                const float4 seed = four(vq);
 #pragma unroll
-                        for (int j = 0; j < 2; j++) mrow[i][j] = (scol[Q + j] > 0.f ? Mp : Mm) + (P + i) * LD;
-                    for (int k = R0 + kSub; k < MB; k += 4) {
-                        const float4 v0 = *reinterpret_cast<const float4 *>(VC + Q * LD + k);
-                        const float4 v1 = *reinterpret_cast<const float4 *>(VC + (Q + 1) * LD + k);
+                for (int p = 3; p >= 0; p--) {
+                    float x = c[p][q] + el(seed, p);
 #pragma unroll
-                        for (int i = 0; i < 4; i++) {
-                            const float4 x0 = *reinterpret_cast<const float4 *>(mrow[i][0] + k);
-                            const float4 x1 = *reinterpret_cast<const float4 *>(mrow[i][1] + k);
-                            acc[i][0] = fmaf(x0.x, v0.x, fmaf(x0.y, v0.y, fmaf(x0.z, v0.z, fmaf(x0.w, v0.w, acc[i][0]))));
-                            acc[i][1] = fmaf(x1.x, v1.x, fmaf(x1.y, v1.y, fmaf(x1.z, v1.z, fmaf(x1.w, v1.w, acc[i][1]))));
-                        }
-                    }
+                    for (int k = 0; k < q; k++) x = fmaf(c[p][k], sp[p] ? el(np[q], k) : el(nm[q], k), x);
 #pragma unroll
-                    for (int i = 0; i < 4; i++)
-#pragma unroll
-                        for (int j = 0; j < 2; j++) VC[(Q + j) * LD + P + i] = acc[i][j];
-                } else {
-                    // row parts of rows R0+2mr.. x columns C0+4mc..: sum over k < 16b
-                    const int m = w - 32;
-                    const int P = R0 + 2 * (m % 8), Q = C0 + 4 * (m / 8);
-                    float acc[2][4] = {};
-                    const float *ncol[2][4];
-#pragma unroll
-                    for (int i = 0; i < 2; i++)
-#pragma unroll
-                        for (int j = 0; j < 4; j++) ncol[i][j] = (srow[P + i] > 0.f ? Np : Nm) + (Q + j) * LD;
-                    for (int k = 0; k < C0; k += 4) {
-                        const float4 v0 = *reinterpret_cast<const float4 *>(VR + P * LD + k);
-                        const float4 v1 = *reinterpret_cast<const float4 *>(VR + (P + 1) * LD + k);
-#pragma unroll
-                        for (int j = 0; j < 4; j++) {
-                            const float4 y0 = *reinterpret_cast<const float4 *>(ncol[0][j] + k);
-                            const float4 y1 = *reinterpret_cast<const float4 *>(ncol[1][j] + k);
-                            acc[0][j] = fmaf(v0.x, y0.x, fmaf(v0.y, y0.y, fmaf(v0.z, y0.z, fmaf(v0.w, y0.w, acc[0][j]))));
-                            acc[1][j] = fmaf(v1.x, y1.x, fmaf(v1.y, y1.y, fmaf(v1.z, y1.z, fmaf(v1.w, y1.w, acc[1][j]))));
-                        }
-                    }
-#pragma unroll
-                    for (int i = 0; i < 2; i++)
-#pragma unroll
-                        for (int j = 0; j < 4; j++) VR[(P + i) * LD + Q + j] += acc[i][j];
+                    for (int k = 3; k > p; k--) x = fmaf(sq[q] ? -el(mp[p], k) : -el(mm[p], k), c[k][q], x);
+                    c[p][q] = x * rd[p][q];
                 }
+                *reinterpret_cast<float4 *>(vq) = make_float4(c[0][q], c[1][q], c[2][q], c[3][q]);
             }
-            __syncthreads();
-        }
-        if (warp < nblk) {
-            const int b = blo + warp, a = kNSub - 1 - s + b;
-            if (b * kSub < bj) subblock_solve(Mp, Mm, Np, Nm, VC, VR, srow, scol, drow, dcol, a * kSub, b * kSub, lane);
         }
         __syncthreads();
+        if (ph < mine) {
+            // the micro-blocks solved now in the same rows (K, to the left) and in
+            // the same columns (L, below)
+            const int K = ph - (kMicros - 1) + mr, L = kMicros - 1 + mc - ph;
+            if (K >= 0) {
+                const float *v = Vs + (mr * kMicros + K) * PT;
+                const int o = tri_index(K, mc) * PT;
+                const float4 v0 = four(v), v1 = four(v + 4), v2 = four(v + 8), v3 = four(v + 12);
+                const float w[4][4] = {{v0.x, v1.x, v2.x, v3.x}, {v0.y, v1.y, v2.y, v3.y},
+                                       {v0.z, v1.z, v2.z, v3.z}, {v0.w, v1.w, v2.w, v3.w}};
+#pragma unroll
+                for (int q = 0; q < 4; q++) {
+                    const float4 a = four(Np + o + q * kMicro), b = four(Nm + o + q * kMicro);
+#pragma unroll
+                    for (int p = 0; p < 4; p++) {
+                        c[p][q] = fmaf(w[p][0], sp[p] ? a.x : b.x, c[p][q]);
+                        c[p][q] = fmaf(w[p][1], sp[p] ? a.y : b.y, c[p][q]);
+                        c[p][q] = fmaf(w[p][2], sp[p] ? a.z : b.z, c[p][q]);
+                        c[p][q] = fmaf(w[p][3], sp[p] ? a.w : b.w, c[p][q]);
+                    }
+                }
+            }
+            if (L < kMicros) {
+                const float *v = Vs + (L * kMicros + mc) * PT;
+                const int o = tri_index(mr, L) * PT;
+                float4 w[4];
+#pragma unroll
+                for (int q = 0; q < 4; q++) w[q] = four(v + q * kMicro);
+#pragma unroll
+                for (int p = 0; p < 4; p++) {
+                    const float4 a = four(Mp + o + p * kMicro), b = four(Mm + o + p * kMicro);
+#pragma unroll
+                    for (int q = 0; q < 4; q++) {
+                        c[p][q] = fmaf(sq[q] ? -a.x : -b.x, w[q].x, c[p][q]);
+                        c[p][q] = fmaf(sq[q] ? -a.y : -b.y, w[q].y, c[p][q]);
+                        c[p][q] = fmaf(sq[q] ? -a.z : -b.z, w[q].z, c[p][q]);
+                        c[p][q] = fmaf(sq[q] ? -a.w : -b.w, w[q].w, c[p][q]);
+                    }
+                }
+            }
+        }
     }
+    // (the last phase's barrier was passed after its values were stored)
 
     // V (float64) and its 16-bit splits in the blocked slice layout: row
     // slices tile (I, J) of Vr[s] (row-major), column slices tile (J, I) of
@@ -461,26 +383,24 @@ mixed_leaf_kernel(int n, const double *__restrict__ T, int ldt, double *__restri
     const float sc = f16 ? sigma : 1.f;
     const size_t tr = ((size_t)I * nbk + J) * MB * MB, tc = ((size_t)J * nbk + I) * MB * MB;
     const size_t sstride = (size_t)nbk * nbk * MB * MB;
-    // four consecutive entries per thread and store: column form (and V) from
-    // VC, row form from VR
+    // four consecutive entries per thread and store
     for (int idx = threadIdx.x; idx < MB * MB / 4; idx += kLeafThreads) {
-        const int pr = 4 * (idx % (MB / 4)), q = idx / (MB / 4);
+        const int m = idx % kMicros, q = idx / kMicros;   // rows 4 m .., column q
         if (q < bj) {
-            const float4 r = *reinterpret_cast<const float4 *>(VC + q * LD + pr);
-            double *vo = &SGT_AT(V, ldv, r0 + pr, c0 + q);
-            vo[0] = r.x; vo[1] = r.y; vo[2] = r.z; vo[3] = r.w;
-            split_store4(make_float4(r.x * sc, r.y * sc, r.z * sc, r.w * sc), S, f16, Vc + tc + q * MB + pr, sstride);
+            const float4 r = four(Vs + (m * kMicros + q / kMicro) * PT + q % kMicro * kMicro);
+            double *vo = &SGT_AT(V, ldv, r0 + kMicro * m, c0 + q);
+            vo[0] = f32_to_f64_bits(r.x);
+            vo[1] = f32_to_f64_bits(r.y);
+            vo[2] = f32_to_f64_bits(r.z);
+            vo[3] = f32_to_f64_bits(r.w);
+            split_store4(make_float4(r.x * sc, r.y * sc, r.z * sc, r.w * sc), S, f16, Vc + tc + q * MB + kMicro * m, sstride);
         }
     }
     for (int idx = threadIdx.x; idx < MB * MB / 4; idx += kLeafThreads) {
-        const int q = 4 * (idx % (MB / 4)), pr = idx / (MB / 4);
-        if (q < bj) {
-            // columns at or beyond bj stay zero: a partial group keeps them so
-            float4 r = *reinterpret_cast<const float4 *>(VR + pr * LD + q);
-            if (q + 1 >= bj) r.y = 0.f;
-            if (q + 2 >= bj) r.z = 0.f;
-            if (q + 3 >= bj) r.w = 0.f;
-            split_store4(make_float4(r.x * sc, r.y * sc, r.z * sc, r.w * sc), S, f16, Vr + tr + pr * MB + q, sstride);
+        const int m = idx % kMicros, pr = idx / kMicros;   // row pr, columns 4 m .. (beyond n: 0)
+        if (kMicro * m < bj) {
+            const float *v = Vs + (pr / kMicro * kMicros + m) * PT + pr % kMicro;
+            split_store4(make_float4(v[0] * sc, v[4] * sc, v[8] * sc, v[12] * sc), S, f16, Vr + tr + pr * MB + kMicro * m, sstride);
         }
     }
 }
@@ -887,6 +807,7 @@ struct MixedCtx {
     // bf16 splits (S slices) of T and of the unknowns, row and column forms,
     // blocked layout (each 64 x 64 tile contiguous)
     __nv_bfloat16 *Tr, *Tc, *Ur, *Uc, *Er, *Ec;
+    float *SEED;                // the leaves' seeds of one anti-diagonal
     float *OPS, *DIAG;          // per-sign fp32 operators of the diagonal blocks for the leaves, fp32 diagonal
     // exact slices of the strictly upper parts of T and U in the gathered
     // layout (residual products): ng gathered positions, rows_g allocated
@@ -947,7 +868,8 @@ size_t bytes_for(int n, int S)
     b += 2 * maxjobs * 16384 * 8 + 2 * 256;                             // partials
     b += 2 * (size_t)n * n * 8 + 2 * 256;                               // E, R (= Rs)
     b += 64 + 256;                                                      // norms
-    b += 4 * nb * MB * MB * sizeof(float) + nb * MB * sizeof(float) + 2 * 256;   // leaf operators, diagonal
+    // leaf operators, seeds, diagonal
+    b += nb * (4 * kMicro * kMicro * kTri + MB * MB + MB) * sizeof(float) + 3 * 256;
     b += 3 * (np + 64) * sizeof(float) + 64 + 4 * 256;                  // fp16 split scales, max slot
     const size_t pairs_max = ngr / 128 + 2 * (size_t)((n + kSuper - 1) / kSuper) + 2;
     b += pairs_max * pairs_max * sizeof(TcJob) + 256;                   // needed-residual jobs
@@ -1039,7 +961,7 @@ signtri_status sweep(MixedCtx &c, const double *T, int ldt, double *V, int ldv, 
                      __nv_bfloat16 *Vc, const double *U0, int ldu0)
 {
     const int n = c.n, nb = c.sc.nb;
-    const size_t leaf_smem = (size_t)kLeafBufs * MB * kLeafLD * sizeof(float);
+    const size_t leaf_smem = kLeafSmem;
     SGT_CUDA_TRY(cudaFuncSetAttribute(mixed_leaf_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)leaf_smem));
     SGT_CUDA_TRY(cudaFuncSetAttribute(mixed_leaf_kernel<MODE>, cudaFuncAttributePreferredSharedMemoryCarveout,
@@ -1168,9 +1090,22 @@ signtri_status sweep(MixedCtx &c, const double *T, int ldt, double *V, int ldv, 
             }
         }
         ProfScope ps(MODE == 0 ? SIGNTRI_KC_OFFDIAG_LEAF_F32 : SIGNTRI_KC_CORRECTION, c.st);
-        mixed_leaf_kernel<MODE><<<ntiles, kLeafThreads, leaf_smem, c.st>>>(
-            n, T, ldt, V, ldv, c.OPS, c.DIAG, c.res_c, c.res_s, n, d, leaf_slots, leaf_slots2, c.PA, c.PB, Vr, Vc,
-            c.S, nb, c.f16 ? (MODE == 0 ? c.sU : c.sE) : 0.f);
+        leaf_seed_kernel<MODE><<<dim3(ntiles, MB * MB / kLeafThreads), kLeafThreads, 0, c.st>>>(
+            n, T, ldt, c.DIAG, c.res_c, c.res_s, n, d, leaf_slots, leaf_slots2, c.PA, c.PB, c.SEED);
+        SGT_LAUNCH_CHECK();
+        cudaLaunchAttribute attr{};
+        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr.val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(ntiles);
+        cfg.blockDim = dim3(kLeafThreads);
+        cfg.dynamicSmemBytes = leaf_smem;
+        cfg.stream = c.st;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        SGT_CUDA_TRY(cudaLaunchKernelEx(&cfg, mixed_leaf_kernel<MODE>, n, V, ldv, (const float *)c.OPS,
+                                        (const float *)c.DIAG, d, (const float *)c.SEED, Vr, Vc, c.S, nb,
+                                        c.f16 ? (MODE == 0 ? c.sU : c.sE) : 0.f));
         SGT_LAUNCH_CHECK();
     }
     return SIGNTRI_OK;
@@ -1493,7 +1428,9 @@ signtri_status mixed_run(int n, const double *T, int ldt, double *U, int ldu, in
     const size_t maxjobs = (size_t)std::max({c.sc.max_jobs, c.scA.max_jobs, c.scB.max_jobs, c.scC.max_jobs, 1});
     c.PA = take<double>(ws, maxjobs * 16384); c.PB = take<double>(ws, maxjobs * 16384);
     c.E = take<double>(ws, (size_t)n * n); c.R = take<double>(ws, (size_t)n * n);
-    c.OPS = take<float>(ws, (size_t)4 * nb * MB * MB); c.DIAG = take<float>(ws, (size_t)nb * MB);
+    c.OPS = take<float>(ws, (size_t)4 * nb * kMicro * kMicro * kTri);
+    c.SEED = take<float>(ws, (size_t)nb * MB * MB);
+    c.DIAG = take<float>(ws, (size_t)nb * MB);
     c.invT = take<float>(ws, np + 64); c.invU = take<float>(ws, np + 64); c.invE = take<float>(ws, np + 64);
     c.amax = take<unsigned>(ws, 16);
     if (!c.invT || !c.invU || !c.invE || !c.amax) return SIGNTRI_ERR_NO_WORKSPACE;
@@ -1532,7 +1469,7 @@ signtri_status mixed_run(int n, const double *T, int ldt, double *U, int ldu, in
         !c.NUc || !c.d_full_jobs || !c.sTr ||
         !c.sTc || !c.sUr || !c.sUc || !c.gTr || !c.gTc || !c.gUr || !c.gUc || !c.gmap || !c.ginv || !c.pos ||
         !c.tmpmax || !c.tmpmax2 || !c.PA || !c.PB || !c.E || !c.R || !c.RA || !c.RB || !c.norms || !c.d_res_jobs ||
-        !c.d_pairs_split || !c.d_pairs_oz || !c.OPS || !c.DIAG || !c.sbbase)
+        !c.d_pairs_split || !c.d_pairs_oz || !c.OPS || !c.SEED || !c.DIAG || !c.sbbase)
         return SIGNTRI_ERR_NO_WORKSPACE;
     c.pairs_split = split_pairs(S);
     c.pairs_oz = ozaki_pairs_impl(kOzakiSlices, kOzakiBits);

@@ -46,6 +46,9 @@ constexpr int kLevelThreads = 2 * LT;
 constexpr int LD = LB + 1;      // shared-memory pitch of a block
 constexpr int BLK = LB * LD;    // doubles per staged block
 
+// What a launch before may still be writing when a kernel starts (U, the slabs)
+// is passed without __restrict__: a restricted pointer's loads may be moved
+// above the wait.
 // Wait for the launch this one programmatically depends on (all of it, with
 // its writes visible); let the next launch start its independent part.
 __device__ __forceinline__ void dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
@@ -156,8 +159,8 @@ constexpr size_t level_workspace_bytes(int n)
 // barrier), and add up at the end; the next K-block is in flight in registers
 // while one is summed.
 template <bool general, class S>
-__device__ __forceinline__ void far_sums(int n, const S *__restrict__ T, int ldt, const S *__restrict__ U,
-                                         int ldu, int I, int J, int kb0, int kb1, S *__restrict__ slab,
+__device__ __forceinline__ void far_sums(int n, const S *__restrict__ T, int ldt, const S *U,
+                                         int ldu, int I, int J, int kb0, int kb1, S *slab,
                                          Smem<S> &sm)
 {
     const int r0 = I * LB, c0 = J * LB;
@@ -317,8 +320,8 @@ __device__ __forceinline__ void solve16(S acc, S base, S rinv, unsigned long lon
 // dependency_wait(); for d <= 2 the blocks next to the diagonal are not yet
 // among it.  Run by the first half of the CTA.
 template <bool general, class S>
-__device__ __forceinline__ void leaf(int n, const S *__restrict__ T, int ldt, S *__restrict__ U, int ldu,
-                                     int I, int J, int nslab, const S *__restrict__ slab0, Smem<S> &sm)
+__device__ __forceinline__ void leaf(int n, const S *__restrict__ T, int ldt, S *U, int ldu,
+                                     int I, int J, int nslab, const S *slab0, Smem<S> &sm)
 {
     auto &s = sm.leaf;
     const S zero = real_value<S>(0.0);
@@ -468,9 +471,9 @@ __device__ __forceinline__ void diag_leaf(int n, const double *__restrict__ T, i
 // `out` (split sout).
 template <bool general, class S>
 __global__ void __launch_bounds__(kLevelThreads)
-level_kernel(int n, const S *__restrict__ T, int ldt, S *__restrict__ U, int ldu, int d, int leaves,
-             const __grid_constant__ Split sin, const S *__restrict__ in,
-             const __grid_constant__ Split sout, S *__restrict__ out)
+level_kernel(int n, const S *__restrict__ T, int ldt, S *U, int ldu, int d, int leaves,
+             const __grid_constant__ Split sin, const S *in,
+             const __grid_constant__ Split sout, S *out)
 {
     extern __shared__ __align__(16) unsigned char raw[];
     Smem<S> &sm = *reinterpret_cast<Smem<S> *>(raw);

@@ -321,7 +321,7 @@ constexpr CrtConst make_crt_const()
 __constant__ CrtConst c_crt = make_crt_const();
 
 // The product an entry's residues stand for (16 bytes, 16 KB apart).
-__device__ __forceinline__ double crt(const int8_t *__restrict__ y)
+__device__ __forceinline__ double crt(const int8_t *y)
 {
     unsigned long long a0 = 0, a1 = 0, a2 = 0;
 #pragma unroll
@@ -403,12 +403,12 @@ union WaveSmem {
     } far;
 };
 
-__device__ __forceinline__ double at_or_zero(const double *__restrict__ M, int ld, int i, int j, int ni, int nj)
+__device__ __forceinline__ double at_or_zero(const double *M, int ld, int i, int j, int ni, int nj)
 {
     return i < ni && j < nj ? SGT_AT(M, ld, i, j) : 0.0;
 }
 
-__device__ __forceinline__ void wave_far(const Wave &wv, int b, int l, double *__restrict__ slabs, WaveSmem &sm)
+__device__ __forceinline__ void wave_far(const Wave &wv, int b, int l, double *slabs, WaveSmem &sm)
 {
     const WaveBlock k = wave_block(wv, b / kParts, l);
     const Problem &w = k.p;
@@ -461,7 +461,7 @@ __device__ __forceinline__ void wave_far(const Wave &wv, int b, int l, double *_
     slabs[(((size_t)k.t * SB + k.jj) * kParts + part) * LT + p + q * LB] = acc;
 }
 
-__device__ __forceinline__ void wave_leaf(const Wave &wv, int b, int l, bool first, const double *__restrict__ slabs,
+__device__ __forceinline__ void wave_leaf(const Wave &wv, int b, int l, bool first, const double *slabs,
                                           WaveSmem &sm)
 {
     auto &s = sm.leaf;
@@ -560,7 +560,7 @@ __device__ __forceinline__ void wave_leaf(const Wave &wv, int b, int l, bool fir
 // Step l of every superblock of the launch: its leaves, and beside them the
 // sums of step l + 1 over finished blocks that this step does not change.
 __global__ void __launch_bounds__(kThreads)
-wave_kernel(const __grid_constant__ Wave w, int l, bool first, const double *__restrict__ in, double *__restrict__ out)
+wave_kernel(const __grid_constant__ Wave w, int l, bool first, const double *in, double *out)
 {
     __shared__ WaveSmem sm;
     const int leaves = w.tiles * wave_blocks(l), b = blockIdx.x;
