@@ -123,7 +123,6 @@ int current_cutoff();
 
 // Recursive Parlett-Higham, float64 (ph_fp64.cu)
 size_t ph_fp64_workspace_bytes(int n, int b);
-signtri_status diag_leaves_f64(int n, const double *T, int ldt, double *U, int ldu, int b, cudaStream_t st);
 // every off-diagonal block of U in blocks of 16, the diagonal blocks being
 // solved; general: U = phi(T), every entry from TU = UT.  Workspace:
 // ph_fp64_workspace_bytes(n, 16)

@@ -406,47 +406,61 @@ mixed_leaf_kernel(int n, double *__restrict__ V, int ldv, const float *__restric
 }
 
 // Correction on the diagonal blocks: the recurrences above restricted to one
-// block, by anti-diagonal, float64.
+// block, by anti-diagonal, float64, each entry's terms split over four
+// neighbouring lanes (a chain of dependent float64 operations takes 74 cycles
+// for each: one lane an entry took 0.5 ms).
 __global__ void __launch_bounds__(kLeafThreads)
 corr_diag_leaf_kernel(int n, const double *__restrict__ T, int ldt, const double *__restrict__ U0, int ldu0,
                       const double *__restrict__ Rc, const double *__restrict__ Rs, int ldr, double *__restrict__ E,
                       int lde)
 {
     constexpr int LD = MB + 1;
+    static_assert(kLeafThreads == 4 * MB, "four lanes per entry of an anti-diagonal");
     extern __shared__ double dsm[];
     double *Ts = dsm;
     double *Us = Ts + MB * LD;
-    double *Es = Us + MB * LD;
+    double *Es = Us + MB * LD;   // -Rc or -Rs until the entry is solved
     const int r0 = blockIdx.x * MB;
     const int bs = min(MB, n - r0);
     for (int idx = threadIdx.x; idx < bs * bs; idx += kLeafThreads) {
         const int i = idx % bs, j = idx / bs;
         Ts[i + j * LD] = (i <= j) ? SGT_AT(T, ldt, r0 + i, r0 + j) : 0.0;
         Us[i + j * LD] = (i <= j) ? SGT_AT(U0, ldu0, r0 + i, r0 + j) : 0.0;
-        Es[i + j * LD] = 0.0;
     }
     __syncthreads();
+    for (int idx = threadIdx.x; idx < bs * bs; idx += kLeafThreads) {
+        const int i = idx % bs, j = idx / bs;
+        const bool opp = (Ts[i + i * LD] > 0.0) != (Ts[j + j * LD] > 0.0);
+        Es[i + j * LD] = i < j ? -SGT_AT(opp ? Rc : Rs, ldr, r0 + i, r0 + j) : 0.0;
+    }
+    __syncthreads();
+    const int i = threadIdx.x / 4, part = threadIdx.x % 4;
     for (int dd = 1; dd < bs; dd++) {
-        for (int i = threadIdx.x; i < bs - dd; i += kLeafThreads) {
-            const int j = i + dd;
-            const double si = Ts[i + i * LD] > 0.0 ? 1.0 : -1.0, sj = Ts[j + j * LD] > 0.0 ? 1.0 : -1.0;
-            double e;
-            if (si + sj == 0.0) {
-                double s = -SGT_AT(Rc, ldr, r0 + i, r0 + j);
-                for (int k = i + 1; k < j; k++) s += Es[i + k * LD] * Ts[k + j * LD] - Ts[i + k * LD] * Es[k + j * LD];
-                e = s / (Ts[i + i * LD] - Ts[j + j * LD]);
-            } else {
-                double s = -SGT_AT(Rs, ldr, r0 + i, r0 + j);
-                for (int k = i + 1; k < j; k++) s -= Us[i + k * LD] * Es[k + j * LD] + Es[i + k * LD] * Us[k + j * LD];
-                e = s / (si + sj);
+        const int j = i + dd;
+        const bool live = j < bs;
+        double s = 0.0;
+        bool opp = false;
+        if (live) {
+            opp = (Ts[i + i * LD] > 0.0) != (Ts[j + j * LD] > 0.0);
+            // signs differ: e t - t e; agree: - u e - e u
+            const double *M = opp ? Ts : Us;
+            for (int k = i + 1 + part; k < j; k += 4) {
+                s = fma(-M[i + k * LD], Es[k + j * LD], s);
+                s = fma(opp ? Es[i + k * LD] : -Es[i + k * LD], M[k + j * LD], s);
             }
-            Es[i + j * LD] = e;
+        }
+        s += __shfl_xor_sync(0xffffffffu, s, 1);
+        s += __shfl_xor_sync(0xffffffffu, s, 2);
+        if (live && part == 0) {
+            const double si = Ts[i + i * LD] > 0.0 ? 1.0 : -1.0;
+            s += Es[i + j * LD];
+            Es[i + j * LD] = opp ? s / (Ts[i + i * LD] - Ts[j + j * LD]) : s * (0.5 * si);
         }
         __syncthreads();
     }
     for (int idx = threadIdx.x; idx < bs * bs; idx += kLeafThreads) {
-        const int i = idx % bs, j = idx / bs;
-        if (i < j) SGT_AT(E, lde, r0 + i, r0 + j) = Es[i + j * LD];
+        const int i2 = idx % bs, j2 = idx / bs;
+        if (i2 < j2) SGT_AT(E, lde, r0 + i2, r0 + j2) = Es[i2 + j2 * LD];
     }
 }
 
@@ -868,6 +882,7 @@ size_t bytes_for(int n, int S)
     b += 2 * maxjobs * 16384 * 8 + 2 * 256;                             // partials
     b += 2 * (size_t)n * n * 8 + 2 * 256;                               // E, R (= Rs)
     b += 64 + 256;                                                      // norms
+    b += ph_fp64_workspace_bytes(n, 16) + 512;                         // diagonal blocks' partial sums
     // leaf operators, seeds, diagonal
     b += nb * (4 * kMicro * kMicro * kTri + MB * MB + MB) * sizeof(float) + 3 * 256;
     b += 3 * (np + 64) * sizeof(float) + 64 + 4 * 256;                  // fp16 split scales, max slot
@@ -1571,8 +1586,13 @@ signtri_status mixed_run(int n, const double *T, int ldt, double *U, int ldu, in
         return rs;
 
     // 1. low-precision solve: diagonal blocks in float64, the rest by sweep
-    if ((rs = launch_zero_strict_lower(n, U, ldu, st)) != SIGNTRI_OK) return rs;
-    if ((rs = diag_leaves_f64(n, T, ldt, U, ldu, MB, st)) != SIGNTRI_OK) return rs;
+    // the diagonal 64 x 64 blocks, by leaves of 16 (block anti-diagonals 0 .. 3,
+    // what they hold beyond the blocks to be overwritten)
+    {
+        const size_t mark = ws.used;
+        if ((rs = ph_fp64_near_run(n, T, ldt, U, ldu, MB / 16 - 1, ws, st)) != SIGNTRI_OK) return rs;
+        ws.used = mark;
+    }
     if (c.f16) {
         // U's scale from its diagonal blocks, largest entry to 2^12 .. 2^13:
         // room for off-diagonal entries up to 8x larger
