@@ -56,7 +56,10 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kQrThreads = 512;
 constexpr int kMaxSweepsPerEigenvalue = 100;
-constexpr long long kRotationBudget = 1LL << 15;   // rotations per launch of the QR kernel (then a sweep's end)
+constexpr long long kRotationBudget = 1LL << 13;   // rotations per launch of the QR kernel (then a sweep's end)
+// rotations (and sweeps) a launch's log holds: two sweeps of a full window
+// always fit
+inline size_t rotation_room(int n) { return ((size_t)1 << 15) + 2 * (size_t)n + 2; }
 
 #define SGT_A(M, ld, i, j) (M)[(size_t)(i) + (size_t)(j) * (size_t)(ld)]
 
@@ -315,39 +318,42 @@ __global__ void qr_state_init_kernel(int n, QrState *st)
     st->rotations = 0;
 }
 
-// One cluster of CL CTAs runs the sweeps, one or two bulges at a time.
-// Two bulges: both eigenvalues of the window's trailing 2 x 2 as shifts
-// (Francis's double shift, in complex arithmetic as two single shifts), the
-// second bulge started 3 steps behind the first; mathematically the two
-// sweeps one after the other (the rotations of the front sweep that touch
-// the rear bulge's rows and columns are all done before it gets there, and
-// the later ones act on disjoint rows and columns), with half the dependent
-// steps.  On GB300 a float64 warp instruction holds its SM sub-partition's
-// float64 pipe for ~64 cycles whatever the number of active lanes (and
-// rsqrt or a division for ~430), so the kernel is laid out around float64
-// instruction counts:
-//  * CTA 0's warp b (chief warp of bulge b) runs that chase's serial part
-//    alone on its sub-partition: the 2 x 2 block at (k, k) and row k+2 of
+// One cluster of CL CTAs runs the sweeps, up to kMaxBulges bulges at a time,
+// each started 3 steps behind the one before it: mathematically single-shift
+// sweeps one after the other (the rotations of a front sweep that touch a
+// rear bulge's rows and columns are all done before it gets there, and the
+// later ones act on disjoint rows and columns), in 1 / kMaxBulges of the
+// dependent steps.  Three bulges and more take the eigenvalues of the
+// window's trailing block of as many rows as shifts (small_eigs, single
+// precision: a shift only steers the convergence, to a factor ~1e-7 a sweep),
+// two the eigenvalues of the trailing 2 x 2 in float64, which is also what a
+// window goes back to after 6 sweeps without a deflation (a graded block's
+// small eigenvalues are lost in single precision).
+// A step is bounded by latencies.  A float64 instruction takes ~74 cycles and
+// a warp has one in flight, an SM starts one every 16-20 cycles, so the kernel
+// is laid out around the float64 instructions of its longest chain:
+//  * a chief warp per bulge (kChiefs per CTA, in CTAs 0..kChiefCtas-1) runs
+//    that chase's serial part: the 2 x 2 block at (k, k) and row k+2 of
 //    columns k, k+1, where the next rotation's inputs (h_{k+1,k}, h_{k+2,k})
-//    are formed, lane-parallel (one real output per lane: 8 lanes for G's
-//    action on the block's two columns, 12 for G^H's on its three rows, 3
-//    float64 instructions each), kept in registers from step to step; the
-//    entry left of the block (h_{k,k-1}, zeroing the old bulge) from the
-//    rotation's own inputs; then the next rotation, its two reciprocal
-//    square roots in lanes 0 and 1 at once, stored into every CTA's shared
+//    are formed, one real output per lane (8 lanes for G's action on the
+//    block's two columns, 12 for G^H's on its three rows, 3 float64
+//    instructions each), kept in registers from step to step; then the next
+//    rotation (one reciprocal square root), stored into every CTA's shared
 //    memory (two slots per bulge, alternating).  The one entry of the next
 //    block that another thread writes, h_{k+1,k+2} (row op of column k+2),
 //    comes through shared memory; the front chase loads the entries no step
-//    touches before (h_{k+2,k+2}, h_{k+3,k+2}) two steps ahead, the rear
-//    chase takes them from the front chief, who wrote them one and zero
-//    steps before (h_{k+2,k+2} as its block's corner, h_{k+3,k+2} as the
-//    entry left of its block), or from T once the front chase has ended.
-//  * CTAs 1.. do the rest of every rotation (rows k, k+1 across the window,
-//    columns k, k+1 above the block) and, with two bulges, the 2 x 2 block
-//    at the rear bulge's rows and the front bulge's columns, which takes the
-//    rear rotation from the left and the front one from the right; entry e
-//    goes to warp e / 32 of a sequence that alternates CTAs and
-//    sub-partitions, so the work fills whole warps spread over the cluster.
+//    touches before (h_{k+2,k+2}, h_{k+3,k+2}) two steps ahead, a rear
+//    chase takes them from the bulge in front, whose warps wrote them one and
+//    zero steps before (h_{k+2,k+2} as its block's corner, h_{k+3,k+2} as the
+//    entry left of its block), or from T once that chase has ended.
+//  * a helper warp per bulge forms the entry left of the block (h_{k,k-1},
+//    zeroing the old bulge) and logs the rotation, off the chief's chain.
+//  * the other CTAs do the rest of every rotation: a warp takes 32 columns of
+//    rows k, k+1 or 32 rows of columns k, k+1 of one bulge (whole warps of
+//    one kind: mixed ones ran each kind's loads and arithmetic in turn), and
+//    a few warps the 2 x 2 blocks at a rear bulge's rows and a front bulge's
+//    columns, which take the rear rotation from the left and the front one
+//    from the right.
 // One cluster barrier per step; no entry is written by one thread while
 // another reads it.  CTA 0 alone takes every decision (deflation, shifts,
 // stop) and broadcasts it, so all CTAs run the same barriers.  T is read with
@@ -355,53 +361,61 @@ __global__ void qr_state_init_kernel(int n, QrState *st)
 // action on the columns right of the window (rows there are never read by a
 // later sweep: the window only shrinks) and on Q is left to
 // apply_rotations_kernel, which runs on other SMs alongside the next launch:
-// this kernel logs each sweep and its rotations instead (the rear sweep after
-// the front one).
-constexpr int kMaxBulges = 2;
-enum { kActSweep = 0, kActDeflate = 1, kActStop = 2 };
+// this kernel logs each sweep and its rotations instead (a rear sweep after
+// the one in front of it).
+constexpr int kMaxBulges = 8;
+constexpr int kChiefs = 2;   // chief warps (and as many helpers) of a chief CTA
+constexpr int kChiefCtas = (kMaxBulges + kChiefs - 1) / kChiefs;
+constexpr int kCross = kMaxBulges * (kMaxBulges - 1) / 2;   // pairs of bulges
+constexpr int kCrossWarps = (kCross + 15) / 16;             // two lanes per pair
+enum { kActSweep = 0, kActStop = 2 };
 
 __device__ __forceinline__ double2 ldT(const double2 *p) { return __ldcg(p); }
 // the unbiased exponent field of |x| (integer operations only)
-__device__ __forceinline__ int exp_field(double x)
+__device__ __forceinline__ int exp_field(double x) { return ((__double2hiint(x) >> 20) & 0x7ff) - 1023; }
+
+// 1 / sqrt(a) for a normal a > 0: with a = 4^h m, m in [1, 4), a single-
+// precision reciprocal root r of m (relative error below 2^-20 with m's
+// mantissa cut to 23 bits) and one step of the third-order iteration
+// r (1 + e / 2 + 3 e^2 / 8), e = 1 - m r^2, from the binomial series of
+// (1 - e)^(-1/2): the series' next term is below 2^-60.  Five float64
+// instructions; the powers of two are moved by integer operations.
+__device__ __forceinline__ double rsqrt_normal(double a)
 {
-    return (int)(((unsigned long long)__double_as_longlong(x) >> 52) & 0x7ff) - 1023;
+    const int hi = __double2hiint(a), lo = __double2loint(a);
+    const int h = ((hi >> 20) - 1023) >> 1;
+    const int mh = hi - (h << 21);
+    const float r0 = rsqrtf(__int_as_float((int)(((unsigned)(mh - (896 << 20)) << 3) | ((unsigned)lo >> 29))));
+    const unsigned rb = (unsigned)__float_as_int(r0);
+    const double m = __hiloint2double(mh, lo);
+    const double r = __hiloint2double((int)(rb >> 3) + (896 << 20), (int)(rb << 29));
+    const double e = fma(-(m * r), r, 1.0);
+    const double y = fma(fma(0.375, e, 0.5), r * e, r);
+    return __hiloint2double(__double2hiint(y) - (h << 20), __double2loint(y));
 }
 
-__device__ __forceinline__ bool is_zero2(double2 v)
+// make_rotation for a chief warp, lane-parallel.  v: in every lane the
+// operands of one product sum p q + u w, by lane & 3 of 0 |x|^2, 1 |y|^2,
+// 2 Re x conj(y), 3 Im x conj(y).  With f = (|x|^2 (|x|^2 + |y|^2))^(-1/2):
+// c = |x|^2 f, s = x conj(y) f, every lane's product its own output, passed
+// by shuffles.  Only where x's and y's exponents lie in [-200, 200], so that
+// no product leaves the normal range; else make_rotation.
+__device__ __forceinline__ void make_rotation_warp(double p, double q, double u, double w, int lane, double &c,
+                                                   double2 &s)
 {
-    return (((unsigned long long)__double_as_longlong(v.x) | (unsigned long long)__double_as_longlong(v.y)) << 1) == 0;
-}
-
-// make_rotation for the chief warp (x, y the same in every lane; every lane
-// gets (c, s)): zero tests and the exponent-range test by integer operations
-// on the bits; without scaling when every component's exponent lies in
-// [-400, 400] (else make_rotation); |x|^2 and |y|^2, the two reciprocal
-// square roots, and the two parts of x conj(y) f each in lanes 0 and 1 of
-// one instruction stream.
-__device__ __forceinline__ void make_rotation_warp(double2 x, double2 y, int lane, double &c, double2 &s)
-{
-    if (is_zero2(y)) {
-        c = 1.0;
-        s = make_double2(0.0, 0.0);
-        return;
-    }
-    const int em = max(max(exp_field(y.x), exp_field(y.y)), max(exp_field(x.x), exp_field(x.y)));
-    if (em > 400 || em < -400 || is_zero2(x)) {
+    const int em = max(exp_field(p), exp_field(u));   // lane 0: x's exponent, lane 1: y's
+    const unsigned fine = __ballot_sync(0xffffffffu, em <= 200 && em >= -200);
+    if ((fine & 3u) != 3u) {
+        const double2 x = make_double2(__shfl_sync(0xffffffffu, p, 0), __shfl_sync(0xffffffffu, u, 0));
+        const double2 y = make_double2(__shfl_sync(0xffffffffu, p, 1), __shfl_sync(0xffffffffu, u, 1));
         make_rotation(x, y, c, s);
         return;
     }
-    const bool l1 = lane & 1;
-    const double2 v = l1 ? y : x;
-    const double sq = fma(v.x, v.x, v.y * v.y);   // lane 0 |x|^2, lane 1 |y|^2
-    const double ax2 = __shfl_sync(0xffffffffu, sq, 0), ay2 = __shfl_sync(0xffffffffu, sq, 1);
-    // lane 0: Re(x conj(y)) = x.x y.x + x.y y.y; lane 1: Im = x.y y.x - x.x y.y
-    const double tt = fma(l1 ? x.y : x.x, y.x, (l1 ? -x.x : x.y) * y.y);
-    const double r = rsqrt(l1 ? ax2 : ax2 + ay2);   // lane 0 1/nrm, lane 1 1/|x|
-    const double inv_n = __shfl_sync(0xffffffffu, r, 0), inv_ax = __shfl_sync(0xffffffffu, r, 1);
-    const double f = inv_ax * inv_n;
-    c = ax2 * f;
-    const double sp = tt * f;
-    s = make_double2(__shfl_sync(0xffffffffu, sp, 0), __shfl_sync(0xffffffffu, sp, 1));
+    const double val = fma(p, q, u * w);
+    const double ax2 = __shfl_sync(0xffffffffu, val, 0), ay2 = __shfl_sync(0xffffffffu, val, 1);
+    const double out = val * rsqrt_normal(ax2 * (ax2 + ay2));
+    c = __shfl_sync(0xffffffffu, out, 0);
+    s = make_double2(__shfl_sync(0xffffffffu, out, 2), __shfl_sync(0xffffffffu, out, 3));
 }
 
 // One real output of G or G^H acting on a pair, in one of the chief warp's
@@ -412,78 +426,257 @@ __device__ __forceinline__ double pair_part(double c, double alpha, double beta,
     return fma(c, alpha, fma(beta, gamma, delta * epsilon));
 }
 
+// The eigenvalues of [a b; c d]: with x = (a - d) / 2 and y = sqrt(x^2 + bc)
+// signed so that |x + y| is the larger, the one nearer d is d - bc / (x + y)
+// (Wilkinson's shift), the other a + d minus it.  Scaled by a power of two to
+// entries of at most 2; roots and quotients by reciprocal square roots (a
+// division or hypot is a long chain of float64 latencies).
+__device__ __forceinline__ void wilkinson(double2 a, double2 b, double2 c, double2 d, double2 &near, double2 &other)
+{
+    int em = max(max(exp_field(a.x), exp_field(a.y)), max(exp_field(b.x), exp_field(b.y)));
+    em = max(em, max(max(exp_field(c.x), exp_field(c.y)), max(exp_field(d.x), exp_field(d.y))));
+    em = min(max(em, -1000), 1000);
+    const double sc = __hiloint2double((1023 - em) << 20, 0);
+    const double2 x = make_double2(0.5 * (a.x * sc - d.x * sc), 0.5 * (a.y * sc - d.y * sc));
+    const double2 bc = cmul(make_double2(b.x * sc, b.y * sc), make_double2(c.x * sc, c.y * sc));
+    const double2 xx = cmul(x, x);
+    const double2 z = make_double2(xx.x + bc.x, xx.y + bc.y);
+    // y = sqrt(z): with t = (|z| + |Re z|) / 2, sqrt(t) is the larger part,
+    // Im z / (2 sqrt(t)) the other
+    constexpr double kTiny = 0x1p-900;
+    double2 y = make_double2(0.0, 0.0);
+    const double z2 = fma(z.x, z.x, z.y * z.y);
+    const double t = 0.5 * ((z2 > kTiny ? z2 * rsqrt(z2) : 0.0) + fabs(z.x));
+    if (t > kTiny) {
+        const double r = rsqrt(t), big = t * r, small = 0.5 * z.y * r;
+        y = z.x >= 0.0 ? make_double2(big, small) : make_double2(fabs(small), copysign(big, z.y));
+    }
+    if (x.x * y.x + x.y * y.y < 0.0) y = make_double2(-y.x, -y.y);
+    const double2 xy = make_double2(x.x + y.x, x.y + y.y);
+    const double d2 = fma(xy.x, xy.x, xy.y * xy.y);
+    near = d;
+    if (d2 > kTiny) {
+        const double r = rsqrt(d2), rr = r * r;
+        const double2 q = cmul(bc, make_double2(xy.x * rr, -xy.y * rr));
+        const double un = __hiloint2double((1023 + em) << 20, 0);
+        near = make_double2(d.x - q.x * un, d.y - q.y * un);
+    }
+    other = make_double2(a.x + d.x - near.x, a.y + d.y - near.y);
+}
+
+__device__ __forceinline__ float2 cmulf(float2 a, float2 b)
+{
+    return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+}
+
+// A warp's eigenvalues of the m x m Hessenberg block h (entries of at most
+// 2), in single precision: single-shift QR sweeps over the block's own
+// window, a lane per column and then per row.  eig[q] is where the diagonal
+// entry q converged; after 8 sweeps without a deflation the diagonal is taken
+// as it stands (these are shifts: any value is valid).
+__device__ void small_eigs(float2 (*h)[kMaxBulges + 1], int m, int lane, float2 *eig)
+{
+    int i = m - 1, its = 0;
+    while (i >= 0) {
+        bool small = false;
+        if (lane >= 1 && lane <= i) {
+            const float2 s = h[lane][lane - 1], u = h[lane - 1][lane - 1], v = h[lane][lane];
+            small = fabsf(s.x) + fabsf(s.y) <= 1e-6f * (fabsf(u.x) + fabsf(u.y) + fabsf(v.x) + fabsf(v.y));
+        }
+        const unsigned mask = __ballot_sync(0xffffffffu, small);
+        const int l = mask ? 31 - __clz((int)mask) : 0;
+        if (l == i || its >= 8) {
+            if (lane == 0) eig[i] = h[i][i];
+            i--;
+            if (its < 8) its = 0;
+            continue;
+        }
+        const float2 a = h[i - 1][i - 1], b = h[i - 1][i], c = h[i][i - 1], d = h[i][i];
+        const float2 x = make_float2(0.5f * (a.x - d.x), 0.5f * (a.y - d.y));
+        const float2 bc = cmulf(b, c), xx = cmulf(x, x);
+        const float2 z = make_float2(xx.x + bc.x, xx.y + bc.y);
+        const float t = 0.5f * (sqrtf(z.x * z.x + z.y * z.y) + fabsf(z.x));
+        float2 y = make_float2(0.0f, 0.0f);
+        if (t > 0.0f) {
+            const float r = rsqrtf(t), big = t * r, sm = 0.5f * z.y * r;
+            y = z.x >= 0.0f ? make_float2(big, sm) : make_float2(fabsf(sm), copysignf(big, z.y));
+        }
+        if (x.x * y.x + x.y * y.y < 0.0f) y = make_float2(-y.x, -y.y);
+        const float2 xy = make_float2(x.x + y.x, x.y + y.y);
+        const float d2 = xy.x * xy.x + xy.y * xy.y;
+        float2 sh = d;
+        if (d2 > 0.0f) {
+            const float2 q = cmulf(bc, make_float2(xy.x / d2, -xy.y / d2));
+            sh = make_float2(d.x - q.x, d.y - q.y);
+        }
+        if (l == i - 1) {
+            if (lane == 0) {
+                eig[i] = sh;
+                eig[i - 1] = make_float2(a.x + d.x - sh.x, a.y + d.y - sh.y);
+            }
+            i -= 2;
+            its = 0;
+            continue;
+        }
+        its++;
+        for (int k = l; k < i; k++) {
+            float2 p = h[k][max(k - 1, l)], q = h[k + 1][max(k - 1, l)];
+            if (k == l) p = make_float2(p.x - sh.x, p.y - sh.y);
+            const float p2 = p.x * p.x + p.y * p.y, q2 = q.x * q.x + q.y * q.y;
+            float cc = 1.0f;
+            float2 s = make_float2(0.0f, 0.0f);
+            if (q2 > 1e-30f) {
+                const float in = rsqrtf(p2 + q2);
+                if (p2 > 1e-30f) {
+                    const float ip = rsqrtf(p2);
+                    cc = p2 * ip * in;
+                    s = cmulf(p, make_float2(q.x, -q.y));
+                    s = make_float2(s.x * ip * in, s.y * ip * in);
+                } else {
+                    cc = 0.0f;
+                    s = make_float2(q.x * in, -q.y * in);
+                }
+            }
+            __syncwarp();
+            if (lane >= max(k - 1, l) && lane <= i) {
+                const float2 u = h[k][lane], v = h[k + 1][lane];
+                const float2 sv = cmulf(s, v), su = cmulf(make_float2(s.x, -s.y), u);
+                h[k][lane] = make_float2(cc * u.x + sv.x, cc * u.y + sv.y);
+                h[k + 1][lane] = make_float2(cc * v.x - su.x, cc * v.y - su.y);
+            }
+            __syncwarp();
+            if (lane >= l && lane <= min(k + 2, i)) {
+                const float2 u = h[lane][k], v = h[lane][k + 1];
+                const float2 sv = cmulf(make_float2(s.x, -s.y), v), su = cmulf(s, u);
+                h[lane][k] = make_float2(cc * u.x + sv.x, cc * u.y + sv.y);
+                h[lane][k + 1] = make_float2(cc * v.x - su.x, cc * v.y - su.y);
+            }
+            __syncwarp();
+        }
+    }
+    __syncwarp();
+}
+
 template <int CL>
 __global__ void __launch_bounds__(kQrThreads)
-schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ st, long long budget,
+schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ st, long long budget, long long room,
                 SweepRec *__restrict__ sweeplog, double *__restrict__ rclog, double2 *__restrict__ rslog,
                 int *__restrict__ nlogged)
 {
     namespace cg = cooperative_groups;
-    constexpr int kWorkers = CL - 1, kWorkerThreads = kWorkers * kQrThreads;   // CTAs 1..
+    constexpr int kWorkers = CL - kChiefCtas, kWarps = kQrThreads / 32, kWorkerWarps = kWorkers * kWarps;
+    static_assert(kWorkers > 0 && kWarps >= 2 * kChiefs && kWorkers >= kCrossWarps, "roles");
     cg::cluster_group cl = cg::this_cluster();
-    __shared__ int redi[kQrThreads / 32];
+    __shared__ int redi[kWarps];
     __shared__ double rc[kMaxBulges][2];
     __shared__ double2 rs[kMaxBulges][2];
-    __shared__ double2 bslot[kMaxBulges][2];   // CTA 0: h_{k+1,k+2} after a step, per bulge
-    __shared__ double2 handF[2], handH[2];       // CTA 0: the front chief's corner and left entry, per step
-    __shared__ double2 sig1;                     // CTA 0: the rear bulge's shift
-    __shared__ int ctl[4];                       // action, l, i, bulges (CTA 0's decision)
+    __shared__ double2 bslot[kMaxBulges][2];              // h_{k+1,k+2} after a step, in the bulge's chief CTA
+    __shared__ double inp[kMaxBulges][2][4];              // a rotation's inputs x, y, for the helper
+    __shared__ double2 handF[kMaxBulges][2], handH[kMaxBulges][2];   // from the bulge in front: its corner and left entry
+    __shared__ double2 sig[kMaxBulges];                   // the bulges' shifts
+    __shared__ float2 blk[kMaxBulges][kMaxBulges + 1], eig[kMaxBulges];
+    __shared__ int ctl[4];                                // action, l, i, bulges (CTA 0's decision)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const unsigned crank = cl.block_rank();
-    const int cb = (crank == 0 && warp < kMaxBulges) ? warp : -1;   // the bulge of a chief warp
+    const int crank = (int)cl.block_rank();
+    const int my = crank * kChiefs + warp % kChiefs;      // the bulge of a chief or helper warp
+    const bool chief_cta = crank < kChiefCtas;
+    const bool chief = chief_cta && warp < kChiefs && my < kMaxBulges;
+    const bool helper = chief_cta && warp >= kChiefs && warp < 2 * kChiefs && my < kMaxBulges;
     const bool chief0 = crank == 0 && warp == 0;
-    // this worker thread's first entry and the stride (CTAs 1.. only)
-    const int e0 = ((warp * kWorkers + ((int)crank - 1)) << 5) + lane;
+    // a worker's warp number: consecutive ones alternate CTAs; the last
+    // kCrossWarps take the pairs of bulges, two lanes a pair
+    const int w = warp * kWorkers + (crank - kChiefCtas);
+    const bool crosser = !chief_cta && w >= kWorkerWarps - kCrossWarps;
+    int pa = 0, pb = 0;                                   // this lane's pair: pa in front of pb
+    if (crosser) {
+        const int pair = (w - (kWorkerWarps - kCrossWarps)) * 16 + (lane >> 1);
+        if (pair < kCross) {
+            pb = 1;
+            while (pair >= pb * (pb + 1) / 2) pb++;
+            pa = pair - pb * (pb - 1) / 2;
+        }
+    }
     int i = st->ihi, its = st->its, status = st->status;
     long long logged = 0, rot = 0;
     const double eps = DBL_EPSILON;
     const double tiny = DBL_MIN * ((double)n / DBL_EPSILON);
     const double2 zero = make_double2(0.0, 0.0);
-    // a chief warp's registers, the same in every lane: the block (A B; E F)
-    // at (k, k), Hh = h_{k+2,k+1}, the rotation of the step and its inputs
-    // (X, Y) = (h_{k,k-1}, h_{k+1,k-1})
-    double2 A = zero, B = zero, E = zero, F = zero, Hh = zero, X = zero, Y = zero, s_cur = zero;
-    double c_cur = 1.0;
+    const int part = lane & 3;
+    const bool odd = part & 1, hi = part >= 2, col1 = (lane >> 2) & 1;
+    const int row = min(lane >> 2, 2);
+    // A chief warp's registers.  Lane 4 col + part holds the column col of
+    // the block (A B; E F) at (k, k): top A or B, bottom E or F, each as its
+    // part `odd` and the other one; every lane Hh = h_{k+2,k+1} likewise, and
+    // the step's rotation.
+    double to = 0.0, te = 0.0, bo = 0.0, be = 0.0, ho = 0.0, he = 0.0, c_cur = 1.0;
+    double2 s_cur = zero;
     double2 pf_f = zero, pf_h = zero;   // front chase: h_{k+2,k+2}, h_{k+3,k+2} for step k+1, loaded early
-    auto put_rotation = [&](int b, int slot, double c, double2 s) {
+    auto put_rotation = [&](int b, int slot) {
         // lanes 0..CL-1 of a chief warp store into CTA `lane`
         if (lane < CL) {
-            *cl.map_shared_rank(&rc[b][slot], lane) = c;
-            *cl.map_shared_rank(&rs[b][slot], lane) = s;
+            *cl.map_shared_rank(&rc[b][slot], lane) = c_cur;
+            *cl.map_shared_rank(&rs[b][slot], lane) = s_cur;
         }
+    };
+    // a chase's first block and rotation, at (l, l) with the shift sg
+    auto start_chase = [&](int b, int slot, int l, int last, double2 sg) {
+        const double2 top = ldT(&SGT_A(T, ldt, l, l + (col1 ? 1 : 0)));
+        const double2 bot = ldT(&SGT_A(T, ldt, l + 1, l + (col1 ? 1 : 0)));
+        const double2 A = ldT(&SGT_A(T, ldt, l, l)), E = ldT(&SGT_A(T, ldt, l + 1, l));
+        if (b == 0) {
+            const double2 H = (l + 2 <= last) ? ldT(&SGT_A(T, ldt, l + 2, l + 1)) : zero;
+            pf_f = (l + 2 <= last) ? ldT(&SGT_A(T, ldt, l + 2, l + 2)) : zero;
+            pf_h = (l + 3 <= last) ? ldT(&SGT_A(T, ldt, l + 3, l + 2)) : zero;
+            ho = odd ? H.y : H.x;
+            he = odd ? H.x : H.y;
+        }
+        to = odd ? top.y : top.x;
+        te = odd ? top.x : top.y;
+        bo = odd ? bot.y : bot.x;
+        be = odd ? bot.x : bot.y;
+        const double2 X = make_double2(A.x - sg.x, A.y - sg.y);
+        const double2 v = part == 1 ? E : X, u = part == 0 ? X : E;
+        // parts 0, 1: v.x v.x + v.y v.y; 2: X.x E.x + X.y E.y; 3: X.y E.x - X.x E.y
+        make_rotation_warp(part == 3 ? X.y : v.x, part < 2 ? v.x : u.x, part == 3 ? -X.x : v.y, part < 2 ? v.y : u.y,
+                           lane, c_cur, s_cur);
+        put_rotation(b, slot);
     };
     for (;;) {
         if (crank == 0) {
-            // l: the largest k in [1, i] whose h_{k,k-1} is negligible, else 0
-            int lk = 0;
-            for (int k = 1 + tid; k <= i; k += kQrThreads) {
-                const double sub = cabs1(ldT(&SGT_A(T, ldt, k, k - 1)));
-                const double ref = cabs1(ldT(&SGT_A(T, ldt, k - 1, k - 1))) + cabs1(ldT(&SGT_A(T, ldt, k, k)));
-                if (sub <= fmax(eps * ref, tiny)) lk = k;
+            int l;
+            for (;;) {
+                // l: the largest k in [1, i] whose h_{k,k-1} is negligible, else 0
+                int lk = 0;
+                for (int k = 1 + tid; k <= i; k += kQrThreads) {
+                    const double sub = cabs1(ldT(&SGT_A(T, ldt, k, k - 1)));
+                    const double ref = cabs1(ldT(&SGT_A(T, ldt, k - 1, k - 1))) + cabs1(ldT(&SGT_A(T, ldt, k, k)));
+                    if (sub <= fmax(eps * ref, tiny)) lk = k;
+                }
+                lk = __reduce_max_sync(0xffffffffu, lk);
+                if (lane == 0) redi[warp] = lk;
+                __syncthreads();
+                l = __reduce_max_sync(0xffffffffu, lane < kWarps ? redi[lane] : 0);
+                __syncthreads();
+                if (status != 0 || i <= 0 || l < i) break;
+                // the window's last row has converged
+                if (tid == 0) SGT_A(T, ldt, i, i - 1) = zero;
+                i--;
+                its = 0;
             }
-            for (int o = 16; o > 0; o >>= 1) lk = max(lk, __shfl_xor_sync(0xffffffffu, lk, o));
-            if (lane == 0) redi[warp] = lk;
-            __syncthreads();
             if (chief0) {
-                int l = 0;
-                for (int w = 0; w < kQrThreads / 32; w++) l = max(l, redi[w]);
-                int act, nbul = 1;
+                int act = kActSweep, nbul = 1;
                 if (status != 0 || i <= 0) {
                     act = kActStop;
                     if (status == 0) {
                         status = 1;
                         i = -1;
                     }
-                } else if (l == i) {
-                    act = kActDeflate;   // the window's last row has converged
-                    if (lane == 0) SGT_A(T, ldt, i, i - 1) = zero;
-                } else if (rot >= budget) {
+                } else if (rot >= budget || (rot > 0 && rot + (long long)kMaxBulges * (i - l) > room)) {
                     act = kActStop;
                 } else if (its >= kMaxSweepsPerEigenvalue) {
                     act = kActStop;
                     status = 2;
                 } else {
-                    act = kActSweep;
                     if (l > 0 && lane == 0) SGT_A(T, ldt, l, l - 1) = zero;
                     const int sw_its = its + 1;
                     double2 sigma;
@@ -496,46 +689,46 @@ schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ s
                         const double e = top ? ldT(&SGT_A(T, ldt, l + 1, l)).x : ldT(&SGT_A(T, ldt, i, i - 1)).x;
                         sigma = make_double2(d.x + 0.75 * fabs(e), d.y);
                     } else {
-                        // Wilkinson: with x = (a - d) / 2 and y = sqrt(x^2 + bc)
-                        // signed so that |x + y| is the larger, the eigenvalue
-                        // of [a b; c d] nearer d is d - bc / (x + y); the
-                        // other one, a + d minus it, shifts the rear bulge
-                        const double2 a = ldT(&SGT_A(T, ldt, i - 1, i - 1)), b = ldT(&SGT_A(T, ldt, i - 1, i));
-                        const double2 cc = ldT(&SGT_A(T, ldt, i, i - 1)), d = ldT(&SGT_A(T, ldt, i, i));
-                        const double2 x = make_double2(0.5 * (a.x - d.x), 0.5 * (a.y - d.y));
-                        const double2 bc = cmul(b, cc);
-                        const double2 xx = cmul(x, x);
-                        double2 y = csqrt_p(make_double2(xx.x + bc.x, xx.y + bc.y));
-                        if (x.x * y.x + x.y * y.y < 0.0) y = make_double2(-y.x, -y.y);
-                        const double2 xy = make_double2(x.x + y.x, x.y + y.y);
-                        if (xy.x == 0.0 && xy.y == 0.0) {
-                            sigma = d;
+                        // a bulge per three rows; two where the log has no
+                        // room for more
+                        if (i - l >= 3) nbul = sw_its > 6 ? 2 : min(kMaxBulges, max(2, (i - l + 1) / 3));
+                        if ((long long)nbul * (i - l) > room) nbul = min(nbul, 2);
+                        if (nbul <= 2) {
+                            double2 other;
+                            wilkinson(ldT(&SGT_A(T, ldt, i - 1, i - 1)), ldT(&SGT_A(T, ldt, i - 1, i)),
+                                      ldT(&SGT_A(T, ldt, i, i - 1)), ldT(&SGT_A(T, ldt, i, i)), sigma, other);
+                            if (lane < kChiefCtas) *cl.map_shared_rank(&sig[1], lane) = other;
                         } else {
-                            const double2 q = cdiv(bc, xy);
-                            sigma = make_double2(d.x - q.x, d.y - q.y);
-                        }
-                        if (i - l >= 3) {
-                            nbul = 2;
-                            if (lane == 0) sig1 = make_double2(a.x + d.x - sigma.x, a.y + d.y - sigma.y);
+                            const int r0 = i - nbul + 1;
+                            int em = -1000;
+                            for (int t = lane; t < nbul * nbul; t += 32) {
+                                const int r = t % nbul, q = t / nbul;
+                                if (r > q + 1) continue;
+                                const double2 v = ldT(&SGT_A(T, ldt, r0 + r, r0 + q));
+                                em = max(em, max(exp_field(v.x), exp_field(v.y)));
+                            }
+                            em = min(__reduce_max_sync(0xffffffffu, em), 1000);
+                            const double sc = __hiloint2double((1023 - em) << 20, 0);
+                            for (int t = lane; t < nbul * nbul; t += 32) {
+                                const int r = t % nbul, q = t / nbul;
+                                const double2 v = r > q + 1 ? zero : ldT(&SGT_A(T, ldt, r0 + r, r0 + q));
+                                blk[r][q] = make_float2((float)(v.x * sc), (float)(v.y * sc));
+                            }
+                            __syncwarp();
+                            small_eigs(blk, nbul, lane, eig);
+                            // the last row's eigenvalue goes first
+                            const double un = __hiloint2double((1023 + em) << 20, 0);
+                            if (lane < nbul) {
+                                const float2 v = eig[nbul - 1 - lane];
+                                const double2 sg = make_double2(v.x * un, v.y * un);
+                                for (int r = 0; r < kChiefCtas; r++) *cl.map_shared_rank(&sig[lane], r) = sg;
+                            }
+                            const float2 v0 = eig[nbul - 1];
+                            sigma = make_double2(v0.x * un, v0.y * un);
                         }
                     }
-                    A = ldT(&SGT_A(T, ldt, l, l));
-                    B = ldT(&SGT_A(T, ldt, l, l + 1));
-                    E = ldT(&SGT_A(T, ldt, l + 1, l));
-                    F = ldT(&SGT_A(T, ldt, l + 1, l + 1));
-                    Hh = (l + 2 <= i) ? ldT(&SGT_A(T, ldt, l + 2, l + 1)) : zero;
-                    pf_f = (l + 2 <= i) ? ldT(&SGT_A(T, ldt, l + 2, l + 2)) : zero;
-                    pf_h = (l + 3 <= i) ? ldT(&SGT_A(T, ldt, l + 3, l + 2)) : zero;
-                    X = make_double2(A.x - sigma.x, A.y - sigma.y);
-                    Y = E;
-                    make_rotation_warp(X, Y, lane, c_cur, s_cur);
-                    put_rotation(0, 0, c_cur, s_cur);
-                    if (lane == 0) {
-                        sweeplog[logged] = SweepRec{l, i, rot};
-                        if (nbul == 2) sweeplog[logged + 1] = SweepRec{l, i, rot + (i - l)};
-                        rclog[rot] = c_cur;
-                        rslog[rot] = s_cur;
-                    }
+                    start_chase(0, 0, l, i, sigma);
+                    if (lane < nbul) sweeplog[logged + lane] = SweepRec{l, i, rot + (long long)lane * (i - l)};
                 }
                 if (lane < CL) {
                     int *rem = cl.map_shared_rank(ctl, lane);
@@ -550,111 +743,77 @@ schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ s
         const int act = ctl[0], l = ctl[1], nbul = ctl[3];
         i = ctl[2];
         if (act == kActStop) break;
-        if (act == kActDeflate) {
-            i--;
-            its = 0;
-            continue;
-        }
         its++;
         const int L = i - l, S = L + 3 * (nbul - 1);
-        double2 Fnext = zero;   // rear chief: its block's next corner
+        // this worker warp's bulge, its first piece of 32 there and the stride
+        const int wq = (kWorkerWarps - kCrossWarps) / nbul;
+        const int wb = w % nbul;
+        const bool worker = !chief_cta && w < wq * nbul;
+        double2 Fnext = zero;   // a rear chief: its block's next corner
         for (int s = 0; s < S; s++) {
-            const int k0 = l + s, k1 = l + s - 3;
-            const bool a0 = s < L;                    // front bulge at k0
-            const bool a1 = nbul > 1 && s >= 3;       // rear bulge at k1 (s - 3 < L always)
-            if (crank > 0) {
-                const double c0 = rc[0][s & 1], c1 = rc[1][s & 1];
-                const double2 s0 = rs[0][s & 1], s1 = rs[1][s & 1];
-                // items: the 2 x 2 block where the two chases meet (rows
-                // k1, k1+1 x columns k0, k0+1: the rear rotation from the
-                // left, the front one from the right; two items, lanes 0
-                // and 1 of the first warp, one column and then one row each);
-                // front rows k0, k0+1 at columns k0+2..i; front columns k0,
-                // k0+1 at rows 0..k0-1 (the rear rows apart); rear rows at
-                // columns k1+2..i (the front columns apart); rear columns at
-                // rows 0..k1-1
-                const int xn = (a0 && a1) ? 2 : 0;
-                const int r0n = a0 ? max(i - k0 - 1, 0) : 0, c0n = a0 ? k0 : 0;
-                const int r1n = a1 ? max(i - k1 - 1, 0) : 0, c1n = a1 ? k1 : 0;
-                const int wtot = xn + r0n + c0n + r1n + c1n;
-                for (int e = e0; e < wtot; e += kWorkerThreads) {
-                    int f = e;
-                    if (f < xn) {
-                        // lane f: column k0 + f through the rear rotation, then
-                        // row k1 + f through the front one
-                        const int j = k0 + f;
-                        double2 a = ldT(&SGT_A(T, ldt, k1, j)), b = ldT(&SGT_A(T, ldt, k1 + 1, j));
-                        rot_rows(c1, s1, a, b);
-                        // lane 0 holds (row k1, row k1+1) of column k0, lane 1
-                        // of column k0+1; row k1 + f needs both columns
-                        const double2 mine = f ? b : a, theirs = f ? a : b;
-                        const double2 other = make_double2(__shfl_xor_sync(0x3u, theirs.x, 1),
-                                                           __shfl_xor_sync(0x3u, theirs.y, 1));
-                        double2 p = f ? other : mine, q = f ? mine : other;
-                        rot_cols(c0, s0, p, q);
-                        SGT_A(T, ldt, k1 + f, k0) = p;
-                        SGT_A(T, ldt, k1 + f, k0 + 1) = q;
-                        continue;
-                    }
-                    f -= xn;
-                    if (f < r0n) {
-                        const int j = k0 + 2 + f;
-                        double2 a = ldT(&SGT_A(T, ldt, k0, j)), b = ldT(&SGT_A(T, ldt, k0 + 1, j));
-                        rot_rows(c0, s0, a, b);
-                        SGT_A(T, ldt, k0, j) = a;
-                        SGT_A(T, ldt, k0 + 1, j) = b;
-                        if (f == 0) *cl.map_shared_rank(&bslot[0][(s + 1) & 1], 0) = b;
-                        continue;
-                    }
-                    f -= r0n;
-                    if (f < c0n) {
-                        if (a1 && (f == k1 || f == k1 + 1)) continue;
-                        double2 a = ldT(&SGT_A(T, ldt, f, k0)), b = ldT(&SGT_A(T, ldt, f, k0 + 1));
-                        rot_cols(c0, s0, a, b);
-                        SGT_A(T, ldt, f, k0) = a;
-                        SGT_A(T, ldt, f, k0 + 1) = b;
-                        continue;
-                    }
-                    f -= c0n;
-                    if (f < r1n) {
-                        const int j = k1 + 2 + f;
-                        if (a0 && (j == k0 || j == k0 + 1)) continue;
-                        double2 a = ldT(&SGT_A(T, ldt, k1, j)), b = ldT(&SGT_A(T, ldt, k1 + 1, j));
-                        rot_rows(c1, s1, a, b);
-                        SGT_A(T, ldt, k1, j) = a;
-                        SGT_A(T, ldt, k1 + 1, j) = b;
-                        if (f == 0) *cl.map_shared_rank(&bslot[1][(s + 1) & 1], 0) = b;
-                        continue;
-                    }
-                    f -= r1n;
-                    double2 a = ldT(&SGT_A(T, ldt, f, k1)), b = ldT(&SGT_A(T, ldt, f, k1 + 1));
-                    rot_cols(c1, s1, a, b);
-                    SGT_A(T, ldt, f, k1) = a;
-                    SGT_A(T, ldt, f, k1 + 1) = b;
-                }
-            } else if (cb >= 0 && cb < nbul) {
-                const int b = cb;
-                if (b == 1 && s == 2) {
-                    // the rear chase starts next step at (l, l): entries final
-                    // since step 1 (h_{l+2,l+1} comes after this step, from the
-                    // front chief), its first rotation from its own shift
-                    A = ldT(&SGT_A(T, ldt, l, l));
-                    B = ldT(&SGT_A(T, ldt, l, l + 1));
-                    E = ldT(&SGT_A(T, ldt, l + 1, l));
-                    F = ldT(&SGT_A(T, ldt, l + 1, l + 1));
-                    const double2 sg = sig1;
-                    X = make_double2(A.x - sg.x, A.y - sg.y);
-                    Y = E;
-                    make_rotation_warp(X, Y, lane, c_cur, s_cur);
-                    put_rotation(1, 1, c_cur, s_cur);
-                    if (lane == 0) {
-                        rclog[rot + L] = c_cur;
-                        rslog[rot + L] = s_cur;
+            if (worker) {
+                const int k = l + s - 3 * wb;
+                if (s >= 3 * wb && s < L + 3 * wb) {
+                    const double c0 = rc[wb][s & 1];
+                    const double2 s0 = rs[wb][s & 1];
+                    const int rw = (i - k - 1 + 31) >> 5, cw = (k + 31) >> 5;
+                    for (int q = w / nbul; q < rw + cw; q += wq) {
+                        if (q < rw) {
+                            // rows k, k+1 at column j, but for the columns of
+                            // the bulges in front, k + 3 t and k + 3 t + 1
+                            const int d = 2 + (q << 5) + lane, j = k + d, t = d / 3;
+                            const bool cross = d >= 3 && t <= wb && d - 3 * t < 2 && s < L + 3 * (wb - t);
+                            if (j <= i && !cross) {
+                                double2 a = ldT(&SGT_A(T, ldt, k, j)), b = ldT(&SGT_A(T, ldt, k + 1, j));
+                                rot_rows(c0, s0, a, b);
+                                SGT_A(T, ldt, k, j) = a;
+                                SGT_A(T, ldt, k + 1, j) = b;
+                                if (d == 2) *cl.map_shared_rank(&bslot[wb][(s + 1) & 1], wb / kChiefs) = b;
+                            }
+                        } else {
+                            // columns k, k+1 at row r < k, but for the rows of
+                            // the bulges behind, k - 3 t and k - 3 t + 1
+                            const int r = ((q - rw) << 5) + lane, g = k - r + 1, t = g / 3;
+                            const bool cross = t >= 1 && t <= nbul - 1 - wb && g - 3 * t < 2 && k - 3 * t >= l;
+                            if (r < k && !cross) {
+                                double2 a = ldT(&SGT_A(T, ldt, r, k)), b = ldT(&SGT_A(T, ldt, r, k + 1));
+                                rot_cols(c0, s0, a, b);
+                                SGT_A(T, ldt, r, k) = a;
+                                SGT_A(T, ldt, r, k + 1) = b;
+                            }
+                        }
                     }
                 }
-                const bool act_b = (b == 0) ? a0 : a1;
-                if (act_b) {
-                    const int kb = (b == 0) ? k0 : k1;
+            } else if (crosser) {
+                // lane f of a pair: column k0 + f through the rear rotation,
+                // then row k1 + f through the front one
+                const int k0 = l + s - 3 * pa, k1 = l + s - 3 * pb, f = lane & 1;
+                const bool on = pb > pa && pb < nbul && s >= 3 * pb && s < L + 3 * pa;
+                double2 a = zero, b = zero;
+                if (on) {
+                    a = ldT(&SGT_A(T, ldt, k1, k0 + f));
+                    b = ldT(&SGT_A(T, ldt, k1 + 1, k0 + f));
+                    rot_rows(rc[pb][s & 1], rs[pb][s & 1], a, b);
+                }
+                // lane 0 holds (row k1, row k1+1) of column k0, lane 1
+                // of column k0+1; row k1 + f needs both columns
+                const double2 mine = f ? b : a, theirs = f ? a : b;
+                const double2 got = make_double2(__shfl_xor_sync(0xffffffffu, theirs.x, 1),
+                                                 __shfl_xor_sync(0xffffffffu, theirs.y, 1));
+                if (on) {
+                    double2 p = f ? got : mine, q = f ? mine : got;
+                    rot_cols(rc[pa][s & 1], rs[pa][s & 1], p, q);
+                    SGT_A(T, ldt, k1 + f, k0) = p;
+                    SGT_A(T, ldt, k1 + f, k0 + 1) = q;
+                }
+            } else if (chief && my < nbul) {
+                const int b = my, kb = l + s - 3 * b;
+                if (b > 0 && s == 3 * b - 1) {
+                    // this chase starts next step at (l, l): entries final
+                    // since the last step (h_{l+2,l+1} comes after this step,
+                    // from the bulge in front)
+                    start_chase(b, (s + 1) & 1, l, i, sig[b]);
+                } else if (s >= 3 * b && s < L + 3 * b) {
                     const double c = c_cur;
                     const double2 sn = s_cur;
                     double2 F2 = zero, H2 = zero;
@@ -664,99 +823,107 @@ schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ s
                         pf_f = (kb + 3 <= i) ? ldT(&SGT_A(T, ldt, kb + 3, kb + 3)) : zero;
                         pf_h = (kb + 4 <= i) ? ldT(&SGT_A(T, ldt, kb + 4, kb + 3)) : zero;
                     } else if (kb + 2 <= i) {
-                        // the next corner h_{k+2,k+2}: the front chief's block
-                        // corner of the previous step, or T once that chase ended
-                        Fnext = (s - 1 < L) ? handF[(s - 1) & 1] : ldT(&SGT_A(T, ldt, kb + 2, kb + 2));
+                        // the next corner h_{k+2,k+2}: the block corner of the
+                        // bulge in front, of the previous step, or T once that
+                        // chase ended
+                        Fnext = (s - 1 < L + 3 * (b - 1)) ? handF[b][(s - 1) & 1]
+                                                          : ldT(&SGT_A(T, ldt, kb + 2, kb + 2));
                     }
-                    const int part = lane & 3;
-                    const bool odd = part & 1, hi = part >= 2;
-                    if (kb > l) {
-                        // h_{k,k-1} = c X + s Y (the entry the rotation keeps),
-                        // h_{k+1,k-1} = 0 (the bulge it zeroes): lanes 0-3
-                        const double rz = pair_part(c, odd ? X.y : X.x, sn.x, odd ? Y.y : Y.x, odd ? sn.y : -sn.y,
-                                                    odd ? Y.x : Y.y);
-                        if (lane < 4)
-                            reinterpret_cast<double *>(&SGT_A(T, ldt, kb + (hi ? 1 : 0), kb - 1))[odd ? 1 : 0] =
-                                hi ? 0.0 : rz;
-                        if (b == 0) {
-                            const double2 r = make_double2(__shfl_sync(0xffffffffu, rz, 0),
-                                                           __shfl_sync(0xffffffffu, rz, 1));
-                            if (lane == 0) handH[s & 1] = r;
-                        }
+                    // G on the block's columns: lane 4 col + part gives part
+                    // (0 top.x, 1 top.y, 2 bottom.x, 3 bottom.y) of its column
+                    const double bx = hi ? -sn.x : sn.x, dy = odd ? sn.y : -sn.y;
+                    const double r1 = pair_part(c, hi ? bo : to, bx, hi ? to : bo, dy, hi ? te : be);
+                    // G^H on the rows k, k+1, k+2: lane 4 row + part gives part
+                    // (0 p.x, 1 p.y, 2 q.x, 3 q.y) of row (p, q): the block's
+                    // two rows after G, and (0, Hh)
+                    const int sp = 2 * row + (odd ? 1 : 0) + (hi ? 0 : 4), sq = sp ^ 4;
+                    double ga = __shfl_sync(0xffffffffu, r1, sp & 31);
+                    double ep = __shfl_sync(0xffffffffu, r1, (sp ^ 1) & 31);
+                    double al = __shfl_sync(0xffffffffu, r1, sq & 31);
+                    if (row == 2) {
+                        al = hi ? ho : 0.0;
+                        ga = hi ? 0.0 : ho;
+                        ep = hi ? 0.0 : he;
                     }
-                    // G on the block's columns: lane 4 col + part holds part
-                    // (0 top.x, 1 top.y, 2 bottom.x, 3 bottom.y) of column col
-                    // (0: (A, E), 1: (B, F)) -- one real output per lane
-                    // (operands picked by selects, no branches: all lanes run
-                    // the same three float64 instructions)
-                    const bool cl1 = (lane >> 2) & 1;
-                    const double2 tp = cl1 ? B : A, bt = cl1 ? F : E;
-                    const double2 u1 = hi ? bt : tp, v1 = hi ? tp : bt;
-                    const double r1 = pair_part(c, odd ? u1.y : u1.x, hi ? -sn.x : sn.x, odd ? v1.y : v1.x,
-                                                odd ? sn.y : -sn.y, odd ? v1.x : v1.y);
-                    const double2 A1 = make_double2(__shfl_sync(0xffffffffu, r1, 0), __shfl_sync(0xffffffffu, r1, 1));
-                    const double2 E1 = make_double2(__shfl_sync(0xffffffffu, r1, 2), __shfl_sync(0xffffffffu, r1, 3));
-                    const double2 B1 = make_double2(__shfl_sync(0xffffffffu, r1, 4), __shfl_sync(0xffffffffu, r1, 5));
-                    const double2 F1 = make_double2(__shfl_sync(0xffffffffu, r1, 6), __shfl_sync(0xffffffffu, r1, 7));
-                    // G^H on the rows k, k+1, k+2: lane 4 row + part holds part
-                    // (0 p.x, 1 p.y, 2 q.x, 3 q.y) of row (p, q): (A1, B1),
-                    // (E1, F1), (0, Hh)
-                    const int row = min(lane >> 2, 2);
-                    const double2 pp = row == 0 ? A1 : (row == 1 ? E1 : zero);
-                    const double2 qq = row == 0 ? B1 : (row == 1 ? F1 : Hh);
-                    const double2 u2 = hi ? qq : pp, v2 = hi ? pp : qq;
-                    const double r2 = pair_part(c, odd ? u2.y : u2.x, hi ? -sn.x : sn.x, odd ? v2.y : v2.x,
-                                                odd ? -sn.y : sn.y, odd ? v2.x : v2.y);
-                    if (lane < 8 || (lane < 12 && kb + 2 <= i))
-                        reinterpret_cast<double *>(&SGT_A(T, ldt, kb + (lane >> 2), kb + (part >> 1)))[part & 1] = r2;
-                    if (b == 0) {
-                        // the block's corner h_kk, for the rear chief two steps on
-                        const double2 corner = make_double2(__shfl_sync(0xffffffffu, r2, 0),
-                                                            __shfl_sync(0xffffffffu, r2, 1));
-                        if (lane == 0) handF[s & 1] = corner;
-                    }
+                    const double r2 = pair_part(c, al, bx, ga, -dy, ep);
                     if (kb + 2 <= i) {
                         // the next rotation zeroes the bulge h_{k+2,k} (lanes 8, 9)
                         // against h_{k+1,k} (lanes 4, 5)
-                        const double2 x = make_double2(__shfl_sync(0xffffffffu, r2, 4), __shfl_sync(0xffffffffu, r2, 5));
-                        const double2 y = make_double2(__shfl_sync(0xffffffffu, r2, 8), __shfl_sync(0xffffffffu, r2, 9));
-                        const double2 f1 = make_double2(__shfl_sync(0xffffffffu, r2, 6), __shfl_sync(0xffffffffu, r2, 7));
-                        const double2 h1 = make_double2(__shfl_sync(0xffffffffu, r2, 10), __shfl_sync(0xffffffffu, r2, 11));
-                        make_rotation_warp(x, y, lane, c_cur, s_cur);
-                        put_rotation(b, (s + 1) & 1, c_cur, s_cur);
-                        if (lane == 0) {
-                            const long long at = rot + (long long)b * L + (kb + 1 - l);
-                            rclog[at] = c_cur;
-                            rslog[at] = s_cur;
-                        }
-                        X = x;
-                        Y = y;
-                        // the block at (k+1, k+1): (h_{k+1,k+1}, h_{k+1,k+2};
-                        // h_{k+2,k+1}, h_{k+2,k+2}), h_{k+1,k+2} from bslot after
-                        // the barrier, and h_{k+3,k+2}
-                        A = f1;
-                        E = h1;
-                        F = (b == 0) ? F2 : Fnext;
-                        if (b == 0) Hh = H2;
+                        const double p = __shfl_sync(0xffffffffu, r2, part == 1 ? 8 : (part == 3 ? 5 : 4));
+                        const double q = __shfl_sync(0xffffffffu, r2, part == 0 ? 4 : 8);
+                        double u = __shfl_sync(0xffffffffu, r2, part == 1 ? 9 : (part == 3 ? 4 : 5));
+                        const double v = __shfl_sync(0xffffffffu, r2, part == 0 ? 5 : 9);
+                        if (part == 3) u = -u;
+                        make_rotation_warp(p, q, u, v, lane, c_cur, s_cur);
+                        put_rotation(b, (s + 1) & 1);
+                        if (lane == 4 || lane == 5 || lane == 8 || lane == 9)
+                            inp[b][(s + 1) & 1][(lane & 1) | (lane >> 2 & 2)] = r2;
+                    }
+                    if (lane < 8 || (lane < 12 && kb + 2 <= i))
+                        reinterpret_cast<double *>(&SGT_A(T, ldt, kb + (lane >> 2), kb + (part >> 1)))[part & 1] = r2;
+                    // the block's corner h_kk, for the bulge behind
+                    if (lane < 2 && b + 1 < nbul)
+                        reinterpret_cast<double *>(
+                            cl.map_shared_rank(&handF[b + 1][s & 1], (b + 1) / kChiefs))[lane] = r2;
+                    // the block at (k+1, k+1): (h_{k+1,k+1}, h_{k+1,k+2};
+                    // h_{k+2,k+1}, h_{k+2,k+2}), h_{k+1,k+2} from bslot after
+                    // the barrier, and h_{k+3,k+2}
+                    const double2 F = (b == 0) ? F2 : Fnext;
+                    const double ao = __shfl_sync(0xffffffffu, r2, odd ? 7 : 6);
+                    const double ae = __shfl_sync(0xffffffffu, r2, odd ? 6 : 7);
+                    const double eo = __shfl_sync(0xffffffffu, r2, odd ? 11 : 10);
+                    const double ee = __shfl_sync(0xffffffffu, r2, odd ? 10 : 11);
+                    to = ao;
+                    te = ae;
+                    bo = col1 ? (odd ? F.y : F.x) : eo;
+                    be = col1 ? (odd ? F.x : F.y) : ee;
+                    if (b == 0) {
+                        ho = odd ? H2.y : H2.x;
+                        he = odd ? H2.x : H2.y;
+                    }
+                }
+            } else if (helper && my < nbul) {
+                const int b = my, kb = l + s - 3 * b;
+                if (s >= 3 * b && s < L + 3 * b) {
+                    const double c = rc[b][s & 1];
+                    const double2 sn = rs[b][s & 1];
+                    if (lane == 0) {
+                        const long long at = rot + (long long)b * L + (kb - l);
+                        rclog[at] = c;
+                        rslog[at] = sn;
+                    }
+                    if (kb > l && lane < 4) {
+                        // h_{k,k-1} = c x + s y (the entry the rotation keeps,
+                        // lanes 0, 1), h_{k+1,k-1} = 0 (the bulge it zeroes)
+                        const double *xy = inp[b][s & 1];
+                        const double rz = pair_part(c, odd ? xy[1] : xy[0], sn.x, odd ? xy[3] : xy[2],
+                                                    odd ? sn.y : -sn.y, odd ? xy[2] : xy[3]);
+                        reinterpret_cast<double *>(&SGT_A(T, ldt, kb + (hi ? 1 : 0), kb - 1))[odd ? 1 : 0] =
+                            hi ? 0.0 : rz;
+                        if (lane < 2 && b + 1 < nbul)
+                            reinterpret_cast<double *>(
+                                cl.map_shared_rank(&handH[b + 1][s & 1], (b + 1) / kChiefs))[lane] = rz;
                     }
                 }
             }
             cl.sync();
-            if (cb >= 0 && cb < nbul) {
-                const int b = cb;
-                const bool act_b = (b == 0) ? a0 : a1;
-                const int kb = (b == 0) ? k0 : k1;
-                if (act_b && kb + 1 < i) B = bslot[b][(s + 1) & 1];
-                if (b == 1) {
-                    if (s == 2) {
-                        Hh = (l + 2 <= i) ? handH[0] : zero;   // the front chief's h_{l+2,l+1} of step 2
-                    } else if (a1 && kb + 3 <= i) {
-                        // h_{k+3,k+2} for the next step: the front chief's
-                        // left entry of this step, or T once that chase ended
-                        Hh = a0 ? handH[s & 1] : ldT(&SGT_A(T, ldt, kb + 3, kb + 2));
-                    } else if (a1) {
-                        Hh = zero;
-                    }
+            if (chief && my < nbul) {
+                const int b = my, kb = l + s - 3 * b;
+                const bool on = s >= 3 * b && s < L + 3 * b;
+                if (on && kb + 1 < i && col1) {
+                    const double2 B = bslot[b][(s + 1) & 1];
+                    to = odd ? B.y : B.x;
+                    te = odd ? B.x : B.y;
+                }
+                if (b > 0 && (on || s == 3 * b - 1)) {
+                    // h_{k+3,k+2} for the next step (h_{l+2,l+1} before the
+                    // first): the left entry of the bulge in front, of this
+                    // step, or T once that chase ended
+                    double2 H = zero;
+                    if (kb + 3 <= i)
+                        H = (s < L + 3 * (b - 1)) ? handH[b][s & 1] : ldT(&SGT_A(T, ldt, kb + 3, kb + 2));
+                    ho = odd ? H.y : H.x;
+                    he = odd ? H.x : H.y;
                 }
             }
         }
@@ -871,15 +1038,15 @@ int qr_cluster_size()
     return clusters >= 1 ? 16 : 8;
 }
 
-cudaError_t launch_qr(int cl, int n, double2 *T, int ldt, QrState *st, long long budget, SweepRec *sweeplog,
-                      double *rclog, double2 *rslog, int *nlogged, cudaStream_t stream)
+cudaError_t launch_qr(int cl, int n, double2 *T, int ldt, QrState *st, SweepRec *sweeplog, double *rclog, double2 *rslog,
+                      int *nlogged, cudaStream_t stream)
 {
     cudaLaunchAttribute at[1];
     const cudaLaunchConfig_t cfg = qr_config(cl, stream, at);
-    return cl == 16 ? cudaLaunchKernelEx(&cfg, schur_qr_kernel<16>, n, T, ldt, st, budget, sweeplog, rclog, rslog,
-                                         nlogged)
-                    : cudaLaunchKernelEx(&cfg, schur_qr_kernel<8>, n, T, ldt, st, budget, sweeplog, rclog, rslog,
-                                         nlogged);
+    return cl == 16 ? cudaLaunchKernelEx(&cfg, schur_qr_kernel<16>, n, T, ldt, st, kRotationBudget,
+                                         (long long)rotation_room(n), sweeplog, rclog, rslog, nlogged)
+                    : cudaLaunchKernelEx(&cfg, schur_qr_kernel<8>, n, T, ldt, st, kRotationBudget,
+                                         (long long)rotation_room(n), sweeplog, rclog, rslog, nlogged);
 }
 
 // The second stream of schur_run and its events.  Destroyed on every
@@ -917,7 +1084,7 @@ size_t schur_workspace_bytes(int n)
     if (n <= 0) return 0;
     // eleven takes, each rounded up to 256 bytes; two logs of one launch each
     const size_t nn = (size_t)n * n;
-    const size_t nlog = (size_t)kRotationBudget + (size_t)kMaxBulges * n + 2;
+    const size_t nlog = rotation_room(n);
     return 2 * nn * sizeof(double) + 3 * (size_t)n * sizeof(double) + sizeof(double) + sizeof(int) + sizeof(QrState) +
            2 * nlog * (sizeof(SweepRec) + sizeof(double) + sizeof(double2)) + 2 * sizeof(int) + 11 * 256;
 }
@@ -937,7 +1104,7 @@ signtri_status schur_run(int n, const double *A, int lda, double *Q, int ldq, do
     // a launch logs fewer than budget + 2n rotations (it starts a multi-sweep
     // only below the budget, a multi-sweep has at most 2 (n - 1)) and no
     // more sweeps; launches alternate between two logs
-    const size_t nlog = (size_t)kRotationBudget + (size_t)kMaxBulges * n + 2;
+    const size_t nlog = rotation_room(n);
     auto *sweeplog = static_cast<SweepRec *>(ws.take(2 * nlog * sizeof(SweepRec)));
     auto *rclog = static_cast<double *>(ws.take(2 * nlog * sizeof(double)));
     auto *rslog = static_cast<double2 *>(ws.take(2 * nlog * sizeof(double2)));
@@ -1018,8 +1185,7 @@ signtri_status schur_run(int n, const double *A, int lda, double *Q, int ldq, do
         if (it >= 2) SGT_CUDA_TRY(cudaStreamWaitEvent(st, ap.applied[p], 0));
         {
             ProfScope ps(SIGNTRI_KC_SCHUR, st);
-            SGT_CUDA_TRY(launch_qr(qr_cl, n, Tc, ldt, qs, kRotationBudget, sweeplog + lo, rclog + lo, rslog + lo,
-                                   nlogged + p, st));
+            SGT_CUDA_TRY(launch_qr(qr_cl, n, Tc, ldt, qs, sweeplog + lo, rclog + lo, rslog + lo, nlogged + p, st));
         }
         SGT_CUDA_TRY(cudaEventRecord(ap.swept[p], st));
         if (it >= 1) {
