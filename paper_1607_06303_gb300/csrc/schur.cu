@@ -846,6 +846,14 @@ schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ s
                         ep = hi ? 0.0 : he;
                     }
                     const double r2 = pair_part(c, al, bx, ga, -dy, ep);
+                    // stored before the next rotation is formed, so that the
+                    // barrier does not wait for them
+                    if (lane < 8 || (lane < 12 && kb + 2 <= i))
+                        reinterpret_cast<double *>(&SGT_A(T, ldt, kb + (lane >> 2), kb + (part >> 1)))[part & 1] = r2;
+                    // the block's corner h_kk, for the bulge behind
+                    if (lane < 2 && b + 1 < nbul)
+                        reinterpret_cast<double *>(
+                            cl.map_shared_rank(&handF[b + 1][s & 1], (b + 1) / kChiefs))[lane] = r2;
                     if (kb + 2 <= i) {
                         // the next rotation zeroes the bulge h_{k+2,k} (lanes 8, 9)
                         // against h_{k+1,k} (lanes 4, 5)
@@ -859,12 +867,6 @@ schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ s
                         if (lane == 4 || lane == 5 || lane == 8 || lane == 9)
                             inp[b][(s + 1) & 1][(lane & 1) | (lane >> 2 & 2)] = r2;
                     }
-                    if (lane < 8 || (lane < 12 && kb + 2 <= i))
-                        reinterpret_cast<double *>(&SGT_A(T, ldt, kb + (lane >> 2), kb + (part >> 1)))[part & 1] = r2;
-                    // the block's corner h_kk, for the bulge behind
-                    if (lane < 2 && b + 1 < nbul)
-                        reinterpret_cast<double *>(
-                            cl.map_shared_rank(&handF[b + 1][s & 1], (b + 1) / kChiefs))[lane] = r2;
                     // the block at (k+1, k+1): (h_{k+1,k+1}, h_{k+1,k+2};
                     // h_{k+2,k+1}, h_{k+2,k+2}), h_{k+1,k+2} from bslot after
                     // the barrier, and h_{k+3,k+2}
@@ -945,43 +947,76 @@ schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ s
 // window ends above it (u > i), down the column with the carried row; unit
 // u >= n is row u - n of Q, which takes every sweep's column rotations along
 // the row.  In log order, so each entry sees its rotations in the order of
-// the QR iteration.  Four lanes per unit, each computing one real output of
-// a rotation (3 float64 instructions, where GB300's float64 pipe, not the
-// memory, bounds this kernel), the carried entry passed by shuffles; the
-// next entry is loaded an iteration ahead.
-__global__ void apply_rotations_kernel(int n, double2 *__restrict__ T, int ldt, double2 *__restrict__ Q, int ldq,
-                                       const int *__restrict__ nlogged, const SweepRec *__restrict__ sweeplog,
-                                       const double *__restrict__ rclog, const double2 *__restrict__ rslog)
+// the QR iteration.  The chain of rotations along a line bounds this kernel,
+// so a warp per line runs up to eight consecutive sweeps of one window in a
+// wavefront: group g of four lanes takes sweep g two steps behind group g - 1,
+// whose finished entry it gets by shuffles; group 0 reads the line, the last
+// one writes it.  Each lane computes one real output of a rotation (3 float64
+// instructions, 24 lanes' rotations in one).  The next steps' rotations and
+// entries are loaded two steps ahead.
+__global__ void __launch_bounds__(kThreads)
+apply_rotations_kernel(int n, double2 *T, int ldt, double2 *Q, int ldq, const int *__restrict__ nlogged,
+                       const SweepRec *__restrict__ sweeplog, const double *__restrict__ rclog,
+                       const double2 *__restrict__ rslog)
 {
-    const int g = blockIdx.x * blockDim.x + threadIdx.x;
-    const int unit = g >> 2, part = g & 3;
-    if (unit >= 2 * n) return;   // the four lanes of a unit leave together
-    const unsigned gmask = 0xFu << (threadIdx.x & 28);
+    const int unit = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (unit >= 2 * n) return;   // a warp's lanes leave together
+    const int g = lane >> 2, part = lane & 3, base = lane & 28;
     const bool odd = part & 1, hi = part >= 2;
     const bool isT = unit < n;
     // entry k of the unit's line: T(k, j) (stride 1) or Q(r, k) (stride ldq)
     double2 *line = isT ? &SGT_A(T, ldt, 0, unit) : &SGT_A(Q, ldq, unit - n, 0);
     const size_t stride = isT ? 1 : (size_t)ldq;
     const int logged = *nlogged;
-    for (int w = 0; w < logged; w++) {
-        const SweepRec sr = sweeplog[w];
-        if (isT && unit <= sr.i) continue;
-        double2 a = line[(size_t)sr.l * stride];
-        double2 b = line[(size_t)(sr.l + 1) * stride];
-        for (int k = sr.l; k < sr.i; k++) {
-            const double c = rclog[sr.off + (k - sr.l)];
-            const double2 s = rslog[sr.off + (k - sr.l)];
-            const double2 bn = (k + 2 <= sr.i) ? line[(size_t)(k + 2) * stride] : b;
+    const double2 zero = make_double2(0.0, 0.0);
+    for (int w = 0; w < logged;) {
+        const int mine = min(w + g, logged - 1);
+        const SweepRec sr = sweeplog[mine], s0 = {__shfl_sync(0xffffffffu, sr.l, 0), __shfl_sync(0xffffffffu, sr.i, 0), 0};
+        const unsigned same = __ballot_sync(0xffffffffu, w + g < logged && sr.l == s0.l && sr.i == s0.i);
+        const int nb = __ffs((int)~same) == 0 ? 8 : (__ffs((int)~same) - 1) >> 2;   // sweeps of this window in a row
+        w += nb;
+        if (isT && unit <= s0.i) continue;
+        const int l = s0.l, L = s0.i - s0.l;
+        // step t of group g: u = t - 2 g; u = 0 takes the entry l over, u in
+        // [1, L] is rotation l + u - 1, u = L + 1 passes the last entry on
+        auto load_c = [&](int u) { return u >= 1 && u <= L ? rclog[sr.off + u - 1] : 1.0; };
+        auto load_s = [&](int u) { return u >= 1 && u <= L ? rslog[sr.off + u - 1] : zero; };
+        auto load_e = [&](int t) { return g == 0 && t <= L ? line[(size_t)(l + t) * stride] : zero; };
+        double r = 0.0;
+        double c0 = load_c(-2 * g), c1 = load_c(1 - 2 * g);
+        double2 q0 = load_s(-2 * g), q1 = load_s(1 - 2 * g);
+        double2 e0 = load_e(0), e1 = load_e(1);
+        const int steps = L + 2 + 2 * (nb - 1);
+        for (int t = 0; t < steps; t++) {
+            const int u = t - 2 * g;
+            const double c = c0;
+            const double2 s = q0, e = e0;
+            c0 = c1;
+            q0 = q1;
+            e0 = e1;
+            c1 = load_c(u + 2);
+            q1 = load_s(u + 2);
+            e1 = load_e(t + 2);
+            // the carried entry a (this group's parts 2, 3) and the incoming b
+            // (parts 0, 1 of the group in front), each as its part `odd` and
+            // the other one
+            const double ao = __shfl_sync(0xffffffffu, r, base + 2 + (odd ? 1 : 0));
+            const double ae = __shfl_sync(0xffffffffu, r, base + 2 + (odd ? 0 : 1));
+            double bo = __shfl_sync(0xffffffffu, r, (base + 28 + (odd ? 1 : 0)) & 31);
+            double be = __shfl_sync(0xffffffffu, r, (base + 28 + (odd ? 0 : 1)) & 31);
+            if (g == 0) {
+                bo = odd ? e.y : e.x;
+                be = odd ? e.x : e.y;
+            }
             // G (T's rows) or G^H (Q's columns) on (a, b): lane part gives
             // part 0 a'.x, 1 a'.y, 2 b'.x, 3 b'.y
-            const double2 u = hi ? b : a, v = hi ? a : b;
-            const double sy = isT ? (odd ? s.y : -s.y) : (odd ? -s.y : s.y);
-            const double r = pair_part(c, odd ? u.y : u.x, hi ? -s.x : s.x, odd ? v.y : v.x, sy, odd ? v.x : v.y);
-            if (!hi) reinterpret_cast<double *>(&line[(size_t)k * stride])[part] = r;
-            a = make_double2(__shfl_sync(gmask, r, 2, 4), __shfl_sync(gmask, r, 3, 4));
-            b = bn;
+            const double sy = isT == odd ? s.y : -s.y;
+            const double v = pair_part(c, hi ? bo : ao, hi ? -s.x : s.x, hi ? ao : bo, sy, hi ? ae : be);
+            r = u >= 1 && u <= L ? v : (hi ? bo : ao);
+            if (g == nb - 1 && u >= 1 && u <= L + 1 && !hi)
+                reinterpret_cast<double *>(&line[(size_t)(l + u - 1) * stride])[part] = r;
         }
-        if (part == 0) line[(size_t)sr.i * stride] = a;
+        __syncwarp();   // the next window's reads of entries other lanes wrote
     }
 }
 
@@ -1169,7 +1204,7 @@ signtri_status schur_run(int n, const double *A, int lda, double *Q, int ldq, do
         SGT_CUDA_TRY(cudaStreamWaitEvent(ap.s, ap.swept[p], 0));
         {
             ProfScope ps(SIGNTRI_KC_SCHUR, ap.s);
-            apply_rotations_kernel<<<(8 * n + kThreads - 1) / kThreads, kThreads, 0, ap.s>>>(
+            apply_rotations_kernel<<<(int)((64LL * n + kThreads - 1) / kThreads), kThreads, 0, ap.s>>>(
                 n, Tc, ldt, Qc, ldq, nlogged + p, sweeplog + lo, rclog + lo, rslog + lo);
             SGT_LAUNCH_CHECK();
         }
