@@ -54,7 +54,7 @@ namespace signtri {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kQrThreads = 512;
+constexpr int kQrThreads = 256;
 constexpr int kMaxSweepsPerEigenvalue = 100;
 constexpr long long kRotationBudget = 1LL << 13;   // rotations per launch of the QR kernel (then a sweep's end)
 // rotations (and sweeps) a launch's log holds: two sweeps of a full window
@@ -341,13 +341,13 @@ __global__ void qr_state_init_kernel(int n, QrState *st)
 //    rotation (one reciprocal square root), stored into every CTA's shared
 //    memory (two slots per bulge, alternating).  The one entry of the next
 //    block that another thread writes, h_{k+1,k+2} (row op of column k+2),
-//    comes through shared memory; the front chase loads the entries no step
-//    touches before (h_{k+2,k+2}, h_{k+3,k+2}) two steps ahead, a rear
-//    chase takes them from the bulge in front, whose warps wrote them one and
-//    zero steps before (h_{k+2,k+2} as its block's corner, h_{k+3,k+2} as the
-//    entry left of its block), or from T once that chase has ended.
+//    comes through shared memory, and so do h_{k+2,k+2} and h_{k+3,k+2},
+//    which the bulge in front wrote one and zero steps before (as its block's
+//    corner and as the entry left of its block).
 //  * a helper warp per bulge forms the entry left of the block (h_{k,k-1},
-//    zeroing the old bulge) and logs the rotation, off the chief's chain.
+//    zeroing the old bulge), logs the rotation, and fetches from T what no
+//    bulge in front hands on (for the front chase, and for the others once the
+//    chase in front has ended), off the chief's chain.
 //  * the other CTAs do the rest of every rotation: a warp takes 32 columns of
 //    rows k, k+1 or 32 rows of columns k, k+1 of one bulge (whole warps of
 //    one kind: mixed ones ran each kind's loads and arithmetic in turn), and
@@ -364,10 +364,10 @@ __global__ void qr_state_init_kernel(int n, QrState *st)
 // this kernel logs each sweep and its rotations instead (a rear sweep after
 // the one in front of it).
 constexpr int kMaxBulges = 8;
-constexpr int kChiefs = 2;   // chief warps (and as many helpers) of a chief CTA
+constexpr int kChiefs = 4;   // chief warps (and as many helpers) of a chief CTA
 constexpr int kChiefCtas = (kMaxBulges + kChiefs - 1) / kChiefs;
 constexpr int kCross = kMaxBulges * (kMaxBulges - 1) / 2;   // pairs of bulges
-constexpr int kCrossWarps = (kCross + 15) / 16;             // two lanes per pair
+constexpr int kCrossWarps = (kCross + 3) / 4;               // eight lanes per pair
 enum { kActSweep = 0, kActStop = 2 };
 
 __device__ __forceinline__ double2 ldT(const double2 *p) { return __ldcg(p); }
@@ -557,6 +557,18 @@ __device__ void small_eigs(float2 (*h)[kMaxBulges + 1], int m, int lane, float2 
     __syncwarp();
 }
 
+// The cluster barrier of a step: the warps that stored something order it
+// before their arrival by a fence, the others do not wait for any memory
+// (arriving with release semantics in every thread measured 850-1500 cycles
+// at 16 CTAs, this 120 without stores, ~650 with stores to shared memory and
+// ~1000 with stores to global memory).
+__device__ __forceinline__ void step_barrier(bool wrote)
+{
+    if (wrote) asm volatile("fence.acq_rel.cluster;" ::: "memory");
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
 template <int CL>
 __global__ void __launch_bounds__(kQrThreads)
 schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ st, long long budget, long long room,
@@ -565,14 +577,14 @@ schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ s
 {
     namespace cg = cooperative_groups;
     constexpr int kWorkers = CL - kChiefCtas, kWarps = kQrThreads / 32, kWorkerWarps = kWorkers * kWarps;
-    static_assert(kWorkers > 0 && kWarps >= 2 * kChiefs && kWorkers >= kCrossWarps, "roles");
+    static_assert(kWorkers > 0 && kWarps >= 2 * kChiefs && kWorkerWarps >= kCrossWarps + kMaxBulges, "roles");
     cg::cluster_group cl = cg::this_cluster();
     __shared__ int redi[kWarps];
     __shared__ double rc[kMaxBulges][2];
     __shared__ double2 rs[kMaxBulges][2];
     __shared__ double2 bslot[kMaxBulges][2];              // h_{k+1,k+2} after a step, in the bulge's chief CTA
     __shared__ double inp[kMaxBulges][2][4];              // a rotation's inputs x, y, for the helper
-    __shared__ double2 handF[kMaxBulges][2], handH[kMaxBulges][2];   // from the bulge in front: its corner and left entry
+    __shared__ double2 handF[kMaxBulges][4], handH[kMaxBulges][2];   // h_{k+2,k+2} a step ahead, h_{k+3,k+2} (four and two slots)
     __shared__ double2 sig[kMaxBulges];                   // the bulges' shifts
     __shared__ float2 blk[kMaxBulges][kMaxBulges + 1], eig[kMaxBulges];
     __shared__ int ctl[4];                                // action, l, i, bulges (CTA 0's decision)
@@ -584,12 +596,12 @@ schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ s
     const bool helper = chief_cta && warp >= kChiefs && warp < 2 * kChiefs && my < kMaxBulges;
     const bool chief0 = crank == 0 && warp == 0;
     // a worker's warp number: consecutive ones alternate CTAs; the last
-    // kCrossWarps take the pairs of bulges, two lanes a pair
+    // kCrossWarps take the pairs of bulges, eight lanes a pair
     const int w = warp * kWorkers + (crank - kChiefCtas);
     const bool crosser = !chief_cta && w >= kWorkerWarps - kCrossWarps;
     int pa = 0, pb = 0;                                   // this lane's pair: pa in front of pb
     if (crosser) {
-        const int pair = (w - (kWorkerWarps - kCrossWarps)) * 16 + (lane >> 1);
+        const int pair = (w - (kWorkerWarps - kCrossWarps)) * 4 + (lane >> 3);
         if (pair < kCross) {
             pb = 1;
             while (pair >= pb * (pb + 1) / 2) pb++;
@@ -604,13 +616,15 @@ schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ s
     const int part = lane & 3;
     const bool odd = part & 1, hi = part >= 2, col1 = (lane >> 2) & 1;
     const int row = min(lane >> 2, 2);
-    // A chief warp's registers.  Lane 4 col + part holds the column col of
-    // the block (A B; E F) at (k, k): top A or B, bottom E or F, each as its
-    // part `odd` and the other one; every lane Hh = h_{k+2,k+1} likewise, and
-    // the step's rotation.
-    double to = 0.0, te = 0.0, bo = 0.0, be = 0.0, ho = 0.0, he = 0.0, c_cur = 1.0;
+    // A chief warp's registers.  Lane 4 col + part forms the real output part
+    // (0 top.x, 1 top.y, 2 bottom.x, 3 bottom.y) of G on the block's column
+    // col ((A, E) or (B, F), the block (A B; E F) at (k, k)): al, ga, ep are
+    // its operands in pair_part; ho, he are h_{k+2,k+1}'s part `odd` and the
+    // other one; the step's rotation.
+    double al = 0.0, ga = 0.0, ep = 0.0, ho = 0.0, he = 0.0, c_cur = 1.0;
     double2 s_cur = zero;
-    double2 pf_f = zero, pf_h = zero;   // front chase: h_{k+2,k+2}, h_{k+3,k+2} for step k+1, loaded early
+    auto as_double = [](double2 *q) { return reinterpret_cast<double *>(q); };
+    const int po = odd ? 1 : 0, pe = odd ? 0 : 1;
     auto put_rotation = [&](int b, int slot) {
         // lanes 0..CL-1 of a chief warp store into CTA `lane`
         if (lane < CL) {
@@ -625,15 +639,15 @@ schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ s
         const double2 A = ldT(&SGT_A(T, ldt, l, l)), E = ldT(&SGT_A(T, ldt, l + 1, l));
         if (b == 0) {
             const double2 H = (l + 2 <= last) ? ldT(&SGT_A(T, ldt, l + 2, l + 1)) : zero;
-            pf_f = (l + 2 <= last) ? ldT(&SGT_A(T, ldt, l + 2, l + 2)) : zero;
-            pf_h = (l + 3 <= last) ? ldT(&SGT_A(T, ldt, l + 3, l + 2)) : zero;
+            const double2 F = (l + 2 <= last) ? ldT(&SGT_A(T, ldt, l + 2, l + 2)) : zero;
+            if (lane == 0) handF[0][3] = F;
             ho = odd ? H.y : H.x;
             he = odd ? H.x : H.y;
         }
-        to = odd ? top.y : top.x;
-        te = odd ? top.x : top.y;
-        bo = odd ? bot.y : bot.x;
-        be = odd ? bot.x : bot.y;
+        const double2 u1 = hi ? bot : top, v1 = hi ? top : bot;
+        al = odd ? u1.y : u1.x;
+        ga = odd ? v1.y : v1.x;
+        ep = odd ? v1.x : v1.y;
         const double2 X = make_double2(A.x - sg.x, A.y - sg.y);
         const double2 v = part == 1 ? E : X, u = part == 0 ? X : E;
         // parts 0, 1: v.x v.x + v.y v.y; 2: X.x E.x + X.y E.y; 3: X.y E.x - X.x E.y
@@ -749,14 +763,15 @@ schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ s
         const int wq = (kWorkerWarps - kCrossWarps) / nbul;
         const int wb = w % nbul;
         const bool worker = !chief_cta && w < wq * nbul;
-        double2 Fnext = zero;   // a rear chief: its block's next corner
         for (int s = 0; s < S; s++) {
+            bool wrote = false;   // this warp has stores for the others to see
             if (worker) {
                 const int k = l + s - 3 * wb;
                 if (s >= 3 * wb && s < L + 3 * wb) {
                     const double c0 = rc[wb][s & 1];
                     const double2 s0 = rs[wb][s & 1];
                     const int rw = (i - k - 1 + 31) >> 5, cw = (k + 31) >> 5;
+                    wrote = true;
                     for (int q = w / nbul; q < rw + cw; q += wq) {
                         if (q < rw) {
                             // rows k, k+1 at column j, but for the columns of
@@ -785,26 +800,33 @@ schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ s
                     }
                 }
             } else if (crosser) {
-                // lane f of a pair: column k0 + f through the rear rotation,
-                // then row k1 + f through the front one
-                const int k0 = l + s - 3 * pa, k1 = l + s - 3 * pb, f = lane & 1;
+                // lane 4 f + part of a pair's eight: column k0 + f through the
+                // rear rotation, then row k1 + f through the front one, an
+                // output each (as in the chief's block)
+                const int k0 = l + s - 3 * pa, k1 = l + s - 3 * pb, f = (lane >> 2) & 1;
                 const bool on = pb > pa && pb < nbul && s >= 3 * pb && s < L + 3 * pa;
-                double2 a = zero, b = zero;
-                if (on) {
-                    a = ldT(&SGT_A(T, ldt, k1, k0 + f));
-                    b = ldT(&SGT_A(T, ldt, k1 + 1, k0 + f));
-                    rot_rows(rc[pb][s & 1], rs[pb][s & 1], a, b);
-                }
-                // lane 0 holds (row k1, row k1+1) of column k0, lane 1
-                // of column k0+1; row k1 + f needs both columns
-                const double2 mine = f ? b : a, theirs = f ? a : b;
-                const double2 got = make_double2(__shfl_xor_sync(0xffffffffu, theirs.x, 1),
-                                                 __shfl_xor_sync(0xffffffffu, theirs.y, 1));
-                if (on) {
-                    double2 p = f ? got : mine, q = f ? mine : got;
-                    rot_cols(rc[pa][s & 1], rs[pa][s & 1], p, q);
-                    SGT_A(T, ldt, k1 + f, k0) = p;
-                    SGT_A(T, ldt, k1 + f, k0 + 1) = q;
+                wrote = __any_sync(0xffffffffu, on);
+                if (wrote) {
+                    double2 a = zero, b = zero, sr = zero, sc = zero;
+                    double cr = 1.0, cc = 1.0;
+                    if (on) {
+                        a = ldT(&SGT_A(T, ldt, k1, k0 + f));
+                        b = ldT(&SGT_A(T, ldt, k1 + 1, k0 + f));
+                        cr = rc[pb][s & 1];
+                        sr = rs[pb][s & 1];
+                        cc = rc[pa][s & 1];
+                        sc = rs[pa][s & 1];
+                    }
+                    const double2 u = hi ? b : a, v = hi ? a : b;
+                    const double r1 = pair_part(cr, odd ? u.y : u.x, hi ? -sr.x : sr.x, odd ? v.y : v.x,
+                                                odd ? sr.y : -sr.y, odd ? v.x : v.y);
+                    // row f: part of its entry in column k0 (lanes 2 f + .. of
+                    // the pair) and in column k0 + 1 (4 lanes on)
+                    const int at = (lane & 24) + 2 * f + po + (hi ? 0 : 4);
+                    const double g2 = __shfl_sync(0xffffffffu, r1, at), e2 = __shfl_sync(0xffffffffu, r1, at ^ 1);
+                    const double a2 = __shfl_sync(0xffffffffu, r1, at ^ 4);
+                    const double r2 = pair_part(cc, a2, hi ? -sc.x : sc.x, g2, odd ? -sc.y : sc.y, e2);
+                    if (on) as_double(&SGT_A(T, ldt, k1 + f, k0 + (part >> 1)))[part & 1] = r2;
                 }
             } else if (chief && my < nbul) {
                 const int b = my, kb = l + s - 3 * b;
@@ -813,47 +835,26 @@ schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ s
                     // since the last step (h_{l+2,l+1} comes after this step,
                     // from the bulge in front)
                     start_chase(b, (s + 1) & 1, l, i, sig[b]);
+                    wrote = true;
                 } else if (s >= 3 * b && s < L + 3 * b) {
                     const double c = c_cur;
                     const double2 sn = s_cur;
-                    double2 F2 = zero, H2 = zero;
-                    if (b == 0) {
-                        F2 = pf_f;
-                        H2 = pf_h;
-                        pf_f = (kb + 3 <= i) ? ldT(&SGT_A(T, ldt, kb + 3, kb + 3)) : zero;
-                        pf_h = (kb + 4 <= i) ? ldT(&SGT_A(T, ldt, kb + 4, kb + 3)) : zero;
-                    } else if (kb + 2 <= i) {
-                        // the next corner h_{k+2,k+2}: the block corner of the
-                        // bulge in front, of the previous step, or T once that
-                        // chase ended
-                        Fnext = (s - 1 < L + 3 * (b - 1)) ? handF[b][(s - 1) & 1]
-                                                          : ldT(&SGT_A(T, ldt, kb + 2, kb + 2));
-                    }
-                    // G on the block's columns: lane 4 col + part gives part
-                    // (0 top.x, 1 top.y, 2 bottom.x, 3 bottom.y) of its column
+                    wrote = true;
+                    // G on the block's columns
                     const double bx = hi ? -sn.x : sn.x, dy = odd ? sn.y : -sn.y;
-                    const double r1 = pair_part(c, hi ? bo : to, bx, hi ? to : bo, dy, hi ? te : be);
+                    const double r1 = pair_part(c, al, bx, ga, dy, ep);
                     // G^H on the rows k, k+1, k+2: lane 4 row + part gives part
                     // (0 p.x, 1 p.y, 2 q.x, 3 q.y) of row (p, q): the block's
-                    // two rows after G, and (0, Hh)
-                    const int sp = 2 * row + (odd ? 1 : 0) + (hi ? 0 : 4), sq = sp ^ 4;
-                    double ga = __shfl_sync(0xffffffffu, r1, sp & 31);
-                    double ep = __shfl_sync(0xffffffffu, r1, (sp ^ 1) & 31);
-                    double al = __shfl_sync(0xffffffffu, r1, sq & 31);
+                    // two rows after G, and (0, h_{k+2,k+1})
+                    const int sp = (2 * row + po + (hi ? 0 : 4)) & 31;
+                    double g2 = __shfl_sync(0xffffffffu, r1, sp), e2 = __shfl_sync(0xffffffffu, r1, sp ^ 1);
+                    double a2 = __shfl_sync(0xffffffffu, r1, sp ^ 4);
                     if (row == 2) {
-                        al = hi ? ho : 0.0;
-                        ga = hi ? 0.0 : ho;
-                        ep = hi ? 0.0 : he;
+                        a2 = hi ? ho : 0.0;
+                        g2 = hi ? 0.0 : ho;
+                        e2 = hi ? 0.0 : he;
                     }
-                    const double r2 = pair_part(c, al, bx, ga, -dy, ep);
-                    // stored before the next rotation is formed, so that the
-                    // barrier does not wait for them
-                    if (lane < 8 || (lane < 12 && kb + 2 <= i))
-                        reinterpret_cast<double *>(&SGT_A(T, ldt, kb + (lane >> 2), kb + (part >> 1)))[part & 1] = r2;
-                    // the block's corner h_kk, for the bulge behind
-                    if (lane < 2 && b + 1 < nbul)
-                        reinterpret_cast<double *>(
-                            cl.map_shared_rank(&handF[b + 1][s & 1], (b + 1) / kChiefs))[lane] = r2;
+                    const double r2 = pair_part(c, a2, bx, g2, -dy, e2);
                     if (kb + 2 <= i) {
                         // the next rotation zeroes the bulge h_{k+2,k} (lanes 8, 9)
                         // against h_{k+1,k} (lanes 4, 5)
@@ -862,26 +863,25 @@ schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ s
                         double u = __shfl_sync(0xffffffffu, r2, part == 1 ? 9 : (part == 3 ? 4 : 5));
                         const double v = __shfl_sync(0xffffffffu, r2, part == 0 ? 5 : 9);
                         if (part == 3) u = -u;
-                        make_rotation_warp(p, q, u, v, lane, c_cur, s_cur);
-                        put_rotation(b, (s + 1) & 1);
+                        // what r2 holds already goes out before the rotation is
+                        // formed, so that the barrier does not wait for it
+                        if (lane < 12) as_double(&SGT_A(T, ldt, kb + (lane >> 2), kb + (part >> 1)))[part & 1] = r2;
                         if (lane == 4 || lane == 5 || lane == 8 || lane == 9)
                             inp[b][(s + 1) & 1][(lane & 1) | (lane >> 2 & 2)] = r2;
-                    }
-                    // the block at (k+1, k+1): (h_{k+1,k+1}, h_{k+1,k+2};
-                    // h_{k+2,k+1}, h_{k+2,k+2}), h_{k+1,k+2} from bslot after
-                    // the barrier, and h_{k+3,k+2}
-                    const double2 F = (b == 0) ? F2 : Fnext;
-                    const double ao = __shfl_sync(0xffffffffu, r2, odd ? 7 : 6);
-                    const double ae = __shfl_sync(0xffffffffu, r2, odd ? 6 : 7);
-                    const double eo = __shfl_sync(0xffffffffu, r2, odd ? 11 : 10);
-                    const double ee = __shfl_sync(0xffffffffu, r2, odd ? 10 : 11);
-                    to = ao;
-                    te = ae;
-                    bo = col1 ? (odd ? F.y : F.x) : eo;
-                    be = col1 ? (odd ? F.x : F.y) : ee;
-                    if (b == 0) {
-                        ho = odd ? H2.y : H2.x;
-                        he = odd ? H2.x : H2.y;
+                        // the block's corner h_kk, for the bulge behind
+                        if (lane < 2 && b + 1 < nbul)
+                            as_double(cl.map_shared_rank(&handF[b + 1][s & 3], (b + 1) / kChiefs))[lane] = r2;
+                        make_rotation_warp(p, q, u, v, lane, c_cur, s_cur);
+                        put_rotation(b, (s + 1) & 1);
+                        // the next block's first column, (h_{k+1,k+1}, h_{k+2,k+1})
+                        // (lanes 6, 7 and 10, 11); its second one after the barrier
+                        al = __shfl_sync(0xffffffffu, r2, (hi ? 10 : 6) + po);
+                        ga = __shfl_sync(0xffffffffu, r2, (hi ? 6 : 10) + po);
+                        ep = __shfl_sync(0xffffffffu, r2, (hi ? 6 : 10) + pe);
+                    } else {
+                        if (lane < 8) as_double(&SGT_A(T, ldt, kb + (lane >> 2), kb + (part >> 1)))[part & 1] = r2;
+                        if (lane < 2 && b + 1 < nbul)
+                            as_double(cl.map_shared_rank(&handF[b + 1][s & 3], (b + 1) / kChiefs))[lane] = r2;
                     }
                 }
             } else if (helper && my < nbul) {
@@ -889,6 +889,7 @@ schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ s
                 if (s >= 3 * b && s < L + 3 * b) {
                     const double c = rc[b][s & 1];
                     const double2 sn = rs[b][s & 1];
+                    wrote = true;
                     if (lane == 0) {
                         const long long at = rot + (long long)b * L + (kb - l);
                         rclog[at] = c;
@@ -903,29 +904,35 @@ schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ s
                         reinterpret_cast<double *>(&SGT_A(T, ldt, kb + (hi ? 1 : 0), kb - 1))[odd ? 1 : 0] =
                             hi ? 0.0 : rz;
                         if (lane < 2 && b + 1 < nbul)
-                            reinterpret_cast<double *>(
-                                cl.map_shared_rank(&handH[b + 1][s & 1], (b + 1) / kChiefs))[lane] = rz;
+                            as_double(cl.map_shared_rank(&handH[b + 1][s & 1], (b + 1) / kChiefs))[lane] = rz;
+                    }
+                    if ((b == 0 || s >= L + 3 * (b - 1)) && kb + 3 <= i && lane >= 4 && lane < 6) {
+                        // the front chase, or the one in front has ended (its
+                        // last entries, a step old)
+                        if (lane == 4)
+                            handF[b][s & 3] = ldT(&SGT_A(T, ldt, kb + 3, kb + 3));
+                        else
+                            handH[b][s & 1] = ldT(&SGT_A(T, ldt, kb + 3, kb + 2));
                     }
                 }
             }
-            cl.sync();
+            step_barrier(wrote);
             if (chief && my < nbul) {
-                const int b = my, kb = l + s - 3 * b;
+                const int b = my;
                 const bool on = s >= 3 * b && s < L + 3 * b;
-                if (on && kb + 1 < i && col1) {
-                    const double2 B = bslot[b][(s + 1) & 1];
-                    to = odd ? B.y : B.x;
-                    te = odd ? B.x : B.y;
+                if (on && col1) {
+                    // the block's second column for the next step:
+                    // (h_{k+1,k+2}, h_{k+2,k+2})
+                    const double *bs = as_double(&bslot[b][(s + 1) & 1]), *hf = as_double(&handF[b][(s - 1) & 3]);
+                    al = (hi ? hf : bs)[po];
+                    ga = (hi ? bs : hf)[po];
+                    ep = (hi ? bs : hf)[pe];
                 }
-                if (b > 0 && (on || s == 3 * b - 1)) {
-                    // h_{k+3,k+2} for the next step (h_{l+2,l+1} before the
-                    // first): the left entry of the bulge in front, of this
-                    // step, or T once that chase ended
-                    double2 H = zero;
-                    if (kb + 3 <= i)
-                        H = (s < L + 3 * (b - 1)) ? handH[b][s & 1] : ldT(&SGT_A(T, ldt, kb + 3, kb + 2));
-                    ho = odd ? H.y : H.x;
-                    he = odd ? H.x : H.y;
+                if (on || s == 3 * b - 1) {
+                    // h_{k+3,k+2} (h_{l+2,l+1} before the first step)
+                    const double *hh = as_double(&handH[b][s & 1]);
+                    ho = hh[po];
+                    he = hh[pe];
                 }
             }
         }
