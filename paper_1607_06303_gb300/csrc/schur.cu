@@ -151,15 +151,11 @@ __global__ void finite_check_kernel(int n, const double *__restrict__ A, int lda
         if (!isfinite(SGT_A(A, lda, i, j))) atomicMin(bad, j);
 }
 
-// H = A (a working copy), Q0 = I
-__global__ void hess_init_kernel(int n, const double *__restrict__ A, int lda, double *__restrict__ H,
-                                 double *__restrict__ Q0)
+// H = A (a working copy)
+__global__ void hess_init_kernel(int n, const double *__restrict__ A, int lda, double *__restrict__ H)
 {
     const int j = blockIdx.x;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        SGT_A(H, n, i, j) = SGT_A(A, lda, i, j);
-        SGT_A(Q0, n, i, j) = (i == j) ? 1.0 : 0.0;
-    }
+    for (int i = threadIdx.x; i < n; i += blockDim.x) SGT_A(H, n, i, j) = SGT_A(A, lda, i, j);
 }
 
 __device__ __forceinline__ double block_sum(double x, double *red)
@@ -236,15 +232,14 @@ __global__ void house_left_kernel(int n, int k, double *__restrict__ H, const do
     for (int i = threadIdx.x; i < m; i += blockDim.x) col[i] = fma(-v[i], w, col[i]);
 }
 
-// The right application M[r, k+1:] -= tau (M[r, k+1:] v) v^T to the rows of
-// H (r < n) and of Q0 (r >= n), in two launches: y_r = tau M[r, k+1:] v with
-// 32 rows per CTA (lane = row, so each column's 32 entries are one
+// The right application H[r, k+1:] -= tau (H[r, k+1:] v) v^T in two
+// launches: y_r = tau H[r, k+1:] v with 32 rows per CTA (lane = row, so each column's 32 entries are one
 // coalesced read) and the columns split over the 8 warps, then the rank-1
 // update with a CTA per column.
 constexpr int kGemvWarps = 8;
 __global__ void __launch_bounds__(32 * kGemvWarps)
-house_gemv_kernel(int n, int k, const double *__restrict__ H, const double *__restrict__ Q0,
-                  const double *__restrict__ v, const double *__restrict__ tau, double *__restrict__ y)
+house_gemv_kernel(int n, int k, const double *__restrict__ H, const double *__restrict__ v,
+                  const double *__restrict__ tau, double *__restrict__ y)
 {
     __shared__ double part[kGemvWarps][32];
     const double t = *tau;
@@ -253,43 +248,198 @@ house_gemv_kernel(int n, int k, const double *__restrict__ H, const double *__re
     const int g = blockIdx.x * 32 + lane;
     const int m = n - k - 1;
     double acc = 0.0;
-    if (g < 2 * n) {
-        const double *M = g < n ? H : Q0;
-        const int r = g < n ? g : g - n;
-        for (int j = w; j < m; j += kGemvWarps) acc = fma(SGT_A(M, n, r, k + 1 + j), v[j], acc);
-    }
+    if (g < n)
+        for (int j = w; j < m; j += kGemvWarps) acc = fma(SGT_A(H, n, g, k + 1 + j), v[j], acc);
     part[w][lane] = acc;
     __syncthreads();
-    if (w == 0 && g < 2 * n) {
+    if (w == 0 && g < n) {
         double sum = 0.0;
         for (int q = 0; q < kGemvWarps; q++) sum += part[q][lane];
         y[g] = t * sum;
     }
 }
 
-__global__ void house_rank1_kernel(int n, int k, double *__restrict__ H, double *__restrict__ Q0,
-                                   const double *__restrict__ v, const double *__restrict__ tau,
-                                   const double *__restrict__ y)
+__global__ void house_rank1_kernel(int n, int k, double *__restrict__ H, const double *__restrict__ v,
+                                   const double *__restrict__ tau, const double *__restrict__ y)
 {
     if (*tau == 0.0) return;
     const int j = k + 1 + blockIdx.x;
     const double vj = v[blockIdx.x];
-    for (int g = threadIdx.x; g < 2 * n; g += blockDim.x) {
-        double *M = g < n ? H : Q0;
-        const int r = g < n ? g : g - n;
-        SGT_A(M, n, r, j) = fma(-y[g], vj, SGT_A(M, n, r, j));
-    }
+    for (int g = threadIdx.x; g < n; g += blockDim.x) SGT_A(H, n, g, j) = fma(-y[g], vj, SGT_A(H, n, g, j));
 }
 
-// complex T = H with its entries below the subdiagonal exactly 0; complex Q = Q0
-__global__ void to_complex_kernel(int n, const double *__restrict__ H, const double *__restrict__ Q0,
-                                  double2 *__restrict__ T, int ldt, double2 *__restrict__ Q, int ldq)
+// The whole reduction in one cluster of CL CTAs with H in their shared
+// memory (column j in CTA j % CL), where it fits (n up to 650 for 16 CTAs):
+// per column the launches above took ~52 us at n = 200, most of it their
+// starts and ends; here it is three cluster barriers and the float64 chains
+// between them (~1 ms for all columns instead of 10.3).  Step k: the owner
+// of column k forms the reflector (scaled by the power of two of its largest
+// entry); every CTA fetches v, applies the reflector to its columns from the
+// left (a warp per column) and sums its columns' share of H v; the shares
+// are added by rows (16 lanes a row, a lane per CTA) and sent to every CTA,
+// which updates its columns from the right.  v goes to V's column k (rows
+// k+1..), tau to taus[k]; T = H, complex.
+constexpr int kHessThreads = 512;
+inline size_t hess_smem(int n, int cl) { return ((size_t)((n + cl - 1) / cl) * n + 3 * (size_t)n) * sizeof(double); }
+constexpr size_t kHessSmemMax = 225 * 1024;
+
+template <int CL>
+__global__ void __launch_bounds__(kHessThreads)
+hess_cluster_kernel(int n, const double *__restrict__ A, int lda, double2 *__restrict__ T, int ldt,
+                    double *__restrict__ V, double *__restrict__ taus)
+{
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    extern __shared__ double hess_sh[];
+    constexpr int kWarps = kHessThreads / 32;
+    __shared__ double red[kWarps], out[3];   // out: 1 / (alpha - beta), tau, beta (scaled)
+    __shared__ int redi[kWarps];
+    __shared__ double tau_own;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, me = (int)cl.block_rank();
+    const int cols = (n + CL - 1) / CL;
+    double *Hc = hess_sh, *v = Hc + (size_t)cols * n, *ypart = v + n, *y = ypart + n;
+    for (int c = 0; me + c * CL < n; c++)
+        for (int i = tid; i < n; i += kHessThreads) Hc[(size_t)c * n + i] = SGT_A(A, lda, i, me + c * CL);
+    __syncthreads();
+    for (int k = 0; k + 2 < n; k++) {
+        const int owner = k % CL;
+        if (me == owner) {
+            double *x = Hc + (size_t)(k / CL) * n;
+            int em = -1000, nz = 0;
+            for (int i = k + 1 + tid; i < n; i += kHessThreads) {
+                em = max(em, ((__double2hiint(x[i]) >> 20) & 0x7ff) - 1023);
+                nz |= i > k + 1 && x[i] != 0.0;
+            }
+            em = __reduce_max_sync(0xffffffffu, em);
+            if (lane == 0) redi[warp] = em;
+            nz = __syncthreads_or(nz);
+            if (nz) {
+                em = min(__reduce_max_sync(0xffffffffu, redi[lane % kWarps]), 1000);
+                const double sc = __hiloint2double((1023 - em) << 20, 0);
+                double ss = 0.0;
+                for (int i = k + 1 + tid; i < n; i += kHessThreads) {
+                    const double t = x[i] * sc;
+                    ss = fma(t, t, ss);
+                }
+                for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+                if (lane == 0) red[warp] = ss;
+                __syncthreads();
+                if (warp == 0) {
+                    ss = lane < kWarps ? red[lane] : 0.0;
+                    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+                    const double alpha = x[k + 1] * sc;
+                    const double beta = -copysign(sqrt(ss), alpha);
+                    // lane 0: 1 / (alpha - beta); lane 1: (beta - alpha) / beta
+                    const double d = lane ? beta : alpha - beta;
+                    const double q = (lane ? beta - alpha : 1.0) / d;
+                    if (lane < 2) out[lane] = q;
+                    if (lane == 2) out[2] = beta * __hiloint2double((1023 + em) << 20, 0);
+                }
+                __syncthreads();
+                const double scal = out[0];
+                const double tau = out[1], beta = out[2];
+                for (int i = k + 1 + tid; i < n; i += kHessThreads) {
+                    const double vi = i == k + 1 ? 1.0 : x[i] * sc * scal;
+                    v[i] = vi;
+                    SGT_A(V, n, i, k) = vi;
+                    x[i] = i == k + 1 ? beta : 0.0;
+                }
+                if (tid == 0) {
+                    tau_own = tau;
+                    taus[k] = tau;
+                }
+            } else if (tid == 0) {
+                tau_own = 0.0;
+                taus[k] = 0.0;
+            }
+        }
+        cl.sync();
+        const double tau = *cl.map_shared_rank(&tau_own, owner);
+        if (me != owner) {
+            const double *vo = cl.map_shared_rank(v, owner);
+            for (int i = k + 1 + tid; i < n; i += kHessThreads) v[i] = vo[i];
+        }
+        if (tau == 0.0) continue;   // the same in every CTA
+        __syncthreads();
+        const int c0 = (k + 1 - me + CL - 1) / CL;   // the first of this CTA's columns right of k
+        const int first = c0 > 0 ? c0 : 0;
+        for (int c = first + warp; me + c * CL < n; c += kWarps) {
+            double *x = Hc + (size_t)c * n;
+            double w = 0.0;
+            for (int i = k + 1 + lane; i < n; i += 32) w = fma(v[i], x[i], w);
+            for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+            w *= tau;
+            for (int i = k + 1 + lane; i < n; i += 32) x[i] = fma(-v[i], w, x[i]);
+        }
+        __syncthreads();
+        for (int r = tid; r < n; r += kHessThreads) {
+            double a = 0.0;
+            for (int c = first; me + c * CL < n; c++) a = fma(Hc[(size_t)c * n + r], v[me + c * CL], a);
+            ypart[r] = a;
+        }
+        cl.sync();
+        for (int r0 = me * (kHessThreads / CL); r0 < n; r0 += kHessThreads) {
+            const int r = r0 + tid / CL, q = tid % CL;
+            double a = r < n ? cl.map_shared_rank(ypart, q)[r] : 0.0;
+            for (int o = CL / 2; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+            if (r < n) cl.map_shared_rank(y, q)[r] = tau * a;
+        }
+        cl.sync();
+        for (int r = tid; r < n; r += kHessThreads) {
+            const double yr = y[r];
+            for (int c = first; me + c * CL < n; c++) {
+                double &h = Hc[(size_t)c * n + r];
+                h = fma(-yr, v[me + c * CL], h);
+            }
+        }
+        __syncthreads();
+    }
+    for (int c = 0; me + c * CL < n; c++) {
+        const int j = me + c * CL;
+        for (int i = tid; i < n; i += kHessThreads)
+            SGT_A(T, ldt, i, j) = make_double2(i <= j + 1 ? Hc[(size_t)c * n + i] : 0.0, 0.0);
+    }
+    cl.sync();   // no CTA leaves while another reads its shared memory
+}
+
+// Q = P_0 P_1 .. P_{n-3}, complex: a row of Q takes every reflector from the
+// right by itself, so a warp per row runs through them without a barrier (lane
+// owns the columns lane + 32 t), the row in shared memory or, above kQRowsMax,
+// in `rows` (n x n).
+constexpr int kFormWarps = 4;
+constexpr int kQRowsMax = 5120;
+
+__global__ void __launch_bounds__(32 * kFormWarps)
+form_q_kernel(int n, const double *__restrict__ V, const double *__restrict__ taus, double *rows,
+              double2 *__restrict__ Q, int ldq)
+{
+    extern __shared__ double form_sh[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, r = blockIdx.x * kFormWarps + warp;
+    if (r >= n) return;
+    double *q = n <= kQRowsMax ? form_sh + (size_t)warp * n : rows + (size_t)r * n;
+    for (int i = lane; i < n; i += 32) q[i] = i == r ? 1.0 : 0.0;
+    for (int k = 0; k + 2 < n; k++) {
+        const double t = taus[k];
+        if (t == 0.0) continue;
+        const double *vk = V + (size_t)k * n;
+        const int i0 = ((k + 1) & ~31) + lane;
+        double w = 0.0;
+        for (int i = i0; i < n; i += 32)
+            if (i > k) w = fma(q[i], vk[i], w);
+        for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+        w *= t;
+        for (int i = i0; i < n; i += 32)
+            if (i > k) q[i] = fma(-w, vk[i], q[i]);
+    }
+    for (int i = lane; i < n; i += 32) SGT_A(Q, ldq, r, i) = make_double2(q[i], 0.0);
+}
+
+// complex T = H with its entries below the subdiagonal exactly 0
+__global__ void to_complex_kernel(int n, const double *__restrict__ H, double2 *__restrict__ T, int ldt)
 {
     const int j = blockIdx.x;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    for (int i = threadIdx.x; i < n; i += blockDim.x)
         SGT_A(T, ldt, i, j) = make_double2(i <= j + 1 ? SGT_A(H, n, i, j) : 0.0, 0.0);
-        SGT_A(Q, ldq, i, j) = make_double2(SGT_A(Q0, n, i, j), 0.0);
-    }
 }
 
 // ---------------------------------------------------------- QR iteration --
@@ -1044,16 +1194,16 @@ __global__ void real_part_kernel(int n, const double2 *__restrict__ Sc, double *
 
 namespace {
 
-// The QR sweeps' cluster: 16 CTAs (a non-portable size: 15 worker CTAs
-// halve the float64 work of each step's row and column updates, which the
-// worker SMs' float64 pipes bound) where the device can place such a cluster
-// of the kernel, else 8.
-cudaLaunchConfig_t qr_config(int cl, cudaStream_t st, cudaLaunchAttribute *at)
+// The cluster of the QR sweeps and of the reduction to Hessenberg form: 16
+// CTAs (a non-portable size: the float64 pipes of the CTAs bound the work
+// beside the chains) where the device can place such a cluster of both
+// kernels, else 8.
+cudaLaunchConfig_t cluster_config(int cl, int threads, size_t smem, cudaStream_t st, cudaLaunchAttribute *at)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(cl, 1, 1);
-    cfg.blockDim = dim3(kQrThreads, 1, 1);
-    cfg.dynamicSmemBytes = 0;
+    cfg.blockDim = dim3(threads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = cl;
@@ -1064,27 +1214,43 @@ cudaLaunchConfig_t qr_config(int cl, cudaStream_t st, cudaLaunchAttribute *at)
     return cfg;
 }
 
-int qr_cluster_size()
+bool places_16(const void *kernel, int threads, size_t smem)
 {
-    if (cudaFuncSetAttribute(schur_qr_kernel<16>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
-        cudaGetLastError();
-        return 8;
-    }
     cudaLaunchAttribute at[1];
-    const cudaLaunchConfig_t cfg = qr_config(16, nullptr, at);
+    const cudaLaunchConfig_t cfg = cluster_config(16, threads, smem, nullptr, at);
     int clusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&clusters, schur_qr_kernel<16>, &cfg) != cudaSuccess) {
-        cudaGetLastError();
-        return 8;
-    }
-    return clusters >= 1 ? 16 : 8;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess &&
+        cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) == cudaSuccess && clusters >= 1)
+        return true;
+    cudaGetLastError();
+    return false;
+}
+
+int cluster_size()
+{
+    return places_16((const void *)schur_qr_kernel<16>, kQrThreads, 0) &&
+                   places_16((const void *)hess_cluster_kernel<16>, kHessThreads, kHessSmemMax)
+               ? 16
+               : 8;
+}
+
+cudaError_t launch_hess(int cl, int n, const double *A, int lda, double2 *T, int ldt, double *V, double *taus,
+                        cudaStream_t stream)
+{
+    cudaLaunchAttribute at[1];
+    const cudaLaunchConfig_t cfg = cluster_config(cl, kHessThreads, hess_smem(n, cl), stream, at);
+    if (cl == 16) return cudaLaunchKernelEx(&cfg, hess_cluster_kernel<16>, n, A, lda, T, ldt, V, taus);
+    const cudaError_t e = cudaFuncSetAttribute(hess_cluster_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)kHessSmemMax);
+    return e == cudaSuccess ? cudaLaunchKernelEx(&cfg, hess_cluster_kernel<8>, n, A, lda, T, ldt, V, taus) : e;
 }
 
 cudaError_t launch_qr(int cl, int n, double2 *T, int ldt, QrState *st, SweepRec *sweeplog, double *rclog, double2 *rslog,
                       int *nlogged, cudaStream_t stream)
 {
     cudaLaunchAttribute at[1];
-    const cudaLaunchConfig_t cfg = qr_config(cl, stream, at);
+    const cudaLaunchConfig_t cfg = cluster_config(cl, kQrThreads, 0, stream, at);
     return cl == 16 ? cudaLaunchKernelEx(&cfg, schur_qr_kernel<16>, n, T, ldt, st, kRotationBudget,
                                          (long long)rotation_room(n), sweeplog, rclog, rslog, nlogged)
                     : cudaLaunchKernelEx(&cfg, schur_qr_kernel<8>, n, T, ldt, st, kRotationBudget,
@@ -1137,10 +1303,9 @@ signtri_status schur_run(int n, const double *A, int lda, double *Q, int ldq, do
     if (n <= 0) return SIGNTRI_OK;
     const size_t nn = (size_t)n * n;
     auto *H = static_cast<double *>(ws.take(nn * sizeof(double)));
-    auto *Q0 = static_cast<double *>(ws.take(nn * sizeof(double)));
-    auto *v = static_cast<double *>(ws.take((size_t)n * sizeof(double)));
+    auto *V = static_cast<double *>(ws.take(nn * sizeof(double)));   // the reflectors, column k in rows k+1..
+    auto *taus = static_cast<double *>(ws.take((size_t)n * sizeof(double)));
     auto *y = static_cast<double *>(ws.take((size_t)2 * n * sizeof(double)));
-    auto *tau = static_cast<double *>(ws.take(sizeof(double)));
     auto *bad = static_cast<int *>(ws.take(sizeof(int)));
     auto *qs = static_cast<QrState *>(ws.take(sizeof(QrState)));
     // a launch logs fewer than budget + 2n rotations (it starts a multi-sweep
@@ -1151,7 +1316,7 @@ signtri_status schur_run(int n, const double *A, int lda, double *Q, int ldq, do
     auto *rclog = static_cast<double *>(ws.take(2 * nlog * sizeof(double)));
     auto *rslog = static_cast<double2 *>(ws.take(2 * nlog * sizeof(double2)));
     auto *nlogged = static_cast<int *>(ws.take(2 * sizeof(int)));
-    if (!H || !Q0 || !v || !y || !tau || !bad || !qs || !sweeplog || !rclog || !rslog || !nlogged)
+    if (!H || !V || !taus || !y || !bad || !qs || !sweeplog || !rclog || !rslog || !nlogged)
         return SIGNTRI_ERR_NO_WORKSPACE;
     const int big = INT_MAX;
     SGT_CUDA_TRY(cudaMemcpyAsync(bad, &big, sizeof(int), cudaMemcpyHostToDevice, st));
@@ -1167,29 +1332,37 @@ signtri_status schur_run(int n, const double *A, int lda, double *Q, int ldq, do
         if (bad_index) *bad_index = first_bad;
         return SIGNTRI_ERR_NONFINITE;
     }
-    {
-        ProfScope ps(SIGNTRI_KC_FILL, st);
-        hess_init_kernel<<<n, kThreads, 0, st>>>(n, A, lda, H, Q0);
-        SGT_LAUNCH_CHECK();
-    }
-    for (int k = 0; k + 2 < n; k++) {
-        ProfScope ps(SIGNTRI_KC_HESSENBERG, st, true, false);
-        prof_count(SIGNTRI_KC_HESSENBERG, 4);
-        house_kernel<<<1, 1024, 0, st>>>(n, k, H, v, tau);
-        SGT_LAUNCH_CHECK();
-        house_left_kernel<<<n - k - 1, kThreads, 0, st>>>(n, k, H, v, tau);
-        SGT_LAUNCH_CHECK();
-        house_gemv_kernel<<<(2 * n + 31) / 32, 32 * kGemvWarps, 0, st>>>(n, k, H, Q0, v, tau, y);
-        SGT_LAUNCH_CHECK();
-        house_rank1_kernel<<<n - k - 1, kThreads, 0, st>>>(n, k, H, Q0, v, tau, y);
-        SGT_LAUNCH_CHECK();
-    }
     auto *Tc = reinterpret_cast<double2 *>(T);
     auto *Qc = reinterpret_cast<double2 *>(Q);
+    const int cl = cluster_size();
+    if (hess_smem(n, cl) <= kHessSmemMax) {
+        ProfScope ps(SIGNTRI_KC_HESSENBERG, st);
+        SGT_CUDA_TRY(launch_hess(cl, n, A, lda, Tc, ldt, V, taus, st));
+    } else {
+        {
+            ProfScope ps(SIGNTRI_KC_FILL, st);
+            hess_init_kernel<<<n, kThreads, 0, st>>>(n, A, lda, H);
+            SGT_LAUNCH_CHECK();
+        }
+        for (int k = 0; k + 2 < n; k++) {
+            ProfScope ps(SIGNTRI_KC_HESSENBERG, st, true, false);
+            prof_count(SIGNTRI_KC_HESSENBERG, 4);
+            double *v = V + (size_t)k * n + k + 1, *tau = taus + k;
+            house_kernel<<<1, 1024, 0, st>>>(n, k, H, v, tau);
+            SGT_LAUNCH_CHECK();
+            house_left_kernel<<<n - k - 1, kThreads, 0, st>>>(n, k, H, v, tau);
+            SGT_LAUNCH_CHECK();
+            house_gemv_kernel<<<(n + 31) / 32, 32 * kGemvWarps, 0, st>>>(n, k, H, v, tau, y);
+            SGT_LAUNCH_CHECK();
+            house_rank1_kernel<<<n - k - 1, kThreads, 0, st>>>(n, k, H, v, tau, y);
+            SGT_LAUNCH_CHECK();
+        }
+        ProfScope ps(SIGNTRI_KC_FILL, st);
+        to_complex_kernel<<<n, kThreads, 0, st>>>(n, H, Tc, ldt);
+        SGT_LAUNCH_CHECK();
+    }
     {
         ProfScope ps(SIGNTRI_KC_FILL, st);
-        to_complex_kernel<<<n, kThreads, 0, st>>>(n, H, Q0, Tc, ldt, Qc, ldq);
-        SGT_LAUNCH_CHECK();
         qr_state_init_kernel<<<1, 1, 0, st>>>(n, qs);
         SGT_LAUNCH_CHECK();
     }
@@ -1205,7 +1378,18 @@ signtri_status schur_run(int n, const double *A, int lda, double *Q, int ldq, do
     // cluster finds its SMs free (a QR CTA takes a whole SM's registers).
     ApplyStream ap;
     SGT_CUDA_TRY(ap.init());
-    const int qr_cl = qr_cluster_size();
+    // Q's reflectors on the second stream as well, while the sweeps begin
+    SGT_CUDA_TRY(cudaEventRecord(ap.swept[0], st));
+    SGT_CUDA_TRY(cudaStreamWaitEvent(ap.s, ap.swept[0], 0));
+    auto form_q = [&]() -> signtri_status {
+        const size_t smem = n <= kQRowsMax ? (size_t)kFormWarps * n * sizeof(double) : 0;
+        SGT_CUDA_TRY(cudaFuncSetAttribute(form_q_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)(kFormWarps * kQRowsMax * sizeof(double))));
+        ProfScope ps(SIGNTRI_KC_HESSENBERG, ap.s);
+        form_q_kernel<<<(n + kFormWarps - 1) / kFormWarps, 32 * kFormWarps, smem, ap.s>>>(n, V, taus, H, Qc, ldq);
+        SGT_LAUNCH_CHECK();
+        return SIGNTRI_OK;
+    };
     auto apply = [&](int p) -> signtri_status {
         const size_t lo = p * nlog;
         SGT_CUDA_TRY(cudaStreamWaitEvent(ap.s, ap.swept[p], 0));
@@ -1227,10 +1411,13 @@ signtri_status schur_run(int n, const double *A, int lda, double *Q, int ldq, do
         if (it >= 2) SGT_CUDA_TRY(cudaStreamWaitEvent(st, ap.applied[p], 0));
         {
             ProfScope ps(SIGNTRI_KC_SCHUR, st);
-            SGT_CUDA_TRY(launch_qr(qr_cl, n, Tc, ldt, qs, sweeplog + lo, rclog + lo, rslog + lo, nlogged + p, st));
+            SGT_CUDA_TRY(launch_qr(cl, n, Tc, ldt, qs, sweeplog + lo, rclog + lo, rslog + lo, nlogged + p, st));
         }
         SGT_CUDA_TRY(cudaEventRecord(ap.swept[p], st));
-        if (it >= 1) {
+        if (it == 0) {
+            const signtri_status rq = form_q();
+            if (rq != SIGNTRI_OK) return rq;
+        } else {
             const signtri_status ra = apply(1 - p);
             if (ra != SIGNTRI_OK) return ra;
         }
