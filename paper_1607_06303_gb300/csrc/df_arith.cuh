@@ -113,4 +113,27 @@ __device__ __forceinline__ void df_rot(float ch, float cl, float uh, float ul, f
     df_add2(ph, pl, qh, ql, h, l);
 }
 
+// the unbiased exponent field of |x| (integer operations only)
+__device__ __forceinline__ int exp_field(double x) { return ((__double2hiint(x) >> 20) & 0x7ff) - 1023; }
+
+// 1 / sqrt(a) for a normal a > 0: with a = 4^h m, m in [1, 4), a single-
+// precision reciprocal root r of m (relative error below 2^-20 with m's
+// mantissa cut to 23 bits) and one step of the third-order iteration
+// r (1 + e / 2 + 3 e^2 / 8), e = 1 - m r^2, from the binomial series of
+// (1 - e)^(-1/2): the series' next term is below 2^-60.  Five float64
+// instructions; the powers of two are moved by integer operations.
+__device__ __forceinline__ double rsqrt_normal(double a)
+{
+    const int hi = __double2hiint(a), lo = __double2loint(a);
+    const int h = ((hi >> 20) - 1023) >> 1;
+    const int mh = hi - (h << 21);
+    const float r0 = rsqrtf(__int_as_float((int)(((unsigned)(mh - (896 << 20)) << 3) | ((unsigned)lo >> 29))));
+    const unsigned rb = (unsigned)__float_as_int(r0);
+    const double m = __hiloint2double(mh, lo);
+    const double r = __hiloint2double((int)(rb >> 3) + (896 << 20), (int)(rb << 29));
+    const double e = fma(-(m * r), r, 1.0);
+    const double y = fma(fma(0.375, e, 0.5), r * e, r);
+    return __hiloint2double(__double2hiint(y) - (h << 20), __double2loint(y));
+}
+
 }  // namespace signtri

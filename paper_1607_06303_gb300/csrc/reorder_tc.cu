@@ -8,8 +8,8 @@
 // window keeps the diagonal block T[W, W] in shared memory, runs the swaps as
 // odd-even rounds there (each rotation as in ps_fp64.cu: G's first column the
 // eigenvector of the entry moving up, the 2 x 2 diagonal block swapped
-// exactly) and logs them; it then forms the window's orthogonal factor Z_W =
-// G_1 G_2 ... by applying the logged rotations to the identity.  The rest of
+// exactly) and logs them; four CTAs a window then form its orthogonal factor
+// Z_W = G_1 G_2 ... by applying the logged rotations to the identity.  The rest of
 // T and Q receive the window's rotations at once, as products:
 //   T[W, right of W] <- Z_W^T T[W, right of W]
 //   T[above W, W]    <- T[above W, W] Z_W
@@ -22,6 +22,7 @@
 #include <algorithm>
 #include <vector>
 
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
 #include "df_arith.cuh"
@@ -45,207 +46,301 @@ constexpr int kWinThreads = 512;
 constexpr int kSlices = 6;
 constexpr int kBits = 8;
 
-// Shared memory of a window: its block as double-float planes (hi, lo), the
-// logged rotations (c, s as double-float pairs, and k), the exact diagonal.
-size_t window_smem_bytes()
-{
-    return 2 * (size_t)kWin * kWinLD * sizeof(float) + 4 * (size_t)kMaxRot * sizeof(float) +
-           (size_t)kWin * sizeof(double) + (size_t)kMaxRot * sizeof(short);
-}
+// The rotations of a window's rounds, read by window_factor_kernel: round
+// r's are [off[r], off[r + 1]), each (c, s) as double-float pairs and its
+// first position k.
+struct WindowLog {
+    float4 rot[kMaxRot];   // c hi, c lo, s hi, s lo
+    short k[kMaxRot];
+    int off[2 * kWin + 8];
+    int rounds;
+};
 
-// One window per CTA: stable partition of T[W, W] by swaps, then Z_W as the
-// exact column slices the products read -- ZC[s][a + j][a + i] = slice s of
-// Z_W[i][j] under the column's power-of-two scale sZ[a + j] (rp rows of
-// pitch kp per slice).  Entries of ZC outside the windows' blocks are never
-// read (the products' K ranges stay inside the window).
+// Shared memory of a window's sort: its block as double-float planes (hi, lo)
+size_t window_smem_bytes() { return 2 * (size_t)kWin * kWinLD * sizeof(float); }
+
+// One window per CTA: stable partition of T[W, W] by swaps, the rotations
+// logged for window_factor_kernel.
 // GB300's float64 rate is about 1/64 of its fp32 rate, and a window is one
 // SM's work, so the rotations are applied in double-float (df_arith.cuh:
 // about 2^-47 per operation) to the block held as hi/lo planes; the
 // diagonal stays float64 (swapped exactly) and each rotation's (c, s) is
-// computed in float64 from it and the coupling, one thread per pair.
+// computed in float64 from it and the coupling, one thread per pair (one
+// reciprocal square root: hypot and two divisions were ~3,000 of a round's
+// ~6,000 cycles).
+// The rounds form a chain: a round's rotations need the couplings that the
+// round before leaves.  So two chief warps (a thread per pair of the next
+// round) apply the few rotations that change those couplings, find the next
+// round's pairs and form its rotations, while the other warps apply the rest
+// of the round; one barrier a round.
+constexpr int kChiefThreads = 64;
+
 __global__ void __launch_bounds__(kWinThreads)
-window_sort_kernel(double *__restrict__ Tr, int ldt, const int2 *__restrict__ wins, __nv_bfloat16 *__restrict__ ZC,
-                   float *__restrict__ sZ, int rp, int kp)
+window_sort_kernel(double *__restrict__ Tr, int ldt, const int2 *__restrict__ wins, WindowLog *__restrict__ logs)
 {
-    extern __shared__ double wsm[];
-    double *dg = wsm;                                        // dg[i] = T[a + i, a + i]
-    float *Bh = reinterpret_cast<float *>(dg + kWin);        // Bh/Bl[i + j * kWinLD]: T[a + i, a + j], i < j
-    float *Bl = Bh + kWin * kWinLD;
-    float *lch = Bl + kWin * kWinLD, *lcl = lch + kMaxRot;   // logged rotations, round by round
-    float *lsh = lcl + kMaxRot, *lsl = lsh + kMaxRot;
-    short *lk = reinterpret_cast<short *>(lsl + kMaxRot);
-    __shared__ signed char sg[kWin];
-    __shared__ short pm[kWin];                        // log index of the round's pair holding position i, or -1
-    __shared__ int roff[2 * kWin + 4];
-    __shared__ int nlog, nround, quiet[2];
+    extern __shared__ float wsm[];
+    float *Bh = wsm, *Bl = Bh + kWin * kWinLD;               // Bh/Bl[i + j * kWinLD]: T[a + i, a + j], i < j
+    // of the round at work and the next one, by the round's parity: the
+    // diagonal, each pair's rotation and first position, the pair (its index
+    // in the round) holding a position or -1, the pairs
+    __shared__ double dg[2][kWin + 2];
+    __shared__ float4 rot[2][kWin / 2];
+    __shared__ short first[2][kWin / 2], pm[2][kWin + 2];
+    __shared__ int wc[2][2], cnt[2];
     const int a = wins[blockIdx.x].x, w = wins[blockIdx.x].y;
-    for (int idx = threadIdx.x; idx < kWin * kWin; idx += kWinThreads) {
+    WindowLog *log = logs + blockIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int idx = tid; idx < kWin * kWin; idx += kWinThreads) {
         const int i = idx % kWin, j = idx / kWin;
         const double v = (i < j && j < w) ? SGT_AT(Tr, ldt, a + i, a + j) : 0.0;
         split_df(v, Bh[i + j * kWinLD], Bl[i + j * kWinLD]);
-        if (i == j) dg[i] = (j < w) ? SGT_AT(Tr, ldt, a + i, a + i) : 1.0;
+        if (i == j) dg[1][i] = (j < w) ? SGT_AT(Tr, ldt, a + i, a + i) : 1.0;
     }
+    if (tid < 2) {
+        dg[tid][kWin] = dg[tid][kWin + 1] = 1.0;
+        cnt[tid] = 0;
+    }
+    for (int i = tid; i < kWin + 2; i += kWinThreads) pm[0][i] = pm[1][i] = -1;
     __syncthreads();
-    for (int i = threadIdx.x; i < kWin; i += kWinThreads) sg[i] = (i < w && dg[i] > 0.0) ? 1 : -1;
-    if (threadIdx.x == 0) {
-        nlog = 0;
-        nround = 0;
-        quiet[0] = quiet[1] = 0;
+    int r = -1, base = 0;   // round -1 has no pairs; the chiefs find round 0's
+    for (;; r++) {
+        const int cur = r & 1, nxt = cur ^ 1;
+        const int P = cnt[cur];
+        if (tid < kChiefThreads) {
+            // the next round's pair slot (k, k + 1); of this round, the pair A
+            // = (k - 1, k) and the pair C = (k + 1, k + 2)
+            const int k = 2 * tid + nxt;
+            const int eA = k > 0 ? pm[cur][k] : -1, eC = k + 1 < kWin ? pm[cur][k + 1] : -1;
+            float bh = 0.f, bl = 0.f;   // the coupling (k, k + 1) after this round
+            if (k + 1 < w) {
+                const int at = k + (k + 1) * kWinLD;
+                bh = Bh[at];
+                bl = Bl[at];
+                float uh = 0.f, ul = 0.f;   // row k - 1 of column k + 1
+                if (eA >= 0) {
+                    const float4 g = rot[cur][eA];
+                    const float ph = Bh[at - 1], pl = Bl[at - 1];
+                    df_rot(g.x, g.y, ph, pl, g.z, g.w, bh, bl, uh, ul);        // c u + s v
+                    df_rot(-g.z, -g.w, ph, pl, g.x, g.y, bh, bl, bh, bl);      // -s u + c v
+                }
+                if (eC >= 0) {
+                    const float4 g2 = rot[cur][eC];
+                    const int at2 = at + kWinLD;
+                    float qh = Bh[at2], ql = Bl[at2];   // row k of column k + 2
+                    if (eA >= 0) {
+                        const float4 g = rot[cur][eA];
+                        const float ph = Bh[at2 - 1], pl = Bl[at2 - 1];
+                        float th, tl;
+                        df_rot(g.x, g.y, ph, pl, g.z, g.w, qh, ql, th, tl);
+                        df_rot(-g.z, -g.w, ph, pl, g.x, g.y, qh, ql, qh, ql);
+                        float xh, xl;
+                        df_rot(g2.x, g2.y, uh, ul, g2.z, g2.w, th, tl, xh, xl);            // u c + v s
+                        df_rot(-g2.z, -g2.w, uh, ul, g2.x, g2.y, th, tl, Bh[at2 - 1], Bl[at2 - 1]);   // -u s + v c
+                        uh = xh;
+                        ul = xl;
+                    }
+                    const float vh = bh, vl = bl;
+                    df_rot(g2.x, g2.y, vh, vl, g2.z, g2.w, qh, ql, bh, bl);
+                    df_rot(-g2.z, -g2.w, vh, vl, g2.x, g2.y, qh, ql, Bh[at2], Bl[at2]);
+                }
+                if (eA >= 0) {
+                    Bh[at - 1] = uh;
+                    Bl[at - 1] = ul;
+                }
+                if (eA >= 0 || eC >= 0) {
+                    Bh[at] = bh;
+                    Bl[at] = bl;
+                }
+            }
+            // the diagonal after the round's swaps (exact)
+            const double d0 = eA >= 0 ? dg[cur][k - 1] : dg[cur][k];
+            const double d1 = eC >= 0 ? dg[cur][k + 2] : dg[cur][k + 1];
+            dg[nxt][k] = d0;
+            dg[nxt][k + 1] = d1;
+            if (nxt == 1 && tid == 0) {
+                dg[1][0] = eA >= 0 ? dg[0][1] : dg[0][0];
+                pm[1][0] = -1;
+            }
+            const bool on = k + 1 < w && !(d0 > 0.0) && d1 > 0.0;
+            const unsigned bal = __ballot_sync(0xffffffffu, on);
+            if (lane == 0) wc[nxt][warp] = __popc(bal);
+            asm volatile("bar.sync 1, %0;" ::"n"(kChiefThreads) : "memory");
+            const int pos = (warp ? wc[nxt][0] : 0) + __popc(bal & ((1u << lane) - 1u));
+            const int total = wc[nxt][0] + wc[nxt][1];
+            pm[nxt][k] = pm[nxt][k + 1] = on ? (short)pos : (short)-1;
+            if (tid == 0) {
+                cnt[nxt] = total;
+                log->off[r + 1] = base;
+            }
+            if (on) {
+                // G's first column is the eigenvector of the entry moving up:
+                // (bb, d) / |(bb, d)|
+                const double bb = df_to_double(bh, bl), d = d1 - d0;
+                const int em = max(exp_field(bb), exp_field(d));
+                double c, s;
+                if (em > -500 && em < 500) {
+                    const double rh = rsqrt_normal(fma(bb, bb, d * d));
+                    c = bb * rh;
+                    s = d * rh;
+                } else {
+                    const double h = hypot(bb, d);
+                    c = bb / h;
+                    s = d / h;
+                }
+                float4 g;
+                split_df(c, g.x, g.y);
+                split_df(s, g.z, g.w);
+                rot[nxt][pos] = g;
+                first[nxt][pos] = (short)k;
+                log->rot[base + pos] = g;
+                log->k[base + pos] = (short)k;
+            }
+            base += total;
+        } else {
+            // the rest of round r, four warps' items a pair e = (k, k + 1),
+            // one per position x: x right of the pair -- G^T on rows k, k+1 of
+            // column x, and, where x is in a pair itself, that pair's G on
+            // columns x, x+1 (the two columns in neighbouring lanes); x left
+            // of the pair and in none -- G on columns k, k+1 of row x.  What
+            // touches the couplings next to the pair is the chiefs'.
+            for (int task = warp - kChiefThreads / 32; task < 4 * P; task += (kWinThreads - kChiefThreads) / 32) {
+                const int k = first[cur][task >> 2];
+                const int x = (((task & 3) << 5) + lane + cur) & (kWin - 1);
+                const int q = pm[cur][x];
+                const bool right = x < w && (q < 0 ? x >= k + 3 : first[cur][q] >= k + 4);
+                const bool left = q < 0 && x <= k - 2;
+                const float4 g = rot[cur][task >> 2];
+                const int i0 = right ? k + x * kWinLD : x + k * kWinLD, i1 = i0 + (right ? 1 : kWinLD);
+                float uh = 0.f, ul = 0.f, vh = 0.f, vl = 0.f, sh, sl, th, tl;
+                if (right || left) {
+                    uh = Bh[i0];
+                    ul = Bl[i0];
+                    vh = Bh[i1];
+                    vl = Bl[i1];
+                }
+                df_rot(g.x, g.y, uh, ul, g.z, g.w, vh, vl, sh, sl);        // c u + s v
+                df_rot(-g.z, -g.w, uh, ul, g.x, g.y, vh, vl, th, tl);      // -s u + c v
+                const bool both = right && q >= 0;
+                if (__any_sync(0xffffffffu, both)) {
+                    const float osh = __shfl_xor_sync(0xffffffffu, sh, 1), osl = __shfl_xor_sync(0xffffffffu, sl, 1);
+                    const float oth = __shfl_xor_sync(0xffffffffu, th, 1), otl = __shfl_xor_sync(0xffffffffu, tl, 1);
+                    if (both) {
+                        // first column u c + v s, second -u s + v c
+                        float4 g2 = rot[cur][q];
+                        if (lane & 1) {
+                            g2.z = -g2.z;
+                            g2.w = -g2.w;
+                        }
+                        df_rot(g2.x, g2.y, sh, sl, g2.z, g2.w, osh, osl, sh, sl);
+                        df_rot(g2.x, g2.y, th, tl, g2.z, g2.w, oth, otl, th, tl);
+                    }
+                }
+                if (right || left) {
+                    Bh[i0] = sh;
+                    Bl[i0] = sl;
+                    Bh[i1] = th;
+                    Bl[i1] = tl;
+                }
+            }
+        }
+        __syncthreads();
+        // two rounds in a row without a swap end the sort (at most w + 1 rounds)
+        if ((r >= 0 && P == 0 && cnt[nxt] == 0) || r >= 2 * kWin) break;
     }
-    __syncthreads();
-    // odd-even rounds until two in a row swap nothing (at most w + 1 rounds).
-    // The count of quiet rounds is double-buffered: round r writes slot
-    // r & 1 while the loop test of round r reads slot (r - 1) & 1.
-    for (int r = 0; r < 2 * kWin + 2; r++) {
-        if (r > 0 && quiet[(r - 1) & 1] >= 2) break;
-        if (threadIdx.x < 32) {
-            // warp 0 finds the round's pairs (positions 4 lane .. 4 lane + 3),
-            // logs them in position order (a prefix count by shuffles) and
-            // marks both positions of each pair in pm
-            const int lane = threadIdx.x, base = nlog;
-            bool on[4];
-            int c = 0;
-#pragma unroll
-            for (int q = 0; q < 4; q++) {
-                const int k = 4 * lane + q;
-                on[q] = (k & 1) == (r & 1) && k + 1 < w && sg[k] < 0 && sg[k + 1] > 0;
-                c += on[q];
-            }
-            int incl = c;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int t = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += t;
-            }
-            int e = base + incl - c, mine[4];
-#pragma unroll
-            for (int q = 0; q < 4; q++) {
-                mine[q] = -1;
-                if (on[q]) {
-                    lk[e] = (short)(4 * lane + q);
-                    mine[q] = e++;
-                }
-            }
-            const int prev = __shfl_up_sync(0xffffffffu, mine[3], 1);
-#pragma unroll
-            for (int q = 0; q < 4; q++) {
-                const int left = q > 0 ? mine[q - 1] : (lane > 0 ? prev : -1);
-                pm[4 * lane + q] = (short)(mine[q] >= 0 ? mine[q] : left);
-            }
-            const int total = __shfl_sync(0xffffffffu, incl, 31);
-            if (lane == 0) {
-                roff[r] = base;
-                nlog = base + total;
-                quiet[r & 1] = total ? 0 : (r > 0 ? quiet[(r - 1) & 1] : 0) + 1;
-                nround = r + 1;
-            }
-        }
-        __syncthreads();
-        const int e0 = roff[r], P = nlog - e0;
-        // each pair's rotation, in float64 from the exact diagonal and the
-        // coupling: G's first column is the eigenvector of the entry moving up
-        for (int t = threadIdx.x; t < P; t += kWinThreads) {
-            const int e = e0 + t, k = lk[e];
-            const double aa = dg[k], cc = dg[k + 1];
-            const double bb = df_to_double(Bh[k + (k + 1) * kWinLD], Bl[k + (k + 1) * kWinLD]);
-            const double d = cc - aa, h = hypot(bb, d);
-            split_df(bb / h, lch[e], lcl[e]);
-            split_df(d / h, lsh[e], lsl[e]);
-        }
-        __syncthreads();
-        // the round's rotations, one item per (pair, position x): x right of
-        // the pair -- G^T on rows k, k+1 of column x (with G_q on columns x,
-        // x+1 as well when x starts pair q); x left of the pair -- G on
-        // columns k, k+1 of row x (rows inside a pair are done from that
-        // pair's side); x = k -- the exact swap of the 2 x 2 diagonal block,
-        // whose coupling is unchanged.  No two items touch the same entry.
-        for (int idx = threadIdx.x; idx < P * kWin; idx += kWinThreads) {
-            const int e = e0 + idx / kWin, x = idx % kWin, k = lk[e];
-            if (x >= w) continue;
-            const float ch = lch[e], cl = lcl[e], sh = lsh[e], sl = lsl[e];
-            if (x >= k + 2) {
-                const int q = pm[x];
-                if (q < 0) {
-                    const int i0 = k + x * kWinLD, i1 = i0 + 1;
-                    const float uh = Bh[i0], ul = Bl[i0], vh = Bh[i1], vl = Bl[i1];
-                    df_rot(ch, cl, uh, ul, sh, sl, vh, vl, Bh[i0], Bl[i0]);          // c u + s v
-                    df_rot(-sh, -sl, uh, ul, ch, cl, vh, vl, Bh[i1], Bl[i1]);        // -s u + c v
-                } else if (lk[q] == x) {
-                    const float c2h = lch[q], c2l = lcl[q], s2h = lsh[q], s2l = lsl[q];
-                    const int i00 = k + x * kWinLD, i10 = i00 + 1, i01 = i00 + kWinLD, i11 = i01 + 1;
-                    float r00h, r00l, r10h, r10l, r01h, r01l, r11h, r11l;
-                    df_rot(ch, cl, Bh[i00], Bl[i00], sh, sl, Bh[i10], Bl[i10], r00h, r00l);
-                    df_rot(-sh, -sl, Bh[i00], Bl[i00], ch, cl, Bh[i10], Bl[i10], r10h, r10l);
-                    df_rot(ch, cl, Bh[i01], Bl[i01], sh, sl, Bh[i11], Bl[i11], r01h, r01l);
-                    df_rot(-sh, -sl, Bh[i01], Bl[i01], ch, cl, Bh[i11], Bl[i11], r11h, r11l);
-                    df_rot(c2h, c2l, r00h, r00l, s2h, s2l, r01h, r01l, Bh[i00], Bl[i00]);    // u c + v s
-                    df_rot(-s2h, -s2l, r00h, r00l, c2h, c2l, r01h, r01l, Bh[i01], Bl[i01]);  // -u s + v c
-                    df_rot(c2h, c2l, r10h, r10l, s2h, s2l, r11h, r11l, Bh[i10], Bl[i10]);
-                    df_rot(-s2h, -s2l, r10h, r10l, c2h, c2l, r11h, r11l, Bh[i11], Bl[i11]);
-                }
-            } else if (x < k) {
-                if (pm[x] < 0) {
-                    const int i0 = x + k * kWinLD, i1 = i0 + kWinLD;
-                    const float uh = Bh[i0], ul = Bl[i0], vh = Bh[i1], vl = Bl[i1];
-                    df_rot(ch, cl, uh, ul, sh, sl, vh, vl, Bh[i0], Bl[i0]);          // u c + v s
-                    df_rot(-sh, -sl, uh, ul, ch, cl, vh, vl, Bh[i1], Bl[i1]);        // -u s + v c
-                }
-            } else if (x == k) {
-                const double t0 = dg[k];
-                dg[k] = dg[k + 1];
-                dg[k + 1] = t0;
-                sg[k] = 1;
-                sg[k + 1] = -1;
-            }
-        }
-        __syncthreads();
+    // round r + 1 is the last one logged, and empty
+    if (tid == 0) {
+        log->off[r + 2] = base;
+        log->rounds = r + 2;
     }
-    if (threadIdx.x == 0) roff[nround] = nlog;
-    for (int idx = threadIdx.x; idx < kWin * kWin; idx += kWinThreads) {
+    const double *dl = dg[(r & 1) ^ 1];
+    for (int idx = tid; idx < kWin * kWin; idx += kWinThreads) {
         const int i = idx % kWin, j = idx / kWin;
         if (j < w && i < j) SGT_AT(Tr, ldt, a + i, a + j) = df_to_double(Bh[i + j * kWinLD], Bl[i + j * kWinLD]);
-        else if (j < w && i == j) SGT_AT(Tr, ldt, a + i, a + i) = dg[i];
+        else if (j < w && i == j) SGT_AT(Tr, ldt, a + i, a + i) = dl[i];
+    }
+}
+
+// The window's orthogonal factor Z_W = I G_1 G_2 ... as the exact column
+// slices the products read -- ZC[s][a + j][a + i] = slice s of Z_W[i][j]
+// under the column's power-of-two scale sZ[a + j] (rp rows of pitch kp per
+// slice).  Entries of ZC outside the windows' blocks are never read (the
+// products' K ranges stay inside the window).  A row of Z takes every
+// rotation by itself, so a cluster of kFactorCtas CTAs takes 32 rows each (a
+// sweep has n / 128 windows, far fewer than SMs): a warp per pair of a round,
+// a row per lane; the columns' maxima meet in shared memory.
+constexpr int kFactorCtas = kWin / 32;
+constexpr int kFactorLD = 33;
+
+size_t factor_smem_bytes()
+{
+    return (size_t)kMaxRot * (sizeof(float4) + sizeof(short)) + 2 * (size_t)kWin * kFactorLD * sizeof(float);
+}
+
+__global__ void __cluster_dims__(kFactorCtas, 1, 1) __launch_bounds__(kWinThreads)
+window_factor_kernel(const int2 *__restrict__ wins, const WindowLog *__restrict__ logs, __nv_bfloat16 *__restrict__ ZC,
+                     float *__restrict__ sZ, int rp, int kp)
+{
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    extern __shared__ float4 fsm[];
+    float4 *rot = fsm;
+    float *Zh = reinterpret_cast<float *>(rot + kMaxRot), *Zl = Zh + kWin * kFactorLD;   // [i + j * kFactorLD]
+    short *first = reinterpret_cast<short *>(Zl + kWin * kFactorLD);
+    __shared__ int off[2 * kWin + 8], cexp[kWin];
+    __shared__ float cmax[kWin];
+    const int win = blockIdx.x / kFactorCtas, a = wins[win].x, w = wins[win].y;
+    const int part = (int)cl.block_rank(), row0 = 32 * part;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const WindowLog *log = logs + win;
+    const int rounds = log->rounds, nlog = log->off[rounds];
+    for (int r = tid; r <= rounds; r += kWinThreads) off[r] = log->off[r];
+    for (int e = tid; e < nlog; e += kWinThreads) {
+        rot[e] = log->rot[e];
+        first[e] = log->k[e];
+    }
+    for (int idx = tid; idx < 32 * kWin; idx += kWinThreads) {
+        const int i = idx & 31, j = idx >> 5;
+        Zh[i + j * kFactorLD] = (row0 + i == j) ? 1.f : 0.f;
+        Zl[i + j * kFactorLD] = 0.f;
     }
     __syncthreads();
-    // Z = I G_1 G_2 ..., round by round (a round's rotations act on disjoint columns)
-    for (int idx = threadIdx.x; idx < kWin * kWin; idx += kWinThreads) {
-        const int i = idx % kWin, j = idx / kWin;
-        Bh[i + j * kWinLD] = (i == j) ? 1.f : 0.f;
-        Bl[i + j * kWinLD] = 0.f;
-    }
-    __syncthreads();
-    for (int r = 0; r < nround; r++) {
-        const int e0 = roff[r], e1 = roff[r + 1];
-        for (int idx = threadIdx.x; idx < (e1 - e0) * kWin; idx += kWinThreads) {
-            const int e = e0 + idx / kWin, i = idx % kWin;
-            const int k = lk[e];
-            const int i0 = i + k * kWinLD, i1 = i0 + kWinLD;
-            const float uh = Bh[i0], ul = Bl[i0], vh = Bh[i1], vl = Bl[i1];
-            df_rot(lch[e], lcl[e], uh, ul, lsh[e], lsl[e], vh, vl, Bh[i0], Bl[i0]);
-            df_rot(-lsh[e], -lsl[e], uh, ul, lch[e], lcl[e], vh, vl, Bh[i1], Bl[i1]);
+    // round by round (a round's rotations act on disjoint columns)
+    for (int r = 0; r < rounds; r++) {
+        for (int e = off[r] + warp; e < off[r + 1]; e += kWinThreads / 32) {
+            const float4 g = rot[e];
+            const int i0 = lane + first[e] * kFactorLD, i1 = i0 + kFactorLD;
+            const float uh = Zh[i0], ul = Zl[i0], vh = Zh[i1], vl = Zl[i1];
+            df_rot(g.x, g.y, uh, ul, g.z, g.w, vh, vl, Zh[i0], Zl[i0]);
+            df_rot(-g.z, -g.w, uh, ul, g.x, g.y, vh, vl, Zh[i1], Zl[i1]);
         }
         __syncthreads();
     }
     // per column of Z: the power-of-two scale above its largest entry (an
     // orthogonal column: between 1 / sqrt(w) and 1; |hi + lo| < 2^e whenever
     // |hi| < 2^e, lo being at most half an ulp of hi), then its exact slices
-    __shared__ int cexp[kWin];
-    for (int j = threadIdx.x; j < w; j += kWinThreads) {
+    for (int j = warp; j < w; j += kWinThreads / 32) {
+        float mx = row0 + lane < w ? fabsf(Zh[lane + j * kFactorLD]) : 0.f;
+        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        if (lane == 0) cmax[j] = mx;
+    }
+    cl.sync();
+    for (int j = tid; j < w; j += kWinThreads) {
         float mx = 0.f;
-        for (int i = 0; i < w; i++) mx = fmaxf(mx, fabsf(Bh[i + j * kWinLD]));
+        for (int q = 0; q < kFactorCtas; q++) mx = fmaxf(mx, cl.map_shared_rank(cmax, q)[j]);
         int e = 0;
         frexpf(mx, &e);
         cexp[j] = e;
-        sZ[a + j] = ldexpf(1.f, e);
+        if (part == 0) sZ[a + j] = ldexpf(1.f, e);
     }
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < w * w; idx += kWinThreads) {
-        const int i = idx % w, j = idx / w;
+    cl.sync();   // also: no CTA leaves while another reads its maxima
+    for (int idx = tid; idx < 32 * w; idx += kWinThreads) {
+        const int i = idx & 31, j = idx >> 5;
+        if (row0 + i >= w) continue;
         float q[kSlices];
-        exact_slices<kSlices>(df_to_double(Bh[i + j * kWinLD], Bl[i + j * kWinLD]), cexp[j], kSlices, kBits, q);
+        exact_slices<kSlices>(df_to_double(Zh[i + j * kFactorLD], Zl[i + j * kFactorLD]), cexp[j], kSlices, kBits, q);
 #pragma unroll
         for (int sl = 0; sl < kSlices; sl++)
-            ZC[((size_t)sl * rp + a + j) * kp + a + i] = __float2bfloat16_rn(q[sl]);
+            ZC[((size_t)sl * rp + a + j) * kp + a + row0 + i] = __float2bfloat16_rn(q[sl]);
     }
 }
 
@@ -469,6 +564,14 @@ signtri_status reorder_blocked_run(int n, const double *T, int ldt, double *Tr, 
         SGT_CUDA_TRY(cudaMemsetAsync(ZC, 0, (size_t)kSlices * rp * kp * 2, st));
         const size_t smem = window_smem_bytes();
         SGT_CUDA_TRY(cudaFuncSetAttribute(window_sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        SGT_CUDA_TRY(cudaFuncSetAttribute(window_factor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)factor_smem_bytes()));
+        // the windows' rotation logs lie in T's column slices, which each
+        // sweep writes after its factors are formed (rp x kp >= 128 x 64, and
+        // a sweep has at most n / 128 + 2 windows)
+        size_t nw_max = 0;
+        for (const Sweep &p : plan) nw_max = std::max(nw_max, (size_t)p.nw);
+        if (nw_max * sizeof(WindowLog) > (size_t)kSlices * rp * kp * 2) return SIGNTRI_ERR_NO_WORKSPACE;
         const TcSource srcZ{ZC, kSlices, rp, kp, kp, sZ}, srcTc{TC, kSlices, rp, kp, kp, sTc};
         const TcSource srcTr{TR, kSlices, rp, kp, kp, sTr}, srcQ{QR, kSlices, rp, kp, kp, sQ};
         const TcQuadOut toT{{Tr, Tr, Tr, Tr}, ldtr, n, n, 0}, toQ{{Q, Q, Q, Q}, ldq, n, n, 0};
@@ -506,7 +609,12 @@ signtri_status reorder_blocked_run(int n, const double *T, int ldt, double *Tr, 
             SGT_CUDA_TRY(cudaMemsetAsync(mx, 0, 3 * (size_t)rp * sizeof(unsigned long long), st));
             {
                 ProfScope ps(SIGNTRI_KC_GIVENS, st);
-                window_sort_kernel<<<p.nw, kWinThreads, smem, st>>>(Tr, ldtr, d_wins + p.w0, ZC, sZ, rp, kp);
+                // the logs lie where T's column slices follow
+                auto *logs = reinterpret_cast<WindowLog *>(TC);
+                window_sort_kernel<<<p.nw, kWinThreads, smem, st>>>(Tr, ldtr, d_wins + p.w0, logs);
+                SGT_LAUNCH_CHECK();
+                window_factor_kernel<<<p.nw * kFactorCtas, kWinThreads, factor_smem_bytes(), st>>>(
+                    d_wins + p.w0, logs, ZC, sZ, rp, kp);
                 SGT_LAUNCH_CHECK();
             }
             // Q is read by its own product only: slice it alongside T's columns

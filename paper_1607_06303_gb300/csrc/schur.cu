@@ -47,6 +47,7 @@
 
 #include <cooperative_groups.h>
 
+#include "df_arith.cuh"
 #include "internal.cuh"
 
 namespace signtri {
@@ -521,28 +522,6 @@ constexpr int kCrossWarps = (kCross + 3) / 4;               // eight lanes per p
 enum { kActSweep = 0, kActStop = 2 };
 
 __device__ __forceinline__ double2 ldT(const double2 *p) { return __ldcg(p); }
-// the unbiased exponent field of |x| (integer operations only)
-__device__ __forceinline__ int exp_field(double x) { return ((__double2hiint(x) >> 20) & 0x7ff) - 1023; }
-
-// 1 / sqrt(a) for a normal a > 0: with a = 4^h m, m in [1, 4), a single-
-// precision reciprocal root r of m (relative error below 2^-20 with m's
-// mantissa cut to 23 bits) and one step of the third-order iteration
-// r (1 + e / 2 + 3 e^2 / 8), e = 1 - m r^2, from the binomial series of
-// (1 - e)^(-1/2): the series' next term is below 2^-60.  Five float64
-// instructions; the powers of two are moved by integer operations.
-__device__ __forceinline__ double rsqrt_normal(double a)
-{
-    const int hi = __double2hiint(a), lo = __double2loint(a);
-    const int h = ((hi >> 20) - 1023) >> 1;
-    const int mh = hi - (h << 21);
-    const float r0 = rsqrtf(__int_as_float((int)(((unsigned)(mh - (896 << 20)) << 3) | ((unsigned)lo >> 29))));
-    const unsigned rb = (unsigned)__float_as_int(r0);
-    const double m = __hiloint2double(mh, lo);
-    const double r = __hiloint2double((int)(rb >> 3) + (896 << 20), (int)(rb << 29));
-    const double e = fma(-(m * r), r, 1.0);
-    const double y = fma(fma(0.375, e, 0.5), r * e, r);
-    return __hiloint2double(__double2hiint(y) - (h << 20), __double2loint(y));
-}
 
 // make_rotation for a chief warp, lane-parallel.  v: in every lane the
 // operands of one product sum p q + u w, by lane & 3 of 0 |x|^2, 1 |y|^2,
