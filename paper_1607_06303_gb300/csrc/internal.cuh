@@ -253,4 +253,33 @@ size_t mixed_workspace_bytes(int n, int S);
 signtri_status mixed_run(int n, const double *T, int ldt, double *U, int ldu, int S, const MixedParams &prm,
                          MixedReport &rep, Arena &ws, int *d_err, double *norms_host, cudaStream_t st);
 
+// A second stream for the work of one call, and events to pass between it and
+// the caller's.  Destroyed on every return of that call, after the stream's
+// work has finished (the caller may reuse the workspace as soon as the call
+// returns).
+struct CallStream {
+    cudaStream_t s = nullptr;
+    cudaEvent_t ready[2] = {}, done[2] = {};
+    cudaError_t init()
+    {
+        cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+        for (int p = 0; p < 2 && e == cudaSuccess; p++) {
+            e = cudaEventCreateWithFlags(&ready[p], cudaEventDisableTiming);
+            if (e == cudaSuccess) e = cudaEventCreateWithFlags(&done[p], cudaEventDisableTiming);
+        }
+        return e;
+    }
+    ~CallStream()
+    {
+        if (s) {
+            cudaStreamSynchronize(s);
+            cudaStreamDestroy(s);
+        }
+        for (int p = 0; p < 2; p++) {
+            if (ready[p]) cudaEventDestroy(ready[p]);
+            if (done[p]) cudaEventDestroy(done[p]);
+        }
+    }
+};
+
 }  // namespace signtri

@@ -1236,34 +1236,6 @@ cudaError_t launch_qr(int cl, int n, double2 *T, int ldt, QrState *st, SweepRec 
                                          (long long)rotation_room(n), sweeplog, rclog, rslog, nlogged);
 }
 
-// The second stream of schur_run and its events.  Destroyed on every
-// return, after the stream's work has finished (the caller may reuse the
-// workspace the applies read and write as soon as schur_run returns).
-struct ApplyStream {
-    cudaStream_t s = nullptr;
-    cudaEvent_t swept[2] = {}, applied[2] = {};
-    cudaError_t init()
-    {
-        cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
-        for (int p = 0; p < 2 && e == cudaSuccess; p++) {
-            e = cudaEventCreateWithFlags(&swept[p], cudaEventDisableTiming);
-            if (e == cudaSuccess) e = cudaEventCreateWithFlags(&applied[p], cudaEventDisableTiming);
-        }
-        return e;
-    }
-    ~ApplyStream()
-    {
-        if (s) {
-            cudaStreamSynchronize(s);
-            cudaStreamDestroy(s);
-        }
-        for (int p = 0; p < 2; p++) {
-            if (swept[p]) cudaEventDestroy(swept[p]);
-            if (applied[p]) cudaEventDestroy(applied[p]);
-        }
-    }
-};
-
 }  // namespace
 
 size_t schur_workspace_bytes(int n)
@@ -1355,11 +1327,11 @@ signtri_status schur_run(int n, const double *A, int lda, double *Q, int ldq, do
     // launch m's log only after its apply.
     // Each launch's applies are issued after the next QR launch, so that the
     // cluster finds its SMs free (a QR CTA takes a whole SM's registers).
-    ApplyStream ap;
+    CallStream ap;
     SGT_CUDA_TRY(ap.init());
     // Q's reflectors on the second stream as well, while the sweeps begin
-    SGT_CUDA_TRY(cudaEventRecord(ap.swept[0], st));
-    SGT_CUDA_TRY(cudaStreamWaitEvent(ap.s, ap.swept[0], 0));
+    SGT_CUDA_TRY(cudaEventRecord(ap.ready[0], st));
+    SGT_CUDA_TRY(cudaStreamWaitEvent(ap.s, ap.ready[0], 0));
     auto form_q = [&]() -> signtri_status {
         const size_t smem = n <= kQRowsMax ? (size_t)kFormWarps * n * sizeof(double) : 0;
         SGT_CUDA_TRY(cudaFuncSetAttribute(form_q_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1371,14 +1343,14 @@ signtri_status schur_run(int n, const double *A, int lda, double *Q, int ldq, do
     };
     auto apply = [&](int p) -> signtri_status {
         const size_t lo = p * nlog;
-        SGT_CUDA_TRY(cudaStreamWaitEvent(ap.s, ap.swept[p], 0));
+        SGT_CUDA_TRY(cudaStreamWaitEvent(ap.s, ap.ready[p], 0));
         {
             ProfScope ps(SIGNTRI_KC_SCHUR, ap.s);
             apply_rotations_kernel<<<(int)((64LL * n + kThreads - 1) / kThreads), kThreads, 0, ap.s>>>(
                 n, Tc, ldt, Qc, ldq, nlogged + p, sweeplog + lo, rclog + lo, rslog + lo);
             SGT_LAUNCH_CHECK();
         }
-        SGT_CUDA_TRY(cudaEventRecord(ap.applied[p], ap.s));
+        SGT_CUDA_TRY(cudaEventRecord(ap.done[p], ap.s));
         return SIGNTRI_OK;
     };
     QrState h{};
@@ -1387,12 +1359,12 @@ signtri_status schur_run(int n, const double *A, int lda, double *Q, int ldq, do
         if (it >= max_launches) return SIGNTRI_ERR_NO_CONVERGENCE;
         const int p = (int)(it & 1);
         const size_t lo = p * nlog;
-        if (it >= 2) SGT_CUDA_TRY(cudaStreamWaitEvent(st, ap.applied[p], 0));
+        if (it >= 2) SGT_CUDA_TRY(cudaStreamWaitEvent(st, ap.done[p], 0));
         {
             ProfScope ps(SIGNTRI_KC_SCHUR, st);
             SGT_CUDA_TRY(launch_qr(cl, n, Tc, ldt, qs, sweeplog + lo, rclog + lo, rslog + lo, nlogged + p, st));
         }
-        SGT_CUDA_TRY(cudaEventRecord(ap.swept[p], st));
+        SGT_CUDA_TRY(cudaEventRecord(ap.ready[p], st));
         if (it == 0) {
             const signtri_status rq = form_q();
             if (rq != SIGNTRI_OK) return rq;
