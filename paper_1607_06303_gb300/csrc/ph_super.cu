@@ -51,6 +51,14 @@ constexpr int kNoExp = INT_MIN / 2;
 constexpr int kHeadroom = 2;
 constexpr int kMinExp = -900;     // keeps 2^(bits - exp) a normal number
 constexpr int kWideBits = 24;
+// Where a level's products are summed ahead, beside the wave before: in runs of
+// kAheadLevels levels with sums or more, beside waves of at most kAheadTiles
+// superblocks.  Wider waves fill the float64 pipes and lose by the company (a
+// batch of 300, hundreds of superblocks a level: 47.7 ms, with every level
+// ahead 49.6); limits of 24, 40 and 128 measured 36.6, 35.4 and 35.4 ms at
+// n = 8192.
+constexpr size_t kAheadTiles = 64;
+constexpr int kAheadLevels = 4;
 
 namespace {
 
@@ -291,9 +299,13 @@ __global__ void tiles_kernel(const Problem *__restrict__ probs, const Super *__r
     const Super t = list[i];
     const Problem &p = probs[t.k];
     rns::Tile *o = tiles + (size_t)products * i;
-    o[0] = {3 * t.k, t.A, t.B, p.triangular ? 2 * t.A : 0, 2 * t.B};
-    o[1] = {3 * t.k + 1, t.A, t.B, 2 * (t.A + 1), p.triangular ? 2 * (t.B + 1) : p.nkbr};
-    if (products == 3) o[2] = {3 * t.k + 2, t.A, t.B, 2 * (t.A + 1), 2 * t.B};
+    // of V, the level before this one solves the superblocks (A, B - 1) and
+    // (A + 1, B); the rest may be summed beside it
+    const int k0 = p.triangular ? 2 * t.A : 0, k1 = p.triangular ? 2 * (t.B + 1) : p.nkbr;
+    const int below = 2 * (t.A + 2), left = 2 * (t.B - 1);
+    o[0] = {3 * t.k, t.A, t.B, k0, 2 * t.B, k0, left};
+    o[1] = {3 * t.k + 1, t.A, t.B, 2 * (t.A + 1), k1, below, k1};
+    if (products == 3) o[2] = {3 * t.k + 2, t.A, t.B, 2 * (t.A + 1), 2 * t.B, below, left};
 }
 
 struct CrtConst {
@@ -600,8 +612,8 @@ int panels_of(int n) { return (n + SP - 1) / SP; }
 size_t run_bytes(size_t problems, size_t superblocks, size_t ops, size_t widest, int products)
 {
     return problems * (sizeof(Problem) + 3 * sizeof(rns::Source) + sizeof(int)) + (superblocks + ops) * sizeof(Super) +
-           superblocks * products * sizeof(rns::Tile) + widest * products * rns::kMods * SP * SP +
-           2 * wave_slab_bytes(widest) + 10 * 256;
+           superblocks * products * sizeof(rns::Tile) + 3 * widest * products * rns::kMods * SP * SP +
+           2 * wave_slab_bytes(widest) + 12 * 256;
 }
 // A problem's exponents, growth marks and forms.
 size_t problem_bytes(int nr, int nc, bool forms)
@@ -663,6 +675,8 @@ struct Run {
         auto *d_list = static_cast<Super *>(ws.take(all.size() * sizeof(Super)));
         auto *tiles = static_cast<rns::Tile *>(ws.take(list.size() * products * sizeof(rns::Tile)));
         auto *res = static_cast<int8_t *>(ws.take(widest * products * rns::kMods * SP * SP));
+        int8_t *ahead[2];
+        for (int8_t *&h : ahead) h = static_cast<int8_t *>(ws.take(widest * products * rns::kMods * SP * SP));
         auto *slab0 = static_cast<double *>(ws.take(wave_slab_bytes(widest)));
         auto *slab1 = static_cast<double *>(ws.take(wave_slab_bytes(widest)));
         if (!slab1) return SIGNTRI_ERR_NO_WORKSPACE;
@@ -670,9 +684,9 @@ struct Run {
         for (int k = 0; k < np; k++) {
             Problem &p = probs[k];
             p.flags = d_flags + k;
-            src[3 * k] = {p.vr, p.fn, p.nkbc, p.nkbc};
-            src[3 * k + 1] = {p.fm, p.vc, p.nkbr, p.nkbr};
-            src[3 * k + 2] = {p.vr, p.vc, p.nkbc, p.nkbr};
+            src[3 * k] = {p.vr, p.fn, p.nkbc, p.nkbc, p.rgrown, nullptr};
+            src[3 * k + 1] = {p.fm, p.vc, p.nkbr, p.nkbr, nullptr, p.cgrown};
+            src[3 * k + 2] = {p.vr, p.vc, p.nkbc, p.nkbr, p.rgrown, p.cgrown};
         }
         SGT_CUDA_TRY(cudaMemcpyAsync(d_probs, probs.data(), np * sizeof(Problem), cudaMemcpyHostToDevice, st));
         SGT_CUDA_TRY(cudaMemcpyAsync(d_src, src.data(), src.size() * sizeof(rns::Source), cudaMemcpyHostToDevice, st));
@@ -716,13 +730,35 @@ struct Run {
             SGT_LAUNCH_CHECK();
             if ((rs = join(l, diagonal.size(), 1)) != SIGNTRI_OK) return rs;
         }
+        // The products stream their operands from memory, the waves wait on
+        // float64 chains: so, beside a level's wave, the next level's products
+        // sum on a second stream what that wave does not change, and only the
+        // K-blocks of two superblocks are left between the waves (n = 8192:
+        // 38.6 -> 35.4 ms; Sylvester equation of a sorted diagonal 21.1 -> 18.5).
+        CallStream side;
+        bool summed_ahead = false;
+        const bool overlap = levels - sums_from >= kAheadLevels;
+        if (overlap) SGT_CUDA_TRY(side.init());
         for (int l = 0; l < levels; l++) {
             const size_t n = off[l + 1] - off[l];
             const Super *at = d_list + off[l];
             const bool with_sums = l >= sums_from;
             if (with_sums) {
-                rs = rns::gemm(d_src, tiles + products * off[l], (int)(products * n), products, res, d_err, cls_sums, st);
+                const bool have = summed_ahead;
+                summed_ahead = false;
+                if (have) SGT_CUDA_TRY(cudaStreamWaitEvent(st, side.done[l & 1], 0));
+                rs = rns::gemm(d_src, tiles + products * off[l], (int)(products * n), products, false,
+                               have ? ahead[l & 1] : nullptr, res, d_err, cls_sums, st);
                 if (rs != SIGNTRI_OK) return rs;
+            }
+            if (overlap && l + 1 < levels && l + 1 >= sums_from + 2 && n <= kAheadTiles) {
+                summed_ahead = true;
+                SGT_CUDA_TRY(cudaEventRecord(side.ready[l & 1], st));
+                SGT_CUDA_TRY(cudaStreamWaitEvent(side.s, side.ready[l & 1], 0));
+                rs = rns::gemm(d_src, tiles + products * off[l + 1], (int)(products * (off[l + 2] - off[l + 1])), products,
+                               true, ahead[(l + 1) & 1], nullptr, d_err, cls_sums, side.s);
+                if (rs != SIGNTRI_OK) return rs;
+                SGT_CUDA_TRY(cudaEventRecord(side.done[(l + 1) & 1], side.s));
             }
             // the steps that hold blocks: ragged panels have fewer rows or columns
             int nbr = 0, nbc = 0;

@@ -18,9 +18,9 @@
 //
 // rns_gemm_kernel: persistent CTAs; a task is one (tile, modulus).  Warp 0
 // loads K-blocks of 64 of both panels, 16 KB each, stored in the swizzled
-// layout so that a plain bulk copy brings them, into a ring of 6; one thread
+// layout so that a plain bulk copy brings them, into a ring of 4; one thread
 // of warp 1 issues M = N = 128 MMAs into 4 TMEM buffers, one per up to 15
-// K-blocks; 16 warps drain them, reduce modulo m and add.  Bound by the
+// K-blocks; 8 warps drain them, reduce modulo m and add.  Bound by the
 // operands' bytes (32 KB per K-block and 2 x 128^2 x 64 operations).
 #include <algorithm>
 
@@ -32,10 +32,14 @@ namespace rns {
 
 namespace {
 
-constexpr int kStages = 6;
+constexpr int kStages = 4;      // leaves shared memory for the kernels this one runs beside
 constexpr int kStageBytes = 32768;
-constexpr int kThreads = 576;
+constexpr int kThreads = 320;   // and at most 102 registers each: room for two CTAs of the waves beside it
 constexpr int kBufs = 4;
+// CTAs of an early launch, which runs beside another kernel: half the SMs keep
+// up with memory (n = 8192 in all: 152 CTAs 40.9 ms, 100 36.7, 84 36.2, 76 35.4,
+// 64 35.6, 48 40.0)
+constexpr int kEarlyCtas = 76;
 constexpr int kChunkKb = 15;    // 960 products of residues of at most 129: below 2^24
 constexpr int kSmemBytes = kStages * kStageBytes + 1024 + 256;
 
@@ -103,6 +107,23 @@ __device__ __forceinline__ void mbar_drain(uint64_t *bar, uint32_t parity)
     }
 }
 
+// The K-blocks of a task: n0 from a0 on, then the rest from a1 on.
+struct Span {
+    int a0, n0, a1, n;
+    bool ahead;   // the others are summed already
+    __device__ __forceinline__ int operator[](int i) const { return i < n0 ? a0 + i : a1 + i - n0; }
+};
+__device__ __forceinline__ Span span_of(const Tile &t, const Source &s, bool early, bool ahead)
+{
+    const int n = max(t.e1 - t.e0, 0);
+    if (early) return {t.e0, n, 0, n, false};
+    if (!ahead || n == 0 || (s.grownA && s.grownA[t.pa]) || (s.grownB && s.grownB[t.pb])) {
+        const int all = max(t.kb1 - t.kb0, 0);
+        return {t.kb0, all, 0, all, false};
+    }
+    return {t.kb0, t.e0 - t.kb0, t.e1, t.e0 - t.kb0 + t.kb1 - t.e1, true};
+}
+
 struct Task {
     int tile, mod;
 };
@@ -111,9 +132,9 @@ __device__ __forceinline__ Task task_of(int id, int per)
     return {id / (per * kMods) * per + id % per, id / per % kMods};
 }
 
-__global__ void __launch_bounds__(kThreads, 1)
-rns_gemm_kernel(const Source *__restrict__ src, const Tile *__restrict__ tiles, int ntasks, int per,
-                int8_t *__restrict__ out, int *__restrict__ err)
+__global__ void __launch_bounds__(kThreads, 2)
+rns_gemm_kernel(const Source *__restrict__ src, const Tile *__restrict__ tiles, int ntasks, int per, bool early,
+                const int8_t *__restrict__ ahead, int8_t *__restrict__ out, int *__restrict__ err)
 {
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -127,7 +148,7 @@ rns_gemm_kernel(const Source *__restrict__ src, const Tile *__restrict__ tiles, 
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; s++) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
-        for (int b = 0; b < kBufs; b++) { mbar_init(&tfull[b], 1); mbar_init(&tempty[b], 16); }
+        for (int b = 0; b < kBufs; b++) { mbar_init(&tfull[b], 1); mbar_init(&tempty[b], 8); }
         mbar_init(done_bar, 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -154,7 +175,9 @@ rns_gemm_kernel(const Source *__restrict__ src, const Tile *__restrict__ tiles, 
                 const Source s = src[t.src];
                 const __nv_bfloat16 *a = s.A + ((size_t)t.pa * kMods + k.mod) * s.nkbA * kTileElems;
                 const __nv_bfloat16 *b = s.B + ((size_t)t.pb * kMods + k.mod) * s.nkbB * kTileElems;
-                for (int kb = t.kb0; kb < t.kb1; kb++) {
+                const Span ks = span_of(t, s, early, ahead != nullptr);
+                for (int i = 0; i < ks.n; i++) {
+                    const int kb = ks[i];
                     if (!mbar_wait(&empty[stage], phase ^ 1, abort_flag)) { ok = false; break; }
                     unsigned char *base = smem + stage * kStageBytes;
                     mbar_expect_tx(&full[stage], kStageBytes);
@@ -182,12 +205,13 @@ rns_gemm_kernel(const Source *__restrict__ src, const Tile *__restrict__ tiles, 
             bool ok = true;
             for (int id = blockIdx.x; id < ntasks && ok; id += gridDim.x) {
                 const Tile t = tiles[task_of(id, per).tile];
-                for (int kc = t.kb0; kc < t.kb1 && ok; kc += kChunkKb, g++) {
+                const Span ks = span_of(t, src[t.src], early, ahead != nullptr);
+                for (int kc = 0; kc < ks.n && ok; kc += kChunkKb, g++) {
                     const int buf = g % kBufs;
                     if (!mbar_wait(&tempty[buf], (uint32_t)((g / kBufs) & 1) ^ 1, abort_flag)) { ok = false; break; }
                     fence_after();
                     const uint32_t d = tmem_base + (uint32_t)(buf * 128);
-                    const int ke = min(kc + kChunkKb, t.kb1);
+                    const int ke = min(kc + kChunkKb, ks.n);
                     for (int kb = kc; kb < ke; kb++) {
                         if (!mbar_wait(&full[stage], phase, abort_flag)) { ok = false; break; }
                         fence_after();
@@ -213,51 +237,65 @@ rns_gemm_kernel(const Source *__restrict__ src, const Tile *__restrict__ tiles, 
         }
     } else {
         const int q = warp & 3;                 // TMEM lane quadrant this warp may read
-        const int cg = (warp - 2) >> 2;         // 32-column group 0..3
-        const uint32_t lane_base = tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(cg * 32);
+        const int cg = (warp - 2) >> 2;         // 64-column group 0, 1
+        const uint32_t lane_base = tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(cg * 64);
         bool ok = true;
         int g = 0;
         for (int id = blockIdx.x; id < ntasks && ok; id += gridDim.x) {
             const Task k = task_of(id, per);
             const Tile t = tiles[k.tile];
             const float m = c_gemm.m[k.mod], rm = c_gemm.rm[k.mod], inv = c_gemm.inv[k.mod];
-            float acc[32];
+            const Span ks = span_of(t, src[t.src], early, ahead != nullptr);
+            if (early && ks.n == 0) continue;
+            const size_t at = (((size_t)k.tile * kMods + k.mod) * kPanel + 32 * q + lane) * kPanel + 64 * cg;
+            float acc[64];
+            if (ks.ahead) {
+                const char4 *h = reinterpret_cast<const char4 *>(ahead + at);
 #pragma unroll
-            for (int i = 0; i < 32; i++) acc[i] = 0.f;
-            for (int kc = t.kb0; kc < t.kb1 && ok; kc += kChunkKb, g++) {
+                for (int i = 0; i < 16; i++) {
+                    const char4 c = h[i];
+                    acc[4 * i] = (float)(signed char)c.x;
+                    acc[4 * i + 1] = (float)(signed char)c.y;
+                    acc[4 * i + 2] = (float)(signed char)c.z;
+                    acc[4 * i + 3] = (float)(signed char)c.w;
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < 64; i++) acc[i] = 0.f;
+            }
+            for (int kc = 0; kc < ks.n && ok; kc += kChunkKb, g++) {
                 const int buf = g % kBufs;
                 if (!mbar_wait(&tfull[buf], (uint32_t)((g / kBufs) & 1), abort_flag)) { ok = false; break; }
                 fence_after();
-                uint32_t r0[16], r1[16];
-                tmem_ld16_nowait(lane_base + (uint32_t)(buf * 128), r0);
-                tmem_ld16_nowait(lane_base + (uint32_t)(buf * 128) + 16, r1);
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                for (int cc = 0; cc < 64; cc += 16) {
+                    uint32_t r[16];
+                    tmem_ld16_nowait(lane_base + (uint32_t)(buf * 128 + cc), r);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                    for (int i = 0; i < 16; i++) acc[cc + i] += reduce(__uint_as_float(r[i]), m, rm);
+                }
                 fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&tempty[buf]);
-#pragma unroll
-                for (int i = 0; i < 16; i++) {
-                    acc[i] += reduce(__uint_as_float(r0[i]), m, rm);
-                    acc[16 + i] += reduce(__uint_as_float(r1[i]), m, rm);
-                }
             }
             if (!ok) break;
-            int4 v[2];
+            int4 v[4];
             int *w = reinterpret_cast<int *>(v);
 #pragma unroll
-            for (int i = 0; i < 32; i += 4) {
+            for (int i = 0; i < 64; i += 4) {
                 unsigned x = 0;
 #pragma unroll
                 for (int j = 0; j < 4; j++) {
-                    const float y = reduce(__fmul_rn(reduce(acc[i + j], m, rm), inv), m, rm);
+                    float y = reduce(acc[i + j], m, rm);
+                    if (!early) y = reduce(__fmul_rn(y, inv), m, rm);
                     x |= ((unsigned)(int)y & 0xffu) << (8 * j);
                 }
                 w[i / 4] = (int)x;
             }
-            int4 *o = reinterpret_cast<int4 *>(out + (((size_t)k.tile * kMods + k.mod) * kPanel + 32 * q + lane) * kPanel +
-                                               32 * cg);
-            o[0] = v[0];
-            o[1] = v[1];
+            int4 *o = reinterpret_cast<int4 *>(out + at);
+#pragma unroll
+            for (int i = 0; i < 4; i++) o[i] = v[i];
         }
         if (!ok) {
             *abort_flag = 1;
@@ -277,14 +315,15 @@ rns_gemm_kernel(const Source *__restrict__ src, const Tile *__restrict__ tiles, 
 
 }  // namespace
 
-signtri_status gemm(const Source *d_src, const Tile *d_tiles, int ntiles, int per, int8_t *out, int *d_err, int cls,
-                    cudaStream_t st)
+signtri_status gemm(const Source *d_src, const Tile *d_tiles, int ntiles, int per, bool early, int8_t *ahead,
+                    int8_t *out, int *d_err, int cls, cudaStream_t st)
 {
     if (ntiles <= 0) return SIGNTRI_OK;
     SGT_CUDA_TRY(cudaFuncSetAttribute(rns_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
     const int ntasks = ntiles * kMods;
     ProfScope ps(cls, st);
-    rns_gemm_kernel<<<std::min(ntasks, 152), kThreads, kSmemBytes, st>>>(d_src, d_tiles, ntasks, per, out, d_err);
+    rns_gemm_kernel<<<std::min(ntasks, early ? kEarlyCtas : 152), kThreads, kSmemBytes, st>>>(
+        d_src, d_tiles, ntasks, per, early, early ? nullptr : ahead, early ? ahead : out, d_err);
     SGT_LAUNCH_CHECK();
     return SIGNTRI_OK;
 }

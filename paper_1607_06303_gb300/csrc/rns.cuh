@@ -36,20 +36,25 @@ struct Form {
 inline size_t form_tile_bytes(int panels, int nkb) { return (size_t)panels * kMods * nkb * kTileElems * 2; }
 
 // One 128 x 128 product: panel pa of source number `src`'s A form times panel pb of
-// its B form over K-blocks [kb0, kb1).
+// its B form over K-blocks [kb0, kb1), of which [e0, e1) may be summed ahead.
 struct Tile {
-    int src, pa, pb, kb0, kb1;
+    int src, pa, pb, kb0, kb1, e0, e1;
 };
+// grownA[pa], grownB[pb] (where not null): the panel has been converted anew
+// since the K-blocks [e0, e1) were summed, so that sum is of no use.
 struct Source {
     const __nv_bfloat16 *A, *B;
     int nkbA, nkbB;
+    const int *grownA, *grownB;
 };
 
 // Residues of tiles [0, ntiles) of d_tiles, `per` consecutive tiles sharing
-// panels: out[tile][modulus][row][column], int8, already multiplied by the
-// modulus's cofactor inverse.
-signtri_status gemm(const Source *d_src, const Tile *d_tiles, int ntiles, int per, int8_t *out, int *d_err, int cls,
-                    cudaStream_t st);
+// panels, in [tile][modulus][row][column], int8.
+//   early: the K-blocks [e0, e1) alone, into `ahead`;
+//   else:  all K-blocks, the ones in `ahead` (where not null) from there,
+//          already multiplied by the modulus's cofactor inverse, into out.
+signtri_status gemm(const Source *d_src, const Tile *d_tiles, int ntiles, int per, bool early, int8_t *ahead,
+                    int8_t *out, int *d_err, int cls, cudaStream_t st);
 
 }  // namespace rns
 }  // namespace signtri

@@ -101,6 +101,20 @@ def test_superblocks_leave_graded_and_nonfinite_data_to_the_plain_path(gpu_lib):
         assert np.isnan(U[0, j]) == (s[0] != s[j])
 
 
+# rows and columns that outgrow their scales every few superblocks: the sums
+# formed ahead of a level are then of no use and formed anew.  An entry's error
+# is within a few 2^-53 of its row's and column's largest, at most 2^8 times
+# the entries of its size: the norm's tolerance holds 2^3 of these
+@pytest.mark.gpu
+def test_superblocks_that_outgrow_their_scales(gpu_lib):
+    n = 1800
+    T0 = make_T(n, 0.4, seed=6)
+    g = np.round(np.linspace(0.0, 8.0, n)).astype(int)
+    U = _super(gpu_lib, np.asfortranarray(np.ldexp(T0, g[None, :] - g[:, None])))
+    U0 = _plain(gpu_lib, T0)
+    assert np.linalg.norm(np.ldexp(U, g[:, None] - g[None, :]) - U0) <= n * np.finfo(float).eps * np.linalg.norm(U0)
+
+
 # Parlett-Sylvester on a grouped diagonal: X of T11 X - X T22 = 2 T12 by
 # superblocks, whole ones, ragged rows, ragged columns, a few columns only
 @pytest.mark.gpu
