@@ -507,13 +507,18 @@ __global__ void qr_state_init_kernel(int n, QrState *st)
 //    from the right.
 // One cluster barrier per step; no entry is written by one thread while
 // another reads it.  CTA 0 alone takes every decision (deflation, shifts,
-// stop) and broadcasts it, so all CTAs run the same barriers.  T is read with
-// L2-only loads (another CTA may have written it since).  The rotations'
+// stop) and broadcasts it, so all CTAs run the same barriers.  Where T fits in
+// the cluster's shared memory (kLocal, n up to 440 at 16 CTAs) its columns lie
+// there, column j in CTA j % CL, for the launch's time: a read takes ~440 cycles
+// instead of ~900 and the fence before a barrier ~500 instead of ~1,000.  Else T
+// is read with L2-only loads (another CTA may have written it since).  The rotations'
 // action on the columns right of the window (rows there are never read by a
 // later sweep: the window only shrinks) and on Q is left to
 // apply_rotations_kernel, which runs on other SMs alongside the next launch:
 // this kernel logs each sweep and its rotations instead (a rear sweep after
 // the one in front of it).
+inline size_t qr_smem(int n, int cl) { return (size_t)((n + cl - 1) / cl) * (n | 1) * sizeof(double2); }
+constexpr size_t kQrSmemMax = 200 * 1024;
 constexpr int kMaxBulges = 8;
 constexpr int kChiefs = 4;   // chief warps (and as many helpers) of a chief CTA
 constexpr int kChiefCtas = (kMaxBulges + kChiefs - 1) / kChiefs;
@@ -521,7 +526,6 @@ constexpr int kCross = kMaxBulges * (kMaxBulges - 1) / 2;   // pairs of bulges
 constexpr int kCrossWarps = (kCross + 3) / 4;               // eight lanes per pair
 enum { kActSweep = 0, kActStop = 2 };
 
-__device__ __forceinline__ double2 ldT(const double2 *p) { return __ldcg(p); }
 
 // make_rotation for a chief warp, lane-parallel.  v: in every lane the
 // operands of one product sum p q + u w, by lane & 3 of 0 |x|^2, 1 |y|^2,
@@ -698,7 +702,7 @@ __device__ __forceinline__ void step_barrier(bool wrote)
     asm volatile("barrier.cluster.arrive.relaxed.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-template <int CL>
+template <int CL, bool kLocal>
 __global__ void __launch_bounds__(kQrThreads)
 schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ st, long long budget, long long room,
                 SweepRec *__restrict__ sweeplog, double *__restrict__ rclog, double2 *__restrict__ rslog,
@@ -708,6 +712,7 @@ schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ s
     constexpr int kWorkers = CL - kChiefCtas, kWarps = kQrThreads / 32, kWorkerWarps = kWorkers * kWarps;
     static_assert(kWorkers > 0 && kWarps >= 2 * kChiefs && kWorkerWarps >= kCrossWarps + kMaxBulges, "roles");
     cg::cluster_group cl = cg::this_cluster();
+    extern __shared__ double2 tsm[];                      // kLocal: columns crank, crank + CL, .. of T
     __shared__ int redi[kWarps];
     __shared__ double rc[kMaxBulges][2];
     __shared__ double2 rs[kMaxBulges][2];
@@ -738,6 +743,22 @@ schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ s
         }
     }
     int i = st->ihi, its = st->its, status = st->status;
+    const int lds = n | 1, ihi = i;
+    auto entry = [&](int r, int c) -> double2 * {
+        if constexpr (kLocal) return cl.map_shared_rank(tsm, c % CL) + (c / CL) * lds + r;
+        else return &SGT_A(T, ldt, r, c);
+    };
+    auto ld = [&](const double2 *q) -> double2 {
+        if constexpr (kLocal) return *q;
+        else return __ldcg(q);
+    };
+    if constexpr (kLocal) {
+        // the columns up to the window's last one: those right of it may be at
+        // work in apply_rotations_kernel
+        for (int c = crank; c <= ihi; c += CL)
+            for (int r = tid; r < n; r += kQrThreads) tsm[(c / CL) * lds + r] = SGT_A(T, ldt, r, c);
+        cl.sync();
+    }
     long long logged = 0, rot = 0;
     const double eps = DBL_EPSILON;
     const double tiny = DBL_MIN * ((double)n / DBL_EPSILON);
@@ -763,12 +784,12 @@ schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ s
     };
     // a chase's first block and rotation, at (l, l) with the shift sg
     auto start_chase = [&](int b, int slot, int l, int last, double2 sg) {
-        const double2 top = ldT(&SGT_A(T, ldt, l, l + (col1 ? 1 : 0)));
-        const double2 bot = ldT(&SGT_A(T, ldt, l + 1, l + (col1 ? 1 : 0)));
-        const double2 A = ldT(&SGT_A(T, ldt, l, l)), E = ldT(&SGT_A(T, ldt, l + 1, l));
+        const double2 top = ld(entry(l, l + (col1 ? 1 : 0)));
+        const double2 bot = ld(entry(l + 1, l + (col1 ? 1 : 0)));
+        const double2 A = ld(entry(l, l)), E = ld(entry(l + 1, l));
         if (b == 0) {
-            const double2 H = (l + 2 <= last) ? ldT(&SGT_A(T, ldt, l + 2, l + 1)) : zero;
-            const double2 F = (l + 2 <= last) ? ldT(&SGT_A(T, ldt, l + 2, l + 2)) : zero;
+            const double2 H = (l + 2 <= last) ? ld(entry(l + 2, l + 1)) : zero;
+            const double2 F = (l + 2 <= last) ? ld(entry(l + 2, l + 2)) : zero;
             if (lane == 0) handF[0][3] = F;
             ho = odd ? H.y : H.x;
             he = odd ? H.x : H.y;
@@ -791,8 +812,8 @@ schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ s
                 // l: the largest k in [1, i] whose h_{k,k-1} is negligible, else 0
                 int lk = 0;
                 for (int k = 1 + tid; k <= i; k += kQrThreads) {
-                    const double sub = cabs1(ldT(&SGT_A(T, ldt, k, k - 1)));
-                    const double ref = cabs1(ldT(&SGT_A(T, ldt, k - 1, k - 1))) + cabs1(ldT(&SGT_A(T, ldt, k, k)));
+                    const double sub = cabs1(ld(entry(k, k - 1)));
+                    const double ref = cabs1(ld(entry(k - 1, k - 1))) + cabs1(ld(entry(k, k)));
                     if (sub <= fmax(eps * ref, tiny)) lk = k;
                 }
                 lk = __reduce_max_sync(0xffffffffu, lk);
@@ -802,7 +823,7 @@ schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ s
                 __syncthreads();
                 if (status != 0 || i <= 0 || l < i) break;
                 // the window's last row has converged
-                if (tid == 0) SGT_A(T, ldt, i, i - 1) = zero;
+                if (tid == 0) *entry(i, i - 1) = zero;
                 i--;
                 its = 0;
             }
@@ -820,7 +841,7 @@ schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ s
                     act = kActStop;
                     status = 2;
                 } else {
-                    if (l > 0 && lane == 0) SGT_A(T, ldt, l, l - 1) = zero;
+                    if (l > 0 && lane == 0) *entry(l, l - 1) = zero;
                     const int sw_its = its + 1;
                     double2 sigma;
                     if (sw_its % 10 == 0) {
@@ -828,8 +849,8 @@ schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ s
                         // (sweeps 10, 30, ..) or bottom corner (20, 40, ..)
                         // by 3/4 of a subdiagonal entry's real part
                         const bool top = (sw_its / 10) % 2 == 1;
-                        const double2 d = top ? ldT(&SGT_A(T, ldt, l, l)) : ldT(&SGT_A(T, ldt, i, i));
-                        const double e = top ? ldT(&SGT_A(T, ldt, l + 1, l)).x : ldT(&SGT_A(T, ldt, i, i - 1)).x;
+                        const double2 d = top ? ld(entry(l, l)) : ld(entry(i, i));
+                        const double e = top ? ld(entry(l + 1, l)).x : ld(entry(i, i - 1)).x;
                         sigma = make_double2(d.x + 0.75 * fabs(e), d.y);
                     } else {
                         // a bulge per three rows; two where the log has no
@@ -838,8 +859,8 @@ schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ s
                         if ((long long)nbul * (i - l) > room) nbul = min(nbul, 2);
                         if (nbul <= 2) {
                             double2 other;
-                            wilkinson(ldT(&SGT_A(T, ldt, i - 1, i - 1)), ldT(&SGT_A(T, ldt, i - 1, i)),
-                                      ldT(&SGT_A(T, ldt, i, i - 1)), ldT(&SGT_A(T, ldt, i, i)), sigma, other);
+                            wilkinson(ld(entry(i - 1, i - 1)), ld(entry(i - 1, i)),
+                                      ld(entry(i, i - 1)), ld(entry(i, i)), sigma, other);
                             if (lane < kChiefCtas) *cl.map_shared_rank(&sig[1], lane) = other;
                         } else {
                             const int r0 = i - nbul + 1;
@@ -847,14 +868,14 @@ schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ s
                             for (int t = lane; t < nbul * nbul; t += 32) {
                                 const int r = t % nbul, q = t / nbul;
                                 if (r > q + 1) continue;
-                                const double2 v = ldT(&SGT_A(T, ldt, r0 + r, r0 + q));
+                                const double2 v = ld(entry(r0 + r, r0 + q));
                                 em = max(em, max(exp_field(v.x), exp_field(v.y)));
                             }
                             em = min(__reduce_max_sync(0xffffffffu, em), 1000);
                             const double sc = __hiloint2double((1023 - em) << 20, 0);
                             for (int t = lane; t < nbul * nbul; t += 32) {
                                 const int r = t % nbul, q = t / nbul;
-                                const double2 v = r > q + 1 ? zero : ldT(&SGT_A(T, ldt, r0 + r, r0 + q));
+                                const double2 v = r > q + 1 ? zero : ld(entry(r0 + r, r0 + q));
                                 blk[r][q] = make_float2((float)(v.x * sc), (float)(v.y * sc));
                             }
                             __syncwarp();
@@ -908,10 +929,10 @@ schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ s
                             const int d = 2 + (q << 5) + lane, j = k + d, t = d / 3;
                             const bool cross = d >= 3 && t <= wb && d - 3 * t < 2 && s < L + 3 * (wb - t);
                             if (j <= i && !cross) {
-                                double2 a = ldT(&SGT_A(T, ldt, k, j)), b = ldT(&SGT_A(T, ldt, k + 1, j));
+                                double2 a = ld(entry(k, j)), b = ld(entry(k + 1, j));
                                 rot_rows(c0, s0, a, b);
-                                SGT_A(T, ldt, k, j) = a;
-                                SGT_A(T, ldt, k + 1, j) = b;
+                                *entry(k, j) = a;
+                                *entry(k + 1, j) = b;
                                 if (d == 2) *cl.map_shared_rank(&bslot[wb][(s + 1) & 1], wb / kChiefs) = b;
                             }
                         } else {
@@ -920,10 +941,10 @@ schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ s
                             const int r = ((q - rw) << 5) + lane, g = k - r + 1, t = g / 3;
                             const bool cross = t >= 1 && t <= nbul - 1 - wb && g - 3 * t < 2 && k - 3 * t >= l;
                             if (r < k && !cross) {
-                                double2 a = ldT(&SGT_A(T, ldt, r, k)), b = ldT(&SGT_A(T, ldt, r, k + 1));
+                                double2 a = ld(entry(r, k)), b = ld(entry(r, k + 1));
                                 rot_cols(c0, s0, a, b);
-                                SGT_A(T, ldt, r, k) = a;
-                                SGT_A(T, ldt, r, k + 1) = b;
+                                *entry(r, k) = a;
+                                *entry(r, k + 1) = b;
                             }
                         }
                     }
@@ -939,8 +960,8 @@ schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ s
                     double2 a = zero, b = zero, sr = zero, sc = zero;
                     double cr = 1.0, cc = 1.0;
                     if (on) {
-                        a = ldT(&SGT_A(T, ldt, k1, k0 + f));
-                        b = ldT(&SGT_A(T, ldt, k1 + 1, k0 + f));
+                        a = ld(entry(k1, k0 + f));
+                        b = ld(entry(k1 + 1, k0 + f));
                         cr = rc[pb][s & 1];
                         sr = rs[pb][s & 1];
                         cc = rc[pa][s & 1];
@@ -955,7 +976,7 @@ schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ s
                     const double g2 = __shfl_sync(0xffffffffu, r1, at), e2 = __shfl_sync(0xffffffffu, r1, at ^ 1);
                     const double a2 = __shfl_sync(0xffffffffu, r1, at ^ 4);
                     const double r2 = pair_part(cc, a2, hi ? -sc.x : sc.x, g2, odd ? -sc.y : sc.y, e2);
-                    if (on) as_double(&SGT_A(T, ldt, k1 + f, k0 + (part >> 1)))[part & 1] = r2;
+                    if (on) as_double(entry(k1 + f, k0 + (part >> 1)))[part & 1] = r2;
                 }
             } else if (chief && my < nbul) {
                 const int b = my, kb = l + s - 3 * b;
@@ -994,7 +1015,7 @@ schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ s
                         if (part == 3) u = -u;
                         // what r2 holds already goes out before the rotation is
                         // formed, so that the barrier does not wait for it
-                        if (lane < 12) as_double(&SGT_A(T, ldt, kb + (lane >> 2), kb + (part >> 1)))[part & 1] = r2;
+                        if (lane < 12) as_double(entry(kb + (lane >> 2), kb + (part >> 1)))[part & 1] = r2;
                         if (lane == 4 || lane == 5 || lane == 8 || lane == 9)
                             inp[b][(s + 1) & 1][(lane & 1) | (lane >> 2 & 2)] = r2;
                         // the block's corner h_kk, for the bulge behind
@@ -1008,7 +1029,7 @@ schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ s
                         ga = __shfl_sync(0xffffffffu, r2, (hi ? 6 : 10) + po);
                         ep = __shfl_sync(0xffffffffu, r2, (hi ? 6 : 10) + pe);
                     } else {
-                        if (lane < 8) as_double(&SGT_A(T, ldt, kb + (lane >> 2), kb + (part >> 1)))[part & 1] = r2;
+                        if (lane < 8) as_double(entry(kb + (lane >> 2), kb + (part >> 1)))[part & 1] = r2;
                         if (lane < 2 && b + 1 < nbul)
                             as_double(cl.map_shared_rank(&handF[b + 1][s & 3], (b + 1) / kChiefs))[lane] = r2;
                     }
@@ -1030,7 +1051,7 @@ schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ s
                         const double *xy = inp[b][s & 1];
                         const double rz = pair_part(c, odd ? xy[1] : xy[0], sn.x, odd ? xy[3] : xy[2],
                                                     odd ? sn.y : -sn.y, odd ? xy[2] : xy[3]);
-                        reinterpret_cast<double *>(&SGT_A(T, ldt, kb + (hi ? 1 : 0), kb - 1))[odd ? 1 : 0] =
+                        reinterpret_cast<double *>(entry(kb + (hi ? 1 : 0), kb - 1))[odd ? 1 : 0] =
                             hi ? 0.0 : rz;
                         if (lane < 2 && b + 1 < nbul)
                             as_double(cl.map_shared_rank(&handH[b + 1][s & 1], (b + 1) / kChiefs))[lane] = rz;
@@ -1039,9 +1060,9 @@ schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ s
                         // the front chase, or the one in front has ended (its
                         // last entries, a step old)
                         if (lane == 4)
-                            handF[b][s & 3] = ldT(&SGT_A(T, ldt, kb + 3, kb + 3));
+                            handF[b][s & 3] = ld(entry(kb + 3, kb + 3));
                         else
-                            handH[b][s & 1] = ldT(&SGT_A(T, ldt, kb + 3, kb + 2));
+                            handH[b][s & 1] = ld(entry(kb + 3, kb + 2));
                     }
                 }
             }
@@ -1067,6 +1088,10 @@ schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ s
         }
         rot += (long long)nbul * L;
         logged += nbul;
+    }
+    if constexpr (kLocal) {   // every CTA's stores are in: the barrier of the decision to stop
+        for (int c = crank; c <= ihi; c += CL)
+            for (int r = tid; r < n; r += kQrThreads) SGT_A(T, ldt, r, c) = tsm[(c / CL) * lds + r];
     }
     if (chief0 && lane == 0) {
         st->ihi = i;
@@ -1208,7 +1233,8 @@ bool places_16(const void *kernel, int threads, size_t smem)
 
 int cluster_size()
 {
-    return places_16((const void *)schur_qr_kernel<16>, kQrThreads, 0) &&
+    return places_16((const void *)schur_qr_kernel<16, false>, kQrThreads, 0) &&
+                   places_16((const void *)schur_qr_kernel<16, true>, kQrThreads, kQrSmemMax) &&
                    places_16((const void *)hess_cluster_kernel<16>, kHessThreads, kHessSmemMax)
                ? 16
                : 8;
@@ -1228,12 +1254,19 @@ cudaError_t launch_hess(int cl, int n, const double *A, int lda, double2 *T, int
 cudaError_t launch_qr(int cl, int n, double2 *T, int ldt, QrState *st, SweepRec *sweeplog, double *rclog, double2 *rslog,
                       int *nlogged, cudaStream_t stream)
 {
+    const size_t smem = qr_smem(n, cl);
+    const bool local = smem <= kQrSmemMax;
     cudaLaunchAttribute at[1];
-    const cudaLaunchConfig_t cfg = cluster_config(cl, kQrThreads, 0, stream, at);
-    return cl == 16 ? cudaLaunchKernelEx(&cfg, schur_qr_kernel<16>, n, T, ldt, st, kRotationBudget,
-                                         (long long)rotation_room(n), sweeplog, rclog, rslog, nlogged)
-                    : cudaLaunchKernelEx(&cfg, schur_qr_kernel<8>, n, T, ldt, st, kRotationBudget,
-                                         (long long)rotation_room(n), sweeplog, rclog, rslog, nlogged);
+    const cudaLaunchConfig_t cfg = cluster_config(cl, kQrThreads, local ? smem : 0, stream, at);
+    auto go = [&](auto *kernel) {
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)cfg.dynamicSmemBytes);
+        return e != cudaSuccess ? e
+                                : cudaLaunchKernelEx(&cfg, kernel, n, T, ldt, st, kRotationBudget,
+                                                     (long long)rotation_room(n), sweeplog, rclog, rslog, nlogged);
+    };
+    if (cl == 16) return local ? go(schur_qr_kernel<16, true>) : go(schur_qr_kernel<16, false>);
+    return local ? go(schur_qr_kernel<8, true>) : go(schur_qr_kernel<8, false>);
 }
 
 }  // namespace
