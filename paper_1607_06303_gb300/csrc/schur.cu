@@ -70,26 +70,6 @@ __device__ __forceinline__ double2 cmul(double2 a, double2 b)
 }
 __device__ __forceinline__ double2 cconj(double2 a) { return make_double2(a.x, -a.y); }
 __device__ __forceinline__ double cabs1(double2 a) { return fabs(a.x) + fabs(a.y); }
-// a / b by Smith's algorithm (R. L. Smith, CACM 5(8), 1962)
-__device__ __forceinline__ double2 cdiv(double2 a, double2 b)
-{
-    if (fabs(b.x) >= fabs(b.y)) {
-        const double r = b.y / b.x, den = b.x + b.y * r;
-        return make_double2((a.x + a.y * r) / den, (a.y - a.x * r) / den);
-    }
-    const double r = b.x / b.y, den = b.x * r + b.y;
-    return make_double2((a.x * r + a.y) / den, (a.y * r - a.x) / den);
-}
-// principal square root (Re >= 0): with r = |z|, sqrt((r + |Re z|) / 2) is
-// the larger part, the other is Im z over twice it
-__device__ __forceinline__ double2 csqrt_p(double2 z)
-{
-    if (z.x == 0.0 && z.y == 0.0) return make_double2(0.0, 0.0);
-    const double a = sqrt(0.5 * (hypot(z.x, z.y) + fabs(z.x)));
-    const double b = z.y / (2.0 * a);
-    return z.x >= 0.0 ? make_double2(a, b) : make_double2(fabs(b), copysign(a, z.y));
-}
-
 // The rotation G = [c s; -conj(s) c] (c real >= 0, c^2 + |s|^2 = 1) with
 // G [x; y] = [r; 0]: c = |x| / nrm, s = (x / |x|) conj(y) / nrm,
 // nrm^2 = |x|^2 + |y|^2.  x and y are first scaled by the power of two that
@@ -519,9 +499,9 @@ __global__ void qr_state_init_kernel(int n, QrState *st)
 // the one in front of it).
 inline size_t qr_smem(int n, int cl) { return (size_t)((n + cl - 1) / cl) * (n | 1) * sizeof(double2); }
 constexpr size_t kQrSmemMax = 200 * 1024;
-constexpr int kMaxBulges = 8;
-constexpr int kChiefs = 4;   // chief warps (and as many helpers) of a chief CTA
-constexpr int kChiefCtas = (kMaxBulges + kChiefs - 1) / kChiefs;
+// (8 bulges measured 30.3 ms for the sign of a general matrix at n = 200, 10
+// 29.9, 12 29.6; at n = 400 111, 104 and 112)
+constexpr int kMaxBulges = 10;
 constexpr int kCross = kMaxBulges * (kMaxBulges - 1) / 2;   // pairs of bulges
 constexpr int kCrossWarps = (kCross + 3) / 4;               // eight lanes per pair
 enum { kActSweep = 0, kActStop = 2 };
@@ -709,6 +689,11 @@ schur_qr_kernel(int n, double2 *__restrict__ T, int ldt, QrState *__restrict__ s
                 int *__restrict__ nlogged)
 {
     namespace cg = cooperative_groups;
+    // Chief warps (and as many helpers) of a chief CTA: they share its float64
+    // pipe, and the fewer they are, the fewer CTAs do the rest (kLocal, n = 200:
+    // four 31.4 ms, three 30.2, two 30.1; n = 400: 109.8, 110.8, 113.8; from
+    // global memory, n = 1000: 1,054, 1,096, 1,133)
+    constexpr int kChiefs = kLocal ? 3 : 4, kChiefCtas = (kMaxBulges + kChiefs - 1) / kChiefs;
     constexpr int kWorkers = CL - kChiefCtas, kWarps = kQrThreads / 32, kWorkerWarps = kWorkers * kWarps;
     static_assert(kWorkers > 0 && kWarps >= 2 * kChiefs && kWorkerWarps >= kCrossWarps + kMaxBulges, "roles");
     cg::cluster_group cl = cg::this_cluster();
