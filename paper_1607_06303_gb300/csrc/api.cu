@@ -200,27 +200,33 @@ void work_estimates(int n, const ScanResult &r, double *w_ph, double *w_ps)
     *w_ps = w;
 }
 
-// Times predicted from the Section 3 work of what each variant executes,
-// plus the latency-bound parts, with constants measured on GB300 (float64
-// leaves and the windowed reorder, whose cost is not in the flop counts):
-//  * Parlett-Higham runs the arithmetic-efficient form (Section 5.3: only the
-//    sum each entry needs, exactly the useful count w_ph) at the float64
-//    product rate, and one off-diagonal leaf step per block column (about
-//    0.06, 0.21, 0.7 ms at b = 16, 32, 64);
-//  * Parlett-Sylvester runs the Sylvester block sums (n_- n_+ n flops, in
-//    double-float at about 4e12 flop/s) and one in-block step per block
-//    anti-diagonal (about 0.29 ms); when k > 0,
-//    the reorder and the back-transform (emulated-float64 tensor-core
-//    products, about 6e13 float64 flop/s).  The windowed reorder (n >= 512)
-//    runs sweeps of windows of 128 at offsets 0 / 64: a negative moves at
-//    most 64 places a sweep, so there are about d / 64 sweeps, d = n_+ -
-//    (index of the first negative) the longest distance one travels.  A
-//    sweep costs its window launch (rounds and float64 rotations, growing
-//    with the swaps per window, about 0.1 ms with a few and 0.5 ms with
-//    ~770), plus the products and slicing of its about min(n_-, n / 256)
-//    active windows, each about 0.7e-8 n seconds.  The
-//    unblocked rounds (n < 512) cost 12 n k flops at the Givens rate and two
-//    launches per round.
+// Times predicted from what each variant runs, with constants measured on
+// GB300.  A grouped diagonal (k = 0 swaps) with leaves of 16:
+//  * Parlett-Higham: a launch of 13 us per block column of 16 beside the useful
+//    count at the float64 rate (n = 700: 0.56 ms, 1200: 1.67); by superblocks
+//    (n >= kSuperMin) per level of 128 0.2 ms of dependent steps and 44 ns a
+//    column of products (n = 2000: 4.1 ms, 4096: 10.8, 8192: 33);
+//  * Parlett-Sylvester: 0.2 ms per anti-diagonal of 128 x 128 superblocks and
+//    n_- n_+ n flops of products at 2e13 a second (n = 700: 0.9 to 1.0 ms,
+//    2000: 3.0 to 3.2, 8192: 15.0 with 0.1 n negatives and 20.1 with 0.5 n).
+// The two meet near n = 1200.  Otherwise the estimates of both by their plain
+// forms, which with a few negatives at large n favour Parlett-Sylvester beyond
+// what the two measure now (n = 8192, three negatives: 41.4 ms against 34.7):
+//  * Parlett-Higham: the useful count w_ph at the float64 product rate, and one
+//    off-diagonal leaf step per block column (0.06, 0.21, 0.7 ms at b = 16, 32,
+//    64);
+//  * Parlett-Sylvester: the Sylvester sums at about 4e12 flop/s and an in-block
+//    step per block anti-diagonal of 64 (0.29 ms), the reorder and the
+//    back-transform (emulated-float64 tensor-core products, about 6e13 float64
+//    flop/s).  The windowed reorder (n >= 512) runs sweeps of windows of 128 at
+//    offsets 0 / 64: a negative moves at most 64 places a sweep, so there are
+//    about d / 64 sweeps, d = n_+ - (index of the first negative) the longest
+//    distance one travels.  A sweep costs its window launch (rounds and
+//    rotations, growing with the swaps per window, 0.1 ms with a few and 0.2
+//    to 0.5 ms with ~770), plus the products and slicing of its about min(n_-,
+//    n / 256) active windows, each about 0.7e-8 n seconds.  The unblocked
+//    rounds (n < 512) cost 12 n k flops at the Givens rate and two launches per
+//    round.
 constexpr double kLaunchSeconds = 5e-6;
 double ph_leaf_step_seconds(int b)
 {
@@ -245,6 +251,11 @@ signtri_variant choose_variant(int n, const ScanResult &r)
     work_estimates(n, r, &w_ph, &w_ps);
     const double t_ph = w_ph / g_rate_gemm + nb * ph_leaf_step_seconds(b) + 2.0 * nb * kLaunchSeconds;
     const double np = r.n_pos, nm = r.n_neg, k = (double)r.swaps;
+    if (r.swaps == 0 && b == 16) {
+        const double ph = n >= kSuperMin ? nd / 128.0 * (0.2e-3 + 44e-9 * nd) : w_ph / g_rate_gemm + nb * 13e-6;
+        const double ps = (std::ceil(np / 128.0) + std::ceil(nm / 128.0) - 1.0) * 0.2e-3 + np * nm * nd / 2e13;
+        return ps < ph ? SIGNTRI_PS_FP64 : SIGNTRI_PH_FP64_EFFICIENT;
+    }
     const double sylv_steps = std::ceil(np / 64.0) + std::ceil(nm / 64.0) - 1.0;
     double t_ps = np * nm * nd / kSylvRate + sylv_steps * kSylvStepSeconds;
     if (r.swaps > 0) {
