@@ -269,6 +269,9 @@ __device__ __forceinline__ void far_sums(int n, const S *__restrict__ T, int ldt
     if (half == 0) slab[p + q * LB] = add(acc, part[p + q * LB]);
 }
 
+// Whether a and b, +-1 each, differ, without the float64 pipe.
+__device__ __forceinline__ bool signs_differ(double a, double b) { return (__double2hiint(a) ^ __double2hiint(b)) < 0; }
+
 // Entry number t of a block along its anti-diagonals step = 15 - p + q, from
 // the bottom-left corner.
 __device__ __forceinline__ void entry_of(int t, int &p, int &q)
@@ -354,13 +357,18 @@ __device__ __forceinline__ void leaf(int n, const S *__restrict__ T, int ldt, S 
     const int step = LB - 1 - p + q;
     half_sync(0);
     const S upp = s.urow[p], uqq = s.ucol[q];
-    const bool opp = general || re(upp) + re(uqq) == 0.0;
+    const bool opp = general || signs_differ(re(upp), re(uqq));
     // signs agree: 1 / (u_pp + u_qq) is +-1/2 exactly
     const S rinv = opp ? inv_diff(s.TI[p + p * LD], s.TJ[q + q * LD]) : scaled(upp, 0.5);
     // flips the sign of the row terms where the signs agree
     const unsigned long long flip = opp ? 0ull : 0x8000000000000000ull;
     const S *M = opp ? s.TI : s.UI, *N = opp ? s.TJ : s.UJ;
     const S *M1 = opp ? s.T1 : s.U1, *N2 = opp ? s.T2 : s.U2;
+
+    // the entry's own term (u_ii and u_jj are real)
+    const double ui = re(s.urow[lo]), uj = re(s.ucol[hi]);
+    const bool o = general || signs_differ(ui, uj);
+    s.V[at] = o ? scaled(tij, ui - uj) : zero;
 
     dependency_wait();
     dependency_release();
@@ -395,11 +403,7 @@ __device__ __forceinline__ void leaf(int n, const S *__restrict__ T, int ldt, S 
         s.U1[at] = u1;
         s.U2[at] = u2;
     }
-    // (u_ii and u_jj are real)
-    const double ui = re(s.urow[lo]), uj = re(s.ucol[hi]);
-    const bool o = general || ui + uj == 0.0;
     s.C[at] = o ? sum : flip_sign(sum, 0x8000000000000000ull);
-    s.V[at] = o ? scaled(tij, ui - uj) : zero;
     half_sync(0);
     S acc = s.C[p + q * LD];
     const S base = s.V[p + q * LD];

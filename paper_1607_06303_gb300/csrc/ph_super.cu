@@ -70,7 +70,7 @@ struct Problem {
     double *V;
     int ldrt, ldru, ldct, ldcu, ldc0, ldv;
     int rows, cols;
-    double own;                                 // an entry's own term is own (u_pp - u_qq) C0
+    double own2;                                // an entry's own term is own2 (u_pp - u_qq) / 2 C0
     int bits;
     bool triangular;                            // V strictly upper, rows and columns the same
     int *er0, *ec0, *er1, *ec1;                 // exponents: V's rows, CT's columns, RT's rows, V's columns
@@ -111,6 +111,16 @@ __device__ __forceinline__ Mat matrix_of(const Problem &p, int what)
     if (what == kRowOps) return {p.RT, p.ldrt, p.rows, p.rows, true};
     if (what == kColOps) return {p.CT, p.ldct, p.cols, p.cols, true};
     return {p.V, p.ldv, p.rows, p.cols, p.triangular};
+}
+
+// Every exponent of a problem below any that an entry has (a CTA per problem: six
+// memsets each took 1.7 ms of a batch with 100 of them).
+__global__ void __launch_bounds__(kThreads)
+init_exps_kernel(const Problem *__restrict__ probs)
+{
+    const Problem p = probs[blockIdx.x];
+    for (int i = threadIdx.x; i < p.nkbr / 2 * SP; i += kThreads) p.er0[i] = p.er1[i] = p.rnew[i] = kNoExp;
+    for (int i = threadIdx.x; i < p.nkbc / 2 * SP; i += kThreads) p.ec0[i] = p.ec1[i] = p.cnew[i] = kNoExp;
 }
 
 // The largest exponents of the superblocks' rows (kRowOps), columns (kColOps)
@@ -332,8 +342,13 @@ constexpr CrtConst make_crt_const()
 }
 __constant__ CrtConst c_crt = make_crt_const();
 
-// The product an entry's residues stand for (16 bytes, 16 KB apart).
-__device__ __forceinline__ double crt(const int8_t *y)
+// An unsigned integer of 32 bits as float64, by the bits and one addition: the
+// conversion instructions and the additions share the SM's one float64 pipe, which
+// the leaves fill.
+__device__ __forceinline__ double from_u32(unsigned x) { return __hiloint2double(0x43300000, (int)x) - 0x1p52; }
+
+// 2^k times the product an entry's residues stand for (16 bytes, 16 KB apart).
+__device__ __forceinline__ double crt(const int8_t *y, int k)
 {
     unsigned long long a0 = 0, a1 = 0, a2 = 0;
 #pragma unroll
@@ -346,7 +361,14 @@ __device__ __forceinline__ double crt(const int8_t *y)
     }
     a1 += a0 >> 32;
     const unsigned long long hi = (a2 << 32) + a1;   // top 64 of 96 bits; whole multiples of P drop out
-    return (__ll2double_rn((long long)hi) * 0x1p-64 + (double)(unsigned)a0 * 0x1p-96) * c_crt.P;
+    // (signed) hi + a0 / 2^32: the upper half as 2^84 + 2^32 (h + 2^31), the lower
+    // as 2^52 + l, their excess taken off exactly
+    const double top = __hiloint2double(0x45300000, (int)((unsigned)(hi >> 32) ^ 0x80000000u)) - (0x1p84 + 0x1p63 + 0x1p52);
+    const double x = fma(from_u32((unsigned)a0), 0x1p-32, top + __hiloint2double(0x43300000, (int)(unsigned)hi));
+    // times P 2^(k - 64): exact but for one rounding, the power of two in P's exponent
+    const int e = (__double2hiint(c_crt.P) >> 20) + k - 64;
+    if (e < 1 || e > 2046 - 64) return scalbn(x * (c_crt.P * 0x1p-64), k);
+    return x * __hiloint2double(__double2hiint(c_crt.P) + ((k - 64) << 20), __double2loint(c_crt.P));
 }
 
 // ---- the superblocks' own solve -----------------------------------------------
@@ -367,10 +389,11 @@ __device__ __forceinline__ double residue_sum(const Wave &w, const Problem &pr, 
     if (w.products == 0) return 0.0;
     const int8_t *y = w.res + (size_t)t * w.products * rns::kMods * SP * SP + i * SP + j;
     const int r = s.A * SP + i, c = s.B * SP + j, b2 = 2 * pr.bits;
-    if (!opp)
-        return -scalbn(crt(y + (size_t)2 * rns::kMods * SP * SP), max(pr.er0[r], kMinExp) + max(pr.ec1[c], kMinExp) - b2);
-    return scalbn(crt(y), max(pr.er0[r], kMinExp) + max(pr.ec0[c], kMinExp) - b2) -
-           scalbn(crt(y + (size_t)rns::kMods * SP * SP), max(pr.er1[r], kMinExp) + max(pr.ec1[c], kMinExp) - b2);
+    // both kinds of entry take their first sum in one pass: UT, or UU
+    const int ec1 = max(pr.ec1[c], kMinExp), first = max(pr.er0[r], kMinExp) + (opp ? max(pr.ec0[c], kMinExp) : ec1);
+    const double v = crt(opp ? y : y + (size_t)2 * rns::kMods * SP * SP, first - b2);
+    if (!opp) return -v;
+    return v - crt(y + (size_t)rns::kMods * SP * SP, max(pr.er1[r], kMinExp) + ec1 - b2);
 }
 
 // Blocks (i, j) of a superblock at step l = 7 - i + j.
@@ -450,8 +473,8 @@ __device__ __forceinline__ void wave_far(const Wave &wv, int b, int l, double *s
     fetch(x0);
     const int p = lo, q = hi;
     bool opp = true;
-    if (w.RU) opp = SGT_AT(w.RU, w.ldru, min(r0 + p, w.rows - 1), min(r0 + p, w.rows - 1)) +
-                    SGT_AT(w.CU, w.ldcu, min(c0 + q, w.cols - 1), min(c0 + q, w.cols - 1)) == 0.0;
+    if (w.RU) opp = lvl::signs_differ(SGT_AT(w.RU, w.ldru, min(r0 + p, w.rows - 1), min(r0 + p, w.rows - 1)),
+                                      SGT_AT(w.CU, w.ldcu, min(c0 + q, w.cols - 1), min(c0 + q, w.cols - 1)));
     const unsigned long long flip = opp ? 0ull : 0x8000000000000000ull;
     double acc = 0.0;
     for (int x = x0, buf = 0; x < x1; x++, buf ^= 1) {
@@ -517,14 +540,16 @@ __device__ __forceinline__ void wave_leaf(const Wave &wv, int b, int l, bool fir
     const int step = LB - 1 - p + q;
     __syncthreads();
     const double upp = s.urow[p], uqq = s.ucol[q];
-    const bool opp = upp + uqq == 0.0;
+    const bool opp = lvl::signs_differ(upp, uqq);
     const bool live = r0 + p < w.rows && c0 + q < w.cols;
-    const double rinv = !live ? 0.0 : opp ? 1.0 / (s.TI[p + p * LD] - s.TJ[q + q * LD]) : 0.5 * upp;
+    const double rinv = !live ? 0.0 : opp ? 1.0 / (s.TI[p + p * LD] - s.TJ[q + q * LD]) : copysign(0.5, upp);
     const unsigned long long flip = opp ? 0ull : 0x8000000000000000ull;
     const double *M = opp ? s.TI : s.UI, *N = opp ? s.TJ : s.UJ;
     const double *M1 = opp ? s.T1 : s.U1, *N2 = opp ? s.T2 : s.U2;
     // here a thread takes entry (hi, lo): residues lie row by row
-    s.C[hi + lo * LD] = residue_sum(wv, w, k.s, k.t, (k.I % SB) * LB + hi, (k.J % SB) * LB + lo, s.urow[hi] + s.ucol[lo] == 0.0);
+    s.C[hi + lo * LD] = residue_sum(wv, w, k.s, k.t, (k.I % SB) * LB + hi, (k.J % SB) * LB + lo, lvl::signs_differ(s.urow[hi], s.ucol[lo]));
+    // own (u_ii - u_jj) = +-2 own
+    s.V[at] = lvl::signs_differ(s.urow[lo], s.ucol[hi]) ? lvl::flip_sign(own, (unsigned long long)__double_as_longlong(s.urow[lo]) & 0x8000000000000000ull) * w.own2 : 0.0;
     __syncthreads();
 
     lvl::dependency_wait();
@@ -542,9 +567,7 @@ __device__ __forceinline__ void wave_leaf(const Wave &wv, int b, int l, bool fir
         if (t < nslab) sum += v[t];
     s.X1[at] = x1;
     s.X2[at] = x2;
-    const double ui = s.urow[lo], uj = s.ucol[hi];
     s.C[at] = sum;
-    s.V[at] = ui + uj == 0.0 ? own * (w.own * (ui - uj)) : 0.0;
     __syncthreads();
     double acc = s.C[p + q * LD];
     const double base = s.V[p + q * LD];
@@ -695,10 +718,8 @@ struct Run {
         const bool sums = levels > sums_from;
         {
             ProfScope ps(SIGNTRI_KC_CONVERT, st);
-            for (const Problem &p : probs) {   // below every exponent
-                for (int *e : {p.er0, p.er1, p.rnew}) SGT_CUDA_TRY(cudaMemsetAsync(e, 0xc0, (size_t)p.nkbr / 2 * SP * sizeof(int), st));
-                for (int *e : {p.ec0, p.ec1, p.cnew}) SGT_CUDA_TRY(cudaMemsetAsync(e, 0xc0, (size_t)p.nkbc / 2 * SP * sizeof(int), st));
-            }
+            init_exps_kernel<<<np, kThreads, 0, st>>>(d_probs);
+            SGT_LAUNCH_CHECK();
             if (sums) {
                 tiles_kernel<<<(unsigned)((list.size() + 255) / 256), 256, 0, st>>>(d_probs, d_list, (int)list.size(),
                                                                                     products, tiles);
@@ -818,7 +839,7 @@ signtri_status ph_super_run(int count, const BatchDesc *mats, Arena &ws, int *d_
         p.ldrt = p.ldct = p.ldc0 = m.ldt;
         p.ldru = p.ldcu = p.ldv = m.ldu;
         p.rows = p.cols = m.n;
-        p.own = 1.0;
+        p.own2 = 2.0;
         p.bits = rns::operand_bits(ns * SP);
         p.triangular = true;
         if (!r.reserve(ws, p, ns, ns, true)) return SIGNTRI_ERR_NO_WORKSPACE;
@@ -883,7 +904,7 @@ signtri_status sylvester_super_run(int m, int p, const double *A, int lda, const
     q.ldv = ldx;
     q.rows = m;
     q.cols = p;
-    q.own = 0.5 * cscale;   // (rows and columns stand for u = 1 and -1)
+    q.own2 = cscale;   // (rows and columns stand for u = 1 and -1)
     q.bits = rns::operand_bits(std::max(nr, nc) * SP);
     if (!r.reserve(ws, q, nr, nc, nr + nc > 2)) return SIGNTRI_ERR_NO_WORKSPACE;
     r.probs.push_back(q);
