@@ -136,4 +136,21 @@ __device__ __forceinline__ double rsqrt_normal(double a)
     return __hiloint2double(__double2hiint(y) - (h << 20), __double2loint(y));
 }
 
+// 1 / d.  With r the single-precision reciprocal of d's leading 24 bits under
+// d's own power of two, e = 1 - d r (one rounding of an almost exact value, below
+// 2^-21) and 1 / d = r (1 + e + e^2 + ...), the geometric series: three terms
+// leave 2^-63, so what counts is the last operation's rounding.  Three float64
+// instructions; exponents near the ends of the range by the division.
+__device__ __forceinline__ double recip(double d)
+{
+    const int hi = __double2hiint(d), ex = (hi >> 20) & 0x7ff;
+    if (ex < 64 || ex > 1982) return 1.0 / d;
+    const float m = __int_as_float(0x3f800000 | (hi & 0xfffff) << 3 | (int)((unsigned)__double2loint(d) >> 29));
+    const unsigned rb = (unsigned)__float_as_int(__fdividef(1.f, m));
+    const int rh = (int)(rb >> 3) + ((896 + 1023 - ex) << 20);
+    const double r = __hiloint2double(rh | (hi & (int)0x80000000u), (int)(rb << 29));
+    const double e = fma(-d, r, 1.0);
+    return fma(r, fma(e, e, e), r);
+}
+
 }  // namespace signtri

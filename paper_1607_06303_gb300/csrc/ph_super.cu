@@ -32,6 +32,7 @@
 #include <climits>
 #include <vector>
 
+#include "df_arith.cuh"
 #include "internal.cuh"
 #include "ph_level.cuh"
 #include "rns.cuh"
@@ -542,7 +543,7 @@ __device__ __forceinline__ void wave_leaf(const Wave &wv, int b, int l, bool fir
     const double upp = s.urow[p], uqq = s.ucol[q];
     const bool opp = lvl::signs_differ(upp, uqq);
     const bool live = r0 + p < w.rows && c0 + q < w.cols;
-    const double rinv = !live ? 0.0 : opp ? 1.0 / (s.TI[p + p * LD] - s.TJ[q + q * LD]) : copysign(0.5, upp);
+    const double rinv = !live ? 0.0 : opp ? recip(s.TI[p + p * LD] - s.TJ[q + q * LD]) : copysign(0.5, upp);
     const unsigned long long flip = opp ? 0ull : 0x8000000000000000ull;
     const double *M = opp ? s.TI : s.UI, *N = opp ? s.TJ : s.UJ;
     const double *M1 = opp ? s.T1 : s.U1, *N2 = opp ? s.T2 : s.U2;
@@ -583,7 +584,8 @@ __device__ __forceinline__ void wave_leaf(const Wave &wv, int b, int l, bool fir
     const double x = in ? s.V[at] : 0.0;
     if (in) SGT_AT(w.V, w.ldv, r0 + lo, c0 + hi) = x;
     // a warp holds 16 rows of two columns
-    const int e = x != 0.0 ? exponent_above(x) : kNoExp;
+    const bool some = (__double2hiint(x) << 1 | __double2loint(x)) != 0;   // x != 0, by the bits
+    const int e = some ? exponent_above(x) : kNoExp;
     const int er = max(e, __shfl_xor_sync(0xffffffffu, e, 16));
     int ec = e;
 #pragma unroll
