@@ -1090,8 +1090,16 @@ signtri_status signtri_sylvester(int m, int p, const double *A, int lda, const d
     signtri_status rs = current_state(&s);
     if (rs != SIGNTRI_OK) return rs;
     Arena ws;
-    // a caller's workspace may hold the plain solve's sums only
     const size_t plain = sylvester_workspace_bytes(m, p);
+    // a capture has no room for the superblocks' waits
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(static_cast<cudaStream_t>(stream), &capture) != cudaSuccess) cudaGetLastError();
+    if (capture != cudaStreamCaptureStatusNone) {
+        rs = get_workspace(*s, plain, ws);
+        if (rs != SIGNTRI_OK) return rs;
+        return sylvester_run(m, p, A, lda, B, ldb, C, ldc, 1.0, X, ldx, ws, static_cast<cudaStream_t>(stream));
+    }
+    // a caller's workspace may hold the plain solve's sums only
     rs = get_workspace(*s, std::max(plain, sylvester_super_workspace_bytes(m, p)), ws);
     if (rs == SIGNTRI_ERR_NO_WORKSPACE) rs = get_workspace(*s, plain, ws);
     if (rs != SIGNTRI_OK) return rs;

@@ -20,9 +20,12 @@
 //     n = 512 on the same swaps run by windows instead (reorder_tc.cu).
 //  2. Triangular Sylvester solve A X - X B = C by the element recurrence
 //     (a_ii - b_jj) x_ij = c_ij - sum_{k>i} a_ik x_kj + sum_{k<j} x_ik b_kj,
-//     blocked: b x b blocks by anti-diagonal (bottom-left first), float64 block
-//     sums of the finished blocks (split along K, fixed summation order), then
-//     the recurrence inside each block.
+//     by superblocks of 128 whose mutual sums are residue products on the
+//     tensor cores (ph_super.cu); where one scale per row or column does not
+//     suit the data or the workspace has no room, by 64 x 64 blocks by
+//     anti-diagonal (bottom-left first), double-float block sums of the finished
+//     blocks (split along K, fixed summation order), then the recurrence inside
+//     each block.
 //  3. Back-transform: with Q = [Q1 Q2] (n x n_+, n x n_-),
 //     Q U~ Q^T = I + (Q1 X - 2 Q2) Q2^T = -I + Q1 (2 Q1^T + X Q2^T);
 //     the form with the smaller inner dimension is used, as two

@@ -128,6 +128,30 @@ def test_sylvester_superblocks_vs_oracle(gpu_lib, oracle_mod, n, n_neg):
     assert np.linalg.norm(U - ref) <= n * np.finfo(float).eps * np.linalg.norm(ref)
 
 
+# signtri_sylvester in a stream capture (where the superblocks' waits cannot be)
+# and outside one: the same solution
+@pytest.mark.gpu
+def test_sylvester_in_a_capture(gpu_lib):
+    import torch
+    m, q = 200, 150
+    T = make_T(m + q, seed=9, n_neg=q, order="sorted")
+    A, B, C = (gpu_lib.to_device(np.asfortranarray(M)) for M in (T[:m, :m], T[m:, m:], T[:m, m:]))
+    out = [gpu_lib.to_device(np.zeros((m, q), order="F")) for _ in range(2)]
+
+    def run(X):
+        st = torch.cuda.current_stream().cuda_stream
+        assert gpu_lib.signtri_sylvester(m, q, A.data_ptr(), m, B.data_ptr(), q, C.data_ptr(), m, X.data_ptr(), m, st) == 0
+    run(out[0])
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        run(out[1])
+    g.replay()
+    torch.cuda.synchronize()
+    x, y = (gpu_lib.to_numpy(X) for X in out)
+    assert np.linalg.norm(x - y) <= (m + q) * np.finfo(float).eps * np.linalg.norm(x)
+
+
 # a batch with problems on both sides of the superblocks' least order, ragged
 # ones, a graded one (left to the plain path) and a one-signed one
 @pytest.mark.gpu
