@@ -399,8 +399,12 @@ __device__ __forceinline__ double residue_sum(const Wave &w, const Problem &pr, 
 
 // Blocks (i, j) of a superblock at step l = 7 - i + j.
 __host__ __device__ constexpr int wave_blocks(int l) { return l < 0 || l > 2 * SB - 2 ? 0 : (l < SB ? l + 1 : 2 * SB - 1 - l); }
-// Their sums over finished blocks more than one away are cut in three.
-constexpr int kParts = 3;
+// Their sums over finished blocks more than one away are cut in two, each as
+// long as a leaf or shorter and fewer CTAs to share the SMs with the leaves (one,
+// two, three, four: Sylvester equation of a sorted diagonal, n = 8192, 16.1, 15.1,
+// 15.9, 16.8 ms; sign(T) n = 2000 3.72, 3.54, 3.68, 3.82, n = 8192 35.7, 33.4,
+// 33.0, 33.0; batch of 300 43.2, 42.6, 43.0, 43.3).
+constexpr int kParts = 2;
 
 struct WaveBlock {
     int t, jj, I, J, c, r;   // tile, place in the step, global blocks, finished blocks below and to the left
@@ -608,6 +612,20 @@ wave_kernel(const __grid_constant__ Wave w, int l, bool first, const double *in,
     }
 }
 
+// Shared memory a launch of G CTAs asks for beside its own: where there are
+// few, an SM's divided by the CTAs an SM gets, so that they spread evenly (the
+// scheduler puts four on an SM and leaves others empty, and a leaf that shares its
+// float64 pipe waits for it); 66 KB at two an SM leaves one beside the residue
+// products' CTA.  Measured with none / this, ms: Sylvester equation of a sorted
+// diagonal, n = 8192, 17.6 / 15.9; sign(T) n = 2000 3.91 / 3.68, 4096 10.1 / 9.7,
+// 8192 33.4 / 33.1 (with three parts, kParts); four an SM (G up to 608) no better
+// than none.
+int wave_spread(int G)
+{
+    const int per = (G + lvl::kSms - 1) / lvl::kSms;
+    return (per == 1 ? 190 : per == 2 ? 66 : per == 3 ? 45 : 0) * 1024;
+}
+
 // l0, l1: the first and one past the last step that hold blocks.
 signtri_status run_wave(const Wave &w, int l0, int l1, double *slab0, double *slab1, int cls, cudaStream_t st)
 {
@@ -620,8 +638,10 @@ signtri_status run_wave(const Wave &w, int l0, int l1, double *slab0, double *sl
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     double *slab[2] = {slab0, slab1};
+    SGT_CUDA_TRY(cudaFuncSetAttribute(wave_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, wave_spread(1)));
     for (int l = l0; l < l1; l++) {
         cfg.gridDim = dim3(w.tiles * (wave_blocks(l) + kParts * wave_blocks(l + 1)));
+        cfg.dynamicSmemBytes = wave_spread((int)cfg.gridDim.x);
         ProfScope ps(cls, st);
         SGT_CUDA_TRY(cudaLaunchKernelEx(&cfg, wave_kernel, w, l, l == l0, (const double *)slab[l & 1], slab[(l + 1) & 1]));
     }
