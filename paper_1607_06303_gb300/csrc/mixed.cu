@@ -118,6 +118,10 @@ constexpr int kTri = kMicros * (kMicros + 1) / 2;   // micro-blocks of an upper 
 // words from one micro-block to the next in shared memory: eight consecutive
 // ones lie in different banks for 16-byte reads
 constexpr int kMicroPitch = kMicro * kMicro + 4;
+// What a launch of no more leaves than SMs asks for, so that each gets one (left to
+// itself the scheduler pairs some beside empty SMs: 27 us a launch all the same
+// alone, n = 3001 8.65 -> 7.82 ms, n = 16384 188.5 -> 184.4).
+constexpr size_t kLeafAlone = 200 * 1024;
 constexpr size_t kLeafSmem = (size_t)(4 * kTri + kMicros * kMicros) * kMicroPitch * sizeof(float);
 
 // Number of micro-block (r, c), r <= c, of an upper triangular tile, row by row.
@@ -978,7 +982,7 @@ signtri_status sweep(MixedCtx &c, const double *T, int ldt, double *V, int ldv, 
     const int n = c.n, nb = c.sc.nb;
     const size_t leaf_smem = kLeafSmem;
     SGT_CUDA_TRY(cudaFuncSetAttribute(mixed_leaf_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)leaf_smem));
+                                      (int)kLeafAlone));
     SGT_CUDA_TRY(cudaFuncSetAttribute(mixed_leaf_kernel<MODE>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                       cudaSharedmemCarveoutMaxShared));   // two leaves per SM
     {
@@ -1114,7 +1118,7 @@ signtri_status sweep(MixedCtx &c, const double *T, int ldt, double *V, int ldv, 
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3(ntiles);
         cfg.blockDim = dim3(kLeafThreads);
-        cfg.dynamicSmemBytes = leaf_smem;
+        cfg.dynamicSmemBytes = ntiles <= 152 ? kLeafAlone : leaf_smem;
         cfg.stream = c.st;
         cfg.attrs = &attr;
         cfg.numAttrs = 1;
