@@ -185,10 +185,11 @@ template <int MODE>
 __global__ void __launch_bounds__(kLeafThreads)
 leaf_seed_kernel(int n, const double *__restrict__ T, int ldt, const float *__restrict__ DIAG,
                  const double *__restrict__ Rc, const double *__restrict__ Rs, int ldr, int d,
-                 const int2 *__restrict__ tslot, const int2 *__restrict__ tslot2, const double *__restrict__ PA,
-                 const double *__restrict__ PB, float *__restrict__ SEED)
+                 const int2 *__restrict__ tslot, const int2 *__restrict__ tslot2, const double *PA,
+                 const double *PB, float *__restrict__ SEED)
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the leaves may load their operators
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int I = blockIdx.x, J = I + d;
     const int e = blockIdx.y * kLeafThreads + threadIdx.x, p = e % MB, q = e / MB;
     const int gi = I * MB + p, gj = J * MB + q;
@@ -295,6 +296,7 @@ mixed_leaf_kernel(int n, double *__restrict__ V, int ldv, const float *__restric
     // (SEED is written by the launch before: a restricted pointer's loads could
     // be moved above the wait)
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 #pragma unroll
     for (int q = 0; q < 4; q++) {
         *reinterpret_cast<float4 *>(Vs + own * PT + q * kMicro) =
@@ -1043,7 +1045,7 @@ signtri_status sweep(MixedCtx &c, const double *T, int ldt, double *V, int ldv, 
             const int cls = SIGNTRI_KC_BLOCK_SUMS_TC | kProfUntimed;
             if ((rs = fork()) != SIGNTRI_OK) return rs;
             rs = tc_blocksums(srcV_r, srcT_r, srcT_c, srcV_c, c.dsA.jobs + A.job_off[d], A.job_off[d + 1] - A.job_off[d],
-                              c.pairs_split, c.d_pairs_split, chunk, c.PA, slots, c.d_err, cls, c.st,
+                              c.pairs_split, c.d_pairs_split, chunk, c.PA, slots, c.d_err, cls | kTcFollows, c.st,
                               tc_flops(c.pairs_split.n, sum_kb, 3), c.dsA.cta_off + A.cta_begin[d], A.nctas[d]);
             if (rs == SIGNTRI_OK)
                 rs = tc_blocksums(srcV_r, srcT_r, srcT_c, srcV_c, c.dsB.jobs + B.job_off[e],
@@ -1062,8 +1064,8 @@ signtri_status sweep(MixedCtx &c, const double *T, int ldt, double *V, int ldv, 
             // leaves sum both slot sets
             const Schedule &B = c.scB, &C = c.scC;
             rs = tc_blocksums(srcV_r, srcT_r, srcT_c, srcV_c, c.dsC.jobs + C.job_off[d], C.job_off[d + 1] - C.job_off[d],
-                              c.pairs_split, c.d_pairs_split, chunk, c.PA, slots, c.d_err, SIGNTRI_KC_BLOCK_SUMS_TC,
-                              c.st, tc_flops(c.pairs_split.n, 4LL * ntiles, 3), c.dsC.cta_off + C.cta_begin[d],
+                              c.pairs_split, c.d_pairs_split, chunk, c.PA, slots, c.d_err,
+                              SIGNTRI_KC_BLOCK_SUMS_TC | kTcFollows, c.st, tc_flops(c.pairs_split.n, 4LL * ntiles, 3), c.dsC.cta_off + C.cta_begin[d],
                               C.nctas[d]);
             if (rs != SIGNTRI_OK) return rs;
             prof_add_bytes(SIGNTRI_KC_BLOCK_SUMS_TC, 4.0 * 4.0 * ntiles * kb_bytes);
@@ -1078,7 +1080,7 @@ signtri_status sweep(MixedCtx &c, const double *T, int ldt, double *V, int ldv, 
                 if (MODE == 0) {
                     // [U_I.; T_I.] x [T_.J | U_.J]: TL = U T, TR = U U, BR = T U
                     rs = tc_blocksums(srcV_r, srcT_r, srcT_c, srcV_c, jobs, njobs, c.pairs_split, c.d_pairs_split,
-                                      chunk, c.PA, slots, c.d_err, SIGNTRI_KC_BLOCK_SUMS_TC, c.st,
+                                      chunk, c.PA, slots, c.d_err, SIGNTRI_KC_BLOCK_SUMS_TC | kTcFollows, c.st,
                                       tc_flops(c.pairs_split.n, sum_kb, 3), coff, G);
                     if (rs != SIGNTRI_OK) return rs;
                     prof_add_bytes(SIGNTRI_KC_BLOCK_SUMS_TC, 4.0 * sum_kb * kb_bytes);
@@ -1095,7 +1097,7 @@ signtri_status sweep(MixedCtx &c, const double *T, int ldt, double *V, int ldv, 
                         sy = c.side;
                     }
                     rs = tc_blocksums(srcV_r, srcT_r, srcT_c, srcV_c, jobs, njobs, c.pairs_split, c.d_pairs_split,
-                                      chunk, c.PA, slots, c.d_err, cls, c.st, tc_flops(c.pairs_split.n, sum_kb, 2),
+                                      chunk, c.PA, slots, c.d_err, cls | kTcFollows, c.st, tc_flops(c.pairs_split.n, sum_kb, 2),
                                       coff, G);
                     if (rs == SIGNTRI_OK)
                         rs = tc_blocksums(srcU_r, srcV_r, srcV_c, srcU_c, jobs, njobs, c.pairs_split,
@@ -1109,19 +1111,20 @@ signtri_status sweep(MixedCtx &c, const double *T, int ldt, double *V, int ldv, 
             }
         }
         ProfScope ps(MODE == 0 ? SIGNTRI_KC_OFFDIAG_LEAF_F32 : SIGNTRI_KC_CORRECTION, c.st);
-        leaf_seed_kernel<MODE><<<dim3(ntiles, MB * MB / kLeafThreads), kLeafThreads, 0, c.st>>>(
-            n, T, ldt, c.DIAG, c.res_c, c.res_s, n, d, leaf_slots, leaf_slots2, c.PA, c.PB, c.SEED);
-        SGT_LAUNCH_CHECK();
         cudaLaunchAttribute attr{};
         attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr.val.programmaticStreamSerializationAllowed = 1;
         cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3(ntiles);
+        cfg.gridDim = dim3(ntiles, MB * MB / kLeafThreads);
         cfg.blockDim = dim3(kLeafThreads);
-        cfg.dynamicSmemBytes = ntiles <= 152 ? kLeafAlone : leaf_smem;
         cfg.stream = c.st;
         cfg.attrs = &attr;
         cfg.numAttrs = 1;
+        SGT_CUDA_TRY(cudaLaunchKernelEx(&cfg, leaf_seed_kernel<MODE>, n, T, ldt, (const float *)c.DIAG,
+                                        (const double *)c.res_c, (const double *)c.res_s, n, d, leaf_slots, leaf_slots2,
+                                        (const double *)c.PA, (const double *)c.PB, c.SEED));
+        cfg.gridDim = dim3(ntiles);
+        cfg.dynamicSmemBytes = ntiles <= 152 ? kLeafAlone : leaf_smem;
         SGT_CUDA_TRY(cudaLaunchKernelEx(&cfg, mixed_leaf_kernel<MODE>, n, V, ldv, (const float *)c.OPS,
                                         (const float *)c.DIAG, d, (const float *)c.SEED, Vr, Vc, c.S, nb,
                                         c.f16 ? (MODE == 0 ? c.sU : c.sE) : 0.f));

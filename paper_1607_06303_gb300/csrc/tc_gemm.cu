@@ -164,6 +164,9 @@ tc_blocksum_kernel(const __grid_constant__ CUtensorMap mTop, const __grid_consta
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_holder + 1);
     TcPairs *pairs_s = reinterpret_cast<TcPairs *>(smem + kStages * kStageBytes + 512);
 
+    // (a launch that follows: nothing of the kernel before is read above)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int j0 = job_off ? job_off[blockIdx.x] : (int)blockIdx.x;
     const int j1 = job_off ? job_off[blockIdx.x + 1] : (int)blockIdx.x + 1;
@@ -867,7 +870,8 @@ signtri_status tc_blocksums(const TcSource &top, const TcSource &bot, const TcSo
     const int resident = (same_w && pairs.n > 1 && nsl <= 3 && nsl <= top.nslices && nsl <= bot.nslices &&
                           nsl <= left.nslices && nsl <= right.nslices) ? 1 : 0;
     const bool timed = (kernel_class & kProfUntimed) == 0;
-    kernel_class &= ~kProfUntimed;
+    const bool follows = (kernel_class & kTcFollows) != 0;
+    kernel_class &= ~(kProfUntimed | kTcFollows);
     // grouped pair mode when pairs with unequal weights share A slices
     bool share = false;
     for (int p = 0; p < pairs.n && !share; p++)
@@ -888,10 +892,19 @@ signtri_status tc_blocksums(const TcSource &top, const TcSource &bot, const TcSo
     SGT_CUDA_TRY(cudaFuncSetAttribute(tc_blocksum_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     prof_add_flops(kernel_class, useful_flops);
     ProfScope ps(kernel_class, st, timed);
-    tc_blocksum_kernel<<<d_job_off ? nctas : njobs, kTcThreads, smem, st>>>(
-        mt, mb, ml, mr, top.rows, left.rows, d_jobs, d_job_off, d_pairs, chunk_kb, top.scale, bot.scale, left.scale,
-        right.scale, out, qo, d_err, resident, nsl, blk, top.cols / 64, f16);
-    SGT_LAUNCH_CHECK();
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(d_job_off ? nctas : njobs);
+    cfg.blockDim = dim3(kTcThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = follows ? 1 : 0;
+    SGT_CUDA_TRY(cudaLaunchKernelEx(&cfg, tc_blocksum_kernel, mt, mb, ml, mr, (int)top.rows, (int)left.rows, d_jobs,
+                                    d_job_off, d_pairs, chunk_kb, top.scale, bot.scale, left.scale, right.scale, out, qo,
+                                    d_err, resident, nsl, blk, (int)(top.cols / 64), (int)f16));
     return SIGNTRI_OK;
 }
 

@@ -89,6 +89,11 @@ signtri_status make_gathered_slices(int n, const double *M, int ldm, const int *
 
 // d_job_off (device, nctas + 1 entries): CTA b runs jobs [d_job_off[b],
 // d_job_off[b+1]) back to back; null: one CTA per job.
+// In kernel_class (beside kProfUntimed): the launch may be set up while the kernel
+// before it on the stream ends (what it reads of that kernel's is read after a
+// dependency wait).  In the mixed sweeps, with the seeds likewise: n = 3001 7.82 ->
+// 7.68 ms, n = 16384 184.4 -> 183.5.
+constexpr int kTcFollows = 0x2000;
 signtri_status tc_blocksums(const TcSource &top, const TcSource &bot, const TcSource &left, const TcSource &right,
                             const TcJob *d_jobs, int njobs, const TcPairs &pairs, const TcPairs *d_pairs, int chunk_kb,
                             double *out, const TcQuadOut &qo, int *d_err, int kernel_class, cudaStream_t st,
