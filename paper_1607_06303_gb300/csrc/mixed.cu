@@ -436,7 +436,7 @@ corr_diag_leaf_kernel(int n, const double *__restrict__ T, int ldt, const double
     __syncthreads();
     for (int idx = threadIdx.x; idx < bs * bs; idx += kLeafThreads) {
         const int i = idx % bs, j = idx / bs;
-        const bool opp = (Ts[i + i * LD] > 0.0) != (Ts[j + j * LD] > 0.0);
+        const bool opp = (__double2hiint(Ts[i + i * LD]) ^ __double2hiint(Ts[j + j * LD])) < 0;
         Es[i + j * LD] = i < j ? -SGT_AT(opp ? Rc : Rs, ldr, r0 + i, r0 + j) : 0.0;
     }
     __syncthreads();
@@ -447,7 +447,7 @@ corr_diag_leaf_kernel(int n, const double *__restrict__ T, int ldt, const double
         double s = 0.0;
         bool opp = false;
         if (live) {
-            opp = (Ts[i + i * LD] > 0.0) != (Ts[j + j * LD] > 0.0);
+            opp = (__double2hiint(Ts[i + i * LD]) ^ __double2hiint(Ts[j + j * LD])) < 0;
             // signs differ: e t - t e; agree: - u e - e u
             const double *M = opp ? Ts : Us;
             for (int k = i + 1 + part; k < j; k += 4) {
@@ -458,9 +458,8 @@ corr_diag_leaf_kernel(int n, const double *__restrict__ T, int ldt, const double
         s += __shfl_xor_sync(0xffffffffu, s, 1);
         s += __shfl_xor_sync(0xffffffffu, s, 2);
         if (live && part == 0) {
-            const double si = Ts[i + i * LD] > 0.0 ? 1.0 : -1.0;
             s += Es[i + j * LD];
-            Es[i + j * LD] = opp ? s / (Ts[i + i * LD] - Ts[j + j * LD]) : s * (0.5 * si);
+            Es[i + j * LD] = s * (opp ? recip(Ts[i + i * LD] - Ts[j + j * LD]) : copysign(0.5, Ts[i + i * LD]));
         }
         __syncthreads();
     }
@@ -477,7 +476,8 @@ corr_diag_leaf_kernel(int n, const double *__restrict__ T, int ldt, const double
 // (RA: Y at equal-sign positions, N_T N_U at opposite-sign ones; RB: N_U N_T)
 // plus the diagonal terms.  Only the strictly upper part of R is written: the
 // correction reads nothing else.  Squared Frobenius norms of the used Rc and
-// Rs entries, of T and of U into norms[0..3].
+// Rs entries, of T and of U into norms[0..3].  Bound by the float64 pipes (10
+// instructions an entry; 15 with the diagonal terms written out).
 __global__ void needed_finalize_kernel(int n, const double *__restrict__ T, int ldt, const double *__restrict__ U,
                                        int ldu, const int *__restrict__ gmap, const double *__restrict__ RA,
                                          const double *__restrict__ RB, int ldg, double *__restrict__ R,
@@ -486,19 +486,19 @@ __global__ void needed_finalize_kernel(int n, const double *__restrict__ T, int 
     const int j = blockIdx.x;
     double nc = 0.0, ns = 0.0, nt = 0.0, nu = 0.0;
     const double tjj = SGT_AT(T, ldt, j, j), ujj = SGT_AT(U, ldu, j, j);
+    const double two = 2.0 * ujj;
     const size_t gj = (size_t)gmap[j] * ldg;
     for (int i = threadIdx.x; i < j; i += blockDim.x) {
-        const double tii = SGT_AT(T, ldt, i, i), uii = SGT_AT(U, ldu, i, i);
+        const double tii = SGT_AT(T, ldt, i, i);
         const double tij = SGT_AT(T, ldt, i, j), uij = SGT_AT(U, ldu, i, j);
         const size_t g = (size_t)gmap[i] + gj;
-        double r;
-        if ((tii > 0.0) == (tjj > 0.0)) {
-            r = RA[g] + uii * uij + uij * ujj;
-            ns += r * r;
-        } else {
-            r = RA[g] - RB[g] + (tii * uij - uij * tjj) + (tij * ujj - uii * tij);
-            nc += r * r;
-        }
+        const bool opp = (__double2hiint(tii) ^ __double2hiint(tjj)) < 0;
+        // u_ii = +-1 and u_jj = +-1: u_ii u_ij + u_ij u_jj = 2 u_jj u_ij where they
+        // agree, t_ij u_jj - u_ii t_ij = 2 u_jj t_ij where they differ
+        double r = fma(two, opp ? tij : uij, RA[g]);
+        if (opp) r += fma(tii, uij, -(uij * tjj)) - RB[g];
+        nc = fma(r, opp ? r : 0.0, nc);
+        ns = fma(r, opp ? 0.0 : r, ns);
         nt += tij * tij;
         nu += uij * uij;
         SGT_AT(R, n, i, j) = r;
