@@ -271,6 +271,7 @@ window_sort_kernel(double *__restrict__ Tr, int ldt, const int2 *__restrict__ wi
 constexpr int kFactorCtas = kWin / 32;
 constexpr int kFactorLD = 33;
 
+constexpr size_t kFactorAlone = 200 * 1024;   // where there are SMs enough, a CTA to each
 size_t factor_smem_bytes()
 {
     return (size_t)kMaxRot * (sizeof(float4) + sizeof(short)) + 2 * (size_t)kWin * kFactorLD * sizeof(float);
@@ -567,7 +568,7 @@ signtri_status reorder_blocked_run(int n, const double *T, int ldt, double *Tr, 
         const size_t smem = window_smem_bytes();
         SGT_CUDA_TRY(cudaFuncSetAttribute(window_sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         SGT_CUDA_TRY(cudaFuncSetAttribute(window_factor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)factor_smem_bytes()));
+                                          (int)kFactorAlone));
         // the windows' rotation logs lie in T's column slices, which each
         // sweep writes after its factors are formed (rp x kp >= 128 x 64, and
         // a sweep has at most n / 128 + 2 windows)
@@ -608,36 +609,44 @@ signtri_status reorder_blocked_run(int n, const double *T, int ldt, double *Tr, 
         };
         signtri_status r2;
         // A sweep's sort needs T alone, and few SMs: so Q's slices and product
-        // run on a second stream, beside the T products and the next sweep's
-        // sort; the next factors, which replace Z, wait for them.  (At n = 3001
-        // and 42 sweeps: 28.4 -> 25.4 ms.)
-        int it = 0;
+        // run on a second stream beside the next sweep's sort; its factors,
+        // which replace Z, wait for them.  (At n = 3001 and 42 sweeps: 28.4 ms
+        // in one stream, 25.2 with Q's part beside T's products, 22.6 so.)
+        auto q_part = [&](const Sweep &p) -> signtri_status {
+            SGT_CUDA_TRY(cudaStreamWaitEvent(side.s, side.ready[0], 0));
+            SGT_CUDA_TRY(cudaMemsetAsync(mxQ, 0, (size_t)rp * sizeof(unsigned long long), side.s));
+            signtri_status r3 = convert(kRowsQ, p, Q, ldq, mxQ, QR, sQ, side.s);
+            if (r3 == SIGNTRI_OK) r3 = product(p, 2, srcQ, srcZ, toQ, side.s);
+            if (r3 != SIGNTRI_OK) return r3;
+            SGT_CUDA_TRY(cudaEventRecord(side.done[0], side.s));
+            SGT_CUDA_TRY(cudaStreamWaitEvent(st, side.done[0], 0));
+            return SIGNTRI_OK;
+        };
+        auto *logs = reinterpret_cast<WindowLog *>(TC);   // where T's column slices follow
+        const Sweep *before = nullptr;
         for (const Sweep &p : plan) {
             SGT_CUDA_TRY(cudaMemsetAsync(mx, 0, 2 * (size_t)rp * sizeof(unsigned long long), st));
             {
                 ProfScope ps(SIGNTRI_KC_GIVENS, st);
-                // the logs lie where T's column slices follow
-                auto *logs = reinterpret_cast<WindowLog *>(TC);
                 window_sort_kernel<<<p.nw, kWinThreads, smem, st>>>(Tr, ldtr, d_wins + p.w0, logs);
                 SGT_LAUNCH_CHECK();
-                if (it > 0) SGT_CUDA_TRY(cudaStreamWaitEvent(st, side.done[0], 0));
-                window_factor_kernel<<<p.nw * kFactorCtas, kWinThreads, factor_smem_bytes(), st>>>(
+            }
+            if (before && (r2 = q_part(*before)) != SIGNTRI_OK) return r2;
+            {
+                ProfScope ps(SIGNTRI_KC_GIVENS, st);
+                window_factor_kernel<<<p.nw * kFactorCtas, kWinThreads,
+                                       p.nw * kFactorCtas <= 152 ? kFactorAlone : factor_smem_bytes(), st>>>(
                     d_wins + p.w0, logs, ZC, sZ, rp, kp);
                 SGT_LAUNCH_CHECK();
             }
-            SGT_CUDA_TRY(cudaEventRecord(side.ready[0], st));
             if ((r2 = convert(kColsT, p, Tr, ldtr, mxTc, TC, sTc, st)) != SIGNTRI_OK) return r2;
             if ((r2 = product(p, 0, srcZ, srcTc, toT, st)) != SIGNTRI_OK) return r2;     // rows of T
             if ((r2 = convert(kRowsT, p, Tr, ldtr, mxTr, TR, sTr, st)) != SIGNTRI_OK) return r2;
             if ((r2 = product(p, 1, srcTr, srcZ, toT, st)) != SIGNTRI_OK) return r2;     // columns of T
-            SGT_CUDA_TRY(cudaStreamWaitEvent(side.s, side.ready[0], 0));
-            SGT_CUDA_TRY(cudaMemsetAsync(mxQ, 0, (size_t)rp * sizeof(unsigned long long), side.s));
-            if ((r2 = convert(kRowsQ, p, Q, ldq, mxQ, QR, sQ, side.s)) != SIGNTRI_OK) return r2;
-            if ((r2 = product(p, 2, srcQ, srcZ, toQ, side.s)) != SIGNTRI_OK) return r2;  // columns of Q
-            SGT_CUDA_TRY(cudaEventRecord(side.done[0], side.s));
-            it++;
+            SGT_CUDA_TRY(cudaEventRecord(side.ready[0], st));
+            before = &p;
         }
-        SGT_CUDA_TRY(cudaStreamWaitEvent(st, side.done[0], 0));
+        if (before && (r2 = q_part(*before)) != SIGNTRI_OK) return r2;   // columns of Q
         // the host lists stay alive until the copies above are done; so do the
         // device lists until the last product
         SGT_CUDA_TRY(cudaStreamSynchronize(st));
