@@ -57,7 +57,11 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kQrThreads = 256;
 constexpr int kMaxSweepsPerEigenvalue = 100;
-constexpr long long kRotationBudget = 1LL << 13;   // rotations per launch of the QR kernel (then a sweep's end)
+// rotations per launch of the QR kernel (then a sweep's end); the last launch's
+// are applied alone, so fewer to a launch are better until the launches count
+// (n = 64, 200, 400, ms: 2^11 6.31, 29.96, 110.5; 2^13 6.40, 29.75, 108.0; 2^15
+// 7.08, 30.5)
+constexpr long long kRotationBudget = 1LL << 13;
 // rotations (and sweeps) a launch's log holds: two sweeps of a full window
 // always fit
 inline size_t rotation_room(int n) { return ((size_t)1 << 15) + 2 * (size_t)n + 2; }
