@@ -8,7 +8,8 @@
 //      K = A .. B whose entries are known (the strictly upper parts of the
 //      diagonal superblocks among them), and UU = U_A. U_.B over A < K < B, as
 //      residues (rns.cu: rounding the operands to 53 or more bits of their
-//      row's or column's largest is the only error);
+//      row's or column's largest is the only error), all but the superblocks
+//      of level D - 1 on a second stream beside that level's waves;
 //   2. 15 launches of wave_kernel: the superblocks' 16 x 16 blocks by block
 //      anti-diagonal, from the bottom-left corner, in float64: per entry the
 //      residue sum its signs ask for, UT - TU or - UU, and the terms that hold

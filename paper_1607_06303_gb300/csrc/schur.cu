@@ -8,36 +8,34 @@
 //  1. Householder reduction to upper Hessenberg form H = Q0^T A Q0, float64.
 //     For column k a reflector P = I - tau v v^T (v_0 = 1) maps A[k+1:, k]
 //     onto beta e_1; it is applied from the left to the columns right of k
-//     (one CTA per column: the column's dot product with v, then the
-//     update) and from the right to the rows of A and of Q0 (the products
-//     with v, 32 rows per CTA, then the rank-1 update).  Four launches per
-//     column.
+//     and from the right to the rows of A.  Where A fits in a cluster's shared
+//     memory one kernel runs all columns (hess_cluster_kernel), else four
+//     launches a column; Q0's rows take the kept reflectors one by one in
+//     form_q_kernel, beside the second stage.
 //  2. Implicitly shifted QR iteration on H in complex float64.  A complex
 //     shift needs no double-shift pairing, so every sweep over the active
 //     window [l, i] is a chain of plane rotations: the first from
 //     (h_ll - sigma, h_{l+1,l}), each later one zeroing the bulge
 //     h_{k+1,k-1}; each rotation G acts on rows k, k+1 of H over all columns
 //     and G^H on columns k, k+1 over the rows that hold nonzeros (so H
-//     becomes all of T, not just its diagonal) and on Q's columns.  The
-//     shift is Wilkinson's (the eigenvalue of the window's trailing 2 x 2
-//     nearer its last diagonal entry), with an ad hoc shift every tenth
-//     sweep without a deflation; h_{k,k-1} is negligible, and set to 0, when
+//     becomes all of T, not just its diagonal) and on Q's columns.  Up to ten
+//     sweeps follow one another three rows apart, shifted by the eigenvalues
+//     of the window's trailing block (by those of its trailing 2 x 2 where a
+//     window is small or does not converge), with one ad hoc shift every tenth
+//     time without a deflation; h_{k,k-1} is negligible, and set to 0, when
 //     |h_{k,k-1}| <= eps (|h_{k-1,k-1}| + |h_kk|) (|z| = |Re z| + |Im z|).
 //     Deflation takes the window's last row when its subdiagonal entry is
 //     negligible.  The rotations of a sweep depend on one another (each reads
 //     what the one before wrote), so one cluster of 16 CTAs (8 where the
-//     device cannot place 16) runs the sweeps with a cluster barrier per
-//     rotation or rotation pair, applying each to the active window only
+//     device cannot place 16) runs the sweeps with a cluster barrier per step
+//     of all its bulges, applying each rotation to the active window only
 //     (schur_qr_kernel says how the work is split); a launch runs sweeps
 //     until a rotation budget is spent and logs them, then a kernel on the
 //     other SMs applies the logged rotations to the columns right of each
 //     sweep's window and to Q, on a second stream while the next launch
 //     runs, and the host relaunches until the window is empty.
-//     The chain of rotations bounds the stage: about 3 sweeps per eigenvalue
-//     (4 counting each bulge's), ~1.9 n^2 rotations for n eigenvalues in
-//     ~0.9 n^2 dependent steps (n = 1024), each a few thousand cycles of
-//     float64 latency and a barrier -- the decomposition is the
-//     general-matrix front end, not a tuned hot path.
+//     The chain of steps bounds the stage: ~0.3 n^2 of ~3,300 cycles each
+//     (n = 200: 21 of 29 ms; two bulges at a time took 1.0 n^2 of 6,000).
 //
 // Layout: A real column-major; Q, T complex interleaved (re, im) float64
 // pairs, column-major, leading dimensions counted in complex elements.
@@ -254,7 +252,7 @@ __global__ void house_rank1_kernel(int n, int k, double *__restrict__ H, const d
 }
 
 // The whole reduction in one cluster of CL CTAs with H in their shared
-// memory (column j in CTA j % CL), where it fits (n up to 650 for 16 CTAs):
+// memory (column j in CTA j % CL), where it fits (n up to 654 for 16 CTAs):
 // per column the launches above took ~52 us at n = 200, most of it their
 // starts and ends; here it is three cluster barriers and the float64 chains
 // between them (~1 ms for all columns instead of 10.3).  Step k: the owner
@@ -492,7 +490,7 @@ __global__ void qr_state_init_kernel(int n, QrState *st)
 // One cluster barrier per step; no entry is written by one thread while
 // another reads it.  CTA 0 alone takes every decision (deflation, shifts,
 // stop) and broadcasts it, so all CTAs run the same barriers.  Where T fits in
-// the cluster's shared memory (kLocal, n up to 440 at 16 CTAs) its columns lie
+// the cluster's shared memory (kLocal, n up to 448 at 16 CTAs) its columns lie
 // there, column j in CTA j % CL, for the launch's time: a read takes ~440 cycles
 // instead of ~900 and the fence before a barrier ~500 instead of ~1,000.  Else T
 // is read with L2-only loads (another CTA may have written it since).  The rotations'
