@@ -52,11 +52,12 @@ typedef enum {
        (both X and Y for every entry), with leaves of 16 as
        SIGNTRI_PH_FP64_EFFICIENT.  From n = 1600 on with leaves of 16 the sums
        between superblocks of 128 run on the tensor cores, exact but for
-       rounding their operands to 53 or more bits of their row's or column's
-       largest entry (no larger an error against 64 bits than the float64
-       sums measured); rows or columns that one scale does not suit (graded by
-       more than about 2^24) and non-finite entries of T or U are left to the
-       float64 sums. */
+       rounding their operands to 62 bits (61 above n = 32768) below a
+       power-of-two scale per row or column.  Where that costs a sum more than
+       half a unit in its last place (in a quarter of the entries of any
+       16 x 16 block: rows or columns graded by more than about 2^5, in
+       whatever order), and for non-finite entries of T or U, the float64 sums
+       alone run. */
     SIGNTRI_PH_FP64 = 1,
     /* Parlett-Sylvester for the sign function (Section 2, Section 3,
        Section 5.1): reorder by sign with adjacent Givens swaps, solve
@@ -416,7 +417,8 @@ signtri_status signtri_reorder_by_sign(int n, const double *T, int ldt, double *
    a_ii != b_jj for all i, j; C (m x p).  All device pointers, column-major;
    X must not share an element with A, B or C (SIGNTRI_ERR_BAD_ARG).  Solved by superblocks
    of 128 whose mutual sums run on the tensor cores (as SIGNTRI_PH_FP64's), and
-   where one scale per row or column does not suit the data, the workspace has
+   where one scale per row or column does not suit the data (the rounding of a
+   sum's operands would exceed double-float's, 2^-48 of it), the workspace has
    no room for them or `stream` is being captured, by blocks of 64 with
    double-float sums.  Enqueued on `stream`; for m + p > 256 the host waits for
    it (not in a capture).  m == 0 or p == 0 is a no-op. */

@@ -294,7 +294,7 @@ signtri_status run_ph_fp64(int n, const double *T, int ldt, double *U, int ldu, 
         signtri_status rs = ph_fp64_near_run(n, T, ldt, U, ldu, kSuperNear, ws, st);
         if (rs != SIGNTRI_OK) return rs;
         const BatchDesc m{T, U, n, ldt, ldu, 0};
-        rs = ph_super_run(1, &m, ws, s.err_dev, flags, st);
+        rs = ph_super_run(1, &m, ws, s.err_dev, flags, flags + 1, st);
         if (rs != SIGNTRI_OK) return rs;
         SGT_CUDA_TRY(cudaMemcpyAsync(s.err_host, s.err_dev, sizeof(int), cudaMemcpyDeviceToHost, st));
         SGT_CUDA_TRY(cudaStreamSynchronize(st));
@@ -466,7 +466,7 @@ signtri_status batched_float64(int cnt, const std::vector<BatchDesc> &h, const B
         }
         std::vector<int> flags(run.size());
         Arena mine = ws;
-        rs = ph_super_run((int)run.size(), run.data(), mine, s.err_dev, flags.data(), st);
+        rs = ph_super_run((int)run.size(), run.data(), mine, s.err_dev, flags.data(), nullptr, st);
         if (rs != SIGNTRI_OK) return rs;
         for (size_t q = 0; q < run.size(); q++)
             if (flags[q]) plainly.push_back(large[i0 + q]);
@@ -642,6 +642,16 @@ signtri_status sign_tri_batched(int count, const int *n, const double *const *T,
     std::vector<int> plainly;
     rs = batched_float64(cnt, descs, d_descs, ph_bs, v != SIGNTRI_PH_FP64, ws, plainly, st, *s);
     if (rs != SIGNTRI_OK) return rs;
+    // many of them share their launches again, a few run each on its own
+    if (plainly.size() > 4) {
+        std::vector<int> bs_plain(cnt, 0);
+        for (int k : plainly) bs_plain[k] = ph_bs[k];
+        Arena sub = ws;
+        rs = batched_ph_run(cnt, descs.data(), d_descs, bs_plain.data(), std::vector<char>(cnt, 0).data(),
+                            v != SIGNTRI_PH_FP64, sub, st);
+        if (rs != SIGNTRI_OK) return rs;
+        plainly.clear();
+    }
     for (int k : plainly) {
         rs = run_ph_plain(sizes[k], descs[k].T, descs[k].ldt, descs[k].U, descs[k].ldu, ph_bs[k], true, st, *s);
         if (rs != SIGNTRI_OK) info[owner[k]] = rs;

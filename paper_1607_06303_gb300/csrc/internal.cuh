@@ -133,17 +133,19 @@ signtri_status ph_fp64_near_run(int n, const double *T, int ldt, double *U, int 
 // superblocks of 128, their sums on the tensor cores (ph_super.cu): everything
 // beyond the diagonal superblocks (ph_fp64_near_run with last = 7) of `count`
 // problems.  flags (host): nonzero where a problem's data did not suit one
-// scale per row and it has to be run plainly; waits for the stream.
+// scale per row and it has to be run plainly; waits for the stream.  told: null,
+// or a pinned word by which a single problem's kernels end the run early.
 constexpr int kSuperNear = 7;
 size_t ph_super_workspace_bytes(int count, const int *n);
-signtri_status ph_super_run(int count, const BatchDesc *mats, Arena &ws, int *d_err, int *flags, cudaStream_t st);
+signtri_status ph_super_run(int count, const BatchDesc *mats, Arena &ws, int *d_err, int *flags, int *told,
+                            cudaStream_t st);
 // X of A X - X B = cscale C likewise, from the bottom-left superblock; one
 // superblock needs no products, sets no flag and returns without waiting
 size_t sylvester_super_workspace_bytes(int m, int p);
 size_t sylvester_super_workspace_bound(int n);   // for every m + p = n
 signtri_status sylvester_super_run(int m, int p, const double *A, int lda, const double *B, int ldb, const double *C,
                                    int ldc, double cscale, double *X, int ldx, Arena &ws, int *d_err, int *flags,
-                                   cudaStream_t st);
+                                   int *told, cudaStream_t st);
 signtri_status ph_fp64_run(int n, const double *T, int ldt, double *U, int ldu, int b,
                            Arena &ws, cudaStream_t st);
 // arithmetic-efficient form (one sum per entry)
@@ -279,6 +281,22 @@ struct CallStream {
             if (ready[p]) cudaEventDestroy(ready[p]);
             if (done[p]) cudaEventDestroy(done[p]);
         }
+    }
+};
+
+// A few events of one call.
+struct CallEvents {
+    cudaEvent_t e[4] = {};
+    cudaError_t init(int count)
+    {
+        cudaError_t r = cudaSuccess;
+        for (int i = 0; i < count && r == cudaSuccess; i++) r = cudaEventCreateWithFlags(&e[i], cudaEventDisableTiming);
+        return r;
+    }
+    ~CallEvents()
+    {
+        for (cudaEvent_t x : e)
+            if (x) cudaEventDestroy(x);
     }
 };
 

@@ -7,8 +7,8 @@
 //   1. rns::gemm: UT = U_A. T_.B and TU = T_A. U_.B over the superblocks
 //      K = A .. B whose entries are known (the strictly upper parts of the
 //      diagonal superblocks among them), and UU = U_A. U_.B over A < K < B, as
-//      residues (rns.cu: rounding the operands to 53 or more bits of their
-//      row's or column's largest is the only error), all but the superblocks
+//      residues (rns.cu: rounding the operands to 62 bits below their row's or
+//      column's scale is the only error), all but the superblocks
 //      of level D - 1 on a second stream beside that level's waves;
 //   2. 15 launches of wave_kernel: the superblocks' 16 x 16 blocks by block
 //      anti-diagonal, from the bottom-left corner, in float64: per entry the
@@ -22,9 +22,21 @@
 // Scales: T's rows and columns by their largest entry.  U's are not known in
 // advance: a row starts with two bits of headroom over its first superblock
 // and is converted anew, with two bits again, when a later superblock outgrows
-// them.  Data that does not suit one scale per row (most of a superblock's
-// entries below 2^-24 of their row's or column's largest) or is not finite
-// sets a flag, and the caller runs the plain float64 path instead.
+// them.
+//
+// Whether one scale per row and column suits the data is tested on the results.
+// With an operand's entries rounded to 2^-(bits + 1) of their scale R (of the row)
+// or C (of the column), a sum over k of u_ik t_kj is off by about
+//   E = 2^-(bits + 1) R C sqrt(|t_.j / C|^2 + |u_i. / R|^2),
+// whatever the entries; the squared norms are gathered with the forms.  A leaf
+// compares E with 2^-53 of what its sums and own terms came to, u_ij (t_ii - t_jj)
+// or 2 u_ij: half a unit in the last place, less than a float64 sum's own
+// roundings.  Where more than a quarter of a leaf's entries exceed that (or data
+// is not finite), a flag is set and the caller runs the plain float64 path.
+// Similar matrices D^-1 T D lose the same bits in every entry, so the test sees
+// any such grading, in whatever order; single entries that came out small by
+// cancellation stay below a quarter.  On ungraded data E is 2^-4 of the limit; D of two levels
+// passes up to about 2^5 between them (n = 1792).
 //
 // The kernels work on lists of superblocks of any number of problems (a batch
 // shares its launches), and on A X - X B = C as well, where every entry is of
@@ -52,7 +64,10 @@ constexpr int kThreads = 256;
 constexpr int kNoExp = INT_MIN / 2;
 constexpr int kHeadroom = 2;
 constexpr int kMinExp = -900;     // keeps 2^(bits - exp) a normal number
-constexpr int kWideBits = 24;
+constexpr int kNormBits = 14;     // squared norms count 2^-14
+// An entry's E may be 2^slack times 2^-53 of its sum: for X, whose plain path sums
+// in double-float (48 bits), more.
+constexpr int kSylvSlack = 4;
 // Where a level's products are summed ahead, beside the wave before: in runs of
 // kAheadLevels levels with sums or more, beside waves of at most kAheadTiles
 // superblocks.  Wider waves fill the float64 pipes and lose by the company (a
@@ -61,6 +76,9 @@ constexpr int kWideBits = 24;
 // n = 8192.
 constexpr size_t kAheadTiles = 64;
 constexpr int kAheadLevels = 4;
+// A run of one problem ends kTellLevels levels after a flag was set, where it has
+// kTellMin or more (the host lets no more than so many run ahead of it).
+constexpr int kTellLevels = 3, kTellMin = 8;
 
 namespace {
 
@@ -73,14 +91,16 @@ struct Problem {
     int ldrt, ldru, ldct, ldcu, ldc0, ldv;
     int rows, cols;
     double own2;                                // an entry's own term is own2 (u_pp - u_qq) / 2 C0
-    int bits;
+    int bits, slack;
     bool triangular;                            // V strictly upper, rows and columns the same
     int *er0, *ec0, *er1, *ec1;                 // exponents: V's rows, CT's columns, RT's rows, V's columns
+    unsigned *nr0, *nc0, *nr1, *nc1;            // squared norms of the converted part under these scales, in 2^-kNormBits
     int *rnew, *cnew;                           // of V's newest superblocks
     int *rgrown, *cgrown;                       // panels whose exponents grew
     __nv_bfloat16 *vr, *vc, *fm, *fn;           // row and column forms of V, row form of RT, column form of CT
     int nkbr, nkbc;                             // K-blocks over the rows (vc, fm) and over the columns (vr, fn)
     int *flags;
+    int *told;                                  // null, or the host's copy of "a flag is set"
 };
 
 struct Super {   // superblock (A, B) of problem k
@@ -92,6 +112,13 @@ struct Super {   // superblock (A, B) of problem k
 __device__ __forceinline__ int exponent_above(double x)   // |x| < 2^result
 {
     return ((__double2hiint(x) >> 20) & 0x7ff) - 1022;
+}
+
+// The problem is one for the plain path: 1 not finite, 2 not suited by one scale.
+__device__ __forceinline__ void raise(const Problem &p, int why)
+{
+    atomicOr(p.flags, why);
+    if (p.told) *static_cast<volatile int *>(p.told) = 1;
 }
 
 // A matrix read as rows x cols, or only its strictly upper part.
@@ -121,8 +148,14 @@ __global__ void __launch_bounds__(kThreads)
 init_exps_kernel(const Problem *__restrict__ probs)
 {
     const Problem p = probs[blockIdx.x];
-    for (int i = threadIdx.x; i < p.nkbr / 2 * SP; i += kThreads) p.er0[i] = p.er1[i] = p.rnew[i] = kNoExp;
-    for (int i = threadIdx.x; i < p.nkbc / 2 * SP; i += kThreads) p.ec0[i] = p.ec1[i] = p.cnew[i] = kNoExp;
+    for (int i = threadIdx.x; i < p.nkbr / 2 * SP; i += kThreads) {
+        p.er0[i] = p.er1[i] = p.rnew[i] = kNoExp;
+        p.nr0[i] = p.nr1[i] = 0;
+    }
+    for (int i = threadIdx.x; i < p.nkbc / 2 * SP; i += kThreads) {
+        p.ec0[i] = p.ec1[i] = p.cnew[i] = kNoExp;
+        p.nc0[i] = p.nc1[i] = 0;
+    }
 }
 
 // The largest exponents of the superblocks' rows (kRowOps), columns (kColOps)
@@ -151,7 +184,7 @@ exps_kernel(const Problem *__restrict__ probs, const Super *__restrict__ list, i
         int *re = what == kRowOps ? p.er1 : p.rnew, *ce = what == kColOps ? p.ec0 : p.cnew;
         if (what != kColOps) atomicMax(&re[t.A * SP + i], rmax[i]);
         if (what != kRowOps) atomicMax(&ce[t.B * SP + i], cmax[i]);
-        if (rmax[i] > 1024) atomicOr(p.flags, 1);
+        if (rmax[i] > 1024) raise(p, 1);
     }
 }
 
@@ -167,11 +200,14 @@ grow_exps_kernel(const Problem *__restrict__ probs, const Super *__restrict__ li
     const int er = p.rnew[r], ec = p.cnew[c];
     p.rnew[r] = kNoExp;
     p.cnew[c] = kNoExp;
-    if (er > 1024) atomicOr(p.flags, 1);
+    if (er > 1024) raise(p, 1);
     const bool rg = er > p.er0[r], cg = ec > p.ec1[c];
     if (rg) p.er0[r] = er + kHeadroom;
     if (cg) p.ec1[c] = ec + kHeadroom;
     const int ra = __syncthreads_or(rg), ca = __syncthreads_or(cg);
+    // all of a grown panel is converted anew, and its norms with it
+    if (ra) p.nr0[r] = 0;
+    if (ca) p.nc1[c] = 0;
     if (threadIdx.x == 0) { p.rgrown[t.A] = ra; p.cgrown[t.B] = ca; }
 }
 
@@ -201,9 +237,8 @@ __constant__ ConvConst c_conv = make_conv_const();
 constexpr int kConvParts = SP * SP / 8 / kThreads;
 __device__ __forceinline__ void convert_superblock(const Mat &M, int bits, bool rows,
                                                    int P, int K, int part, const int *__restrict__ exps,
-                                                   __nv_bfloat16 *__restrict__ tiles, int nkb, int *flags)
+                                                   unsigned *norms, __nv_bfloat16 *__restrict__ tiles, int nkb)
 {
-    int small = 0, some = 0;
     const int it = part * kThreads + threadIdx.x;
     {
         // line `i` of the panel, 8 entries along K from 8 ch: eight threads write
@@ -213,6 +248,7 @@ __device__ __forceinline__ void convert_superblock(const Mat &M, int bits, bool 
         const int g = P * SP + i;
         const int e = max(exps[g], kMinExp);
         float dig[8][5];
+        unsigned norm = 0;
 #pragma unroll
         for (int t = 0; t < 8; t++) {
             const int k = K * SP + ch * 8 + t;
@@ -224,10 +260,11 @@ __device__ __forceinline__ void convert_superblock(const Mat &M, int bits, bool 
             const int sh = (e - bits) - (ex - 1075);
             long long v = ex ? (x & 0xfffffffffffffll) | 0x10000000000000ll : 0;
             v = sh <= 0 ? v << min(-sh, 10) : sh < 63 ? (v + (1ll << (sh - 1))) >> sh : 0;
+            // its square, rounded up
+            const unsigned h = (unsigned)(v >> (bits - 12)) + 1;
+            norm += v ? (h * h >> (24 - kNormBits)) + 1 : 0;
             if (x < 0) v = -v;
-            some += ex != 0;
-            small += ex != 0 && ex - 1022 < e - kWideBits;
-            // bits <= 56: five balanced digits of 14 bits
+            // five balanced digits of 14 bits
 #pragma unroll
             for (int d = 0; d < 5; d++) {
                 const int r = ((int)(v & 16383) ^ 8192) - 8192;
@@ -258,9 +295,11 @@ __device__ __forceinline__ void convert_superblock(const Mat &M, int bits, bool 
             }
             *reinterpret_cast<uint4 *>(dst + (size_t)m * nkb * rns::kTileElems) = w;
         }
+        // (whole numbers: the sum does not depend on its order)
+        const int lanes = rows ? 8 : SP / 8;
+        for (int o = 1; o < lanes; o <<= 1) norm += __shfl_xor_sync(0xffffffffu, norm, o);
+        if (it % lanes == 0 && norm) atomicAdd(&norms[g], norm);
     }
-    some = __syncthreads_count(2 * small > some);   // threads most of whose entries are far below their scale
-    if (threadIdx.x == 0 && some > kThreads / 2) atomicOr(flags, 2);
 }
 
 // The operators' superblocks: row form of the rows' (kRowOps), column form of
@@ -271,9 +310,9 @@ convert_ops_kernel(const Problem *__restrict__ probs, const Super *__restrict__ 
     const Super t = list[blockIdx.x];
     const Problem p = probs[t.k];
     if (what == kRowOps)
-        convert_superblock(matrix_of(p, what), p.bits, true, t.A, t.B, blockIdx.y, p.er1, p.fm, p.nkbr, p.flags);
+        convert_superblock(matrix_of(p, what), p.bits, true, t.A, t.B, blockIdx.y, p.er1, p.nr1, p.fm, p.nkbr);
     else
-        convert_superblock(matrix_of(p, what), p.bits, false, t.B, t.A, blockIdx.y, p.ec0, p.fn, p.nkbc, p.flags);
+        convert_superblock(matrix_of(p, what), p.bits, false, t.B, t.A, blockIdx.y, p.ec0, p.nc0, p.fn, p.nkbc);
 }
 
 // V's new superblocks (A, B), and the whole of a panel whose scale grew: of row
@@ -289,11 +328,11 @@ convert_new_kernel(const Problem *__restrict__ probs, const Super *__restrict__ 
     if (blockIdx.z % 2 == 0) {
         const int count = 1 + (p.rgrown[t.A] ? t.B - (p.triangular ? t.A : 0) : 0);
         for (int y = blockIdx.y; y < count; y += gridDim.y)
-            convert_superblock(M, p.bits, true, t.A, t.B - y, part, p.er0, p.vr, p.nkbc, p.flags);
+            convert_superblock(M, p.bits, true, t.A, t.B - y, part, p.er0, p.nr0, p.vr, p.nkbc);
     } else {
         const int count = 1 + (p.cgrown[t.B] ? (p.triangular ? t.B : p.nkbr / 2 - 1) - t.A : 0);
         for (int y = blockIdx.y; y < count; y += gridDim.y)
-            convert_superblock(M, p.bits, false, t.B, t.A + y, part, p.ec1, p.vc, p.nkbr, p.flags);
+            convert_superblock(M, p.bits, false, t.B, t.A + y, part, p.ec1, p.nc1, p.vc, p.nkbr);
     }
 }
 
@@ -349,7 +388,8 @@ __constant__ CrtConst c_crt = make_crt_const();
 // the leaves fill.
 __device__ __forceinline__ double from_u32(unsigned x) { return __hiloint2double(0x43300000, (int)x) - 0x1p52; }
 
-// 2^k times the product an entry's residues stand for (16 bytes, 16 KB apart).
+// 2^k times the product an entry's residues stand for (kMods bytes, 16 KB apart).
+// 96 bits of its quotient by the moduli's product: off by 2^-68 R C.
 __device__ __forceinline__ double crt(const int8_t *y, int k)
 {
     unsigned long long a0 = 0, a1 = 0, a2 = 0;
@@ -384,18 +424,34 @@ struct Wave {
     int tiles, products;
 };
 
-// The residue sums of entry (i, j) of superblock t.
-__device__ __forceinline__ double residue_sum(const Wave &w, const Problem &pr, const Super &s, int t, int i, int j,
-                                              bool opp)
+// The exponent above sqrt(a + b), squared norms in 2^-kNormBits.
+__device__ __forceinline__ int norm_exp(unsigned a, unsigned b)
 {
+    const unsigned long long s = (unsigned long long)a + b;
+    return (65 - __clzll((long long)s) - kNormBits) >> 1;
+}
+
+// The residue sums of entry (i, j) of superblock t; off: the exponent of their
+// error E (far below any where there is none).
+__device__ __forceinline__ double residue_sum(const Wave &w, const Problem &pr, const Super &s, int t, int i, int j,
+                                              bool opp, int &off)
+{
+    off = -4000;
     if (w.products == 0) return 0.0;
     const int8_t *y = w.res + (size_t)t * w.products * rns::kMods * SP * SP + i * SP + j;
     const int r = s.A * SP + i, c = s.B * SP + j, b2 = 2 * pr.bits;
     // both kinds of entry take their first sum in one pass: UT, or UU
-    const int ec1 = max(pr.ec1[c], kMinExp), first = max(pr.er0[r], kMinExp) + (opp ? max(pr.ec0[c], kMinExp) : ec1);
+    const int er0 = max(pr.er0[r], kMinExp), ec1 = max(pr.ec1[c], kMinExp);
+    const int first = er0 + (opp ? max(pr.ec0[c], kMinExp) : ec1);
+    const unsigned nr0 = pr.nr0[r], nc = opp ? pr.nc0[c] : pr.nc1[c];
     const double v = crt(opp ? y : y + (size_t)2 * rns::kMods * SP * SP, first - b2);
+    // (of neighbouring superblocks A, B there are no products U U)
+    if (nr0 && nc && (opp || s.B > s.A + 1)) off = first + norm_exp(nr0, nc) - pr.bits - 1;
     if (!opp) return -v;
-    return v - crt(y + (size_t)rns::kMods * SP * SP, max(pr.er1[r], kMinExp) + ec1 - b2);
+    const int second = max(pr.er1[r], kMinExp) + ec1;
+    const unsigned nr1 = pr.nr1[r], nc1 = pr.nc1[c];
+    if (nr1 && nc1) off = max(off, second + norm_exp(nr1, nc1) - pr.bits - 1);
+    return v - crt(y + (size_t)rns::kMods * SP * SP, second - b2);
 }
 
 // Blocks (i, j) of a superblock at step l = 7 - i + j.
@@ -438,6 +494,7 @@ union WaveSmem {
         double T1[BLK], U1[BLK], T2[BLK], U2[BLK], X1[BLK], X2[BLK];
         double C[BLK], V[BLK];
         double urow[LB], ucol[LB];
+        short off[BLK];                     // residue_sum's errors
     } leaf;
     struct {
         double OT[2][BLK], OU[2][BLK], X[2][BLK];
@@ -553,7 +610,10 @@ __device__ __forceinline__ void wave_leaf(const Wave &wv, int b, int l, bool fir
     const double *M = opp ? s.TI : s.UI, *N = opp ? s.TJ : s.UJ;
     const double *M1 = opp ? s.T1 : s.U1, *N2 = opp ? s.T2 : s.U2;
     // here a thread takes entry (hi, lo): residues lie row by row
-    s.C[hi + lo * LD] = residue_sum(wv, w, k.s, k.t, (k.I % SB) * LB + hi, (k.J % SB) * LB + lo, lvl::signs_differ(s.urow[hi], s.ucol[lo]));
+    int off;
+    s.C[hi + lo * LD] = residue_sum(wv, w, k.s, k.t, (k.I % SB) * LB + hi, (k.J % SB) * LB + lo,
+                                    lvl::signs_differ(s.urow[hi], s.ucol[lo]), off);
+    s.off[hi + lo * LD] = (short)off;
     // own (u_ii - u_jj) = +-2 own
     s.V[at] = lvl::signs_differ(s.urow[lo], s.ucol[hi]) ? lvl::flip_sign(own, (unsigned long long)__double_as_longlong(s.urow[lo]) & 0x8000000000000000ull) * w.own2 : 0.0;
     __syncthreads();
@@ -597,6 +657,11 @@ __device__ __forceinline__ void wave_leaf(const Wave &wv, int b, int l, bool fir
     for (int o = 1; o < LB; o <<= 1) ec = max(ec, __shfl_xor_sync(0xffffffffu, ec, o));
     if ((threadIdx.x & 31) < LB && inr) atomicMax(&w.rnew[r0 + lo], er);
     if (lo == 0 && inc) atomicMax(&w.cnew[c0 + hi], ec);
+    if (wv.products == 0) return;
+    // what the sums and the own term came to: x (t_ii - t_jj) or 2 x
+    const int ev = e + (lvl::signs_differ(s.urow[lo], s.ucol[hi]) ? exponent_above(s.TI[lo * (LD + 1)] - s.TJ[hi * (LD + 1)]) - 1 : 1);
+    const int over = __syncthreads_count(some && s.off[at] > ev - 53 + w.slack);
+    if (threadIdx.x == 0 && 4 * over > min(LB, w.rows - r0) * min(LB, w.cols - c0)) raise(w, 2);
 }
 
 // Step l of every superblock of the launch: its leaves, and beside them the
@@ -664,7 +729,7 @@ size_t run_bytes(size_t problems, size_t superblocks, size_t ops, size_t widest,
 // A problem's exponents, growth marks and forms.
 size_t problem_bytes(int nr, int nc, bool forms)
 {
-    size_t b = 3 * ((size_t)(nr + nc) * SP * sizeof(int) + 512) + (size_t)(nr + nc) * sizeof(int) + 512;
+    size_t b = 5 * ((size_t)(nr + nc) * SP * sizeof(int) + 512) + (size_t)(nr + nc) * sizeof(int) + 512;
     if (forms)
         b += rns::form_tile_bytes(nr, 2 * nr) + rns::form_tile_bytes(nc, 2 * nc) + rns::form_tile_bytes(nr, 2 * nc) +
              rns::form_tile_bytes(nc, 2 * nr) + 4 * 256;
@@ -691,6 +756,10 @@ struct Run {
         p.ec0 = ints((size_t)nc * SP);
         p.ec1 = ints((size_t)nc * SP);
         p.cnew = ints((size_t)nc * SP);
+        p.nr0 = reinterpret_cast<unsigned *>(ints((size_t)nr * SP));
+        p.nr1 = reinterpret_cast<unsigned *>(ints((size_t)nr * SP));
+        p.nc0 = reinterpret_cast<unsigned *>(ints((size_t)nc * SP));
+        p.nc1 = reinterpret_cast<unsigned *>(ints((size_t)nc * SP));
         p.rgrown = ints(nr);
         p.cgrown = ints(nc);
         p.nkbr = 2 * nr;
@@ -707,8 +776,9 @@ struct Run {
     }
 
     // flags (host, one per problem): nonzero where the data did not suit one
-    // scale per row; waits for the stream.
-    signtri_status run(Arena &ws, int *d_err, int *flags, cudaStream_t st)
+    // scale per row; waits for the stream.  told: null, or (one problem) a
+    // pinned word the kernels can write
+    signtri_status run(Arena &ws, int *d_err, int *flags, int *told, cudaStream_t st)
     {
         const int np = (int)probs.size(), levels = (int)off.size() - 1;
         size_t widest = 0;
@@ -730,6 +800,7 @@ struct Run {
         for (int k = 0; k < np; k++) {
             Problem &p = probs[k];
             p.flags = d_flags + k;
+            p.told = told;
             src[3 * k] = {p.vr, p.fn, p.nkbc, p.nkbc, p.rgrown, nullptr};
             src[3 * k + 1] = {p.fm, p.vc, p.nkbr, p.nkbr, nullptr, p.cgrown};
             src[3 * k + 2] = {p.vr, p.vc, p.nkbc, p.nkbr, p.rgrown, p.cgrown};
@@ -783,7 +854,17 @@ struct Run {
         bool summed_ahead = false;
         const bool overlap = levels - sums_from >= kAheadLevels;
         if (overlap) SGT_CUDA_TRY(side.init());
+        const bool tell = told && levels >= kTellMin;
+        CallEvents behind;   // the last levels' ends
+        if (tell) {
+            *told = 0;
+            SGT_CUDA_TRY(behind.init(kTellLevels));
+        }
         for (int l = 0; l < levels; l++) {
+            if (tell && l >= kTellLevels) {
+                SGT_CUDA_TRY(cudaEventSynchronize(behind.e[l % kTellLevels]));
+                if (*static_cast<volatile int *>(told)) break;
+            }
             const size_t n = off[l + 1] - off[l];
             const Super *at = d_list + off[l];
             const bool with_sums = l >= sums_from;
@@ -814,6 +895,7 @@ struct Run {
             const Wave w{d_probs, at, res, (int)n, with_sums ? products : 0};
             if ((rs = run_wave(w, SB - nbr, SB - 1 + nbc, slab0, slab1, cls_leaf, st)) != SIGNTRI_OK) return rs;
             if (l + 1 < levels && (rs = join(at, n, l + 2)) != SIGNTRI_OK) return rs;
+            if (tell) SGT_CUDA_TRY(cudaEventRecord(behind.e[l % kTellLevels], st));
         }
         if (!sums) {   // nothing that could have set a flag
             for (int k = 0; k < np; k++) flags[k] = 0;
@@ -844,7 +926,8 @@ size_t ph_super_workspace_bytes(int count, const int *n)
     return b + run_bytes(count, superblocks, ops, widest, 3);
 }
 
-signtri_status ph_super_run(int count, const BatchDesc *mats, Arena &ws, int *d_err, int *flags, cudaStream_t st)
+signtri_status ph_super_run(int count, const BatchDesc *mats, Arena &ws, int *d_err, int *flags, int *told,
+                            cudaStream_t st)
 {
     using namespace sup;
     Run r;
@@ -878,7 +961,7 @@ signtri_status ph_super_run(int count, const BatchDesc *mats, Arena &ws, int *d_
             for (int A = 0; A + D < panels_of(mats[k].n); A++) r.list.push_back({k, A, A + D});
         r.off.push_back(r.list.size());
     }
-    return r.run(ws, d_err, flags, st);
+    return r.run(ws, d_err, flags, count == 1 ? told : nullptr, st);
 }
 
 // ---- A X - X B = C ----------------------------------------------------------------
@@ -907,7 +990,7 @@ size_t sylvester_super_workspace_bound(int n)
 
 signtri_status sylvester_super_run(int m, int p, const double *A, int lda, const double *B, int ldb, const double *C,
                                    int ldc, double cscale, double *X, int ldx, Arena &ws, int *d_err, int *flags,
-                                   cudaStream_t st)
+                                   int *told, cudaStream_t st)
 {
     using namespace sup;
     const int nr = panels_of(m), nc = panels_of(p);
@@ -929,6 +1012,7 @@ signtri_status sylvester_super_run(int m, int p, const double *A, int lda, const
     q.cols = p;
     q.own2 = cscale;   // (rows and columns stand for u = 1 and -1)
     q.bits = rns::operand_bits(std::max(nr, nc) * SP);
+    q.slack = kSylvSlack;
     if (!r.reserve(ws, q, nr, nc, nr + nc > 2)) return SIGNTRI_ERR_NO_WORKSPACE;
     r.probs.push_back(q);
     for (int a = 0; a < nr; a++)
@@ -939,7 +1023,7 @@ signtri_status sylvester_super_run(int m, int p, const double *A, int lda, const
         for (int b = std::max(0, s - (nr - 1)); b <= std::min(nc - 1, s); b++) r.list.push_back({0, nr - 1 - s + b, b});
         r.off.push_back(r.list.size());
     }
-    return r.run(ws, d_err, flags, st);
+    return r.run(ws, d_err, flags, told, st);
 }
 
 }  // namespace signtri

@@ -426,7 +426,8 @@ signtri_status sylvester_any_run(int m, int p, const double *A, int lda, const d
     const size_t mark = ws.used;
     if (ws.bytes - ws.used >= sylvester_super_workspace_bytes(m, p)) {
         const signtri_status rs =
-            sylvester_super_run(m, p, A, lda, Bm, ldb, C, ldc, cscale, X, ldx, ws, d_err, flags_host, st);
+            sylvester_super_run(m, p, A, lda, Bm, ldb, C, ldc, cscale, X, ldx, ws, d_err, flags_host,
+                                flags_host + 1, st);
         if (rs != SIGNTRI_OK || !*flags_host) return rs;
         ws.used = mark;
     }

@@ -1,20 +1,19 @@
 // rns.cu -- float64 products on the tensor cores through residues.
 //
 // GB300 multiplies float64 at 1.2 TFLOP/s and bf16 at 1.9 PFLOP/s.  A product
-// of integers is formed here modulo 16 pairwise coprime numbers up to 256
+// of integers is formed here modulo 18 pairwise coprime numbers up to 256
 // (the residue number system; Garner, "The residue number system", IRE Trans.
 // EC-8, 1959; for matrix products Ozaki, Uchino and Imamura, "Ozaki scheme
 // II", 2025): residues between -128 and 128 are exact in bf16, and a sum of
 // 960 of their products is an integer below 2^24, exact in the tensor
-// cores' fp32 accumulators.  Entries are first rounded to integers of 55 or so
+// cores' fp32 accumulators.  Entries are first rounded to integers of 62
 // bits under a power-of-two scale per row of the left operand and per column
 // of the right; the integer product, below half the moduli's product, comes
 // back from its residues by the Chinese remainder theorem.  So the only error
-// is that of rounding the entries to 2^-53 or less of their row's or column's
-// largest; the sums are exact.
+// is that of rounding the entries to 2^-63 of their scale; the sums are exact.
 //
-// 16 products instead of the 36 of eight 7-bit slices, and independent ones:
-// a 128 x 128 tile is 16 tasks, so a few tiles already fill the GPU.
+// 18 products instead of the 36 of eight 7-bit slices, and independent ones:
+// a 128 x 128 tile is 18 tasks, so a few tiles already fill the GPU.
 //
 // rns_gemm_kernel: persistent CTAs; a task is one (tile, modulus).  Warp 0
 // loads K-blocks of 64 of both panels, 16 KB each, stored in the swizzled

@@ -8,19 +8,24 @@
 namespace signtri {
 namespace rns {
 
-// Pairwise coprime moduli; their product is 2^125.3.
-constexpr int kMods = 16;
-constexpr int kModulus[kMods] = {256, 255, 253, 251, 247, 241, 239, 233, 229, 227, 223, 217, 211, 199, 197, 193};
+// Pairwise coprime moduli; their product is 2^140.4.  (With the first 16 of
+// them, 2^125.3, operands keep 55 bits at K = 8192 and their rounding is as large
+// as that of float64 sums on ungraded data: no room for data that spreads.)
+constexpr int kMods = 18;
+constexpr int kModulus[kMods] = {256, 255, 253, 251, 247, 241, 239, 233, 229, 227, 223, 217, 211, 199, 197, 193, 191, 181};
 constexpr int kPanel = 128;                    // rows of a panel, and edge of a product tile
 constexpr int kTileElems = kPanel * 64;        // one panel's K-block of 64, one modulus: 16 KB of bf16
 
 // Bits kept of each operand entry below its row's (column's) power-of-two
-// scale: products of K terms then stay below half the moduli's product.
+// scale: sums of K products then stay below half the moduli's product.  62 up to
+// K = 32768 (an entry's 53 bits whole down to 2^-9 of the scale), 61 up to
+// 131072; no more than 62, so that a rounded entry fits 63 bits and its sign.
 constexpr int operand_bits(int K)
 {
     int lg = 0;
-    while ((1 << lg) < K) lg++;
-    return (124 - lg) / 2;
+    while (lg < 30 && (1 << lg) < K) lg++;
+    const int b = (139 - lg) / 2;
+    return b < 62 ? b : 62;
 }
 
 // The residues of a matrix cut into panels of 128 rows (a row form: rows of

@@ -115,6 +115,83 @@ def test_superblocks_that_outgrow_their_scales(gpu_lib):
     assert np.linalg.norm(np.ldexp(U, g[:, None] - g[None, :]) - U0) <= n * np.finfo(float).eps * np.linalg.norm(U0)
 
 
+# T = D^-1 T0 D with D of powers of two, D^-1 sign(T0) D: float64 sums lose
+# nothing by it.  In D's scale every entry is compared: d of two levels, alternating
+# or at random, one index far from the others, and steps; from a level that the
+# residues' spare bits cover to ones that would lose every bit
+def _gradings(n):
+    rng = np.random.Generator(np.random.PCG64(n))
+    out = []
+    for g in (2, 5, 10, 20, 40, 60):
+        out += [np.arange(n) % 2 * g, rng.integers(0, 2, n) * g]
+    one = np.zeros(n, dtype=int)
+    one[n // 2] = 30
+    return out + [one, np.arange(n) // 100 % 3 * 12, -np.round(np.linspace(0.0, 20.0, n)).astype(int)]
+
+
+def _scaled(T0, d):
+    return np.asfortranarray(np.ldexp(T0, d[None, :] - d[:, None]))
+
+
+# an entry's sums round by about a unit in the last place in either form, and
+# pass on as much again: a few eps of the norm
+@pytest.mark.gpu
+def test_superblocks_of_interleaved_scales(gpu_lib):
+    n = 1800
+    T0 = make_T(n, 0.4, seed=8)
+    U0 = _plain(gpu_lib, T0)
+    for k, d in enumerate(_gradings(n)):
+        U = np.ldexp(_super(gpu_lib, _scaled(T0, d)), d[:, None] - d[None, :])
+        err = np.linalg.norm(U - U0) / np.linalg.norm(U0)
+        assert err <= 8 * np.finfo(float).eps, (k, err)
+
+
+@pytest.mark.gpu
+def test_batched_superblocks_of_interleaved_scales(gpu_lib):
+    import torch
+    p, n = gpu_lib, 700
+    T0 = make_T(n, 0.4, seed=9)
+    U0 = _plain(gpu_lib, T0)
+    ds = _gradings(n)
+    dev = [p.to_device(_scaled(T0, d)) for d in ds]
+    out = [torch.empty_like(t) for t in dev]
+    ns = [n] * len(ds)
+    st, info = p.sign_tri_batched(ns, [t.data_ptr() for t in dev], ns, [u.data_ptr() for u in out], ns,
+                                  p.Variant.PH_FP64_EFFICIENT, torch.cuda.current_stream().cuda_stream)
+    assert st == 0 and not any(info)
+    for k, d in enumerate(ds):
+        U = np.ldexp(p.to_numpy(out[k]), d[:, None] - d[None, :])
+        err = np.linalg.norm(U - U0) / np.linalg.norm(U0)
+        assert err <= 8 * np.finfo(float).eps, (k, err)
+
+
+# X of A X - X B = C, graded on either side and, by Parlett-Sylvester, on both.
+# The plain solve's sums are double-float, 48 bits and more: 2^-44
+@pytest.mark.gpu
+def test_sylvester_superblocks_of_interleaved_scales(gpu_lib):
+    import torch
+    p, n, q = gpu_lib, 900, 400
+    m = n - q
+    T0 = make_T(n, seed=10, n_neg=q, order="sorted")
+    U0 = _plain(p, T0)
+
+    def syl(T):
+        A, B, C = (p.to_device(np.asfortranarray(M)) for M in (T[:m, :m], T[m:, m:], T[:m, m:]))
+        X = p.to_device(np.zeros((m, q), order="F"))
+        st = torch.cuda.current_stream().cuda_stream
+        assert p.signtri_sylvester(m, q, A.data_ptr(), m, B.data_ptr(), q, C.data_ptr(), m, X.data_ptr(), m, st) == 0
+        torch.cuda.synchronize()
+        return p.to_numpy(X)
+    for k, d in enumerate(_gradings(n)):
+        T = _scaled(T0, d)
+        U = p.to_numpy(p.sign(p.to_device(T), p.Variant.PS_FP64))
+        torch.cuda.synchronize()
+        for X in (U[:m, m:], 2.0 * syl(T)):
+            X = np.ldexp(X, d[:m, None] - d[None, m:])
+            err = np.linalg.norm(X - U0[:m, m:]) / np.linalg.norm(U0)
+            assert err <= 2.0 ** -44, (k, err)
+
+
 # Parlett-Sylvester on a grouped diagonal: X of T11 X - X T22 = 2 T12 by
 # superblocks, whole ones, ragged rows, ragged columns, a few columns only
 @pytest.mark.gpu
