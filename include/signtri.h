@@ -205,8 +205,9 @@ signtri_status signtri_set_cutoff(int b);
    forms then enqueue their launches and return without waiting for them
    (from n = 1600 on with leaves of 16 they return after U is written);
    Parlett-Sylvester also waits while it builds its swap schedule from the
-   diagonal, and the mixed variants wait a few times (diagonal signs,
-   residual norms) and return after U is written.
+   diagonal and returns after U is written (unless no swap is needed and
+   neither sign has more than 128 eigenvalues), and the mixed variants wait a
+   few times (diagonal signs, residual norms) and return after U is written.
    n == 0 is a no-op returning SIGNTRI_OK.  n == 1 writes sign(t_11).
    If all t_ii > 0 (all < 0) U = I (U = -I) exactly (Section 3). */
 signtri_status sign_tri(int n, const double *T, int ldt, double *U, int ldu,
@@ -420,8 +421,8 @@ signtri_status signtri_reorder_by_sign(int n, const double *T, int ldt, double *
    where one scale per row or column does not suit the data (the rounding of a
    sum's operands would exceed double-float's, 2^-48 of it), the workspace has
    no room for them or `stream` is being captured, by blocks of 64 with
-   double-float sums.  Enqueued on `stream`; for m + p > 256 the host waits for
-   it (not in a capture).  m == 0 or p == 0 is a no-op. */
+   double-float sums.  Enqueued on `stream`; where there is more than one
+   superblock (m > 128 or p > 128) the host waits for it (not in a capture).  m == 0 or p == 0 is a no-op. */
 signtri_status signtri_sylvester(int m, int p, const double *A, int lda, const double *B, int ldb,
                                  const double *C, int ldc, double *X, int ldx, void *stream);
 

@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "internal.cuh"
+#include "super_plan.h"
 
 using namespace signtri;
 
@@ -296,9 +297,6 @@ signtri_status run_ph_fp64(int n, const double *T, int ldt, double *U, int ldu, 
         const BatchDesc m{T, U, n, ldt, ldu, 0};
         rs = ph_super_run(1, &m, ws, s.err_dev, flags, flags + 1, st);
         if (rs != SIGNTRI_OK) return rs;
-        SGT_CUDA_TRY(cudaMemcpyAsync(s.err_host, s.err_dev, sizeof(int), cudaMemcpyDeviceToHost, st));
-        SGT_CUDA_TRY(cudaStreamSynchronize(st));
-        if (*s.err_host) return SIGNTRI_ERR_TIMEOUT;
         if (!*flags) return SIGNTRI_OK;
         // entries that one scale per row does not suit, or not finite
     }
@@ -323,9 +321,9 @@ signtri_status run_variant(int n, const double *T, int ldt, double *U, int ldu, 
         SGT_CUDA_TRY(cudaMemsetAsync(s.err_dev, 0, sizeof(int), st));
         rs = ps_fp64_run(n, T, ldt, U, ldu, r.n_pos, r.swaps, ws, s.err_dev, reinterpret_cast<int *>(s.norms_host), st);
         if (rs != SIGNTRI_OK) return rs;
-        if ((r.swaps > 0 && n >= kBlockedReorderMin) || n > 256) {
-            // the tensor-core products (of the blocked reorder, of the
-            // Sylvester solve's superblocks) wait with a bound
+        if (ps_products(r.n_pos, r.n_neg, r.swaps)) {
+            // the tensor-core products (of the reorder, of the Sylvester
+            // solve's superblocks, of the back-transform) wait with a bound
             SGT_CUDA_TRY(cudaMemcpyAsync(s.err_host, s.err_dev, sizeof(int), cudaMemcpyDeviceToHost, st));
             SGT_CUDA_TRY(cudaStreamSynchronize(st));
             if (*s.err_host) return SIGNTRI_ERR_TIMEOUT;
@@ -471,9 +469,7 @@ signtri_status batched_float64(int cnt, const std::vector<BatchDesc> &h, const B
         for (size_t q = 0; q < run.size(); q++)
             if (flags[q]) plainly.push_back(large[i0 + q]);
     }
-    SGT_CUDA_TRY(cudaMemcpyAsync(s.err_host, s.err_dev, sizeof(int), cudaMemcpyDeviceToHost, st));
-    SGT_CUDA_TRY(cudaStreamSynchronize(st));
-    return *s.err_host ? SIGNTRI_ERR_TIMEOUT : SIGNTRI_OK;
+    return SIGNTRI_OK;
 }
 
 // Synthetic upper-triangular T for the autotuner: counter-based hash
@@ -1117,7 +1113,7 @@ signtri_status signtri_sylvester(int m, int p, const double *A, int lda, const d
     SGT_CUDA_TRY(cudaMemsetAsync(s->err_dev, 0, sizeof(int), st));
     rs = sylvester_any_run(m, p, A, lda, B, ldb, C, ldc, 1.0, X, ldx, ws, s->err_dev,
                            reinterpret_cast<int *>(s->norms_host), st);
-    if (rs != SIGNTRI_OK || m + p <= 256) return rs;
+    if (rs != SIGNTRI_OK || !sylvester_products(m, p)) return rs;
     SGT_CUDA_TRY(cudaMemcpyAsync(s->err_host, s->err_dev, sizeof(int), cudaMemcpyDeviceToHost, st));
     SGT_CUDA_TRY(cudaStreamSynchronize(st));
     return *s->err_host ? SIGNTRI_ERR_TIMEOUT : SIGNTRI_OK;

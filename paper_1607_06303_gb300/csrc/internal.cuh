@@ -133,7 +133,8 @@ signtri_status ph_fp64_near_run(int n, const double *T, int ldt, double *U, int 
 // superblocks of 128, their sums on the tensor cores (ph_super.cu): everything
 // beyond the diagonal superblocks (ph_fp64_near_run with last = 7) of `count`
 // problems.  flags (host): nonzero where a problem's data did not suit one
-// scale per row and it has to be run plainly; waits for the stream.  told: null,
+// scale per row and it has to be run plainly; waits for the stream and returns
+// SIGNTRI_ERR_TIMEOUT where a product's wait ran out.  told: null,
 // or a pinned word by which a single problem's kernels end the run early.
 constexpr int kSuperNear = 7;
 size_t ph_super_workspace_bytes(int count, const int *n);

@@ -49,6 +49,7 @@
 #include "internal.cuh"
 #include "ph_level.cuh"
 #include "rns.cuh"
+#include "super_plan.h"
 
 namespace signtri {
 namespace sup {
@@ -58,7 +59,8 @@ using lvl::LB;
 using lvl::LD;
 using lvl::LT;
 
-constexpr int SP = rns::kPanel;   // superblock edge
+constexpr int SP = kSuperEdge;
+static_assert(SP == rns::kPanel, "a superblock is a product tile");
 constexpr int SB = SP / LB;       // blocks of 16 per edge
 constexpr int kThreads = 256;
 constexpr int kNoExp = INT_MIN / 2;
@@ -717,7 +719,7 @@ size_t wave_slab_bytes(size_t tiles) { return tiles * SB * kParts * LT * sizeof(
 
 // ---- host side -------------------------------------------------------------------
 
-int panels_of(int n) { return (n + SP - 1) / SP; }
+int panels_of(int n) { return super_panels(n); }
 
 // What a run of `levels` of superblocks works in besides its problems' own.
 size_t run_bytes(size_t problems, size_t superblocks, size_t ops, size_t widest, int products)
@@ -776,8 +778,9 @@ struct Run {
     }
 
     // flags (host, one per problem): nonzero where the data did not suit one
-    // scale per row; waits for the stream.  told: null, or (one problem) a
-    // pinned word the kernels can write
+    // scale per row.  Where products run, waits for the stream and reads the
+    // error word of their waits.  told: null, or (one problem) a pinned word the
+    // kernels can write
     signtri_status run(Arena &ws, int *d_err, int *flags, int *told, cudaStream_t st)
     {
         const int np = (int)probs.size(), levels = (int)off.size() - 1;
@@ -901,9 +904,12 @@ struct Run {
             for (int k = 0; k < np; k++) flags[k] = 0;
             return SIGNTRI_OK;
         }
+        int err = 0;
         SGT_CUDA_TRY(cudaMemcpyAsync(flags, d_flags, np * sizeof(int), cudaMemcpyDeviceToHost, st));
+        if (overlap) SGT_CUDA_TRY(cudaStreamSynchronize(side.s));   // products beside the last wave
+        SGT_CUDA_TRY(cudaMemcpyAsync(&err, d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
         SGT_CUDA_TRY(cudaStreamSynchronize(st));
-        return SIGNTRI_OK;
+        return err ? SIGNTRI_ERR_TIMEOUT : SIGNTRI_OK;
     }
 };
 

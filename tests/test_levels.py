@@ -24,6 +24,17 @@ def test_level_split(tmp_path):
     assert out.stdout.startswith("ok ")
 
 
+@pytest.mark.skipif(shutil.which("g++") is None, reason="needs g++")
+def test_calls_with_bounded_waits(tmp_path):
+    exe = str(tmp_path / "super_plan_check")
+    csrc = os.path.join(ROOT, "paper_1607_06303_gb300", "csrc")
+    subprocess.run(["g++", "-std=c++17", "-O2", "-Wall", "-I", csrc,
+                    os.path.join(ROOT, "tests", "super_plan_check.cpp"), "-o", exe], check=True)
+    out = subprocess.run([exe], capture_output=True, text=True)
+    assert out.returncode == 0, out.stdout
+    assert out.stdout.startswith("ok ")
+
+
 # one block and a ragged one (17, 31), the first anti-diagonals whose near
 # blocks coincide or touch the diagonal (33 .. 65), an odd ordinary order, and
 # more leaves than SMs (2449: two CTAs on an SM)
