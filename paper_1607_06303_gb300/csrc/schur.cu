@@ -45,6 +45,7 @@
 
 #include <cooperative_groups.h>
 
+#include "apply_window.h"
 #include "df_arith.cuh"
 #include "internal.cuh"
 
@@ -1127,8 +1128,8 @@ apply_rotations_kernel(int n, double2 *T, int ldt, double2 *Q, int ldq, const in
         const int l = s0.l, L = s0.i - s0.l;
         // step t of group g: u = t - 2 g; u = 0 takes the entry l over, u in
         // [1, L] is rotation l + u - 1, u = L + 1 passes the last entry on
-        auto load_c = [&](int u) { return u >= 1 && u <= L ? rclog[sr.off + u - 1] : 1.0; };
-        auto load_s = [&](int u) { return u >= 1 && u <= L ? rslog[sr.off + u - 1] : zero; };
+        auto load_c = [&](int u) { return apply_reads(g, nb, u, L) ? rclog[sr.off + u - 1] : 1.0; };
+        auto load_s = [&](int u) { return apply_reads(g, nb, u, L) ? rslog[sr.off + u - 1] : zero; };
         auto load_e = [&](int t) { return g == 0 && t <= L ? line[(size_t)(l + t) * stride] : zero; };
         double r = 0.0;
         double c0 = load_c(-2 * g), c1 = load_c(1 - 2 * g);
@@ -1279,9 +1280,10 @@ signtri_status schur_run(int n, const double *A, int lda, double *Q, int ldq, do
     auto *y = static_cast<double *>(ws.take((size_t)2 * n * sizeof(double)));
     auto *bad = static_cast<int *>(ws.take(sizeof(int)));
     auto *qs = static_cast<QrState *>(ws.take(sizeof(QrState)));
-    // a launch logs fewer than budget + 2n rotations (it starts a multi-sweep
-    // only below the budget, a multi-sweep has at most 2 (n - 1)) and no
-    // more sweeps; launches alternate between two logs
+    // a launch's log has room for nlog rotations, and as many sweeps: the kernel
+    // starts a multi-sweep only where all of its bulges' fit, with two bulges
+    // where the window has more than they leave room for (two sweeps of a full
+    // window, 2 (n - 1), always fit); launches alternate between two logs
     const size_t nlog = rotation_room(n);
     auto *sweeplog = static_cast<SweepRec *>(ws.take(2 * nlog * sizeof(SweepRec)));
     auto *rclog = static_cast<double *>(ws.take(2 * nlog * sizeof(double)));

@@ -15,7 +15,10 @@ checked without a GPU:
   - the batched path's per-level task tables (csrc/batched_plan.h: every
     tile's block sums once, slots disjoint) and its workspace bound, which
     must hold for every subset of a batch's matrices, by
-    tests/batched_plan_check.cpp."""
+    tests/batched_plan_check.cpp;
+  - the Schur sweeps' logged rotations that the apply kernel reads
+    (csrc/apply_window.h: inside their own sweep's record, each once), by
+    tests/apply_window_check.cpp."""
 import os
 import shutil
 import subprocess
@@ -63,3 +66,8 @@ def test_reorder_rounds(tmp_path):
 @pytest.mark.skipif(shutil.which("g++") is None, reason="needs g++")
 def test_batched_plan_and_workspace_bound(tmp_path):
     _compile_and_run(tmp_path, "batched_plan_check.cpp")
+
+
+@pytest.mark.skipif(shutil.which("g++") is None, reason="needs g++")
+def test_apply_reads(tmp_path):
+    _compile_and_run(tmp_path, "apply_window_check.cpp")
