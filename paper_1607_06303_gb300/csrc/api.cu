@@ -418,7 +418,9 @@ constexpr size_t kBatchSuperRoom = (size_t)32 << 30;
 bool batch_super(int n, int b) { return b == 16 && n >= kBatchSuperMin; }
 
 // Workspace the superblocks of a batch's problems (orders n, leaf sizes b) are
-// given: all of them at once, up to kBatchSuperRoom.
+// given: all of them at once, up to kBatchSuperRoom.  batched_float64 asks for no
+// more than what is counted here, so that what runs does not depend on how far
+// earlier calls have grown the workspace.
 size_t batch_super_need(const std::vector<int> &n, const std::vector<int> &b)
 {
     std::vector<int> ns;
@@ -443,7 +445,7 @@ signtri_status batched_float64(int cnt, const std::vector<BatchDesc> &h, const B
     std::vector<int> large;
     const size_t room = ws.bytes - ws.used;
     for (int k = 0; k < cnt; k++)
-        if (b[k] && batch_super(h[k].n, b[k]) && ph_super_workspace_bytes(1, &h[k].n) + 4096 <= room) {
+        if (b[k] && batch_super(h[k].n, b[k]) && ph_super_workspace_bytes(1, &h[k].n) <= room) {
             near[k] = 1;
             large.push_back(k);
         }
@@ -459,7 +461,7 @@ signtri_status batched_float64(int cnt, const std::vector<BatchDesc> &h, const B
         const size_t i0 = i;
         while (i < large.size()) {
             ns.push_back(h[large[i]].n);
-            if (!run.empty() && ph_super_workspace_bytes((int)ns.size(), ns.data()) + 4096 > room) break;
+            if (!run.empty() && ph_super_workspace_bytes((int)ns.size(), ns.data()) > room) break;
             run.push_back(h[large[i++]]);
         }
         std::vector<int> flags(run.size());
@@ -581,7 +583,7 @@ signtri_status sign_tri_batched(int count, const int *n, const double *const *T,
         if (!ns.empty()) plan = std::max(plan, batched_workspace_bytes((int)ns.size(), ns.data(), B));
     }
     const size_t fixed = (size_t)cnt * (sizeof(BatchDesc) + sizeof(ScanResult) + sizeof(int) + sizeof(double)) +
-                         8 * 256;
+                         8 * 256;   // (four arrays, each rounded up to 256 bytes)
     Arena ws;
     rs = get_workspace(*s, fixed + std::max(plan, batch_super_need(sizes, bs)), ws);
     if (rs == SIGNTRI_ERR_NO_WORKSPACE) rs = get_workspace(*s, fixed + plan, ws);   // without superblocks

@@ -261,3 +261,39 @@ def test_batched_superblocks_vs_oracle(gpu_lib, oracle_mod):
         if k == 3:   # entries of very different size: compared at one size
             U, ref = np.ldexp(U, g[:, None] - g[None, :]), np.ldexp(ref, g[:, None] - g[None, :])
         assert np.linalg.norm(U - ref) <= ns[k] * np.finfo(float).eps * np.linalg.norm(ref), k
+
+
+# what a batch runs does not depend on how far earlier calls have grown the
+# workspace: the same bits from the first call of a process and after a larger
+# one (superblocks and float64 sums round differently)
+_FIRST_BATCH = """
+import numpy as np, torch
+import paper_1607_06303_gb300 as p
+from paper_1607_06303_gb300.inputs import make_T
+
+def batch(ns):
+    dev = [p.to_device(make_T(n, 0.4, seed=n)) for n in ns]
+    out = [torch.empty_like(t) for t in dev]
+    st, info = p.sign_tri_batched(ns, [t.data_ptr() for t in dev], ns, [u.data_ptr() for u in out], ns,
+                                  p.Variant.PH_FP64_EFFICIENT, torch.cuda.current_stream().cuda_stream)
+    assert st == 0 and not any(info)
+    return out
+
+p.load()
+sizes = [[%s]]
+first = [batch(ns) for ns in sizes]
+p.sign(p.to_device(make_T(3000, 0.4, seed=1)), p.Variant.PH_FP64_EFFICIENT)
+again = [batch(ns) for ns in sizes]
+for a, b in zip(first, again):
+    for x, y in zip(a, b):
+        assert torch.equal(x, y), x.shape
+print("same")
+"""
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("ns", ["1024", "513, 1200, 640, 90"])
+def test_batch_in_a_fresh_process(gpu_lib, ns):
+    import sys
+    out = subprocess.run([sys.executable, "-c", _FIRST_BATCH % ns], capture_output=True, text=True, cwd=ROOT)
+    assert out.returncode == 0 and out.stdout.strip() == "same", out.stderr[-2000:]
