@@ -153,4 +153,29 @@ __device__ __forceinline__ double recip(double d)
     return fma(r, fma(e, e, e), r);
 }
 
+// A divisor as 1 / d = r 2^ex, so that r is a normal number over d's whole range:
+// ex is 0 but for |d| below 2^-959 or from 2^959 on.
+template <class S>
+struct Divisor {
+    S r;
+    int ex;
+};
+__device__ __forceinline__ int divisor_shift(int field)   // of d's exponent field
+{
+    return field < 64 ? 64 : field > 1982 ? -64 : 0;
+}
+__device__ __forceinline__ int exponent_field(double d) { return (__double2hiint(d) >> 20) & 0x7ff; }
+__device__ __forceinline__ double power_of_2(int e) { return __hiloint2double((1023 + e) << 20, 0); }
+// by the division, and by recip
+__device__ __forceinline__ Divisor<double> divisor(double d)
+{
+    const int ex = divisor_shift(exponent_field(d));
+    return {1.0 / (ex ? d * power_of_2(ex) : d), ex};
+}
+__device__ __forceinline__ Divisor<double> divisor_recip(double d)
+{
+    const int ex = divisor_shift(exponent_field(d));
+    return {recip(ex ? d * power_of_2(ex) : d), ex};
+}
+
 }  // namespace signtri

@@ -459,7 +459,8 @@ corr_diag_leaf_kernel(int n, const double *__restrict__ T, int ldt, const double
         s += __shfl_xor_sync(0xffffffffu, s, 2);
         if (live && part == 0) {
             s += Es[i + j * LD];
-            Es[i + j * LD] = s * (opp ? recip(Ts[i + i * LD] - Ts[j + j * LD]) : copysign(0.5, Ts[i + i * LD]));
+            const Divisor<double> dv = divisor_recip(Ts[i + i * LD] - Ts[j + j * LD]);
+            Es[i + j * LD] = opp ? s * dv.r * power_of_2(dv.ex) : s * copysign(0.5, Ts[i + i * LD]);
         }
         __syncthreads();
     }

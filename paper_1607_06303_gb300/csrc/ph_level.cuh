@@ -34,6 +34,7 @@
 
 #include <algorithm>
 
+#include "df_arith.cuh"
 #include "internal.cuh"
 #include "level_split.h"
 #include "ph_bodies.cuh"
@@ -85,17 +86,46 @@ template <>
 __device__ __forceinline__ double real_value<double>(double r) { return r; }
 template <>
 __device__ __forceinline__ double2 real_value<double2>(double r) { return make_double2(r, 0.0); }
-// 1 / (a - b); complex by R. L. Smith's algorithm (CACM 5(8), 1962)
-__device__ __forceinline__ double inv_diff(double a, double b) { return 1.0 / (a - b); }
-__device__ __forceinline__ double2 inv_diff(double2 a, double2 b)
+__device__ __forceinline__ double sub(double a, double b) { return a - b; }
+__device__ __forceinline__ double2 sub(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
+__device__ __forceinline__ bool finite(double a) { return (__double2hiint(a) & 0x7ff00000) != 0x7ff00000; }
+__device__ __forceinline__ bool finite(double2 a) { return finite(a.x) && finite(a.y); }
+// complex 1 / d by R. L. Smith's algorithm (CACM 5(8), 1962)
+__device__ __forceinline__ Divisor<double2> divisor(double2 d)
 {
-    const double x = a.x - b.x, y = a.y - b.y;
+    const int ex = divisor_shift(max((__double2hiint(d.x) >> 20) & 0x7ff, (__double2hiint(d.y) >> 20) & 0x7ff));
+    if (ex) d = scaled(d, power_of_2(ex));
+    const double x = d.x, y = d.y;
     if (fabs(x) >= fabs(y)) {
         const double r = y / x, den = fma(y, r, x);
-        return make_double2(1.0 / den, -r / den);
+        return {make_double2(1.0 / den, -r / den), ex};
     }
     const double r = x / y, den = fma(x, r, y);
-    return make_double2(r / den, -1.0 / den);
+    return {make_double2(r / den, -1.0 / den), ex};
+}
+using signtri::divisor;
+// c + a b with one rounding of c's size (mac of complex entries has two)
+__device__ __forceinline__ double mac_once(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ double2 mac_once(double2 a, double2 b, double2 c)
+{
+    return add(make_double2(fma(a.x, b.x, -(a.y * b.y)), fma(a.x, b.y, a.y * b.x)), c);
+}
+// base / d + sum / d, the first quotient given
+template <class S>
+__device__ __forceinline__ S add_quotient(S sum, const Divisor<S> &dv, S quot)
+{
+    if (dv.ex == 0) return mac_once(sum, dv.r, quot);
+    return add(scaled(mac(sum, dv.r, real_value<S>(0.0)), power_of_2(dv.ex)), quot);
+}
+// base / d: the product with 1 / d and one step of iterative refinement, as
+// accurate as a division
+template <class S>
+__device__ __forceinline__ S quotient(S base, S d, const Divisor<S> &dv)
+{
+    const S zero = real_value<S>(0.0);
+    S x = add_quotient(base, dv, zero);
+    if (dv.ex == 0 && finite(x)) x = mac_once(nmac(d, x, base), dv.r, x);
+    return x;
 }
 
 // barrier of one half of a CTA
@@ -203,7 +233,9 @@ __device__ __forceinline__ void far_sums(int n, const S *__restrict__ T, int ldt
     }
     const bool any_opp = __any_sync(0xffffffffu, opp), all_opp = __all_sync(0xffffffffu, opp);
     // acc restarts every few K-blocks, its sum so far added to `total`: long
-    // sums round as two short chains, at 1 addition in 64 terms
+    // sums round as two short chains, at 1 addition in 64 terms (in 16 products of
+    // one kind where the entries are complex, whose products round twice: error
+    // against 64 bits at n = 1000 7.8e-17 -> 6.3e-17)
     S acc = real_value<S>(0.0), total = acc;
     __syncthreads();   // the buffers may still be read for the CTA's work before
     for (int kb = kb0 + half, buf = 0; kb < kb1; kb += 2, buf ^= 1) {
@@ -215,21 +247,26 @@ __device__ __forceinline__ void far_sums(int n, const S *__restrict__ T, int ldt
         BT[hi * LD + lo] = bt;
         half_sync(half);
         if (kb + 2 < kb1) fetch(kb + 2);
+        S acc2 = real_value<S>(0.0);
         const S *A1 = AU + p, *A2 = AT + p, *B1 = (opp ? BT : BU) + q * LD, *B2 = BU + q * LD;
         if (kb >= I + 2 && kb <= J - 2) {
             if (all_opp) {
 #pragma unroll (sizeof(S) == 8 ? LB : LB / 4)
                 for (int k = 0; k < LB; k++) {
                     acc = mac(A1[k * LB], B1[k], acc);
-                    acc = nmac(A2[k * LB], B2[k], acc);
+                    S &second = sizeof(S) == 16 ? acc2 : acc;
+                    second = nmac(A2[k * LB], B2[k], second);
                 }
+                if (sizeof(S) == 16) acc = add(acc, acc2);
             } else if (any_opp) {
 #pragma unroll 4
                 for (int k = 0; k < LB; k++) {
                     acc = mac(A1[k * LB], B1[k], acc);
-                    const S r = nmac(A2[k * LB], B2[k], acc);
-                    if (opp) acc = r;
+                    S &second = sizeof(S) == 16 ? acc2 : acc;
+                    const S r = nmac(A2[k * LB], B2[k], second);
+                    if (opp) second = r;
                 }
+                if (sizeof(S) == 16) acc = add(acc, acc2);
             } else {
 #pragma unroll (sizeof(S) == 8 ? LB : LB / 4)
                 for (int k = 0; k < LB; k++) acc = mac(A1[k * LB], B1[k], acc);
@@ -254,7 +291,7 @@ __device__ __forceinline__ void far_sums(int n, const S *__restrict__ T, int ldt
                 }
             }
         }
-        if (((kb - kb0) & 6) == 6) {
+        if (sizeof(S) == 16 || ((kb - kb0) & 6) == 6) {
             total = add(total, acc);
             acc = real_value<S>(0.0);
         }
@@ -285,37 +322,58 @@ __device__ __forceinline__ void entry_of(int t, int &p, int &q)
     if (t >= 136) { p = LB - 1 - p; q = LB - 1 - q; }
 }
 
-// The block's solve: the thread's entry (p, q) starts as acc (the sums of all
-// terms outside the block) and base (its own term), and takes
-//   - M[p, k] v_kq (k > p)   and   + v_pk N[k, q] (k < q; sign flipped by flip)
-// as the entries of V are solved, step by step; V must not be in use.  The
-// base is as a rule far larger than the other terms, so it joins them last,
-// when only the terms of one step are still to come.
-template <class S>
-__device__ __forceinline__ void solve16(S acc, S base, S rinv, unsigned long long flip, const S *M, const S *N, S *V,
-                                        int p, int q, int step)
+// The block's solve: the thread's entry (p, q) starts as the quotients by its
+// divisor of its own term (quot) and of `outside`, the sum of all terms outside
+// the block, and takes
+//   - M[p, k] v_kq / d (k > p)   and   + v_pk N[k, q] / d (k < q; sign flipped by flip)
+// as the entries of V are solved, step by step; V must not be in use.  The terms of
+// the block are summed by themselves and the quotients join in the last
+// operation: the sums and the reciprocal then round in proportion to the sums,
+// which are as a rule smaller than the entry's own term.  (Everything added to one sum and
+// multiplied by the reciprocal: errors against 64 bits of 8.1e-17, 8.6e-17,
+// 7.6e-17 at n = 256, 1001, 8192, now 6.1e-17, 6.8e-17, 5.9e-17; complex n = 1000
+// 9.2e-17, now 6.2e-17.)  Complex entries, whose products are separate
+// instructions, add `outside` to the block's sum, so that only one addition
+// rounds by the entry's own size.
+// scaled: a warp with a divisor that is (dv.ex; else dv.ex is not looked at).  A
+// warp's entries have up to five steps: before and after these it forms none
+// (formed under a condition of the lane alone, the quotient's multiply-add is
+// issued by every warp at every step: 15 % of the leaf's float64 instructions).
+template <bool kScaled, class S>
+__device__ __forceinline__ void solve_steps(S outside, S quot, const Divisor<S> &dv, unsigned long long flip,
+                                            const S *M, const S *N, S *V, int p, int q, int step)
 {
-    if (step == 0) acc = add(acc, base);
-    half_sync(0);   // every base is read: V now takes the solution
-    for (int st = 0; st < 2 * LB - 1; st++) {
-        if (step == st || step == st + 1) {
-            // the entry's value, or its base term: one instruction for both
-            // kinds of lane (x * 1 + base and x * rinv - 0 round as the plain
-            // sum and product)
-            const bool now = step == st;
-            acc = mac(acc, now ? rinv : real_value<S>(1.0), now ? real_value<S>(-0.0) : base);
-            if (now) V[p + q * LD] = acc;
+    constexpr bool kComplex = sizeof(S) == 16;
+    auto by_d = [&](S x, S base) { return kScaled ? add_quotient(x, dv, base) : mac_once(x, dv.r, base); };
+    if (!kComplex) quot = by_d(outside, quot);
+    S acc = real_value<S>(0.0);
+    auto take = [&](int st) {
+        const int k1 = LB - 1 + q - st;   // solved at this step in the entry's column ...
+        const int k2 = st - (LB - 1) + p;   // ... and in its row
+        if (k2 >= 0) {
+            acc = mac(flip_sign(V[p + k2 * LD], flip), N[k2 + q * LD], acc);
         }
+        if (k1 < LB) acc = nmac(M[p + k1 * LD], V[k1 + q * LD], acc);
+    };
+    const int lo = __reduce_min_sync(0xffffffffu, step), hi = __reduce_max_sync(0xffffffffu, step);
+    int st = 0;
+    for (; st < lo; st++) {
         half_sync(0);
-        if (st < step) {
-            const int k1 = LB - 1 + q - st;   // solved at this step in the entry's column ...
-            const int k2 = st - (LB - 1) + p;   // ... and in its row
-            if (k2 >= 0) {
-                acc = mac(flip_sign(V[p + k2 * LD], flip), N[k2 + q * LD], acc);
-            }
-            if (k1 < LB) acc = nmac(M[p + k1 * LD], V[k1 + q * LD], acc);
-        }
+        take(st);
     }
+    for (; st <= hi; st++) {
+        if (step == st) V[p + q * LD] = by_d(kComplex ? add(outside, acc) : acc, quot);
+        half_sync(0);
+        if (st < step) take(st);
+    }
+    for (; st < 2 * LB - 1; st++) half_sync(0);
+}
+template <class S>
+__device__ __forceinline__ void solve16(S outside, S quot, const Divisor<S> &dv, bool scaled, unsigned long long flip,
+                                        const S *M, const S *N, S *V, int p, int q, int step)
+{
+    if (!scaled) solve_steps<false>(outside, quot, dv, flip, M, N, V, p, q, step);
+    else solve_steps<true>(outside, quot, dv, flip, M, N, V, p, q, step);
 }
 
 // Leaf of block (I, J): nslab partial slabs from slab0 on, LT doubles each.
@@ -359,7 +417,8 @@ __device__ __forceinline__ void leaf(int n, const S *__restrict__ T, int ldt, S 
     const S upp = s.urow[p], uqq = s.ucol[q];
     const bool opp = general || signs_differ(re(upp), re(uqq));
     // signs agree: 1 / (u_pp + u_qq) is +-1/2 exactly
-    const S rinv = opp ? inv_diff(s.TI[p + p * LD], s.TJ[q + q * LD]) : scaled(upp, 0.5);
+    const S dif = sub(s.TI[p + p * LD], s.TJ[q + q * LD]);
+    const Divisor<S> dv = opp ? divisor(dif) : Divisor<S>{scaled(upp, 0.5), 0};
     // flips the sign of the row terms where the signs agree
     const unsigned long long flip = opp ? 0ull : 0x8000000000000000ull;
     const S *M = opp ? s.TI : s.UI, *N = opp ? s.TJ : s.UJ;
@@ -369,6 +428,9 @@ __device__ __forceinline__ void leaf(int n, const S *__restrict__ T, int ldt, S 
     const double ui = re(s.urow[lo]), uj = re(s.ucol[hi]);
     const bool o = general || signs_differ(ui, uj);
     s.V[at] = o ? scaled(tij, ui - uj) : zero;
+    half_sync(0);
+    const S quot = opp ? quotient(s.V[p + q * LD], dif, dv) : zero;
+    const bool far = __any_sync(0xffffffffu, dv.ex != 0);
 
     dependency_wait();
     dependency_release();
@@ -406,18 +468,19 @@ __device__ __forceinline__ void leaf(int n, const S *__restrict__ T, int ldt, S 
     s.C[at] = o ? sum : flip_sign(sum, 0x8000000000000000ull);
     half_sync(0);
     S acc = s.C[p + q * LD];
-    const S base = s.V[p + q * LD];
     if (d >= 2) {
+        S col = zero, row = zero;
         // (d = 2: both near blocks are the same, and a sum of U U counts it once)
-        const bool row = d > 2 || opp;
+        const bool both = d > 2 || opp;
 #pragma unroll (sizeof(S) == 8 ? 8 : 4)
         for (int k = 0; k < LB; k++) {
-            acc = nmac(M1[p + k * LD], s.X1[k + q * LD], acc);
-            const S r = mac(flip_sign(s.X2[p + k * LD], flip), N2[k + q * LD], acc);
-            if (row) acc = r;
+            col = nmac(M1[p + k * LD], s.X1[k + q * LD], col);
+            row = mac(flip_sign(s.X2[p + k * LD], flip), N2[k + q * LD], row);
         }
+        if (both) col = add(col, row);
+        acc = add(acc, col);
     }
-    solve16(acc, base, rinv, flip, M, N, s.V, p, q, step);
+    solve16(acc, quot, dv, far, flip, M, N, s.V, p, q, step);
     if (in) SGT_AT(U, ldu, r0 + lo, c0 + hi) = s.V[at];
 }
 

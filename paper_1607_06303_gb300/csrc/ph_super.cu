@@ -607,7 +607,9 @@ __device__ __forceinline__ void wave_leaf(const Wave &wv, int b, int l, bool fir
     const double upp = s.urow[p], uqq = s.ucol[q];
     const bool opp = lvl::signs_differ(upp, uqq);
     const bool live = r0 + p < w.rows && c0 + q < w.cols;
-    const double rinv = !live ? 0.0 : opp ? recip(s.TI[p + p * LD] - s.TJ[q + q * LD]) : copysign(0.5, upp);
+    const double dif = s.TI[p + p * LD] - s.TJ[q + q * LD];
+    Divisor<double> dv = !live ? Divisor<double>{0.0, 0}
+                               : opp ? divisor_recip(dif) : Divisor<double>{copysign(0.5, upp), 0};
     const unsigned long long flip = opp ? 0ull : 0x8000000000000000ull;
     const double *M = opp ? s.TI : s.UI, *N = opp ? s.TJ : s.UJ;
     const double *M1 = opp ? s.T1 : s.U1, *N2 = opp ? s.T2 : s.U2;
@@ -619,6 +621,8 @@ __device__ __forceinline__ void wave_leaf(const Wave &wv, int b, int l, bool fir
     // own (u_ii - u_jj) = +-2 own
     s.V[at] = lvl::signs_differ(s.urow[lo], s.ucol[hi]) ? lvl::flip_sign(own, (unsigned long long)__double_as_longlong(s.urow[lo]) & 0x8000000000000000ull) * w.own2 : 0.0;
     __syncthreads();
+    const double quot = opp && live ? lvl::quotient(s.V[p + q * LD], dif, dv) : 0.0;
+    const bool far = __any_sync(0xffffffffu, dv.ex != 0);
 
     lvl::dependency_wait();
     lvl::dependency_release();
@@ -637,8 +641,7 @@ __device__ __forceinline__ void wave_leaf(const Wave &wv, int b, int l, bool fir
     s.X2[at] = x2;
     s.C[at] = sum;
     __syncthreads();
-    double acc = s.C[p + q * LD];
-    const double base = s.V[p + q * LD];
+    double acc = 0.0;
     if (k.c > 0) {
 #pragma unroll 8
         for (int i = 0; i < LB; i++) acc = fma(-M1[p + i * LD], s.X1[i + q * LD], acc);
@@ -647,7 +650,8 @@ __device__ __forceinline__ void wave_leaf(const Wave &wv, int b, int l, bool fir
 #pragma unroll 8
         for (int i = 0; i < LB; i++) acc = fma(lvl::flip_sign(s.X2[p + i * LD], flip), N2[i + q * LD], acc);
     }
-    lvl::solve16(acc, base, rinv, flip, M, N, s.V, p, q, step);
+    if (far && opp && live) dv.ex = divisor_shift(exponent_field(s.TI[p + p * LD] - s.TJ[q + q * LD]));
+    lvl::solve16(s.C[p + q * LD] + acc, quot, dv, far, flip, M, N, s.V, p, q, step);
     const double x = in ? s.V[at] : 0.0;
     if (in) SGT_AT(w.V, w.ldv, r0 + lo, c0 + hi) = x;
     // a warp holds 16 rows of two columns

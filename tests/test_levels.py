@@ -297,3 +297,37 @@ def test_batch_in_a_fresh_process(gpu_lib, ns):
     import sys
     out = subprocess.run([sys.executable, "-c", _FIRST_BATCH % ns], capture_output=True, text=True, cwd=ROOT)
     assert out.returncode == 0 and out.stdout.strip() == "same", out.stderr[-2000:]
+
+
+# T and 2^s T have the same sign: divisors t_ii - t_jj from one end of the range
+# to the other, with entries whose sums are exactly 0 (0 / d, never 0 times an
+# infinite 1 / d).  Entries are whole numbers, so 2^s T is exact.  At 2^-1060 each
+# product u t rounds by 2^-1075, 2^-19 of a divisor (16 or more) or less: n 2^-15
+# holds the sums of n of them; at the other scales the rounding is the usual one
+@pytest.mark.gpu
+@pytest.mark.parametrize("s", [-1060, -1000, 0, 1000, 1018])
+@pytest.mark.parametrize("kind", ["levels", "superblocks", "complex"])
+def test_divisors_over_the_whole_range(gpu_lib, oracle_mod, s, kind):
+    import torch
+    p, n = gpu_lib, 45
+    rng = np.random.Generator(np.random.PCG64(n))
+    T = np.triu(rng.integers(-1, 2, (n, n)), 1).astype(float)
+    T[:6, -20:] = 0.0
+    T[20:30, 30:] = 0.0
+    d = rng.integers(8, 16, n) * np.where(rng.random(n) < 0.5, -1.0, 1.0)
+    if kind == "superblocks":
+        d = np.concatenate([np.abs(d[:25]), -np.abs(d[25:])])
+    T[np.arange(n), np.arange(n)] = d
+    if kind == "complex":
+        T = T + 1j * np.triu(rng.integers(-1, 2, (n, n)) * (T != 0), 0)
+        ref = oracle_mod.sign_tri_complex(T)
+    else:
+        ref = oracle_mod.sign_tri(np.asfortranarray(T), schedule="antidiag")
+    Ts = np.asfortranarray(np.ldexp(T.real, s) + (1j * np.ldexp(T.imag, s) if kind == "complex" else 0.0))
+    if kind == "complex":
+        U = p.to_numpy(p.sign_complex(p.to_device_complex(Ts)))
+    else:
+        U = p.to_numpy(p.sign(p.to_device(Ts), p.Variant.PS_FP64 if kind == "superblocks" else p.Variant.PH_FP64))
+    torch.cuda.synchronize()
+    tol = n * (2.0 ** -15 if s == -1060 else np.finfo(float).eps)
+    assert np.linalg.norm(U - ref) <= tol * np.linalg.norm(ref)
