@@ -149,9 +149,12 @@ const char *signtri_status_string(signtri_status s);
 
 /* Bytes of device workspace sign_tri needs for size n and variant v with the
    current cutoff (0 when none).  Returns 0 for invalid arguments.  The float64
-   Parlett-Higham forms also run in less (a caller's workspace without room
-   for the superblocks' operands), down to the leaves' partial sums, by
-   float64 sums alone. */
+   Parlett-Higham forms from n = 1600 on are given 72 n^2 bytes for the
+   superblocks' operands (4.8 GB at n = 8192, 19.3 GB at 16384; none where that
+   exceeds 80 GB, n about 34,000), kept by the library for later calls.  They
+   also run in less, down to the leaves' partial sums, by float64 sums alone:
+   in a caller's workspace without that room, and where the device does not
+   have it free. */
 size_t signtri_workspace_bytes(int n, signtri_variant v);
 
 /* Use caller-owned device memory [dev_ptr, dev_ptr+bytes) as the workspace of

@@ -97,8 +97,10 @@ signtri_status current_state(DeviceState **out)
     return SIGNTRI_OK;
 }
 
-// Workspace of at least `need` bytes for the current device.
-signtri_status get_workspace(DeviceState &s, size_t need, Arena &a)
+// Workspace of at least `need` bytes for the current device.  optional: the caller
+// can do with less, so the one there is is kept where `need` is more than the device
+// has free.
+signtri_status get_workspace(DeviceState &s, size_t need, Arena &a, bool optional = false)
 {
     a = Arena();
     if (need == 0) return SIGNTRI_OK;
@@ -109,6 +111,11 @@ signtri_status get_workspace(DeviceState &s, size_t need, Arena &a)
         return SIGNTRI_OK;
     }
     if (s.lib_bytes < need) {
+        size_t free_now = 0, total = 0;
+        if (optional && (cudaMemGetInfo(&free_now, &total) != cudaSuccess || free_now + s.lib_bytes < need)) {
+            cudaGetLastError();
+            return SIGNTRI_ERR_NO_WORKSPACE;
+        }
         if (s.lib_ptr) {
             // the previous workspace may still be in use by enqueued work
             if (cudaDeviceSynchronize() != cudaSuccess) return SIGNTRI_ERR_CUDA;
@@ -145,7 +152,14 @@ int current_cutoff_locked()
 // 4.1 / 11.8 / 40.7 ms at n = 1537 / 2000 / 4096 / 8192, against 2.7 / 5.0 /
 // 32 / 270 ms by float64 sums alone (p = 0.3 random).
 constexpr int kSuperMin = 1600;
-bool super_runs(int n, int cutoff) { return n >= kSuperMin && cutoff == 16; }
+// Their operands take 72 n^2 bytes, 9 times T (4.8 GB at n = 8192, 19.3 at 16384,
+// 77 at 32768), kept with the library's workspace; from kSuperRoom on (n about
+// 34,000) float64 sums alone run.
+constexpr size_t kSuperRoom = (size_t)80 << 30;
+bool super_runs(int n, int cutoff)
+{
+    return n >= kSuperMin && cutoff == 16 && ph_super_workspace_bytes(1, &n) <= kSuperRoom;
+}
 
 // What the float64 Parlett-Higham forms work in; with less (a caller's
 // workspace), down to the plain path's, the plain path runs.
@@ -289,7 +303,7 @@ signtri_status run_ph_fp64(int n, const double *T, int ldt, double *U, int ldu, 
                            DeviceState &s)
 {
     Arena ws;
-    if (super_runs(n, b) && get_workspace(s, ph_workspace_need(n, b, split), ws) == SIGNTRI_OK) {
+    if (super_runs(n, b) && get_workspace(s, ph_workspace_need(n, b, split), ws, true) == SIGNTRI_OK) {
         SGT_CUDA_TRY(cudaMemsetAsync(s.err_dev, 0, sizeof(int), st));
         int *flags = reinterpret_cast<int *>(s.norms_host);
         signtri_status rs = ph_fp64_near_run(n, T, ldt, U, ldu, kSuperNear, ws, st);
@@ -312,9 +326,9 @@ signtri_status run_variant(int n, const double *T, int ldt, double *U, int ldu, 
         g_info.cutoff = b;
         return run_ph_fp64(n, T, ldt, U, ldu, b, v == SIGNTRI_PH_FP64_EFFICIENT, st, s);
     }
-    signtri_status rs = get_workspace(s, workspace_need(n, v, r.swaps), ws);
+    signtri_status rs = get_workspace(s, workspace_need(n, v, r.swaps), ws, v == SIGNTRI_PS_FP64);
     if (rs == SIGNTRI_ERR_NO_WORKSPACE && v == SIGNTRI_PS_FP64)
-        rs = get_workspace(s, ps_workspace_bytes(n, r.swaps, false), ws);   // a caller's, without room for superblocks
+        rs = get_workspace(s, ps_workspace_bytes(n, r.swaps, false), ws);   // without room for superblocks
     if (rs != SIGNTRI_OK) return rs;
     switch (v) {
     case SIGNTRI_PS_FP64: {
@@ -415,7 +429,7 @@ int cutoff_for(int n)
 // problems as fit kBatchSuperRoom.
 constexpr int kBatchSuperMin = 512;
 constexpr size_t kBatchSuperRoom = (size_t)32 << 30;
-bool batch_super(int n, int b) { return b == 16 && n >= kBatchSuperMin; }
+bool batch_super(int n, int b) { return b == 16 && n >= kBatchSuperMin && ph_super_workspace_bytes(1, &n) <= kSuperRoom; }
 
 // Workspace the superblocks of a batch's problems (orders n, leaf sizes b) are
 // given: all of them at once, up to kBatchSuperRoom.  batched_float64 asks for no
@@ -585,7 +599,7 @@ signtri_status sign_tri_batched(int count, const int *n, const double *const *T,
     const size_t fixed = (size_t)cnt * (sizeof(BatchDesc) + sizeof(ScanResult) + sizeof(int) + sizeof(double)) +
                          8 * 256;   // (four arrays, each rounded up to 256 bytes)
     Arena ws;
-    rs = get_workspace(*s, fixed + std::max(plan, batch_super_need(sizes, bs)), ws);
+    rs = get_workspace(*s, fixed + std::max(plan, batch_super_need(sizes, bs)), ws, true);
     if (rs == SIGNTRI_ERR_NO_WORKSPACE) rs = get_workspace(*s, fixed + plan, ws);   // without superblocks
     if (rs != SIGNTRI_OK) return rs;
     auto *d_descs = static_cast<BatchDesc *>(ws.take(cnt * sizeof(BatchDesc)));
@@ -723,7 +737,7 @@ signtri_status signtri_autotune(int n_max, void *stream)
         for (int b : {16, 32, 64}) need = std::max(need, batched_workspace_bytes(c, ns.data(), b));
         const size_t with_super = std::max(need, batch_super_need(ns, std::vector<int>(c, 16)));
         Arena ws;
-        rs = get_workspace(*s, with_super + c * sizeof(BatchDesc) + 512, ws);
+        rs = get_workspace(*s, with_super + c * sizeof(BatchDesc) + 512, ws, true);
         if (rs == SIGNTRI_ERR_NO_WORKSPACE) rs = get_workspace(*s, need + c * sizeof(BatchDesc) + 512, ws);
         if (rs != SIGNTRI_OK) break;
         auto *d_h = static_cast<BatchDesc *>(ws.take(c * sizeof(BatchDesc)));
@@ -1108,7 +1122,7 @@ signtri_status signtri_sylvester(int m, int p, const double *A, int lda, const d
         return sylvester_run(m, p, A, lda, B, ldb, C, ldc, 1.0, X, ldx, ws, static_cast<cudaStream_t>(stream));
     }
     // a caller's workspace may hold the plain solve's sums only
-    rs = get_workspace(*s, std::max(plain, sylvester_super_workspace_bytes(m, p)), ws);
+    rs = get_workspace(*s, std::max(plain, sylvester_super_workspace_bytes(m, p)), ws, true);
     if (rs == SIGNTRI_ERR_NO_WORKSPACE) rs = get_workspace(*s, plain, ws);
     if (rs != SIGNTRI_OK) return rs;
     cudaStream_t st = static_cast<cudaStream_t>(stream);

@@ -100,6 +100,7 @@ struct Problem {
     int *rnew, *cnew;                           // of V's newest superblocks
     int *rgrown, *cgrown;                       // panels whose exponents grew
     __nv_bfloat16 *vr, *vc, *fm, *fn;           // row and column forms of V, row form of RT, column form of CT
+    rns::Layout lvr, lvc, lfm, lfn;             // their layouts
     int nkbr, nkbc;                             // K-blocks over the rows (vc, fm) and over the columns (vr, fn)
     int *flags;
     int *told;                                  // null, or the host's copy of "a flag is set"
@@ -234,12 +235,14 @@ constexpr ConvConst make_conv_const()
 }
 __constant__ ConvConst c_conv = make_conv_const();
 
-// Residues of one 128 x 128 superblock of M into panel P's K-blocks 2 K, 2 K + 1.  rows: P holds rows, K counts columns; else P
-// holds columns and K counts rows.  Part `part` of kConvParts of it.
+// Residues of one 128 x 128 superblock of M into panel P's K-blocks 2 K, 2 K + 1.
+// rows: P holds rows, K counts columns; else P holds columns and K counts rows.
+// Part `part` of kConvParts of it.
 constexpr int kConvParts = SP * SP / 8 / kThreads;
 __device__ __forceinline__ void convert_superblock(const Mat &M, int bits, bool rows,
                                                    int P, int K, int part, const int *__restrict__ exps,
-                                                   unsigned *norms, __nv_bfloat16 *__restrict__ tiles, int nkb)
+                                                   unsigned *norms, __nv_bfloat16 *__restrict__ tiles,
+                                                   const rns::Layout &form)
 {
     const int it = part * kThreads + threadIdx.x;
     {
@@ -275,7 +278,8 @@ __device__ __forceinline__ void convert_superblock(const Mat &M, int bits, bool 
             }
         }
         const int kb = 2 * K + ch / 8, c8 = ch & 7;
-        __nv_bfloat16 *dst = tiles + ((size_t)P * rns::kMods * nkb + kb) * rns::kTileElems + i * 64 + ((c8 ^ (i & 7)) * 8);
+        __nv_bfloat16 *dst = tiles + form.tile(P, 0, kb) * rns::kTileElems + i * 64 + ((c8 ^ (i & 7)) * 8);
+        const size_t next = (size_t)form.count(P) * rns::kTileElems;
 #pragma unroll 4
         for (int m = 0; m < rns::kMods; m++) {
             const float mm = c_conv.m[m], rm = c_conv.rm[m];
@@ -295,7 +299,7 @@ __device__ __forceinline__ void convert_superblock(const Mat &M, int bits, bool 
                 const __nv_bfloat162 b = __floats2bfloat162_rn(y[2 * t], y[2 * t + 1]);
                 wp[t] = *reinterpret_cast<const unsigned *>(&b);
             }
-            *reinterpret_cast<uint4 *>(dst + (size_t)m * nkb * rns::kTileElems) = w;
+            *reinterpret_cast<uint4 *>(dst + (size_t)m * next) = w;
         }
         // (whole numbers: the sum does not depend on its order)
         const int lanes = rows ? 8 : SP / 8;
@@ -312,9 +316,9 @@ convert_ops_kernel(const Problem *__restrict__ probs, const Super *__restrict__ 
     const Super t = list[blockIdx.x];
     const Problem p = probs[t.k];
     if (what == kRowOps)
-        convert_superblock(matrix_of(p, what), p.bits, true, t.A, t.B, blockIdx.y, p.er1, p.nr1, p.fm, p.nkbr);
+        convert_superblock(matrix_of(p, what), p.bits, true, t.A, t.B, blockIdx.y, p.er1, p.nr1, p.fm, p.lfm);
     else
-        convert_superblock(matrix_of(p, what), p.bits, false, t.B, t.A, blockIdx.y, p.ec0, p.nc0, p.fn, p.nkbc);
+        convert_superblock(matrix_of(p, what), p.bits, false, t.B, t.A, blockIdx.y, p.ec0, p.nc0, p.fn, p.lfn);
 }
 
 // V's new superblocks (A, B), and the whole of a panel whose scale grew: of row
@@ -330,20 +334,18 @@ convert_new_kernel(const Problem *__restrict__ probs, const Super *__restrict__ 
     if (blockIdx.z % 2 == 0) {
         const int count = 1 + (p.rgrown[t.A] ? t.B - (p.triangular ? t.A : 0) : 0);
         for (int y = blockIdx.y; y < count; y += gridDim.y)
-            convert_superblock(M, p.bits, true, t.A, t.B - y, part, p.er0, p.nr0, p.vr, p.nkbc);
+            convert_superblock(M, p.bits, true, t.A, t.B - y, part, p.er0, p.nr0, p.vr, p.lvr);
     } else {
         const int count = 1 + (p.cgrown[t.B] ? (p.triangular ? t.B : p.nkbr / 2 - 1) - t.A : 0);
         for (int y = blockIdx.y; y < count; y += gridDim.y)
-            convert_superblock(M, p.bits, false, t.B, t.A + y, part, p.ec1, p.nc1, p.vc, p.nkbr);
+            convert_superblock(M, p.bits, false, t.B, t.A + y, part, p.ec1, p.nc1, p.vc, p.lvc);
     }
 }
 
 // ---- products ----------------------------------------------------------------
 
 // Every superblock's products: V N over the finished blocks of its row, M V over
-// those of its column, and, for sign(T), U U.  Triangular V: from the diagonal
-// superblock of the row and to that of the column, whose strictly upper parts
-// are known.
+// those of its column, and, for sign(T), U U.
 __global__ void tiles_kernel(const Problem *__restrict__ probs, const Super *__restrict__ list, int count, int products,
                              rns::Tile *__restrict__ tiles)
 {
@@ -352,13 +354,10 @@ __global__ void tiles_kernel(const Problem *__restrict__ probs, const Super *__r
     const Super t = list[i];
     const Problem &p = probs[t.k];
     rns::Tile *o = tiles + (size_t)products * i;
-    // of V, the level before this one solves the superblocks (A, B - 1) and
-    // (A + 1, B); the rest may be summed beside it
-    const int k0 = p.triangular ? 2 * t.A : 0, k1 = p.triangular ? 2 * (t.B + 1) : p.nkbr;
-    const int below = 2 * (t.A + 2), left = 2 * (t.B - 1);
-    o[0] = {3 * t.k, t.A, t.B, k0, 2 * t.B, k0, left};
-    o[1] = {3 * t.k + 1, t.A, t.B, 2 * (t.A + 1), k1, below, k1};
-    if (products == 3) o[2] = {3 * t.k + 2, t.A, t.B, 2 * (t.A + 1), 2 * t.B, below, left};
+    auto tile = [&](int which, const SuperSpan &k) { return rns::Tile{3 * t.k + which, t.A, t.B, k.k0, k.k1, k.e0, k.e1}; };
+    o[0] = tile(0, span_vn(p.triangular, t.A, t.B));
+    o[1] = tile(1, span_mv(p.triangular, p.nkbr, t.A, t.B));
+    if (products == 3) o[2] = tile(2, span_uu(t.A, t.B));
 }
 
 struct CrtConst {
@@ -732,15 +731,24 @@ size_t run_bytes(size_t problems, size_t superblocks, size_t ops, size_t widest,
            superblocks * products * sizeof(rns::Tile) + 3 * widest * products * rns::kMods * SP * SP +
            2 * wave_slab_bytes(widest) + 12 * 256;
 }
-// A problem's exponents, growth marks and forms.
-size_t problem_bytes(int nr, int nc, bool forms)
+// A problem's exponents, norms and growth marks, and its forms.
+size_t problem_bytes(int nr, int nc)
 {
-    size_t b = 5 * ((size_t)(nr + nc) * SP * sizeof(int) + 512) + (size_t)(nr + nc) * sizeof(int) + 512;
-    if (forms)
-        b += rns::form_tile_bytes(nr, 2 * nr) + rns::form_tile_bytes(nc, 2 * nc) + rns::form_tile_bytes(nr, 2 * nc) +
-             rns::form_tile_bytes(nc, 2 * nr) + 4 * 256;
-    return b;
+    return 5 * ((size_t)(nr + nc) * SP * sizeof(int) + 512) + (size_t)(nr + nc) * sizeof(int) + 512;
 }
+struct Forms {
+    rns::Layout fm, fn, vr, vc;
+    Forms(int nr, int nc, bool triangular)
+        : fm{rns::kUpperRows, 2 * nr}, fn{rns::kUpperCols, 2 * nc},
+          vr{triangular ? rns::kUpperRows : rns::kFull, 2 * nc}, vc{triangular ? rns::kUpperCols : rns::kFull, 2 * nr}
+    {
+    }
+    size_t bytes(int nr, int nc) const
+    {
+        return rns::form_tile_bytes(fm, nr) + rns::form_tile_bytes(fn, nc) + rns::form_tile_bytes(vr, nr) +
+               rns::form_tile_bytes(vc, nc) + 4 * 256;
+    }
+};
 
 // A set of problems whose superblocks are solved level by level, every level's
 // in the same launches.
@@ -771,13 +779,18 @@ struct Run {
         p.nkbr = 2 * nr;
         p.nkbc = 2 * nc;
         if (!forms) return p.cgrown != nullptr;
-        auto form = [&](int panels, int nkb) {
-            return static_cast<__nv_bfloat16 *>(ws.take(rns::form_tile_bytes(panels, nkb)));
+        const Forms l(nr, nc, p.triangular);
+        auto form = [&](const rns::Layout &f, int panels) {
+            return static_cast<__nv_bfloat16 *>(ws.take(rns::form_tile_bytes(f, panels)));
         };
-        p.fm = form(nr, 2 * nr);
-        p.fn = form(nc, 2 * nc);
-        p.vr = form(nr, 2 * nc);
-        p.vc = form(nc, 2 * nr);
+        p.lfm = l.fm;
+        p.lfn = l.fn;
+        p.lvr = l.vr;
+        p.lvc = l.vc;
+        p.fm = form(l.fm, nr);
+        p.fn = form(l.fn, nc);
+        p.vr = form(l.vr, nr);
+        p.vc = form(l.vc, nc);
         return p.vc != nullptr;
     }
 
@@ -808,9 +821,9 @@ struct Run {
             Problem &p = probs[k];
             p.flags = d_flags + k;
             p.told = told;
-            src[3 * k] = {p.vr, p.fn, p.nkbc, p.nkbc, p.rgrown, nullptr};
-            src[3 * k + 1] = {p.fm, p.vc, p.nkbr, p.nkbr, nullptr, p.cgrown};
-            src[3 * k + 2] = {p.vr, p.vc, p.nkbc, p.nkbr, p.rgrown, p.cgrown};
+            src[3 * k] = {p.vr, p.fn, p.lvr, p.lfn, p.rgrown, nullptr};
+            src[3 * k + 1] = {p.fm, p.vc, p.lfm, p.lvc, nullptr, p.cgrown};
+            src[3 * k + 2] = {p.vr, p.vc, p.lvr, p.lvc, p.rgrown, p.cgrown};
         }
         SGT_CUDA_TRY(cudaMemcpyAsync(d_probs, probs.data(), np * sizeof(Problem), cudaMemcpyHostToDevice, st));
         SGT_CUDA_TRY(cudaMemcpyAsync(d_src, src.data(), src.size() * sizeof(rns::Source), cudaMemcpyHostToDevice, st));
@@ -928,7 +941,7 @@ size_t ph_super_workspace_bytes(int count, const int *n)
     size_t b = 0, superblocks = 0, ops = 0, widest = 0;
     for (int k = 0; k < count; k++) {
         const size_t ns = panels_of(n[k]);
-        b += problem_bytes((int)ns, (int)ns, true);
+        b += problem_bytes((int)ns, (int)ns) + Forms((int)ns, (int)ns, true).bytes((int)ns, (int)ns);
         superblocks += ns * (ns - 1) / 2;
         ops += ns * (ns + 1) + ns;
         widest += ns - 1;
@@ -979,22 +992,22 @@ signtri_status ph_super_run(int count, const BatchDesc *mats, Arena &ws, int *d_
 static size_t sylvester_super_bytes(int nr, int nc, int nt)
 {
     using namespace sup;
-    return problem_bytes(nr, nc, nr + nc > 2) +
-           run_bytes(1, (size_t)nr * nc, ((size_t)nr * (nr + 1) + (size_t)nc * (nc + 1)) / 2, nt, 2);
+    return problem_bytes(nr, nc) + run_bytes(1, (size_t)nr * nc, ((size_t)nr * (nr + 1) + (size_t)nc * (nc + 1)) / 2, nt, 2);
 }
 
 size_t sylvester_super_workspace_bytes(int m, int p)
 {
     if (m <= 0 || p <= 0) return 0;
     const int nr = sup::panels_of(m), nc = sup::panels_of(p);
-    return sylvester_super_bytes(nr, nc, std::min(nr, nc));
+    return sylvester_super_bytes(nr, nc, std::min(nr, nc)) + (nr + nc > 2 ? sup::Forms(nr, nc, false).bytes(nr, nc) : 0);
 }
 
-// for every m + p = n: the forms take 2 (nr + nc)^2 tiles of K-blocks
+// for every m + p = n, with k panels in all: the forms hold nr (nr + 1) + nc (nc + 1) + 4 nr nc
+// K-blocks, most at nr = nc
 size_t sylvester_super_workspace_bound(int n)
 {
-    const int k = sup::panels_of(n) + 1;
-    return sylvester_super_bytes(k, 1, k / 2 + 1) +
+    const int k = sup::panels_of(n) + 1, h = (k + 1) / 2;
+    return sylvester_super_bytes(k, 1, k / 2 + 1) + sup::Forms(h, h, false).bytes(h, h) +
            (size_t)k * k / 2 * (2 * sizeof(rns::Tile) + sizeof(sup::Super));
 }
 

@@ -172,8 +172,8 @@ rns_gemm_kernel(const Source *__restrict__ src, const Tile *__restrict__ tiles, 
                 const Task k = task_of(id, per);
                 const Tile t = tiles[k.tile];
                 const Source s = src[t.src];
-                const __nv_bfloat16 *a = s.A + ((size_t)t.pa * kMods + k.mod) * s.nkbA * kTileElems;
-                const __nv_bfloat16 *b = s.B + ((size_t)t.pb * kMods + k.mod) * s.nkbB * kTileElems;
+                const __nv_bfloat16 *a = s.A + s.la.tile(t.pa, k.mod, 0) * kTileElems;
+                const __nv_bfloat16 *b = s.B + s.lb.tile(t.pb, k.mod, 0) * kTileElems;
                 const Span ks = span_of(t, s, early, ahead != nullptr);
                 for (int i = 0; i < ks.n; i++) {
                     const int kb = ks[i];

@@ -4,6 +4,7 @@
 #include <cuda_bf16.h>
 
 #include "internal.cuh"
+#include "super_plan.h"
 
 namespace signtri {
 namespace rns {
@@ -11,7 +12,6 @@ namespace rns {
 // Pairwise coprime moduli; their product is 2^140.4.  (With the first 16 of
 // them, 2^125.3, operands keep 55 bits at K = 8192 and their rounding is as large
 // as that of float64 sums on ungraded data: no room for data that spreads.)
-constexpr int kMods = 18;
 constexpr int kModulus[kMods] = {256, 255, 253, 251, 247, 241, 239, 233, 229, 227, 223, 217, 211, 199, 197, 193, 191, 181};
 constexpr int kPanel = 128;                    // rows of a panel, and edge of a product tile
 constexpr int kTileElems = kPanel * 64;        // one panel's K-block of 64, one modulus: 16 KB of bf16
@@ -28,17 +28,7 @@ constexpr int operand_bits(int K)
     return b < 62 ? b : 62;
 }
 
-// The residues of a matrix cut into panels of 128 rows (a row form: rows of
-// M) or of 128 columns (a column form: columns of M), K-contiguous: tile
-// (panel, modulus, K-block) at ((panel * kMods + modulus) * nkb + kblock) *
-// kTileElems, already in the 128-byte swizzle the MMA descriptor names.
-struct Form {
-    __nv_bfloat16 *tiles;
-    int *exps;      // per row (column): entries are below 2^exps
-    int panels;
-    int nkb;
-};
-inline size_t form_tile_bytes(int panels, int nkb) { return (size_t)panels * kMods * nkb * kTileElems * 2; }
+constexpr size_t form_tile_bytes(const Layout &l, int panels) { return l.before(panels) * kMods * kTileElems * 2; }
 
 // One 128 x 128 product: panel pa of source number `src`'s A form times panel pb of
 // its B form over K-blocks [kb0, kb1), of which [e0, e1) may be summed ahead.
@@ -49,7 +39,7 @@ struct Tile {
 // since the K-blocks [e0, e1) were summed, so that sum is of no use.
 struct Source {
     const __nv_bfloat16 *A, *B;
-    int nkbA, nkbB;
+    Layout la, lb;
     const int *grownA, *grownB;
 };
 

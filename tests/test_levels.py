@@ -331,3 +331,46 @@ def test_divisors_over_the_whole_range(gpu_lib, oracle_mod, s, kind):
     torch.cuda.synchronize()
     tol = n * (2.0 ** -15 if s == -1060 else np.finfo(float).eps)
     assert np.linalg.norm(U - ref) <= tol * np.linalg.norm(ref)
+
+
+# the superblocks' workspace: 9 times T and no more, none beyond 80 GB; and where
+# the device does not have it free, float64 sums in the workspace there is
+@pytest.mark.gpu
+def test_superblock_workspace(gpu_lib):
+    p = gpu_lib
+    for n in (2048, 8192, 16384, 32768):
+        need = p.signtri_workspace_bytes(n, p.Variant.PH_FP64_EFFICIENT)
+        assert 72 * n * n <= need <= 72 * n * n * 1.25 + (64 << 20), n
+    assert p.signtri_workspace_bytes(65536, p.Variant.PH_FP64_EFFICIENT) < (1 << 30)
+
+
+_LITTLE_FREE = """
+import torch
+import paper_1607_06303_gb300 as p
+p.load()
+def sign(n):
+    g = torch.Generator(device="cuda").manual_seed(n)
+    t = torch.randn((n, n), generator=g, device="cuda", dtype=torch.float64).mul_(n ** -0.5).tril_(-1)
+    t.diagonal().copy_((torch.arange(n, device="cuda") % 3 - 0.5).double())
+    u = torch.empty_like(t)
+    def run():
+        p.sign(t, p.Variant.PH_FP64_EFFICIENT, out=u)
+        torch.cuda.synchronize()
+        return u
+    return run
+small, large = sign(2500), sign(9000)
+first = small().clone()
+fill = torch.empty(torch.cuda.mem_get_info()[0] - (4 << 30), dtype=torch.uint8, device="cuda")
+free = torch.cuda.mem_get_info()[0]
+large()
+assert torch.cuda.mem_get_info()[0] == free
+assert torch.equal(small(), first)
+print("kept")
+"""
+
+
+@pytest.mark.gpu
+def test_workspace_is_kept_where_a_larger_one_does_not_fit(gpu_lib):
+    import sys
+    out = subprocess.run([sys.executable, "-c", _LITTLE_FREE], capture_output=True, text=True, cwd=ROOT)
+    assert out.returncode == 0 and out.stdout.strip() == "kept", out.stderr[-2000:]
