@@ -27,6 +27,10 @@
  *     cudaMalloc, or set by signtri_set_workspace).  Calls that share a
  *     workspace must not run concurrently: issue them from one host thread,
  *     or on one stream, at a time.
+ *   - Calls on one device take turns on the host, each until it returns (its
+ *     waits included).  Calls on other devices go on beside them, and so do
+ *     questions about settings and sizes; a call that changes a setting waits
+ *     for the calls under way.
  */
 #ifndef SIGNTRI_H
 #define SIGNTRI_H

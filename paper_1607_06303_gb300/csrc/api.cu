@@ -8,6 +8,7 @@
 #include <algorithm>
 #include <cstring>
 #include <mutex>
+#include <shared_mutex>
 #include <utility>
 #include <vector>
 
@@ -21,6 +22,7 @@ namespace {
 constexpr int kMaxDevices = 64;
 
 struct DeviceState {
+    std::mutex mu;                 // held by the call at work on the device
     void *lib_ptr = nullptr;       // library-owned workspace (cudaMalloc)
     size_t lib_bytes = 0;
     void *user_ptr = nullptr;      // caller-owned workspace, if set
@@ -36,7 +38,13 @@ struct DeviceState {
     bool ready = false;            // every per-device buffer above the workspace allocated
 };
 
-std::mutex g_mu;
+// Guards the settings below.  A call that works on a device shares it, and
+// holds the device's own mutex for its length, waits included: calls on other
+// devices go on beside it, and so do questions about settings.  A call that
+// changes a setting has it alone.
+std::shared_mutex g_mu;
+using SettingsLock = std::unique_lock<std::shared_mutex>;
+using SharedLock = std::shared_lock<std::shared_mutex>;
 DeviceState g_dev[kMaxDevices];
 // 0: kDefaultCutoff; else the leaf size set by signtri_set_cutoff
 int g_cutoff = 0;
@@ -60,12 +68,14 @@ thread_local signtri_info g_info;
 
 bool valid_variant(int v) { return v >= SIGNTRI_AUTO && v <= SIGNTRI_PH_MIXED_FP16; }
 
-signtri_status current_state(DeviceState **out)
+// The current device's state, locked for the caller by lk (after g_mu).
+signtri_status current_state(DeviceState **out, std::unique_lock<std::mutex> &lk)
 {
     int dev = 0;
     SGT_CUDA_TRY(cudaGetDevice(&dev));
     if (dev < 0 || dev >= kMaxDevices) return SIGNTRI_ERR_CUDA;
     DeviceState &s = g_dev[dev];
+    lk = std::unique_lock<std::mutex>(s.mu);
     if (!s.ready) {
         // a piece is stored only once allocated, so a call after a failed
         // attempt allocates what is still missing instead of using a NULL
@@ -518,7 +528,7 @@ __global__ void synth_kernel(int n, double *T, unsigned long long seed)
 
 int signtri::current_cutoff()
 {
-    std::lock_guard<std::mutex> lk(g_mu);
+    SharedLock lk(g_mu);
     return current_cutoff_locked();
 }
 
@@ -544,13 +554,13 @@ const char *signtri_status_string(signtri_status s)
 size_t signtri_workspace_bytes(int n, signtri_variant v)
 {
     if (n < 0 || !valid_variant(v)) return 0;
-    std::lock_guard<std::mutex> lk(g_mu);
+    SharedLock lk(g_mu);
     return workspace_need(n, v, -1);
 }
 
 signtri_status signtri_set_rates(double gemm_flops_per_s, double givens_flops_per_s)
 {
-    std::lock_guard<std::mutex> lk(g_mu);
+    SettingsLock lk(g_mu);
     g_rate_gemm = gemm_flops_per_s > 0 ? gemm_flops_per_s : kDefaultGemmRate;
     g_rate_givens = givens_flops_per_s > 0 ? givens_flops_per_s : kDefaultGivensRate;
     return SIGNTRI_OK;
@@ -563,9 +573,10 @@ signtri_status sign_tri_batched(int count, const int *n, const double *const *T,
     if (count < 0 || !valid_variant(v)) return SIGNTRI_ERR_BAD_ARG;
     if (count == 0) return SIGNTRI_OK;
     if (!n || !T || !ldt || !U || !ldu || !info) return SIGNTRI_ERR_BAD_ARG;
-    std::lock_guard<std::mutex> lk(g_mu);
+    SharedLock lk(g_mu);
+    std::unique_lock<std::mutex> device;
     DeviceState *s = nullptr;
-    signtri_status rs = current_state(&s);
+    signtri_status rs = current_state(&s, device);
     if (rs != SIGNTRI_OK) return rs;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     std::vector<BatchDesc> descs;
@@ -682,7 +693,7 @@ signtri_status signtri_set_cutoff_table(const int *b, int len)
     if (len < 0 || len > 32 || (len > 0 && !b)) return SIGNTRI_ERR_BAD_ARG;
     for (int k = 0; k < len; k++)
         if (b[k] != 0 && b[k] != 16 && b[k] != 32 && b[k] != 64) return SIGNTRI_ERR_BAD_ARG;
-    std::lock_guard<std::mutex> lk(g_mu);
+    SettingsLock lk(g_mu);
     for (int k = 0; k < 32; k++) g_cutoff_table[k] = k < len ? b[k] : 0;
     return SIGNTRI_OK;
 }
@@ -690,7 +701,7 @@ signtri_status signtri_set_cutoff_table(const int *b, int len)
 signtri_status signtri_get_cutoff_table(int *b, int len)
 {
     if (len < 0 || len > 32 || (len > 0 && !b)) return SIGNTRI_ERR_BAD_ARG;
-    std::lock_guard<std::mutex> lk(g_mu);
+    SharedLock lk(g_mu);
     for (int k = 0; k < len; k++) b[k] = g_cutoff_table[k];
     return SIGNTRI_OK;
 }
@@ -698,9 +709,10 @@ signtri_status signtri_get_cutoff_table(int *b, int len)
 signtri_status signtri_autotune(int n_max, void *stream)
 {
     if (n_max < 32 || n_max > 32768) return SIGNTRI_ERR_BAD_ARG;
-    std::lock_guard<std::mutex> lk(g_mu);
+    SettingsLock lk(g_mu);
+    std::unique_lock<std::mutex> device;
     DeviceState *s = nullptr;
-    signtri_status rs = current_state(&s);
+    signtri_status rs = current_state(&s, device);
     if (rs != SIGNTRI_OK) return rs;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     // per size bucket n = 2^k: a batch of c = 2^27 / n^2 problems (at most
@@ -780,7 +792,7 @@ signtri_status signtri_autotune(int n_max, void *stream)
 signtri_status signtri_get_variant_table(int *v, int len)
 {
     if (len < 0 || len > 32 || (len > 0 && !v)) return SIGNTRI_ERR_BAD_ARG;
-    std::lock_guard<std::mutex> lk(g_mu);
+    SharedLock lk(g_mu);
     for (int k = 0; k < len; k++) v[k] = g_variant_table[k];
     return SIGNTRI_OK;
 }
@@ -790,7 +802,7 @@ signtri_status signtri_set_variant_table(const int *v, int len)
     if (len < 0 || len > 32 || (len > 0 && !v)) return SIGNTRI_ERR_BAD_ARG;
     for (int k = 0; k < len; k++)
         if (v[k] != 0 && !(valid_variant(v[k]) && v[k] != SIGNTRI_AUTO)) return SIGNTRI_ERR_BAD_ARG;
-    std::lock_guard<std::mutex> lk(g_mu);
+    SettingsLock lk(g_mu);
     for (int k = 0; k < 32; k++) g_variant_table[k] = k < len ? v[k] : 0;
     return SIGNTRI_OK;
 }
@@ -798,7 +810,7 @@ signtri_status signtri_set_variant_table(const int *v, int len)
 signtri_status signtri_batched_cache_stats(long long *hits, long long *builds)
 {
     if (!hits || !builds) return SIGNTRI_ERR_BAD_ARG;
-    std::lock_guard<std::mutex> lk(g_mu);
+    SettingsLock lk(g_mu);
     batched_cache_stats(hits, builds);
     return SIGNTRI_OK;
 }
@@ -806,9 +818,10 @@ signtri_status signtri_batched_cache_stats(long long *hits, long long *builds)
 signtri_status signtri_selftest_wait(int arrive, long long limit_cycles, void *stream)
 {
     if (limit_cycles <= 0 || limit_cycles > 4000000000LL) return SIGNTRI_ERR_BAD_ARG;
-    std::lock_guard<std::mutex> lk(g_mu);
+    SharedLock lk(g_mu);
+    std::unique_lock<std::mutex> device;
     DeviceState *s = nullptr;
-    signtri_status rs = current_state(&s);
+    signtri_status rs = current_state(&s, device);
     if (rs != SIGNTRI_OK) return rs;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     SGT_CUDA_TRY(cudaMemsetAsync(s->err_dev, 0, sizeof(int), st));
@@ -821,7 +834,7 @@ signtri_status signtri_selftest_wait(int arrive, long long limit_cycles, void *s
 
 signtri_status signtri_set_refinement(double tol, int max_steps)
 {
-    std::lock_guard<std::mutex> lk(g_mu);
+    SettingsLock lk(g_mu);
     g_mixed_tol = tol > 0 ? tol : kDefaultMixedTol;
     g_mixed_max_steps = max_steps;
     return SIGNTRI_OK;
@@ -830,7 +843,7 @@ signtri_status signtri_set_refinement(double tol, int max_steps)
 signtri_status signtri_set_verification(int full)
 {
     if (full != 0 && full != 1) return SIGNTRI_ERR_BAD_ARG;
-    std::lock_guard<std::mutex> lk(g_mu);
+    SettingsLock lk(g_mu);
     g_mixed_verify_full = full;
     return SIGNTRI_OK;
 }
@@ -845,9 +858,10 @@ signtri_status signtri_reorder_by_sign(int n, const double *T, int ldt, double *
     if (blocks_overlap(T, ldt, n, n, Tr, ldtr, n, n) || blocks_overlap(T, ldt, n, n, Q, ldq, n, n) ||
         blocks_overlap(Tr, ldtr, n, n, Q, ldq, n, n))
         return SIGNTRI_ERR_BAD_ARG;
-    std::lock_guard<std::mutex> lk(g_mu);
+    SharedLock lk(g_mu);
+    std::unique_lock<std::mutex> device;
     DeviceState *s = nullptr;
-    signtri_status rs = current_state(&s);
+    signtri_status rs = current_state(&s, device);
     if (rs != SIGNTRI_OK) return rs;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     rs = launch_inertia_scan(n, T, ldt, s->scan_dev, st);
@@ -875,9 +889,10 @@ signtri_status signtri_gemm_emulated(int m, int n, int k, const double *A, int l
     if (!A || !B || !C || lda < m || ldb < std::max(k, 1) || ldc < m) return SIGNTRI_ERR_BAD_ARG;
     if (blocks_overlap(A, lda, m, k, C, ldc, m, n) || blocks_overlap(B, ldb, k, n, C, ldc, m, n))
         return SIGNTRI_ERR_BAD_ARG;
-    std::lock_guard<std::mutex> lk(g_mu);
+    SharedLock lk(g_mu);
+    std::unique_lock<std::mutex> device;
     DeviceState *s = nullptr;
-    signtri_status rs = current_state(&s);
+    signtri_status rs = current_state(&s, device);
     if (rs != SIGNTRI_OK) return rs;
     Arena ws;
     rs = get_workspace(*s, emulated_gemm_workspace_bytes(m, n, k, 8), ws);
@@ -900,7 +915,7 @@ static size_t schur_products_bytes(int n)
 size_t signtri_sign_schur_workspace_bytes(int n, signtri_variant v)
 {
     if (n < 0 || !valid_variant(v)) return 0;
-    std::lock_guard<std::mutex> lk(g_mu);
+    SharedLock lk(g_mu);
     return std::max(workspace_need(n, v, -1), schur_products_bytes(n));
 }
 
@@ -913,9 +928,10 @@ signtri_status signtri_sign_schur(int n, const double *Q, int ldq, const double 
     if (!Q || !T || !S || ldq < n || ldt < n || lds < n) return SIGNTRI_ERR_BAD_ARG;
     if (blocks_overlap(T, ldt, n, n, S, lds, n, n) || blocks_overlap(Q, ldq, n, n, S, lds, n, n))
         return SIGNTRI_ERR_BAD_ARG;
-    std::lock_guard<std::mutex> lk(g_mu);
+    SharedLock lk(g_mu);
+    std::unique_lock<std::mutex> device;
     DeviceState *s = nullptr;
-    signtri_status rs = current_state(&s);
+    signtri_status rs = current_state(&s, device);
     if (rs != SIGNTRI_OK) return rs;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     // U = sign(T), held in S until the second product overwrites it
@@ -962,9 +978,10 @@ signtri_status signtri_sign_tri_complex(int n, const double *T, int ldt, double 
     if (n == 0) return SIGNTRI_OK;
     if (!T || !U || ldt < n || ldu < n) return SIGNTRI_ERR_BAD_ARG;
     if (cblocks_overlap(T, ldt, U, ldu, n)) return SIGNTRI_ERR_BAD_ARG;
-    std::lock_guard<std::mutex> lk(g_mu);
+    SharedLock lk(g_mu);
+    std::unique_lock<std::mutex> device;
     DeviceState *s = nullptr;
-    signtri_status rs = current_state(&s);
+    signtri_status rs = current_state(&s, device);
     if (rs != SIGNTRI_OK) return rs;
     Arena ws;
     rs = get_workspace(*s, complex_workspace_bytes(n), ws);
@@ -986,9 +1003,10 @@ signtri_status signtri_sign_schur_complex(int n, const double *Q, int ldq, const
     if (n == 0) return SIGNTRI_OK;
     if (!Q || !T || !S || ldq < n || ldt < n || lds < n) return SIGNTRI_ERR_BAD_ARG;
     if (cblocks_overlap(T, ldt, S, lds, n) || cblocks_overlap(Q, ldq, S, lds, n)) return SIGNTRI_ERR_BAD_ARG;
-    std::lock_guard<std::mutex> lk(g_mu);
+    SharedLock lk(g_mu);
+    std::unique_lock<std::mutex> device;
     DeviceState *s = nullptr;
-    signtri_status rs = current_state(&s);
+    signtri_status rs = current_state(&s, device);
     if (rs != SIGNTRI_OK) return rs;
     Arena ws;
     rs = get_workspace(*s, complex_schur_workspace_bytes(n), ws);
@@ -1026,9 +1044,10 @@ signtri_status signtri_schur(int n, const double *A, int lda, double *Q, int ldq
     if (blocks_overlap(A, lda, n, n, Q, 2 * ldq, 2 * n, n) || blocks_overlap(A, lda, n, n, T, 2 * ldt, 2 * n, n) ||
         cblocks_overlap(Q, ldq, T, ldt, n))
         return SIGNTRI_ERR_BAD_ARG;
-    std::lock_guard<std::mutex> lk(g_mu);
+    SharedLock lk(g_mu);
+    std::unique_lock<std::mutex> device;
     DeviceState *s = nullptr;
-    signtri_status rs = current_state(&s);
+    signtri_status rs = current_state(&s, device);
     if (rs != SIGNTRI_OK) return rs;
     Arena ws;
     rs = get_workspace(*s, schur_workspace_bytes(n), ws);
@@ -1052,9 +1071,10 @@ signtri_status signtri_sign_general(int n, const double *A, int lda, double *S, 
     if (n == 0) return SIGNTRI_OK;
     if (!A || !S || lda < n || lds < n) return SIGNTRI_ERR_BAD_ARG;
     if (blocks_overlap(A, lda, n, n, S, lds, n, n)) return SIGNTRI_ERR_BAD_ARG;
-    std::lock_guard<std::mutex> lk(g_mu);
+    SharedLock lk(g_mu);
+    std::unique_lock<std::mutex> device;
     DeviceState *s = nullptr;
-    signtri_status rs = current_state(&s);
+    signtri_status rs = current_state(&s, device);
     if (rs != SIGNTRI_OK) return rs;
     Arena ws;
     rs = get_workspace(*s, sign_general_workspace_bytes(n), ws);
@@ -1080,9 +1100,10 @@ signtri_status signtri_funm(int n, const double *T, int ldt, double *F, int ldf,
     if (n == 0) return SIGNTRI_OK;
     if (!T || !F || ldt < n || ldf < n) return SIGNTRI_ERR_BAD_ARG;
     if (blocks_overlap(T, ldt, n, n, F, ldf, n, n)) return SIGNTRI_ERR_BAD_ARG;
-    std::lock_guard<std::mutex> lk(g_mu);
+    SharedLock lk(g_mu);
+    std::unique_lock<std::mutex> device;
     DeviceState *s = nullptr;
-    signtri_status rs = current_state(&s);
+    signtri_status rs = current_state(&s, device);
     if (rs != SIGNTRI_OK) return rs;
     const int b = current_cutoff_locked();
     Arena ws;
@@ -1107,9 +1128,10 @@ signtri_status signtri_sylvester(int m, int p, const double *A, int lda, const d
     if (blocks_overlap(A, lda, m, m, X, ldx, m, p) || blocks_overlap(B, ldb, p, p, X, ldx, m, p) ||
         blocks_overlap(C, ldc, m, p, X, ldx, m, p))
         return SIGNTRI_ERR_BAD_ARG;
-    std::lock_guard<std::mutex> lk(g_mu);
+    SharedLock lk(g_mu);
+    std::unique_lock<std::mutex> device;
     DeviceState *s = nullptr;
-    signtri_status rs = current_state(&s);
+    signtri_status rs = current_state(&s, device);
     if (rs != SIGNTRI_OK) return rs;
     Arena ws;
     const size_t plain = sylvester_workspace_bytes(m, p);
@@ -1138,9 +1160,10 @@ signtri_status signtri_sylvester(int m, int p, const double *A, int lda, const d
 signtri_status signtri_set_workspace(void *dev_ptr, size_t bytes)
 {
     if (dev_ptr && ((uintptr_t)dev_ptr % 256) != 0) return SIGNTRI_ERR_BAD_ARG;
-    std::lock_guard<std::mutex> lk(g_mu);
+    SharedLock lk(g_mu);
+    std::unique_lock<std::mutex> device;
     DeviceState *s = nullptr;
-    signtri_status rs = current_state(&s);
+    signtri_status rs = current_state(&s, device);
     if (rs != SIGNTRI_OK) return rs;
     s->user_ptr = dev_ptr;
     s->user_bytes = dev_ptr ? bytes : 0;
@@ -1150,7 +1173,7 @@ signtri_status signtri_set_workspace(void *dev_ptr, size_t bytes)
 signtri_status signtri_set_cutoff(int b)
 {
     if (b != 0 && b != 16 && b != 32 && b != 64) return SIGNTRI_ERR_BAD_ARG;
-    std::lock_guard<std::mutex> lk(g_mu);
+    SettingsLock lk(g_mu);
     g_cutoff = b;
     return SIGNTRI_OK;
 }
@@ -1163,9 +1186,10 @@ signtri_status sign_tri(int n, const double *T, int ldt, double *U, int ldu, sig
     if (n == 0) return SIGNTRI_OK;
     if (!T || !U || ldt < n || ldu < n) return SIGNTRI_ERR_BAD_ARG;
     if (blocks_overlap(T, ldt, n, n, U, ldu, n, n)) return SIGNTRI_ERR_BAD_ARG;
-    std::lock_guard<std::mutex> lk(g_mu);
+    SharedLock lk(g_mu);
+    std::unique_lock<std::mutex> device;
     DeviceState *s = nullptr;
-    signtri_status rs = current_state(&s);
+    signtri_status rs = current_state(&s, device);
     if (rs != SIGNTRI_OK) return rs;
     return sign_tri_locked(n, T, ldt, U, ldu, v, static_cast<cudaStream_t>(stream), *s);
 }
@@ -1177,9 +1201,10 @@ signtri_status sign_tri_host(int n, const double *T_host, int ldt, double *U_hos
     if (n < 0 || !valid_variant(v)) return SIGNTRI_ERR_BAD_ARG;
     if (n == 0) return SIGNTRI_OK;
     if (!T_host || !U_host || ldt < n || ldu < n) return SIGNTRI_ERR_BAD_ARG;
-    std::lock_guard<std::mutex> lk(g_mu);
+    SharedLock lk(g_mu);
+    std::unique_lock<std::mutex> device;
     DeviceState *s = nullptr;
-    signtri_status rs = current_state(&s);
+    signtri_status rs = current_state(&s, device);
     if (rs != SIGNTRI_OK) return rs;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const size_t elems = (size_t)n * n;
@@ -1233,9 +1258,10 @@ signtri_status signtri_inertia(int n, const double *T, int ldt, int *n_pos, int 
         if (swaps) *swaps = 0;
         return SIGNTRI_OK;
     }
-    std::lock_guard<std::mutex> lk(g_mu);
+    SharedLock lk(g_mu);
+    std::unique_lock<std::mutex> device;
     DeviceState *s = nullptr;
-    signtri_status rs = current_state(&s);
+    signtri_status rs = current_state(&s, device);
     if (rs != SIGNTRI_OK) return rs;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     rs = launch_inertia_scan(n, T, ldt, s->scan_dev, st);

@@ -49,7 +49,7 @@ const char *kClassNames[SIGNTRI_KC_COUNT] = {
     "hessenberg", "host_copies",
 };
 
-bool p_paused = false;
+thread_local bool p_paused = false;   // the thread that captures
 
 }  // namespace
 

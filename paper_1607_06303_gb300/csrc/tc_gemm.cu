@@ -28,6 +28,7 @@
 // buffer and the lo parts in registers.
 // Every mbarrier wait is bounded; on expiry the CTA records an error and
 // returns after draining what it issued.
+#include <atomic>
 #include <algorithm>
 
 #include <cuda.h>
@@ -780,7 +781,7 @@ tc_pair2_kernel(const __grid_constant__ CUtensorMap mTop, const __grid_constant_
     }
 }
 
-PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
+std::atomic<PFN_cuTensorMapEncodeTiled_v12000> g_encode{nullptr};   // calls on two devices may set it at once
 
 signtri_status get_encoder()
 {
@@ -803,7 +804,7 @@ signtri_status make_map(CUtensorMap *m, const __nv_bfloat16 *base, long long row
     cuuint64_t strides[1] = {(cuuint64_t)(ld * 2)};
     cuuint32_t box[2] = {64, 64};
     cuuint32_t estr[2] = {1, 1};
-    CUresult r = g_encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<__nv_bfloat16 *>(base), dims, strides,
+    CUresult r = g_encode.load()(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<__nv_bfloat16 *>(base), dims, strides,
                           box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                           CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? SIGNTRI_OK : SIGNTRI_ERR_CUDA;

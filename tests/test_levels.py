@@ -374,3 +374,36 @@ def test_workspace_is_kept_where_a_larger_one_does_not_fit(gpu_lib):
     import sys
     out = subprocess.run([sys.executable, "-c", _LITTLE_FREE], capture_output=True, text=True, cwd=ROOT)
     assert out.returncode == 0 and out.stdout.strip() == "kept", out.stderr[-2000:]
+
+
+# a question about sizes is answered beside a solve (which waits for its superblocks,
+# 36 ms at n = 8192) and not after it.  The limit is half a solve
+@pytest.mark.gpu
+def test_questions_beside_a_solve(gpu_lib):
+    import threading
+    import time
+    import torch
+    p, n = gpu_lib, 8192
+    t = torch.randn((n, n), device="cuda", dtype=torch.float64).mul_(n ** -0.5).tril_(-1)
+    t.diagonal().copy_((torch.arange(n, device="cuda") % 3 - 0.5).double())
+    u = torch.empty_like(t)
+    p.sign(t, p.Variant.PH_FP64, out=u)
+    torch.cuda.synchronize()
+    took = []
+
+    def solve():
+        with torch.cuda.device(0):
+            for _ in range(8):
+                t0 = time.perf_counter()
+                p.sign(t, p.Variant.PH_FP64, out=u)
+                took.append(time.perf_counter() - t0)
+    th = threading.Thread(target=solve)
+    th.start()
+    longest = 0.0
+    while th.is_alive():
+        t0 = time.perf_counter()
+        p.signtri_workspace_bytes(64, p.Variant.PH_FP64)
+        longest = max(longest, time.perf_counter() - t0)
+        time.sleep(0.001)
+    th.join()
+    assert longest < 0.5 * min(took), (longest, took)
