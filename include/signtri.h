@@ -57,11 +57,11 @@ typedef enum {
        SIGNTRI_PH_FP64_EFFICIENT.  From n = 1600 on with leaves of 16 the sums
        between superblocks of 128 run on the tensor cores, exact but for
        rounding their operands to 62 bits (61 above n = 32768) below a
-       power-of-two scale per row or column.  Where that costs a sum more than
-       half a unit in its last place (in a quarter of the entries of any
-       16 x 16 block: rows or columns graded by more than about 2^5, in
-       whatever order), and for non-finite entries of T or U, the float64 sums
-       alone run. */
+       power-of-two scale per row or column (U's with two bits of headroom).
+       Where that costs a sum more than half a unit in its last place (in a
+       quarter of the entries of any 16 x 16 block: rows or columns graded by
+       more than about 2^5, in whatever order), and for non-finite entries of T
+       or U, the float64 sums alone run. */
     SIGNTRI_PH_FP64 = 1,
     /* Parlett-Sylvester for the sign function (Section 2, Section 3,
        Section 5.1): reorder by sign with adjacent Givens swaps, solve
@@ -340,8 +340,8 @@ size_t signtri_complex_workspace_bytes(int n);
    up to ten bulges at a time and a cluster barrier per step of them all;
    the logged rotations reach the rest of T and Q on a second stream, which
    the call creates and destroys, while the next sweeps run.  The sweeps are
-   a serial chain: on one GB300, sign(A) by this route takes 28 ms at n = 200
-   and 1.04 s at n = 1000.  signtri_sign_general: S = sign(A) for real A, real
+   a serial chain: on one GB300, sign(A) by this route takes 29 ms at n = 200
+   and 1.1 s at n = 1000.  signtri_sign_general: S = sign(A) for real A, real
    n x n (device, column-major): signtri_schur, the complex sign of T
    (signtri_sign_tri_complex), Q U Q^H (as signtri_sign_schur_complex), and
    the real part (A real makes sign(A) real; the imaginary part left is

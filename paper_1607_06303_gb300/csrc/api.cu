@@ -146,9 +146,9 @@ signtri_status get_workspace(DeviceState &s, size_t need, Arena &a, bool optiona
 
 // Leaf size of the float64 forms when none is set.  16 runs one launch per
 // anti-diagonal (ph_level.cuh) and is the fastest measured on GB300 at every
-// size: the efficient form takes 0.22 / 1.0 / 5.0 / 32 / 262 ms at n = 256 /
-// 1001 / 2000 / 4000 / 8192 with leaves of 16, against 1.2 / 5.6 / 14.5 / 51 /
-// 312 ms with 32 and 2.0 / 8.6 / 22 / 65 / 309 ms with 64 (p = 0.3 random).
+// size: by float64 sums alone 0.22 / 1.06 / 5.1 / 33 / 260 ms at n = 256 / 1001 /
+// 2000 / 4000 / 8192, against 1.25 / 5.7 / 14.6 / 51 / 311 ms with 32 and 2.0 /
+// 8.6 / 22 / 64 / 310 ms with 64 (p = 0.3 random).
 constexpr int kDefaultCutoff = 16;
 
 // the leaf size a float64 form runs with (callers hold g_mu)
@@ -158,9 +158,9 @@ int current_cutoff_locked()
 }
 
 // From this order on the float64 Parlett-Higham forms with leaves of 16 run
-// by superblocks with their sums on the tensor cores (ph_super.cu): 2.95 /
-// 4.1 / 11.8 / 40.7 ms at n = 1537 / 2000 / 4096 / 8192, against 2.7 / 5.0 /
-// 32 / 270 ms by float64 sums alone (p = 0.3 random).
+// by superblocks with their sums on the tensor cores (ph_super.cu): 2.6 / 3.5 /
+// 9.8 / 35.5 ms at n = 1600 / 2000 / 4096 / 8192, against 2.9 / 5.1 / 35 / 260
+// ms by float64 sums alone (p = 0.3 random).
 constexpr int kSuperMin = 1600;
 // Their operands take 72 n^2 bytes, 9 times T (4.8 GB at n = 8192, 19.3 at 16384,
 // 77 at 32768), kept with the library's workspace; from kSuperRoom on (n about
@@ -228,15 +228,15 @@ void work_estimates(int n, const ScanResult &r, double *w_ph, double *w_ps)
 // Times predicted from what each variant runs, with constants measured on
 // GB300.  A grouped diagonal (k = 0 swaps) with leaves of 16:
 //  * Parlett-Higham: a launch of 13 us per block column of 16 beside the useful
-//    count at the float64 rate (n = 700: 0.56 ms, 1200: 1.67); by superblocks
+//    count at the float64 rate (n = 700: 0.58 ms, 1200: 1.70); by superblocks
 //    (n >= kSuperMin) per level of 128 0.2 ms of dependent steps and 44 ns a
-//    column of products (n = 2000: 4.1 ms, 4096: 10.8, 8192: 33);
+//    column of products (n = 2000: 3.4 ms, 4096: 9.3, 8192: 33.6);
 //  * Parlett-Sylvester: 0.2 ms per anti-diagonal of 128 x 128 superblocks and
-//    n_- n_+ n flops of products at 2e13 a second (n = 700: 0.9 to 1.0 ms,
-//    2000: 3.0 to 3.2, 8192: 15.0 with 0.1 n negatives and 20.1 with 0.5 n).
+//    n_- n_+ n flops of products at 2e13 a second (n = 700: 0.8 to 1.0 ms,
+//    2000: 2.6 to 2.7, 8192: 12.1 with 0.1 n negatives and 17.4 with 0.5 n).
 // The two meet near n = 1200.  Otherwise the estimates of both by their plain
 // forms, which with a few negatives at large n favour Parlett-Sylvester beyond
-// what the two measure now (n = 8192, three negatives: 41.4 ms against 34.7):
+// what the two measure now (n = 8192, three negatives: 38.2 ms against 35.6):
 //  * Parlett-Higham: the useful count w_ph at the float64 product rate, and one
 //    off-diagonal leaf step per block column (0.06, 0.21, 0.7 ms at b = 16, 32,
 //    64);

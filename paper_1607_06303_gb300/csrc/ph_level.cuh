@@ -26,8 +26,8 @@
 //
 // Inside a leaf one thread owns one entry.  A solved entry is pushed at once
 // into the later entries that need it (one multiply-add for the row, one for
-// the column), so a step's critical path is a product, a barrier and two
-// multiply-adds, whatever the length of the entry's sum; threads are numbered
+// the column), so a step's critical path is three multiply-adds and a barrier,
+// whatever the length of the entry's sum; threads are numbered
 // along the block's anti-diagonals, so whole warps fall idle as the solve
 // proceeds and leave the float64 pipe to the others.
 #pragma once

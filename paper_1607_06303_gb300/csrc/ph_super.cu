@@ -67,15 +67,18 @@ constexpr int kNoExp = INT_MIN / 2;
 constexpr int kHeadroom = 2;
 constexpr int kMinExp = -900;     // keeps 2^(bits - exp) a normal number
 constexpr int kNormBits = 14;     // squared norms count 2^-14
+// A rounded entry is below 2^bits: a 53-bit significand moved up by 10 at most,
+// in a signed 64-bit integer, and five balanced digits of 14 bits.
+static_assert(rns::operand_bits(1) <= 62, "53 + 10 bits with the sign, and 5 x 14 - 1");
 // An entry's E may be 2^slack times 2^-53 of its sum: for X, whose plain path sums
 // in double-float (48 bits), more.
 constexpr int kSylvSlack = 4;
 // Where a level's products are summed ahead, beside the wave before: in runs of
 // kAheadLevels levels with sums or more, beside waves of at most kAheadTiles
 // superblocks.  Wider waves fill the float64 pipes and lose by the company (a
-// batch of 300, hundreds of superblocks a level: 47.7 ms, with every level
-// ahead 49.6); limits of 24, 40 and 128 measured 36.6, 35.4 and 35.4 ms at
-// n = 8192.
+// batch of 300, hundreds of superblocks a level: 44.2 ms, with every level
+// ahead 46.3); limits of 24, 40, 64 and 128 measure 36.6, 36.0, 36.3 and 36.3
+// ms at n = 8192.
 constexpr size_t kAheadTiles = 64;
 constexpr int kAheadLevels = 4;
 // A run of one problem ends kTellLevels levels after a flag was set, where it has
@@ -459,9 +462,9 @@ __device__ __forceinline__ double residue_sum(const Wave &w, const Problem &pr, 
 __host__ __device__ constexpr int wave_blocks(int l) { return l < 0 || l > 2 * SB - 2 ? 0 : (l < SB ? l + 1 : 2 * SB - 1 - l); }
 // Their sums over finished blocks more than one away are cut in two, each as
 // long as a leaf or shorter and fewer CTAs to share the SMs with the leaves (one,
-// two, three, four: Sylvester equation of a sorted diagonal, n = 8192, 16.1, 15.1,
-// 15.9, 16.8 ms; sign(T) n = 2000 3.72, 3.54, 3.68, 3.82, n = 8192 35.7, 33.4,
-// 33.0, 33.0; batch of 300 43.2, 42.6, 43.0, 43.3).
+// two, three, four: Sylvester equation of a sorted diagonal, n = 8192, 16.1, 14.9,
+// 16.0, 16.8 ms; Schur pair n = 2000 4.80, 4.58, 4.77, 4.92; sign(T) n = 8192 38.1,
+// 36.3, 36.3, 36.3; batch of 300 44.6, 44.2, 44.8, 45.3).
 constexpr int kParts = 2;
 
 struct WaveBlock {
@@ -688,9 +691,8 @@ wave_kernel(const __grid_constant__ Wave w, int l, bool first, const double *in,
 // scheduler puts four on an SM and leaves others empty, and a leaf that shares its
 // float64 pipe waits for it); 66 KB at two an SM leaves one beside the residue
 // products' CTA.  Measured with none / this, ms: Sylvester equation of a sorted
-// diagonal, n = 8192, 17.6 / 15.9; sign(T) n = 2000 3.91 / 3.68, 4096 10.1 / 9.7,
-// 8192 33.4 / 33.1 (with three parts, kParts); four an SM (G up to 608) no better
-// than none.
+// diagonal, n = 8192, 17.1 / 14.9; Schur pair n = 2000 4.85 / 4.58; sign(T)
+// n = 8192 36.2 / 36.3; four an SM (G up to 608) no better than none.
 int wave_spread(int G)
 {
     const int per = (G + lvl::kSms - 1) / lvl::kSms;
@@ -869,7 +871,7 @@ struct Run {
         // float64 chains: so, beside a level's wave, the next level's products
         // sum on a second stream what that wave does not change, and only the
         // K-blocks of two superblocks are left between the waves (n = 8192:
-        // 38.6 -> 35.4 ms; Sylvester equation of a sorted diagonal 21.1 -> 18.5).
+        // 37.9 -> 36.3 ms; Sylvester equation of a sorted diagonal 17.8 -> 14.9).
         CallStream side;
         bool summed_ahead = false;
         const bool overlap = levels - sums_from >= kAheadLevels;

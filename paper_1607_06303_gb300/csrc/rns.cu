@@ -36,8 +36,8 @@ constexpr int kStageBytes = 32768;
 constexpr int kThreads = 320;   // and at most 102 registers each: room for two CTAs of the waves beside it
 constexpr int kBufs = 4;
 // CTAs of an early launch, which runs beside another kernel: half the SMs keep
-// up with memory (n = 8192 in all: 152 CTAs 40.9 ms, 100 36.7, 84 36.2, 76 35.4,
-// 64 35.6, 48 40.0)
+// up with memory (n = 8192 in all: 152 CTAs 40.2 ms, 100 37.4, 84 37.1, 76 36.3,
+// 64 37.5, 48 43.8)
 constexpr int kEarlyCtas = 76;
 constexpr int kChunkKb = 15;    // 960 products of residues of at most 129: below 2^24
 constexpr int kSmemBytes = kStages * kStageBytes + 1024 + 256;
