@@ -335,18 +335,21 @@ __device__ __forceinline__ void entry_of(int t, int &p, int &q)
 // 9.2e-17, now 6.2e-17.)  Complex entries, whose products are separate
 // instructions, add `outside` to the block's sum, so that only one addition
 // rounds by the entry's own size.
+// general: the entry is a divided difference, whose own term the sums nearly cancel
+// where eigenvalues are close: `outside` holds that term too, everything is one
+// sum, and the quotient is taken of what is left.
 // scaled: a warp with a divisor that is (dv.ex; else dv.ex is not looked at).  A
 // warp's entries have up to five steps: before and after these it forms none
 // (formed under a condition of the lane alone, the quotient's multiply-add is
 // issued by every warp at every step: 15 % of the leaf's float64 instructions).
-template <bool kScaled, class S>
+template <bool general, bool kScaled, class S>
 __device__ __forceinline__ void solve_steps(S outside, S quot, const Divisor<S> &dv, unsigned long long flip,
                                             const S *M, const S *N, S *V, int p, int q, int step)
 {
-    constexpr bool kComplex = sizeof(S) == 16;
+    constexpr bool kComplex = sizeof(S) == 16 && !general;
     auto by_d = [&](S x, S base) { return kScaled ? add_quotient(x, dv, base) : mac_once(x, dv.r, base); };
-    if (!kComplex) quot = by_d(outside, quot);
-    S acc = real_value<S>(0.0);
+    S acc = general ? outside : real_value<S>(0.0);
+    if (!general && !kComplex) quot = by_d(outside, quot);
     auto take = [&](int st) {
         const int k1 = LB - 1 + q - st;   // solved at this step in the entry's column ...
         const int k2 = st - (LB - 1) + p;   // ... and in its row
@@ -368,12 +371,12 @@ __device__ __forceinline__ void solve_steps(S outside, S quot, const Divisor<S> 
     }
     for (; st < 2 * LB - 1; st++) half_sync(0);
 }
-template <class S>
+template <bool general, class S>
 __device__ __forceinline__ void solve16(S outside, S quot, const Divisor<S> &dv, bool scaled, unsigned long long flip,
                                         const S *M, const S *N, S *V, int p, int q, int step)
 {
-    if (!scaled) solve_steps<false>(outside, quot, dv, flip, M, N, V, p, q, step);
-    else solve_steps<true>(outside, quot, dv, flip, M, N, V, p, q, step);
+    if (!scaled) solve_steps<general, false>(outside, quot, dv, flip, M, N, V, p, q, step);
+    else solve_steps<general, true>(outside, quot, dv, flip, M, N, V, p, q, step);
 }
 
 // Leaf of block (I, J): nslab partial slabs from slab0 on, LT doubles each.
@@ -429,7 +432,7 @@ __device__ __forceinline__ void leaf(int n, const S *__restrict__ T, int ldt, S 
     const bool o = general || signs_differ(ui, uj);
     s.V[at] = o ? scaled(tij, ui - uj) : zero;
     half_sync(0);
-    const S quot = opp ? quotient(s.V[p + q * LD], dif, dv) : zero;
+    const S base = s.V[p + q * LD], quot = !general && opp ? quotient(base, dif, dv) : zero;
     const bool far = __any_sync(0xffffffffu, dv.ex != 0);
 
     dependency_wait();
@@ -480,7 +483,8 @@ __device__ __forceinline__ void leaf(int n, const S *__restrict__ T, int ldt, S 
         if (both) col = add(col, row);
         acc = add(acc, col);
     }
-    solve16(acc, quot, dv, far, flip, M, N, s.V, p, q, step);
+    if (general) acc = add(acc, base);
+    solve16<general>(acc, quot, dv, far, flip, M, N, s.V, p, q, step);
     if (in) SGT_AT(U, ldu, r0 + lo, c0 + hi) = s.V[at];
 }
 

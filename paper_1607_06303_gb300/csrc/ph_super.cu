@@ -653,7 +653,7 @@ __device__ __forceinline__ void wave_leaf(const Wave &wv, int b, int l, bool fir
         for (int i = 0; i < LB; i++) acc = fma(lvl::flip_sign(s.X2[p + i * LD], flip), N2[i + q * LD], acc);
     }
     if (far && opp && live) dv.ex = divisor_shift(exponent_field(s.TI[p + p * LD] - s.TJ[q + q * LD]));
-    lvl::solve16(s.C[p + q * LD] + acc, quot, dv, far, flip, M, N, s.V, p, q, step);
+    lvl::solve16<false>(s.C[p + q * LD] + acc, quot, dv, far, flip, M, N, s.V, p, q, step);
     const double x = in ? s.V[at] : 0.0;
     if (in) SGT_AT(w.V, w.ldv, r0 + lo, c0 + hi) = x;
     // a warp holds 16 rows of two columns
